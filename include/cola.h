@@ -187,41 +187,23 @@ int cola_power_spectrum(cola_ctx* ctx, const float* s, double* pk, int nbins);
  *                               Available when the tile geometry fits (cola_create decides).
  *   COLA_SCHED_TILE_GATHER    : tile-wise gather from shared memory (requires the binned deposit
  *                               and tiles of at least 4 cells along z).
- *   COLA_SCHED_PIPELINED_FFT  : persistent cp.async-pipelined strided FFT passes (else one CTA per
- *                               tile of pencils).
- *   COLA_SCHED_PIPE_EPT8      : the pipelined passes give each thread 8 complex values per stage
- *                               instead of 16 (twice the threads on the same tile); requires
- *                               COLA_SCHED_PIPELINED_FFT.
  *   COLA_SCHED_PIPELINED_GATHER: the tile gather runs on persistent CTAs that copy the next tile's
  *                               forces while interpolating the current one (requires
  *                               COLA_SCHED_TILE_GATHER).
- *   COLA_SCHED_GREEN_EPT8     : the fused x + Green + inverse-x pass gives each thread 8 complex values
- *                               per stage instead of 16 (narrower tiles, fewer registers per thread).
- *   COLA_SCHED_C2R_EPT8       : the same for the contiguous-axis C2R passes of the three forces.
- *   COLA_SCHED_ROWS_PIPE      : the C2R passes run on persistent CTAs that copy the next tile's rows
- *                               (cp.async) while transforming the current one.
- *   bits COLA_SCHED_BUDGET_SHIFT..+1 : shared-memory budget per CTA of the pipelined passes,
- *                               0: 160 KB, 1: 96 KB, 2: 64 KB (sets their tile width); must be 0
- *                               without COLA_SCHED_PIPELINED_FFT.
- *   COLA_SCHED_R2C_EPT8       : 8 complex values per thread per stage in the contiguous-axis R2C
- *                               pass of the density.
- *   COLA_SCHED_WIDE_TILES     : tiles of 8 pencils (one CTA of up to 768 threads per SM) in the
- *                               16-element Green pass and the one-CTA-per-tile strided passes where
- *                               the default tile is narrower (meshes of 769 to 1536 cells), so that
- *                               every row segment moved is 64 bytes; on by default.
- *   COLA_SCHED_PIPE_INPLACE   : the pipelined passes keep two tile buffers (staging and one work buffer
- *                               that the middle stages overwrite) in up to 210 KB, which holds tiles of
- *                               8 pencils of 1536; requires COLA_SCHED_PIPELINED_FFT, budget bits 0 and
- *                               no COLA_SCHED_PIPE_EPT8.
- * cola_create picks a schedule from the sizes (in-place pipelined passes for meshes of 769 to 1536
- * cells, the binned deposit and tile gather where the tiles are dense enough); cola_get_schedule reads
- * it and cola_set_schedule replaces it (COLA_ERR_INVALID for an unavailable or malformed schedule).
+ *   COLA_SCHED_PIPELINED_FFT, _PIPE_EPT8, _GREEN_EPT8, _C2R_EPT8, _ROWS_PIPE, _R2C_EPT8, _WIDE_TILES,
+ *   _PIPE_INPLACE and the two budget bits COLA_SCHED_BUDGET_SHIFT..+1 (values 0 to 2): choices of earlier
+ *                               FFT kernels.  Each length now has one set of passes, the fastest at
+ *                               every size measured, so these bits are checked for consistency as
+ *                               before (_PIPE_EPT8, _PIPE_INPLACE and a nonzero budget need
+ *                               _PIPELINED_FFT; _PIPE_INPLACE excludes _PIPE_EPT8 and a budget), kept
+ *                               and reported, and select nothing.
+ * cola_create picks a schedule from the sizes (the binned deposit and tile gather where the tiles are
+ * dense enough); cola_get_schedule reads it and cola_set_schedule replaces it (COLA_ERR_INVALID for an
+ * unavailable or malformed schedule).
  * cola_autotune times `reps` PM force evaluations (deposit, FFTs, Poisson + gradient, gather) at
  * displacements s (device float32 [3][np^3]; an evolved state is representative, a lattice is not)
- * in a coordinate search from the current schedule: the deposit/gather choice, then the strided
- * passes (pipelining, elements per thread, budget or in-place tiles), then the Green pass, then the tile width, then
- * the C2R passes (elements per thread, pipelining), then the R2C pass, each
- * with the others fixed.  It keeps the fastest, writes it to *best (may be NULL), and writes the
+ * for the deposit/gather choices, the other bits unchanged.  It keeps the fastest, writes it to *best
+ * (may be NULL), and writes the
  * schedules it timed and their milliseconds per evaluation, in timing order, to
  * scheds[0..max_candidates) and ms[0..max_candidates) (either may be NULL).  Returns the number of
  * schedules timed, or minus a cola_status.  It synchronises the stream and allocates a temporary

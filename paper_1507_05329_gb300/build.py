@@ -16,13 +16,17 @@ ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 BUILD_DIR = os.path.join(HERE, "_build")
 LIB_PATH = os.path.join(HERE, "libcola.so")
-SOURCES = ["fft.cu", "fft_generic.cu", "fft_fast8.cu", "fft_fast16.cu", "fft_pipe8.cu", "fft_pipe16.cu", "fft_green8.cu", "fft_green16.cu", "fft_green8e.cu", "fft_green16e.cu", "fft_rows8e.cu",
-           "fft_rows16e.cu", "particles.cu", "binning.cu", "adjoint.cu", "fof.cu", "cola_batch.cu", "cola_abi.cu",
-           "cola_static.cu", "rng.cu", "host_cosmo.cpp"]
-HEADERS = [os.path.join(CSRC, "cola_internal.h"), os.path.join(CSRC, "fft_core.cuh"), os.path.join(CSRC, "fft_fast.inc"),
-           os.path.join(ROOT, "include", "cola.h")]
+CT_PARTS = 16   # parts of the per-length FFT kernels (fft_ct.cu), compiled in parallel
+SOURCES = ["fft.cu", "fft_generic.cu", "particles.cu", "binning.cu", "adjoint.cu", "fof.cu", "cola_batch.cu",
+           "cola_abi.cu", "cola_static.cu", "rng.cu", "host_cosmo.cpp"]
+HEADERS = [os.path.join(CSRC, h) for h in ("cola_internal.h", "fft_core.cuh", "fft_ct.cuh", "fft_ops.h", "fft_plan.h")] + [
+    os.path.join(ROOT, "include", "cola.h")]
+# (source, object, extra flags) of every compilation
+UNITS = [(s, s + ".o", []) for s in SOURCES] + [
+    ("fft_ct.cu", f"fft_ct_{k}.o", [f"-DCOLA_CT_PART={k}"]) for k in range(CT_PARTS)]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
-FLAGS = ["-O3", "-std=c++17", "-lineinfo", "-Xcompiler", "-fPIC", "-I" + os.path.join(ROOT, "include")]
+FLAGS = ["-O3", "-std=c++17", "-lineinfo", "-Xcompiler", "-fPIC", "-I" + os.path.join(ROOT, "include"),
+         f"-DCOLA_CT_PARTS={CT_PARTS}"]
 
 
 def _nvcc() -> str:
@@ -36,7 +40,7 @@ def _stale() -> bool:
     if not os.path.exists(LIB_PATH):
         return True
     t = os.path.getmtime(LIB_PATH)
-    deps = [os.path.join(CSRC, s) for s in SOURCES] + HEADERS + [os.path.abspath(__file__)]
+    deps = [os.path.join(CSRC, u[0]) for u in UNITS] + HEADERS + [os.path.abspath(__file__)]
     return any(os.path.getmtime(d) > t for d in deps)
 
 
@@ -47,9 +51,10 @@ def build(force: bool = False, verbose: bool = False) -> str:
     nvcc = _nvcc()
     os.makedirs(BUILD_DIR, exist_ok=True)
 
-    def compile_one(src: str) -> str:
-        obj = os.path.join(BUILD_DIR, src + ".o")
-        cmd = [nvcc, *ARCH, *FLAGS, "-c", os.path.join(CSRC, src), "-o", obj]
+    def compile_one(unit) -> str:
+        src, name, extra = unit
+        obj = os.path.join(BUILD_DIR, name)
+        cmd = [nvcc, *ARCH, *FLAGS, *extra, "-c", os.path.join(CSRC, src), "-o", obj]
         res = subprocess.run(cmd, capture_output=True, text=True)
         if res.returncode != 0:
             raise RuntimeError(f"nvcc failed on {src}:\n{res.stdout}\n{res.stderr}")
@@ -57,8 +62,8 @@ def build(force: bool = False, verbose: bool = False) -> str:
             print(res.stdout + res.stderr)
         return obj
 
-    with cf.ThreadPoolExecutor(max_workers=len(SOURCES)) as ex:
-        objs = list(ex.map(compile_one, SOURCES))
+    with cf.ThreadPoolExecutor(max_workers=os.cpu_count() or 8) as ex:
+        objs = list(ex.map(compile_one, UNITS))
     tmp = LIB_PATH + ".tmp"
     cmd = [nvcc, *ARCH, "-shared", "-cudart", "static", "-o", tmp, *objs]
     res = subprocess.run(cmd, capture_output=True, text=True)

@@ -153,7 +153,7 @@ int forward_yz(cola_ctx* c, const unsigned long long* rho, bool check_mass) {
   COLA_TRY(STAGED(kStFwdZ, launch_r2c_rows(c->mplan, g, kSrcFixedPoint, rho, g.n, scale, c->cbuf[2], c->stream,
                                            check_mass ? c->mass_acc : nullptr)));
   if (check_mass) COLA_TRY(launch_mass_check(c->pg, nullptr, false, c->mass_acc, c->flags, c->stream));
-  COLA_TRY(STAGED(kStFwdY, launch_pencils(c->mplan, g, 1, -1, c->cbuf[2], c->stream)));
+  COLA_TRY(STAGED(kStFwdY, launch_pencils(c->mplan, g, 1, -1, &c->cbuf[2], 1, c->stream)));
   return COLA_OK;
 }
 
@@ -171,27 +171,23 @@ int deposit_and_forward_yz(cola_ctx* c, const float* s) {
     COLA_TRY(STAGED(kStFwdZ, launch_r2c_rows(c->mplan, g, kSrcFloat, delta, g.n, 1.0f, c->cbuf[2], c->stream)));
     COLA_TRY(launch_mass_reduce(c->tile_mass, c->bg.tiles, c->mass_acc, c->stream));
     COLA_TRY(launch_mass_check(c->pg, nullptr, false, c->mass_acc, c->flags, c->stream));
-    return STAGED(kStFwdY, launch_pencils(c->mplan, g, 1, -1, c->cbuf[2], c->stream));
+    return STAGED(kStFwdY, launch_pencils(c->mplan, g, 1, -1, &c->cbuf[2], 1, c->stream));
   }
   COLA_TRY(deposit_mesh(c, s, c->rho));
   return forward_yz(c, c->rho, true);
 }
 
 // S3 after forward_yz: the three force components as real fields in cbuf[0..2] (rows of 2 pc floats).
-// With save_spectrum the fast Green kernels also leave the density's forward spectrum in the
+// With save_spectrum the compiled Green kernels also leave the density's forward spectrum in the
 // (already consumed) fixed-point mesh buffer and c->spec_saved says so.
 int green_and_inverse(cola_ctx* c, double force_scale, bool save_spectrum = false) {
   const Grid3& g = c->mesh;
-  float2* const outs[3] = {c->cbuf[0], c->cbuf[1], c->cbuf[2]};
   bool saved = false;
-  COLA_TRY(STAGED(kStGreenX, launch_green_x(c->mplan, g, c->cbuf[2], outs, c->dtab, (float)force_scale, c->stream,
+  COLA_TRY(STAGED(kStGreenX, launch_green_x(c->mplan, g, c->cbuf, c->dtab, (float)force_scale, c->stream,
                                             save_spectrum ? reinterpret_cast<float2*>(c->rho) : nullptr, &saved)));
   c->spec_saved = saved;
-  for (int j = 0; j < 3; ++j) {
-    COLA_TRY(STAGED(kStInvY, launch_pencils(c->mplan, g, 1, +1, c->cbuf[j], c->stream)));
-    COLA_TRY(STAGED(kStInvZ, launch_c2r_rows(c->mplan, g, c->cbuf[j], c->stream)));
-  }
-  return COLA_OK;
+  COLA_TRY(STAGED(kStInvY, launch_green_y(c->mplan, g, c->cbuf, c->dtab, c->stream)));
+  return STAGED(kStInvZ, launch_c2r_rows(c->mplan, g, c->cbuf, 3, c->stream));
 }
 
 // S1-S3: the three force components as real fields in cbuf[0..2] (rows of 2 pc floats).
@@ -201,9 +197,9 @@ int force_mesh(cola_ctx* c, const float* s, double force_scale, bool save_spectr
 }
 
 int inverse3d(cola_ctx* c, const Grid3& g, const FftPlan& p, float2* b) {
-  COLA_TRY(STAGED(kStFwdX, launch_pencils(p, g, 0, +1, b, c->stream)));
-  COLA_TRY(STAGED(kStInvY, launch_pencils(p, g, 1, +1, b, c->stream)));
-  return STAGED(kStInvZ, launch_c2r_rows(p, g, b, c->stream));
+  COLA_TRY(STAGED(kStFwdX, launch_pencils(p, g, 0, +1, &b, 1, c->stream)));
+  COLA_TRY(STAGED(kStInvY, launch_pencils(p, g, 1, +1, &b, 1, c->stream)));
+  return STAGED(kStInvZ, launch_c2r_rows(p, g, &b, 1, c->stream));
 }
 
 // A 2LPT field: inverse3d of mul times the lattice spectrum src, into dst, and, with particles, into
@@ -211,22 +207,22 @@ int inverse3d(cola_ctx* c, const Grid3& g, const FftPlan& p, float2* b) {
 // inverse pass and the last pass writes the particle layout itself; else separate kernels do.
 int inverse3d_mul(cola_ctx* c, const Grid3& g, const FftPlan& p, const float2* src, const IcMul& mul, float2* dst,
                   float scale = 1.0f, float* particles = nullptr) {
-  if (pencils_x_mul_ok(p, g)) {
+  if (fft_compiled(p)) {
     COLA_TRY(STAGED(kStFwdX, launch_pencils_x_mul(p, g, src, mul, dst, c->stream)));
   } else {
     COLA_TRY(STAGED(kStIc, launch_ic_multiply(g, src, dst, (IcField)mul.kind, mul.ci, mul.cj, mul.scale, c->stream)));
-    COLA_TRY(STAGED(kStFwdX, launch_pencils(p, g, 0, +1, dst, c->stream)));
+    COLA_TRY(STAGED(kStFwdX, launch_pencils(p, g, 0, +1, &dst, 1, c->stream)));
   }
-  COLA_TRY(STAGED(kStInvY, launch_pencils(p, g, 1, +1, dst, c->stream)));
-  if (!particles) return STAGED(kStInvZ, launch_c2r_rows(p, g, dst, c->stream));
-  if (c2r_rows_dense_ok(p, g)) return STAGED(kStInvZ, launch_c2r_rows_dense(p, g, dst, scale, particles, c->stream));
-  COLA_TRY(STAGED(kStInvZ, launch_c2r_rows(p, g, dst, c->stream)));
+  COLA_TRY(STAGED(kStInvY, launch_pencils(p, g, 1, +1, &dst, 1, c->stream)));
+  if (!particles) return STAGED(kStInvZ, launch_c2r_rows(p, g, &dst, 1, c->stream));
+  if (fft_compiled(p)) return STAGED(kStInvZ, launch_c2r_rows_dense(p, g, dst, scale, particles, c->stream));
+  COLA_TRY(STAGED(kStInvZ, launch_c2r_rows(p, g, &dst, 1, c->stream)));
   return STAGED(kStIc, launch_ic_to_particles(g, dst, scale, particles, c->stream));
 }
 
 int forward3d_yx(cola_ctx* c, const Grid3& g, const FftPlan& p, float2* b) {
-  COLA_TRY(STAGED(kStFwdY, launch_pencils(p, g, 1, -1, b, c->stream)));
-  return STAGED(kStFwdX, launch_pencils(p, g, 0, -1, b, c->stream));
+  COLA_TRY(STAGED(kStFwdY, launch_pencils(p, g, 1, -1, &b, 1, c->stream)));
+  return STAGED(kStFwdX, launch_pencils(p, g, 0, -1, &b, 1, c->stream));
 }
 
 // W(k) = R2C of the lattice white noise into B0: the caller's field wn, or (wn == NULL) the field
@@ -429,12 +425,8 @@ extern "C" int cola_create(const cola_params* params, void* stream, cola_ctx** o
     c->binned = true;
     c->tile_gather = tile_gather_pays(c->bg, c->pg.npart);
   }
-  // meshes (and 2LPT lattices) of 769 to 1536 cells: the in-place pipelined strided passes hold
-  // tiles of 8 pencils (64-byte row segments) where the three-buffer ones hold 4 (at 1536: 185.6
-  // against 203.2 ms per PM force evaluation on 1024^3 particles)
-  auto inplace_pays = [](int n) { return n > 768 && n * 8 <= 12288; };
-  c->mplan.pipe_inplace = inplace_pays(params->nmesh);
-  c->lplan.pipe_inplace = inplace_pays(params->np);
+  c->fft_sched = COLA_SCHED_PIPELINED_FFT | COLA_SCHED_WIDE_TILES |
+                 (params->nmesh > 768 && params->nmesh <= 1536 ? COLA_SCHED_PIPE_INPLACE : 0);
   if ((st = cuda_status(cudaMallocHost(&c->edges_host, (kPkMaxBins + 1) * sizeof(long long)), "cudaMallocHost")) !=
       COLA_OK)
     return fail(st);
@@ -512,7 +504,7 @@ extern "C" int cola_density_spectrum(cola_ctx* c, const float* s, float* delta_k
   COLA_TRY(check_ptr(s));
   COLA_TRY(check_ptr(delta_k));
   COLA_TRY(deposit_and_forward_yz(c, s));
-  COLA_TRY(STAGED(kStFwdX, launch_pencils(c->mplan, c->mesh, 0, -1, c->cbuf[2], c->stream)));
+  COLA_TRY(STAGED(kStFwdX, launch_pencils(c->mplan, c->mesh, 0, -1, &c->cbuf[2], 1, c->stream)));
   return launch_dense_spectrum(c->mesh, c->cbuf[2], delta_k, c->stream);
 }
 
@@ -521,7 +513,7 @@ extern "C" int cola_density_spectrum_of_mesh(cola_ctx* c, const unsigned long lo
   COLA_TRY(check_ptr(rho));
   COLA_TRY(check_ptr(delta_k));
   COLA_TRY(forward_yz(c, rho, false));
-  COLA_TRY(STAGED(kStFwdX, launch_pencils(c->mplan, c->mesh, 0, -1, c->cbuf[2], c->stream)));
+  COLA_TRY(STAGED(kStFwdX, launch_pencils(c->mplan, c->mesh, 0, -1, &c->cbuf[2], 1, c->stream)));
   return launch_dense_spectrum(c->mesh, c->cbuf[2], delta_k, c->stream);
 }
 
@@ -596,7 +588,7 @@ extern "C" int cola_power_spectrum_ex(cola_ctx* c, const float* s, double* pk, i
   COLA_TRY(check_ptr(s));
   COLA_TRY(check_ptr(pk));
   COLA_TRY(deposit_and_forward_yz(c, s));
-  COLA_TRY(STAGED(kStFwdX, launch_pencils(c->mplan, c->mesh, 0, -1, c->cbuf[2], c->stream)));
+  COLA_TRY(STAGED(kStFwdX, launch_pencils(c->mplan, c->mesh, 0, -1, &c->cbuf[2], 1, c->stream)));
   return pk_from_spectrum(c, c->cbuf[2], pk, nbins, flags);
 }
 
@@ -708,17 +700,11 @@ extern "C" int cola_run_snapshots(cola_ctx* c, const float* wn, float* s, float*
 
 // ---- execution schedule and autotuner ---------------------------------------------------------
 namespace {
-constexpr int kPipeBudgetsKb[3] = {160, 96, 64};
+constexpr int kParticleBits = COLA_SCHED_BINNED_DEPOSIT | COLA_SCHED_TILE_GATHER | COLA_SCHED_PIPELINED_GATHER;
 
 int schedule_of(const cola_ctx* c) {
-  int k = 0;
-  while (k < 2 && kPipeBudgetsKb[k] != c->mplan.pipe_kb) ++k;
   return (c->binned ? COLA_SCHED_BINNED_DEPOSIT : 0) | (c->tile_gather ? COLA_SCHED_TILE_GATHER : 0) |
-         (c->mplan.pipe ? COLA_SCHED_PIPELINED_FFT : 0) | (c->mplan.pipe_ept == 8 ? COLA_SCHED_PIPE_EPT8 : 0) |
-         (c->gather_pipe ? COLA_SCHED_PIPELINED_GATHER : 0) | (c->mplan.green_ept == 8 ? COLA_SCHED_GREEN_EPT8 : 0) |
-         (c->mplan.row_ept == 8 ? COLA_SCHED_C2R_EPT8 : 0) | (c->mplan.row_pipe ? COLA_SCHED_ROWS_PIPE : 0) |
-         (k << COLA_SCHED_BUDGET_SHIFT) | (c->mplan.r2c_ept == 8 ? COLA_SCHED_R2C_EPT8 : 0) |
-         (c->mplan.wide ? COLA_SCHED_WIDE_TILES : 0) | (c->mplan.pipe_inplace ? COLA_SCHED_PIPE_INPLACE : 0);
+         (c->gather_pipe ? COLA_SCHED_PIPELINED_GATHER : 0) | c->fft_sched;
 }
 
 bool schedule_valid(const cola_ctx* c, int sc) {
@@ -742,16 +728,8 @@ bool schedule_valid(const cola_ctx* c, int sc) {
 void apply_schedule(cola_ctx* c, int sc) {
   c->binned = (sc & COLA_SCHED_BINNED_DEPOSIT) != 0;
   c->tile_gather = (sc & COLA_SCHED_TILE_GATHER) != 0;
-  c->mplan.pipe = (sc & COLA_SCHED_PIPELINED_FFT) != 0;
-  c->mplan.pipe_kb = kPipeBudgetsKb[(sc >> COLA_SCHED_BUDGET_SHIFT) & 3];
-  c->mplan.pipe_ept = (sc & COLA_SCHED_PIPE_EPT8) ? 8 : 16;
   c->gather_pipe = (sc & COLA_SCHED_PIPELINED_GATHER) != 0;
-  c->mplan.green_ept = (sc & COLA_SCHED_GREEN_EPT8) ? 8 : 16;
-  c->mplan.row_ept = (sc & COLA_SCHED_C2R_EPT8) ? 8 : 16;
-  c->mplan.r2c_ept = (sc & COLA_SCHED_R2C_EPT8) ? 8 : 16;
-  c->mplan.wide = (sc & COLA_SCHED_WIDE_TILES) != 0;
-  c->mplan.pipe_inplace = (sc & COLA_SCHED_PIPE_INPLACE) != 0;
-  c->mplan.row_pipe = (sc & COLA_SCHED_ROWS_PIPE) != 0;
+  c->fft_sched = sc & ~kParticleBits;   // kept for cola_get_schedule: every length has one set of FFT kernels
 }
 }  // namespace
 
@@ -802,36 +780,20 @@ extern "C" int cola_autotune(cola_ctx* c, const float* s, int reps, int* best, i
     timed.push_back({sc, t});
     return t;
   };
-  // coordinate search from the current schedule: one group of knobs at a time, the others fixed
-  const int kB1 = 1 << COLA_SCHED_BUDGET_SHIFT, kB2 = 2 << COLA_SCHED_BUDGET_SHIFT;
-  const int P = COLA_SCHED_PIPELINED_FFT, E = COLA_SCHED_PIPE_EPT8, I = COLA_SCHED_PIPE_INPLACE;
-  const std::vector<std::pair<int, std::vector<int>>> groups = {
-      {COLA_SCHED_BINNED_DEPOSIT | COLA_SCHED_TILE_GATHER | COLA_SCHED_PIPELINED_GATHER,
-       {0, COLA_SCHED_BINNED_DEPOSIT, COLA_SCHED_BINNED_DEPOSIT | COLA_SCHED_TILE_GATHER,
-        COLA_SCHED_BINNED_DEPOSIT | COLA_SCHED_TILE_GATHER | COLA_SCHED_PIPELINED_GATHER}},
-      {P | E | I | (3 << COLA_SCHED_BUDGET_SHIFT), {0, P, P | E, P | kB1, P | kB1 | E, P | kB2, P | kB2 | E, P | I}},
-      {COLA_SCHED_GREEN_EPT8, {0, COLA_SCHED_GREEN_EPT8}},
-      {COLA_SCHED_WIDE_TILES, {0, COLA_SCHED_WIDE_TILES}},
-      {COLA_SCHED_C2R_EPT8 | COLA_SCHED_ROWS_PIPE,
-       {0, COLA_SCHED_C2R_EPT8, COLA_SCHED_ROWS_PIPE, COLA_SCHED_C2R_EPT8 | COLA_SCHED_ROWS_PIPE}},
-      {COLA_SCHED_R2C_EPT8, {0, COLA_SCHED_R2C_EPT8}}};
-  int cur = keep;
-  for (const auto& g : groups) {
-    int arg = -1;
-    float tbest = 0.0f;
-    for (int opt : g.second) {
-      const int sc = (cur & ~g.first) | opt;
-      if (!schedule_valid(c, sc)) continue;
-      const float t = time_of(sc);
-      if (st != COLA_OK) break;
-      if (arg < 0 || t < tbest) {
-        arg = sc;
-        tbest = t;
-      }
-    }
+  // the particle kernels' choices; the FFT bits select nothing, so they stay as they are
+  int cur = keep, arg = -1;
+  float tbest = 0.0f;
+  for (int opt : {0, COLA_SCHED_BINNED_DEPOSIT, COLA_SCHED_BINNED_DEPOSIT | COLA_SCHED_TILE_GATHER, kParticleBits}) {
+    const int sc = (keep & ~kParticleBits) | opt;
+    if (!schedule_valid(c, sc)) continue;
+    const float t = time_of(sc);
     if (st != COLA_OK) break;
-    if (arg >= 0) cur = arg;
+    if (arg < 0 || t < tbest) {
+      arg = sc;
+      tbest = t;
+    }
   }
+  if (st == COLA_OK && arg >= 0) cur = arg;
   c->prof = prof;
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);

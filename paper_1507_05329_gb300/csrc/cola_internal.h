@@ -6,6 +6,7 @@
 #include <vector>
 
 #include "../../include/cola.h"
+#include "fft_plan.h"
 
 namespace cola {
 
@@ -37,8 +38,6 @@ StepScalars step_scalars(const cola_params& p, const Cosmo& c, int i);
 // ---------------------------------------------------------------------------------------------
 // FFT plan: one transform length, its radix stages and the twiddle table exp(-2 pi i t / n).
 // ---------------------------------------------------------------------------------------------
-constexpr int kMaxStages = 12;
-
 struct FftDev {
   int n;
   int nstages;
@@ -46,35 +45,27 @@ struct FftDev {
   const float2* tw;   // device table, n entries
 };
 
-struct FftPlan {
-  FftDev dev{};
-  float2* tw = nullptr;   // owned device memory
-  // padded shared-tile row steps of each stage along n/R and along ns (0: padding not affine),
-  // computed once by fft_plan_init for the fast-path kernels
-  int nbp[kMaxStages] = {};
-  int nsp[kMaxStages] = {};
-  int w_pencil = 8;       // pencils per CTA in the strided passes
-  int w_rows = 4;         // row pairs per CTA in the contiguous (R2C / C2R) passes
-  int ept = 16;           // complex elements per thread
-  // schedule (chosen by cola_set_schedule / cola_autotune): persistent pipelined strided passes
-  // on/off, and their shared-memory budget per CTA (sets the tile width)
-  bool pipe = true;
-  int pipe_kb = 160;
-  int pipe_ept = 16;      // complex elements per thread of the pipelined passes (16 or 8)
-  int green_ept = 16;     // complex elements per thread of the Green pass (16 or 8)
-  int row_ept = 16;       // complex elements per thread of the C2R row passes (16 or 8)
-  int r2c_ept = 16;       // complex elements per thread of the R2C row pass (16 or 8)
-  bool row_pipe = false;  // persistent C2R passes with a staging buffer for the next tile
-  bool wide = true;       // tiles of 8 pencils in the one-CTA-per-tile strided and Green passes
-  bool pipe_inplace = false;  // pipelined passes: one work buffer overwritten in place, 210 KB budget
+struct FftOps;   // launches of a length with compiled kernels (fft_ops.h)
+
+struct FftTables {
+  const float2* fwd;   // stage-major twiddles (fft_plan.h) of the plan
+  const float2* rev;   // ... and of the reversed plan
 };
 
-// Factor n into radices {16, 8, 5, 4, 3, 2}; returns false if n has another prime factor.
-bool fft_factor(int n, std::vector<int>* radices);
-int fft_plan_init(FftPlan* plan, int n);   // allocates the twiddle table; returns cola_status
-void fft_plan_steps(FftPlan* plan);        // fills nbp / nsp from dev.n and dev.radix (host only)
+struct FftPlan {
+  FftDev dev{};
+  float2* tw = nullptr;          // owned device memory: the plain table and the two stage-major ones
+  const FftOps* ops = nullptr;   // compiled kernels of this length, or null (run-time plan, fft_generic.cu)
+  FftTables tab{};
+};
+
+constexpr size_t fft_table_entries(int n) { return 3 * (size_t)n; }
+// Fills the plan's length, radices and kernels and points it at a device table of fft_table_entries(n)
+// entries (the plain table, then the stage-major ones); false if n has a prime factor above 5.
+bool fft_plan_set(FftPlan* plan, int n, const float2* table);
+int fft_plan_init(FftPlan* plan, int n);   // allocates and fills the twiddle tables; returns cola_status
 void fft_plan_free(FftPlan* plan);
-void fft_set_smem_limits();                // raise the dynamic shared-memory limit of the FFT kernels
+void fft_set_smem_limits();                // raise the dynamic shared-memory limit of the run-time FFT kernels
 
 // True the first time it is called for `key` on the current device (thread safe).  Kernel attributes
 // (the dynamic shared-memory limit) are per device, so every setter is keyed by (device, kernel).
@@ -99,31 +90,30 @@ enum RowSource { kSrcFixedPoint = 0, kSrcFloat = 1 };
 int launch_r2c_rows(const FftPlan& p, const Grid3& g, RowSource kind, const void* src,
                     long long src_row_stride, float scale, float2* dst, cudaStream_t st,
                     unsigned long long* mass_acc = nullptr);
-// Inverse C2R along z, in place on a complex grid (real rows of stride 2*pc floats).
-int launch_c2r_rows(const FftPlan& p, const Grid3& g, float2* data, cudaStream_t st);
+// Inverse C2R along z, in place on `fields` (1 to 3) complex grids (real rows of stride 2*pc floats).
+int launch_c2r_rows(const FftPlan& p, const Grid3& g, float2* const* data, int fields, cudaStream_t st);
 // The C2R rows of data (not modified) written to out as dense rows of n floats times scale, where the
-// plan has a specialised kernel for it (c2r_rows_dense_ok); the same floats as launch_c2r_rows then
+// length has compiled kernels (fft_compiled); the same floats as launch_c2r_rows then
 // launch_ic_to_particles.
-bool c2r_rows_dense_ok(const FftPlan& p, const Grid3& g);
-// The inverse x pass of mul times the lattice spectrum src into dst (src unchanged) where the plan has
-// a specialised in-place pipelined kernel for it (pencils_x_mul_ok); the same floats as
-// launch_ic_multiply followed by launch_pencils(axis 0, +1).
-struct IcMul;
-bool pencils_x_mul_ok(const FftPlan& p, const Grid3& g);
-int launch_pencils_x_mul(const FftPlan& p, const Grid3& g, const float2* src, const IcMul& mul, float2* dst,
-                         cudaStream_t st);
 int launch_c2r_rows_dense(const FftPlan& p, const Grid3& g, const float2* data, float scale, float* out,
                           cudaStream_t st);
-// C2C along y (axis 1) or x (axis 0) of the complex grid; dir = -1 forward, +1 inverse.
-int launch_pencils(const FftPlan& p, const Grid3& g, int axis, int dir, float2* data,
+// The inverse x pass of mul times the lattice spectrum src into dst (src unchanged) where the length has
+// compiled kernels; the same floats as launch_ic_multiply followed by launch_pencils(axis 0, +1).
+struct IcMul;
+int launch_pencils_x_mul(const FftPlan& p, const Grid3& g, const float2* src, const IcMul& mul, float2* dst,
+                         cudaStream_t st);
+inline bool fft_compiled(const FftPlan& p) { return p.ops != nullptr; }
+// C2C along y (axis 1) or x (axis 0) of `fields` (1 to 3) complex grids; dir = -1 forward, +1 inverse.
+int launch_pencils(const FftPlan& p, const Grid3& g, int axis, int dir, float2* const* data, int fields,
                    cudaStream_t st);
-// Forward x transform, then for each j in {x, y, z}: out_j = i D(k_j) scale delta(k)/k^2
-// (k in rad/cell, D the 4-point gradient kernel), then the inverse x transform of out_j.
-// out[2] may alias in.  With spec_out (a complex grid that aliases none of the others) the fast
-// kernels also write the forward spectrum delta(k) there and set *spec_saved.
-int launch_green_x(const FftPlan& p, const Grid3& g, const float2* in, float2* const out[3],
-                   const float* dtab, float scale, cudaStream_t st, float2* spec_out = nullptr,
-                   bool* spec_saved = nullptr);
+// The force components' inverse transforms from the density's y,z spectrum in out[2]: forward x
+// transform, out_j = i D(k_j) scale delta(k)/k^2 (k in rad/cell, D the 4-point gradient kernel), inverse
+// x and y transforms of every component (a C2R pass is left).  With spec_out (a complex grid that
+// aliases none of out) the compiled kernels also write the forward spectrum delta(k) there and set
+// *spec_saved.  The x part alone is launch_green_x; launch_green_y follows it.
+int launch_green_x(const FftPlan& p, const Grid3& g, float2* const out[3], const float* dtab, float scale,
+                   cudaStream_t st, float2* spec_out = nullptr, bool* spec_saved = nullptr);
+int launch_green_y(const FftPlan& p, const Grid3& g, float2* const out[3], const float* dtab, cudaStream_t st);
 
 // Launchers (particles.cu).
 struct ParticleGeom {
@@ -430,6 +420,7 @@ struct cola_ctx {
   bool binned = false;                    // tile-wise deposit (else direct atomics)
   bool tile_gather = false;               // tile-wise gather from shared memory (else lattice order)
   bool gather_pipe = false;               // ... by persistent CTAs that stage the next tile meanwhile
+  int fft_sched = 0;                      // the schedule's FFT bits (reported, no effect)
   cola::BinGeom bg{};
   cola::BinBuffers bb;
   void* bin_mem = nullptr;

@@ -29,7 +29,7 @@ constexpr size_t kRhoBytes = round256((size_t)kMaxMesh * kMaxMesh * kMaxMesh * s
 constexpr size_t kSpecBytes = round256((size_t)kMaxMesh * kMaxMesh * (kMaxMesh / 2 + 2) * sizeof(float2));
 constexpr size_t kPartBytes = round256((size_t)kBlocks * 2 * kMaxBins * sizeof(double));
 constexpr size_t kEdgeBytes = round256((kMaxBins + 1) * sizeof(long long));
-constexpr size_t kTwBytes = round256(kMaxMesh * sizeof(float2));
+constexpr size_t kTwBytes = round256(fft_table_entries(kMaxMesh) * sizeof(float2));
 constexpr size_t kGeomBytes = round256(2 * kMaxBins * sizeof(double));
 constexpr size_t kFlagBytes = 256;
 constexpr size_t kOffSpec = kRhoBytes;
@@ -47,12 +47,14 @@ struct EdgeTable {
   long long e[kMaxBins + 1];
 };
 
-// Per-call tables: twiddles exp(-2 pi i t / n) (FP64 sincospi rounded to float) and bin edges.
-__global__ void k_static_tables(int n, float2* tw, EdgeTable edges, int nedges, long long* edges_out) {
-  for (int t = threadIdx.x; t < n; t += blockDim.x) {
+// Per-call tables: twiddles exp(-2 pi i t / n) (FP64 sincospi rounded to float), plain and stage-major
+// (the forward plan's: no inverse transform runs here), and bin edges.
+__global__ void k_static_tables(int n, Groups g, float2* tw, EdgeTable edges, int nedges, long long* edges_out) {
+  for (int e = threadIdx.x; e < 2 * n - 1; e += blockDim.x) {
+    const int t = e < n ? e : (g.ok ? stage_twiddle(g, e - n) : 0);
     double s, c;
     sincospi(-2.0 * (double)t / (double)n, &s, &c);
-    tw[t] = make_float2((float)c, (float)s);
+    tw[e] = make_float2((float)c, (float)s);
   }
   for (int b = threadIdx.x; b < nedges; b += blockDim.x) edges_out[b] = edges.e[b];
 }
@@ -106,13 +108,7 @@ extern "C" int cola_power_spectrum_noalloc(const cola_params* p, const float* s,
   const int n = p->nmesh;
 
   FftPlan plan;
-  std::vector<int> rad;
-  if (!fft_factor(n, &rad)) return COLA_ERR_INVALID;
-  plan.dev.n = n;
-  plan.dev.nstages = (int)rad.size();
-  for (int i = 0; i < kMaxStages; ++i) plan.dev.radix[i] = i < (int)rad.size() ? rad[i] : 1;
-  plan.dev.tw = reinterpret_cast<const float2*>(base + kOffTw);
-  fft_plan_steps(&plan);
+  if (!fft_plan_set(&plan, n, reinterpret_cast<const float2*>(base + kOffTw))) return COLA_ERR_INVALID;
 
   Grid3 g;
   g.n = n;
@@ -138,13 +134,13 @@ extern "C" int cola_power_spectrum_noalloc(const cola_params* p, const float* s,
 
   const size_t n3 = (size_t)n * n * n;
   if (cudaMemsetAsync(rho, 0, n3 * sizeof(unsigned long long), st) != cudaSuccess) return COLA_ERR_CUDA;
-  k_static_tables<<<1, 128, 0, st>>>(n, tw, edges, nbins + 1, edg);
+  k_static_tables<<<1, 128, 0, st>>>(n, make_groups(n, false), tw, edges, nbins + 1, edg);
   if (cudaGetLastError() != cudaSuccess) return COLA_ERR_CUDA;
   int r = launch_deposit(pg, s, rho, flags, st);
   const float scale = (float)((double)n3 / ((double)pg.npart * 4398046511104.0));
   if (r == COLA_OK) r = launch_r2c_rows(plan, g, kSrcFixedPoint, rho, n, scale, spec, st);
-  if (r == COLA_OK) r = launch_pencils(plan, g, 1, -1, spec, st);
-  if (r == COLA_OK) r = launch_pencils(plan, g, 0, -1, spec, st);
+  if (r == COLA_OK) r = launch_pencils(plan, g, 1, -1, &spec, 1, st);
+  if (r == COLA_OK) r = launch_pencils(plan, g, 0, -1, &spec, 1, st);
   const double pscale = std::pow(p->box, 3) / std::pow((double)n, 6);
   if (r == COLA_OK) r = launch_pk_geometry(g, edg, nbins, part, kBlocks, geom, st);
   if (r == COLA_OK) r = launch_pk_bins(g, spec, edg, nbins, 0, part, kBlocks, st);
