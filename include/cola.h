@@ -186,19 +186,17 @@ int cola_power_spectrum(cola_ctx* ctx, const float* s, double* pk, int nbins);
  *                               shared memory (else one global 64-bit atomic per CIC corner).
  *                               Available when the tile geometry fits (cola_create decides).
  *   COLA_SCHED_TILE_GATHER    : tile-wise gather from shared memory (requires the binned deposit
- *                               and tiles of at least 4 cells along z).
- *   COLA_SCHED_PIPELINED_GATHER: the tile gather runs on persistent CTAs that copy the next tile's
- *                               forces while interpolating the current one (requires
- *                               COLA_SCHED_TILE_GATHER).
+ *                               and a mesh side that is a multiple of 4).
  *   COLA_SCHED_PIPELINED_FFT, _PIPE_EPT8, _GREEN_EPT8, _C2R_EPT8, _ROWS_PIPE, _R2C_EPT8, _WIDE_TILES,
- *   _PIPE_INPLACE and the two budget bits COLA_SCHED_BUDGET_SHIFT..+1 (values 0 to 2): choices of earlier
- *                               FFT kernels.  Each length now has one set of passes, the fastest at
- *                               every size measured, so these bits are checked for consistency as
- *                               before (_PIPE_EPT8, _PIPE_INPLACE and a nonzero budget need
- *                               _PIPELINED_FFT; _PIPE_INPLACE excludes _PIPE_EPT8 and a budget), kept
- *                               and reported, and select nothing.
- * cola_create picks a schedule from the sizes (the binned deposit and tile gather where the tiles are
- * dense enough); cola_get_schedule reads it and cola_set_schedule replaces it (COLA_ERR_INVALID for an
+ *   _PIPE_INPLACE, _PIPELINED_GATHER and the two budget bits COLA_SCHED_BUDGET_SHIFT..+1 (values 0 to 2):
+ *                               choices of earlier kernels.  Each length has one set of FFT passes and
+ *                               the tile gather one form, the fastest at every size measured, so these
+ *                               bits are checked for consistency as before (_PIPE_EPT8, _PIPE_INPLACE
+ *                               and a nonzero budget need _PIPELINED_FFT, _PIPELINED_GATHER needs
+ *                               _TILE_GATHER; _PIPE_INPLACE excludes _PIPE_EPT8 and a budget), kept and
+ *                               reported, and select nothing.
+ * cola_create picks a schedule from the sizes (the binned deposit and tile gather where the mesh is too
+ * large for the direct deposit's atomics to stay in L2 and the tiles are dense enough); cola_get_schedule reads it and cola_set_schedule replaces it (COLA_ERR_INVALID for an
  * unavailable or malformed schedule).
  * cola_autotune times `reps` PM force evaluations (deposit, FFTs, Poisson + gradient, gather) at
  * displacements s (device float32 [3][np^3]; an evolved state is representative, a lattice is not)

@@ -22,19 +22,25 @@
 #include "cola_internal.h"
 
 #include <cstdio>
-#include <type_traits>
 
 namespace cola {
 namespace {
 
 constexpr int kThreads = 256;
+// Tiles of T x T x TZ mesh cells.  The last tile of an axis is cut off where the mesh side is no multiple
+// of the tile's, so that every mesh has tiles of the same shape (a 360^3 mesh with tiles of the largest
+// power of two dividing its side, 8 x 8 x 8, took 399 us for the deposit and 161 us for the binning of
+// 180^3 particles).  TZ = 64: a tile's particles come in runs of neighbours along the lattice's z, and a
+// longer tile makes longer runs, so that a warp's 18 particle accesses touch fewer lines and its lanes
+// fewer rows of the staged forces (TZ = 32: gather 616 against 531 us at 256^3/384^3, 5465 against
+// 4730 us at 512^3/768^3, 762 against 630 us at 256^3/512^3).
+constexpr int kLt = 3, kT = 1 << kLt, kLz = 6, kTz = 1 << kLz;
+constexpr int kDepositThreads = 512, kGatherThreads = 512;
 // Deposit accumulator columns of TZ + 1 cells: without the pad every column of a tile started on the
 // same shared-memory bank, and a warp's lanes from two columns with equal z conflicted (24.4 against
 // 26.7 ms at 1024^3/1536^3).
-constexpr int kDepositPad = 1;
-#ifndef COLA_DEPOSIT_MIN_BLOCKS
-#define COLA_DEPOSIT_MIN_BLOCKS 8   // resident deposit CTAs per SM the register budget is sized for
-#endif
+constexpr int kCol = kTz + 1;
+constexpr int kAccWords = kT * kT * kCol;
 
 int check_launch(const char* what) {
   const cudaError_t e = cudaGetLastError();
@@ -56,177 +62,158 @@ __device__ __forceinline__ void unpack_q(unsigned e, int np, int* q, long long* 
   *id = ((long long)q[0] * np + q[1]) * np + q[2];
 }
 
-constexpr int kGatherEnt = 1024;   // entries staged in shared memory per tile (4 KB)
-
-// Exact 64-bit shared-memory add from two native 32-bit atomics (low word with carry out).
-__device__ __forceinline__ void smem_add64(unsigned long long* p, unsigned long long w) {
-  unsigned* h = reinterpret_cast<unsigned*>(p);
-  const unsigned lo = (unsigned)w, hi = (unsigned)(w >> 32);
-  const unsigned old = atomicAdd(h, lo);
-  const unsigned carry = (old + lo) < old ? 1u : 0u;
-  if (hi + carry) atomicAdd(h + 1, hi + carry);
-}
-
 // warp-aggregated increment of counter[key] for the lanes whose key >= 0; returns the lane's slot
-// (old value + rank among equal keys) when want_slot.
-__device__ __forceinline__ unsigned agg_inc(unsigned* counter, int key, bool want_slot) {
+// (old value + rank among equal keys).
+__device__ __forceinline__ unsigned agg_inc(unsigned* counter, int key) {
   const unsigned active = __activemask();
   const unsigned grp = __match_any_sync(active, key);
   const int lane = threadIdx.x & 31;
   const int leader = __ffs(grp) - 1;
   unsigned base = 0;
   if (key >= 0 && lane == leader) base = atomicAdd(counter + key, (unsigned)__popc(grp));
-  if (!want_slot) return 0;
   base = __shfl_sync(grp, base, leader);
   return base + __popc(grp & ((1u << lane) - 1u));
 }
 
-// Bin keys of one particle: primary tile and up to seven spill tiles (-1 = none).  Tile index
-// (bx * nt + by) * nz + bz runs fastest along z.
-// LT, LZ: compile-time log2 of the tile sides (the common 8 x 8 x 32 tiles), or 0 to read them from b.
-template <int LT, int LZ>
-__device__ __forceinline__ void tile_keys(const BinGeom& b, int cx, int cy, int cz, int* k) {
-  const int lt = LT ? LT : b.lt, lz = LZ ? LZ : b.lz;
-  const int bx = cx >> lt, by = cy >> lt, bz = cz >> lz;
-  const int m = (1 << lt) - 1, mz = (1 << lz) - 1;
-  // with a single tile along an axis the cloud wraps inside the tile itself: no spill there
-  const bool sx = b.nt > 1 && (cx & m) == m, sy = b.nt > 1 && (cy & m) == m, sz = b.nz > 1 && (cz & mz) == mz;
-  const int bxs[2] = {bx, bx + 1 == b.nt ? 0 : bx + 1};
-  const int bys[2] = {by, by + 1 == b.nt ? 0 : by + 1};
-  const int bzs[2] = {bz, bz + 1 == b.nz ? 0 : bz + 1};
-#pragma unroll
-  for (int c = 0; c < 8; ++c) {
-    const int dx = c >> 2, dy = (c >> 1) & 1, dz = c & 1;
-    const bool ok = (!dx || sx) && (!dy || sy) && (!dz || sz);
-    k[c] = ok ? (bxs[dx] * b.nt + bys[dy]) * b.nz + bzs[dz] : -1;
-  }
+// A particle's tile: its coordinates and which upper faces of the tile its base cell lies on (1: x,
+// 2: y, 4: z), packed as flags << 25 | bx << 16 | by << 7 | bz (nt <= 512, nz <= 128).  Tile index
+// (bx nt + by) nz + bz runs fastest along z.  With a single tile along an axis the cloud wraps inside
+// the tile itself: no upper face there.
+__device__ __forceinline__ unsigned tile_code(const BinGeom& b, int n, int cx, int cy, int cz) {
+  const unsigned sx = b.nt > 1 && ((cx & (kT - 1)) == kT - 1 || cx == n - 1);
+  const unsigned sy = b.nt > 1 && ((cy & (kT - 1)) == kT - 1 || cy == n - 1);
+  const unsigned sz = b.nz > 1 && ((cz & (kTz - 1)) == kTz - 1 || cz == n - 1);
+  return (sx << 25) | (sy << 26) | (sz << 27) | ((unsigned)(cx >> kLt) << 16) | ((unsigned)(cy >> kLt) << 7) |
+         (unsigned)(cz >> kLz);
+}
+__device__ __forceinline__ unsigned code_flags(unsigned code) { return code >> 25; }
+__device__ __forceinline__ int code_key(const BinGeom& b, unsigned code) {
+  return (int)((((code >> 16) & 511u) * b.nt + ((code >> 7) & 511u)) * b.nz + (code & 127u));
+}
+// Calls f(key) for every other tile the cloud of a particle with upper faces reaches (at most seven):
+// the non-empty subsets of its faces.  One face, the usual case, costs one turn.
+template <class F>
+__device__ __forceinline__ void for_spill_keys(const BinGeom& b, unsigned code, F&& f) {
+  const unsigned flags = code_flags(code);
+  const int bx = (code >> 16) & 511u, by = (code >> 7) & 511u, bz = code & 127u;
+  const int key = (bx * b.nt + by) * b.nz + bz;
+  const int col = b.nt * b.nz;
+  const int dx = bx + 1 == b.nt ? -bx * col : col;
+  const int dy = by + 1 == b.nt ? -by * b.nz : b.nz;
+  const int dz = bz + 1 == b.nz ? -bz : 1;
+  for (unsigned sub = flags; sub; sub = (sub - 1u) & flags)
+    f(key + (sub & 1u ? dx : 0) + (sub & 2u ? dy : 0) + (sub & 4u ? dz : 0));
 }
 
-// Spill keys of a particle from its primary tile key and its three upper-face flags (the keys
-// tile_keys gives, without the particle's position).
-__device__ __forceinline__ void keys_from_record(const BinGeom& b, unsigned key, unsigned flags, int* k) {
-  const int bz = (int)(key % (unsigned)b.nz), bxy = (int)(key / (unsigned)b.nz);
-  const int bx = bxy / b.nt, by = bxy - bx * b.nt;
-  const bool sx = flags & 1u, sy = flags & 2u, sz = flags & 4u;
-  const int bxs[2] = {bx, bx + 1 == b.nt ? 0 : bx + 1};
-  const int bys[2] = {by, by + 1 == b.nt ? 0 : by + 1};
-  const int bzs[2] = {bz, bz + 1 == b.nz ? 0 : bz + 1};
-#pragma unroll
-  for (int c = 0; c < 8; ++c) {
-    const int dx = c >> 2, dy = (c >> 1) & 1, dz = c & 1;
-    const bool ok = (!dx || sx) && (!dy || sy) && (!dz || sz);
-    k[c] = ok ? (bxs[dx] * b.nt + bys[dy]) * b.nz + bzs[dz] : -1;
+// Lattice row r of a walk over all rows (qx, qy), as a block's threads of one threadIdx.y take them: the
+// planes in a scattered order (mul is coprime to np, a step of about 0.38 np), the rows of a plane in
+// order.  Rows in flight together then belong to planes far apart and meet on fewer tile counters, while
+// neighbouring rows still get neighbouring places in a tile's list, which the gather's accesses profit
+// from.  32-bit divisions: 64-bit ones were about a third of both passes' instructions.
+struct RowWalk {
+  unsigned np, mul;
+  __device__ __forceinline__ void at(unsigned r, int* qx, int* qy, long long* row) const {
+    const unsigned p = r / np, y = r - p * np, x = (p * mul) % np;
+    *qx = (int)x;
+    *qy = (int)y;
+    *row = ((long long)x * np + y) * np;
   }
-}
+};
 
 // Count pass: per-tile primary and spill counts; every particle's rank within its primary tile (the
-// aggregated atomic's return) is recorded with its tile key and upper-face flags, so that the scatter
-// pass needs neither the positions nor atomics for the primary entries.
-//   rec[id] = rank << 32 | flags << 26 | key   (key < 2^26 tiles, flags: x, y, z upper face)
-template <int LT, int LZ, bool F32>
-__global__ void __launch_bounds__(kThreads) k_bin_count(ParticleGeom pg, BinGeom b, FixedGeo fg,
+// aggregated atomic's return) is recorded with its tile code, so that the scatter pass needs neither the
+// positions nor atomics for the primary entries: rec[id] = rank << 32 | code.
+// Bound by instruction issue and by the atomics' return trips.
+template <bool F32>
+__global__ void __launch_bounds__(kThreads) k_bin_count(ParticleGeom pg, BinGeom b, FixedGeo fg, RowWalk walk,
                                                         const float* __restrict__ s, unsigned* cnt_p, unsigned* cnt_s,
                                                         unsigned long long* __restrict__ rec) {
   const long long n = pg.npart;
   const int np = pg.np;
-  const long long nrows = (long long)np * np;
-  const int lt = LT ? LT : b.lt, lz = LZ ? LZ : b.lz;
-  const int m = (1 << lt) - 1, mz = (1 << lz) - 1;
-  // the block walks (row, chunk) pairs; the positions of the next pair are loaded before this
-  // pair's atomics, so the two latencies overlap
-  const int nch = (np + (int)blockDim.x - 1) / (int)blockDim.x;
-  long long row = blockIdx.x;
-  int ch = 0;
-  float p0 = 0.f, p1 = 0.f, p2 = 0.f;
-  auto load = [&](long long r, int c, float& a0, float& a1, float& a2) {
-    const int qz = c * (int)blockDim.x + (int)threadIdx.x;
-    if (qz < np) {
-      const long long id = r * np + qz;
-      a0 = __ldg(s + id);
-      a1 = __ldg(s + n + id);
-      a2 = __ldg(s + 2 * n + id);
-    }
-  };
-  if (row < nrows) load(row, 0, p0, p1, p2);
-  while (row < nrows) {
-    long long nrow = row;
-    int nchk = ch + 1;
-    if (nchk == nch) {
-      nchk = 0;
-      nrow += gridDim.x;
-    }
-    float n0 = 0.f, n1 = 0.f, n2 = 0.f;
-    if (nrow < nrows) load(nrow, nchk, n0, n1, n2);
-    const int qx = (int)(row / np), qy = (int)(row - (long long)qx * np);
-    // whole warps walk the row together so that the warp-aggregated atomics see full warps
-    const int qz = ch * (int)blockDim.x + (int)threadIdx.x;
-    const bool live = qz < np;
-    int k[8] = {-1, -1, -1, -1, -1, -1, -1, -1};
-    unsigned flags = 0;
-    if (live) {
-      int cx, cy, cz, f;
-      cell_frac<F32>(qx, p0, fg, &cx, &f);
-      cell_frac<F32>(qy, p1, fg, &cy, &f);
-      cell_frac<F32>(qz, p2, fg, &cz, &f);
-      tile_keys<LT, LZ>(b, cx, cy, cz, k);
-      flags = (b.nt > 1 && (cx & m) == m ? 1u : 0u) | (b.nt > 1 && (cy & m) == m ? 2u : 0u) |
-              (b.nz > 1 && (cz & mz) == mz ? 4u : 0u);
-    }
-    if (__any_sync(__activemask(), live)) {
-      // primary keys are shared by runs of lanes: one aggregated atomic per run
-      const unsigned rank = agg_inc(cnt_p, k[0], true);
-      if (live) rec[row * np + qz] = ((unsigned long long)rank << 32) | ((unsigned long long)flags << 26) | (unsigned)k[0];
-    }
-    // spill keys are sparse: one atomic per entry (its result unused)
+  const unsigned nrows = (unsigned)np * np, step = gridDim.x * blockDim.y;
+  unsigned r = blockIdx.x * blockDim.y + threadIdx.y;
+  int qz = threadIdx.x, qx = 0, qy = 0;
+  long long row = 0;
+  float p[3] = {0.f, 0.f, 0.f};
+  auto load = [&](long long first, int z, float (&v)[3]) {
 #pragma unroll
-    for (int e = 1; e < 8; ++e)
-      if (k[e] >= 0) atomicAdd(cnt_s + k[e], 1u);
-    row = nrow;
-    ch = nchk;
-    p0 = n0;
-    p1 = n1;
-    p2 = n2;
+    for (int a = 0; a < 3; ++a) v[a] = z < np ? __ldg(s + a * n + first + z) : 0.f;
+  };
+  if (r < nrows) {
+    walk.at(r, &qx, &qy, &row);
+    load(row, qz, p);
+  }
+  while (r < nrows) {
+    // the next positions are loaded before this chunk's atomics, so the two latencies overlap; whole
+    // warps walk the row together so that the warp-aggregated atomics see full warps
+    unsigned rn = r;
+    int zn = qz + (int)blockDim.x, qxn = qx, qyn = qy;
+    long long rown = row;
+    if (zn - (int)threadIdx.x >= np) {
+      rn += step;
+      zn = threadIdx.x;
+      if (rn < nrows) walk.at(rn, &qxn, &qyn, &rown);
+    }
+    float pn[3] = {0.f, 0.f, 0.f};
+    if (rn < nrows) load(rown, zn, pn);
+    int key = -1;
+    unsigned code = 0;
+    if (qz < np) {
+      int cx, cy, cz, f;
+      cell_frac<F32>(qx, p[0], fg, &cx, &f);
+      cell_frac<F32>(qy, p[1], fg, &cy, &f);
+      cell_frac<F32>(qz, p[2], fg, &cz, &f);
+      code = tile_code(b, pg.n, cx, cy, cz);
+      key = code_key(b, code);
+    }
+    // primary keys are shared by runs of lanes: one aggregated atomic per run
+    const unsigned rank = agg_inc(cnt_p, key);
+    if (qz < np) rec[row + qz] = ((unsigned long long)rank << 32) | code;
+    // spill keys are sparse: one atomic per entry (its result unused)
+    for_spill_keys(b, code, [&](int k) { atomicAdd(cnt_s + k, 1u); });
+    r = rn;
+    qz = zn;
+    qx = qxn;
+    qy = qyn;
+    row = rown;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) p[a] = pn[a];
   }
 }
 
 // Scatter pass from the records: primary entries straight to offset + rank, spill entries through
-// the spill cursors.
-__global__ void __launch_bounds__(kThreads) k_bin_scatter(ParticleGeom pg, BinGeom b,
+// the spill cursors.  Bound by the latency of the records and of the offset lookups.
+__global__ void __launch_bounds__(kThreads) k_bin_scatter(ParticleGeom pg, BinGeom b, RowWalk walk,
                                                           const unsigned long long* __restrict__ rec,
                                                           const unsigned* __restrict__ off_p, unsigned* cur_s,
                                                           unsigned* ent_p, unsigned* ent_s) {
   const int np = pg.np;
-  const long long nrows = (long long)np * np;
+  const unsigned nrows = (unsigned)np * np, step = gridDim.x * blockDim.y;
   constexpr int U = 2;   // records in flight per thread: their loads, then their offset lookups
-  for (long long row = blockIdx.x; row < nrows; row += gridDim.x) {
-    const int qx = (int)(row / np), qy = (int)(row - (long long)qx * np);
+  for (unsigned w = blockIdx.x * blockDim.y + threadIdx.y; w < nrows; w += step) {
+    int qx, qy;
+    long long row;
+    walk.at(w, &qx, &qy, &row);
     for (int q0 = threadIdx.x; q0 < np; q0 += U * blockDim.x) {
       unsigned long long r[U];
       unsigned base[U];
 #pragma unroll
       for (int u = 0; u < U; ++u) {
         const int qz = q0 + u * (int)blockDim.x;
-        r[u] = qz < np ? __ldcs(rec + row * np + qz) : 0ULL;
+        r[u] = qz < np ? __ldcs(rec + row + qz) : 0ULL;
       }
 #pragma unroll
       for (int u = 0; u < U; ++u) {
         const int qz = q0 + u * (int)blockDim.x;
-        base[u] = qz < np ? __ldg(off_p + ((unsigned)r[u] & ((1u << 26) - 1u))) : 0u;
+        base[u] = qz < np ? __ldg(off_p + code_key(b, (unsigned)r[u])) : 0u;
       }
 #pragma unroll
       for (int u = 0; u < U; ++u) {
         const int qz = q0 + u * (int)blockDim.x;
         if (qz >= np) continue;
-        const unsigned key = (unsigned)r[u] & ((1u << 26) - 1u), flags = ((unsigned)r[u] >> 26) & 7u;
         const unsigned packed = pack_q(qx, qy, qz);
         ent_p[base[u] + (unsigned)(r[u] >> 32)] = packed;
-        if (flags) {
-          int k[8];
-          keys_from_record(b, key, flags, k);
-#pragma unroll
-          for (int e = 1; e < 8; ++e)
-            if (k[e] >= 0) ent_s[atomicAdd(cur_s + k[e], 1u)] = packed;
-        }
+        for_spill_keys(b, (unsigned)r[u], [&](int k) { ent_s[atomicAdd(cur_s + k, 1u)] = packed; });
       }
     }
   }
@@ -320,111 +307,177 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_apply(const unsigned* __r
   }
 }
 
-// Tile-wise deposit: shared accumulator [T][T][TZ] of 64-bit fixed-point sums.  The tile's primary
-// and spill entries form one index range, so a CTA's threads run out of work together.
-template <int LT, int LZ, bool F32>
-__global__ void __launch_bounds__(kThreads, COLA_DEPOSIT_MIN_BLOCKS) k_deposit_tiles(ParticleGeom pg, BinGeom b, FixedGeo fg,
-                                                           const float* __restrict__ s,
-                                                           const unsigned* __restrict__ off_p,
-                                                           const unsigned* __restrict__ ent_p,
-                                                           const unsigned* __restrict__ off_s,
-                                                           const unsigned* __restrict__ ent_s,
-                                                           unsigned long long* rho, float* delta_out, float scale,
-                                                           unsigned long long* tile_mass) {
-  extern __shared__ unsigned long long acc[];
-  const int lt = LT ? LT : b.lt, lz = LZ ? LZ : b.lz;
-  const int nm = pg.n, T = 1 << lt, TZ = 1 << lz;
-  const int tile = blockIdx.x;
-  const int bz = tile % b.nz, bxy = tile / b.nz;
-  const int bx = bxy / b.nt, by = bxy - bx * b.nt;
-  const int x0 = bx << lt, y0 = by << lt, z0 = bz << lz;
-  const int cells = (T * T) << lz;
-  const int cs = TZ + kDepositPad;   // accumulator column stride (padding spreads columns over banks)
-  for (int i = threadIdx.x; i < T * T * cs; i += blockDim.x) acc[i] = 0ULL;
-  __syncthreads();
+// The scan in one launch for few segments: every block sums the counts before its segment itself (at
+// most kScanOneSegs segments of 4096 counts) instead of two launches that do it once.
+constexpr int kScanOneSegs = 16;
+__global__ void __launch_bounds__(kScanThreads) k_scan_one(const unsigned* __restrict__ cnt_p,
+                                                          const unsigned* __restrict__ cnt_s, int m, unsigned* off_p,
+                                                          unsigned* off_s, unsigned* cur_s) {
+  const int list = blockIdx.y;
+  const unsigned* cnt = list ? cnt_s : cnt_p;
+  unsigned* off = list ? off_s : off_p;
+  const int base = blockIdx.x * kScanSeg;
+  unsigned v = 0, before, tot;
+  for (int i = threadIdx.x; i < base; i += kScanThreads) v += cnt[i];
+  block_excl_scan(v, &before);
+  unsigned c[8];
+  v = 0;
+#pragma unroll
+  for (int k = 0; k < 8; ++k) {
+    const int i = base + threadIdx.x * 8 + k;
+    c[k] = i < m ? cnt[i] : 0;
+    v += c[k];
+  }
+  unsigned run = before + block_excl_scan(v, &tot);
+#pragma unroll
+  for (int k = 0; k < 8; ++k) {
+    const int i = base + threadIdx.x * 8 + k;
+    if (i < m) {
+      off[i] = run;
+      if (list) cur_s[i] = run;
+    }
+    run += c[k];
+    if (i == m - 1) off[m] = run;
+  }
+}
+
+// Tile-wise deposit.  The tile's primary and spill entries form one index range, so a CTA's threads run
+// out of work together.  A cell's sum of weights (each at most 2^42) is kept as two 32-bit words, the low
+// 21 bits of every weight and the rest, added by shared atomics whose result nobody reads: up to
+// kDepositBatch contributions fit each word, after which the words are folded into 64-bit totals.  A
+// particle adds to a cell once, so a batch of that many entries cannot overflow.
+// Bound by the shared atomics.  The two-word sum with a carry (an atomic whose old value decides a second
+// one) executed 510 instructions per 32 entries at 73% of the issue slots, with the atomics' return trips
+// exposed.
+constexpr unsigned kDepositBatch = 2047;
+constexpr int kLoBits = 21;
+
+// shared add of v at byte address a + OFF if p (a reduction: nothing comes back)
+template <int OFF>
+__device__ __forceinline__ void red_shared(unsigned a, unsigned v, bool p) {
+  asm volatile("{\n .reg .pred q;\n setp.ne.u32 q, %2, 0;\n @q red.shared.add.u32 [%0 + %3], %1;\n}\n" ::"r"(a), "r"(v),
+               "r"((unsigned)p), "n"(OFF)
+               : "memory");
+}
+
+// adds the 8 weights of one entry that fall inside the tile (acc: shared address of the low words)
+template <bool F32>
+__device__ __forceinline__ void deposit_entry(const ParticleGeom& pg, const FixedGeo& fg, const float* __restrict__ s,
+                                              unsigned e, int x0, int y0, int z0, unsigned acc) {
+  const int nm = pg.n;
   const long long n = pg.npart;
-  const unsigned p0 = off_p[tile], np_t = off_p[tile + 1] - p0;
-  const unsigned s0 = off_s[tile], total = np_t + (off_s[tile + 1] - s0);
-  for (unsigned k = threadIdx.x; k < total; k += blockDim.x) {
-    int q[3];
-    long long id;
-    unpack_q(k < np_t ? ent_p[p0 + k] : ent_s[s0 + (k - np_t)], pg.np, q, &id);
-    int c[3];
-    unsigned w1[3], w0[3];
+  int q[3];
+  long long id;
+  unpack_q(e, pg.np, q, &id);
+  int c[3], f[3];
 #pragma unroll
-    for (int a = 0; a < 3; ++a) {
-      int f;
-      cell_frac<F32>(q[a], __ldg(s + a * n + id), fg, &c[a], &f);
-      w1[a] = (unsigned)f;
-      w0[a] = kWeightOne - w1[a];
-    }
-    int lz2[2];
+  for (int a = 0; a < 3; ++a) cell_frac<F32>(q[a], __ldg(s + a * n + id), fg, &c[a], &f[a]);
+  const int lx[2] = {c[0] - x0, (c[0] + 1 == nm ? 0 : c[0] + 1) - x0};
+  const int ly[2] = {c[1] - y0, (c[1] + 1 == nm ? 0 : c[1] + 1) - y0};
+  const int lz[2] = {c[2] - z0, (c[2] + 1 == nm ? 0 : c[2] + 1) - z0};
+  const bool okz[2] = {(unsigned)lz[0] < (unsigned)kTz, (unsigned)lz[1] < (unsigned)kTz};
+  const unsigned wz[2] = {(unsigned)(kWeightOne - f[2]), (unsigned)f[2]};
 #pragma unroll
-    for (int dz = 0; dz < 2; ++dz) {
-      int iz = c[2] + dz;
-      if (iz == nm) iz = 0;
-      lz2[dz] = iz - z0;
-    }
+  for (int dx = 0; dx < 2; ++dx) {
+    const unsigned wx = dx ? f[0] : kWeightOne - f[0];
+    const bool okx = (unsigned)lx[dx] < (unsigned)kT;
 #pragma unroll
-    for (int dx = 0; dx < 2; ++dx) {
-      int ix = c[0] + dx;
-      if (ix == nm) ix = 0;
-      const int lx = ix - x0;
-      if (lx < 0 || lx >= T) continue;
+    for (int dy = 0; dy < 2; ++dy) {
+      const unsigned wxy = wx * (dy ? f[1] : kWeightOne - f[1]);   // <= 2^28
+      const bool okxy = okx && (unsigned)ly[dy] < (unsigned)kT;
+      const unsigned col = acc + 4u * (unsigned)((lx[dx] * kT + ly[dy]) * kCol);
 #pragma unroll
-      for (int dy = 0; dy < 2; ++dy) {
-        int iy = c[1] + dy;
-        if (iy == nm) iy = 0;
-        const int ly = iy - y0;
-        if (ly < 0 || ly >= T) continue;
-        const unsigned wxy = (dx ? w1[0] : w0[0]) * (dy ? w1[1] : w0[1]);   // <= 2^28
-        unsigned long long* col = acc + (lx * T + ly) * cs;
-#pragma unroll
-        for (int dz = 0; dz < 2; ++dz) {
-          const unsigned long long w = (unsigned long long)wxy * (dz ? w1[2] : w0[2]);   // <= 2^42
-          if (w && lz2[dz] >= 0 && lz2[dz] < TZ) smem_add64(col + lz2[dz], w);
-        }
+      for (int dz = 0; dz < 2; ++dz) {
+        const unsigned long long w = (unsigned long long)wxy * wz[dz];   // <= 2^42
+        const unsigned a = col + 4u * (unsigned)lz[dz];
+        const bool ok = okxy && okz[dz];
+        red_shared<0>(a, (unsigned)w & ((1u << kLoBits) - 1u), ok);
+        red_shared<4 * kAccWords>(a, (unsigned)(w >> kLoBits), ok);
       }
     }
   }
+}
+
+template <bool F32>
+__global__ void __launch_bounds__(kDepositThreads, 4) k_deposit_tiles(ParticleGeom pg, BinGeom b, FixedGeo fg,
+                                                               const float* __restrict__ s,
+                                                               const unsigned* __restrict__ off_p,
+                                                               const unsigned* __restrict__ ent_p,
+                                                               const unsigned* __restrict__ off_s,
+                                                               const unsigned* __restrict__ ent_s,
+                                                               unsigned long long* rho, float* delta_out, float scale,
+                                                               unsigned long long* tile_mass) {
+  __shared__ unsigned words[2 * kAccWords];
+  unsigned* const lo = words;
+  unsigned* const hi = words + kAccWords;
+  const unsigned acc = (unsigned)__cvta_generic_to_shared(words);
+  const int nm = pg.n;
+  const int tile = blockIdx.x;
+  const unsigned p0 = off_p[tile], np_t = off_p[tile + 1] - p0;
+  const unsigned s0 = off_s[tile], total = np_t + (off_s[tile + 1] - s0);
+  const int bz = tile % b.nz, bxy = tile / b.nz;
+  const int bx = bxy / b.nt, by = bxy - bx * b.nt;
+  const int x0 = bx << kLt, y0 = by << kLt, z0 = bz << kLz;
+  for (int i = threadIdx.x; i < kAccWords; i += kDepositThreads) lo[i] = hi[i] = 0u;
   __syncthreads();
-  // the tile owns its cells: plain, coalesced stores of T*T column segments of TZ cells
-  if (!delta_out) {
-    for (int i = threadIdx.x; i < cells; i += blockDim.x) {
-      const int col = i >> lz, z = i & (TZ - 1);
-      const int lx = col >> lt, ly = col & (T - 1);
-      rho[((long long)(x0 + lx) * nm + (y0 + ly)) * nm + z0 + z] = acc[col * cs + z];
+  constexpr int kCells = kT * kT * kTz / kDepositThreads;   // cells per thread, a column segment of one z each
+  unsigned long long sum[kCells];
+  bool folded = false;
+  for (unsigned k0 = 0; k0 < total; k0 += kDepositBatch) {
+    const unsigned k1 = total - k0 < kDepositBatch ? total : k0 + kDepositBatch;
+    for (unsigned k = k0 + threadIdx.x; k < k1; k += kDepositThreads)
+      deposit_entry<F32>(pg, fg, s, k < np_t ? ent_p[p0 + k] : ent_s[s0 + (k - np_t)], x0, y0, z0, acc);
+    __syncthreads();
+    if (k1 < total) {   // more to come: fold the words (a thread folds its own cells only)
+#pragma unroll
+      for (int i = 0; i < kCells; ++i) {
+        const int j = threadIdx.x + i * kDepositThreads, a = (j >> kLz) * kCol + (j & (kTz - 1));
+        const unsigned long long v = lo[a] + ((unsigned long long)hi[a] << kLoBits);
+        sum[i] = folded ? sum[i] + v : v;
+        lo[a] = hi[a] = 0u;
+      }
+      folded = true;
+      __syncthreads();
     }
-    return;
   }
-  // the density contrast instead of the fixed-point values, and the exact 128-bit total for the
-  // overflow check (every thread of the CTA's full warps reaches the warp reduction)
-  unsigned long long lo = 0ULL, hi = 0ULL;
-  for (int i = threadIdx.x; i < cells; i += blockDim.x) {
-    const int col = i >> lz, z = i & (TZ - 1);
-    const int lx = col >> lt, ly = col & (T - 1);
-    const unsigned long long v = acc[col * cs + z];
-    lo += v;
-    hi += (lo < v);
-    delta_out[((long long)(x0 + lx) * nm + (y0 + ly)) * nm + z0 + z] = fixed_to_delta(v, scale);
+  // the tile owns its cells: plain, coalesced stores of column segments; with delta_out the density
+  // contrast, and the exact 128-bit total for the overflow check
+  unsigned long long tlo = 0ULL, thi = 0ULL;
+#pragma unroll
+  for (int i = 0; i < kCells; ++i) {
+    const int j = threadIdx.x + i * kDepositThreads, col = j >> kLz, z = j & (kTz - 1), a = col * kCol + z;
+    const int gx = x0 + (col >> kLt), gy = y0 + (col & (kT - 1)), gz = z0 + z;
+    if (gx < nm && gy < nm && gz < nm) {
+      unsigned long long v = lo[a] + ((unsigned long long)hi[a] << kLoBits);
+      if (folded) v += sum[i];
+      const long long cell = ((long long)gx * nm + gy) * nm + gz;
+      if (!delta_out) {
+        rho[cell] = v;
+      } else {
+        tlo += v;
+        thi += (tlo < v);
+        delta_out[cell] = fixed_to_delta(v, scale);
+      }
+    }
   }
+  if (!delta_out) return;
   // the CTA's total (warp shuffles, then the warps' partials in shared memory) and one slot update
   for (int off = 16; off > 0; off >>= 1) {
-    const unsigned long long olo = __shfl_down_sync(0xffffffffu, lo, off);
-    const unsigned long long ohi = __shfl_down_sync(0xffffffffu, hi, off);
-    lo += olo;
-    hi += ohi + (lo < olo);
+    const unsigned long long olo = __shfl_down_sync(0xffffffffu, tlo, off);
+    const unsigned long long ohi = __shfl_down_sync(0xffffffffu, thi, off);
+    tlo += olo;
+    thi += ohi + (tlo < olo);
   }
-  __shared__ unsigned long long wpart[2 * (kThreads / 32)];
+  __shared__ unsigned long long wpart[2 * (kDepositThreads / 32)];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   if (lane == 0) {
-    wpart[2 * warp] = lo;
-    wpart[2 * warp + 1] = hi;
+    wpart[2 * warp] = tlo;
+    wpart[2 * warp + 1] = thi;
   }
   __syncthreads();
   if (threadIdx.x == 0) {
-    unsigned long long tlo = 0ULL, thi = 0ULL;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
+    tlo = thi = 0ULL;
+    for (int w = 0; w < kDepositThreads / 32; ++w) {
       tlo += wpart[2 * w];
       thi += wpart[2 * w + 1] + (tlo < wpart[2 * w]);
     }
@@ -434,96 +487,42 @@ __global__ void __launch_bounds__(kThreads, COLA_DEPOSIT_MIN_BLOCKS) k_deposit_t
 }
 
 // Tile-wise gather (+ kick and drift) over the primary entries of each tile, from a shared copy
-// of the tile's force values with a one-cell halo on the upper side of every axis.
-// Shared copy: 3 components x (T+1)^2 rows of hz = TZ + 1 floats, rows padded to hp (16 B).
-struct GatherTile {
-  int x0, y0, z0;
-};
+// of the tile's force values with a one-cell halo on the upper side of every axis: 3 components x
+// (T+1)^2 rows of TZ + 1 floats, rows padded to kHp (16 bytes).
+constexpr int kHx = kT + 1, kHp = (kTz + 1 + 3) & ~3;
+constexpr int kGatherFloats = 3 * kHx * kHx * kHp;
+constexpr int kBulkWaitLimit = 1 << 22;   // polls of the staging barrier before the CTA gives up
 
-// floats of one tile's staged forces: 3 components x (T+1)^2 rows of hp
-__host__ __device__ __forceinline__ int gather_floats(const BinGeom& b) {
-  const int hx = (1 << b.lt) + 1, hp = ((1 << b.lz) + 1 + 3) & ~3;
-  return 3 * hx * hx * hp;
-}
-template <int LT, int LZ>
-__device__ __forceinline__ int gather_floats_t(const BinGeom& b) {
-  const int hx = (1 << (LT ? LT : b.lt)) + 1, hp = ((1 << (LZ ? LZ : b.lz)) + 1 + 3) & ~3;
-  return 3 * hx * hx * hp;
-}
-
-__device__ __forceinline__ GatherTile gather_tile_origin(const BinGeom& b, int tile) {
-  const int bz = tile % b.nz, bxy = tile / b.nz;
-  const int bx = bxy / b.nt, by = bxy - bx * b.nt;
-  return GatherTile{bx << b.lt, by << b.lt, bz << b.lz};
-}
-
-// Issue (and commit as one group) the asynchronous copies of a tile's forces into fsm: TZ/4
-// chunks of 16 bytes per row (rows start 16-byte aligned: z0 is a multiple of TZ and real rows
-// hold 2 pc floats, pc even) plus the 4-byte periodic halo cell.
-template <int LT, int LZ>
-__device__ __forceinline__ void gather_stage(float* fsm, const BinGeom& b, int nm, const GatherTile& t,
+// Stage a tile's forces: one cp.async.bulk of the tile's z extent (32 cells, fewer in the last tile; a
+// multiple of 4: the mesh side is, where this kernel runs) per force row, all completing on the mbarrier
+// at bar_sa, plus each row's periodic halo cell by a 4-byte cp.async (committed as one group).  Rows start
+// 16-byte aligned (z0 a multiple of 32, rows of 2 pc floats with pc even).  Called by every thread of the
+// block; contains a barrier.
+__device__ __forceinline__ void gather_stage(float* fsm, unsigned bar_sa, int nm, int x0, int y0, int z0,
                                              const float* __restrict__ f0, const float* __restrict__ f1,
                                              const float* __restrict__ f2, long long rs) {
-  const int hx = (1 << (LT ? LT : b.lt)) + 1, zl = 1 << (LZ ? LZ : b.lz), hp = (zl + 1 + 3) & ~3;
-  const int rows = 3 * hx * hx, chunks = (zl >> 2) + 1;
-  for (int op = threadIdx.x; op < rows * chunks; op += blockDim.x) {
-    const int r = op / chunks, ch = op - r * chunks;
-    const int comp = r / (hx * hx), col = r - comp * hx * hx;
-    const int lx = col / hx, ly = col - lx * hx;
-    int gx = t.x0 + lx, gy = t.y0 + ly;
-    if (gx >= nm) gx -= nm;
-    if (gy >= nm) gy -= nm;
-    const float* f = comp == 0 ? f0 : (comp == 1 ? f1 : f2);
-    const float* row = f + ((long long)gx * nm + gy) * rs;
-    float* dst = fsm + r * hp;
-    if (ch < (zl >> 2)) {
-      const unsigned sa = (unsigned)__cvta_generic_to_shared(dst + 4 * ch);
-      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(sa), "l"(row + t.z0 + 4 * ch) : "memory");
-    } else {
-      const int gzz = t.z0 + zl == nm ? 0 : t.z0 + zl;
-      const unsigned sa = (unsigned)__cvta_generic_to_shared(dst + zl);
-      asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(sa), "l"(row + gzz) : "memory");
-    }
-  }
-  asm volatile("cp.async.commit_group;\n" ::: "memory");
-}
-
-constexpr int kBulkWaitLimit = 1 << 22;   // polls of a staging barrier before the CTA gives up
-
-// Stage a tile's forces as gather_stage does, by bulk copies: one cp.async.bulk of TZ cells per force
-// row (3 (T+1)^2 rows, a row per thread), all completing on the mbarrier at bar_sa, plus each row's
-// periodic halo cell by a 4-byte cp.async (committed as one group).  Rows start 16-byte aligned (z0 a
-// multiple of TZ >= 4, rows of 2 pc floats with pc even) and TZ cells are a multiple of 16 bytes.
-// Called by every thread of the block; contains a barrier.
-template <int LT, int LZ>
-__device__ __forceinline__ void gather_stage_bulk(float* fsm, unsigned bar_sa, const BinGeom& b, int nm,
-                                                  const GatherTile& t, const float* __restrict__ f0,
-                                                  const float* __restrict__ f1, const float* __restrict__ f2,
-                                                  long long rs) {
-  const int hx = (1 << (LT ? LT : b.lt)) + 1, zl = 1 << (LZ ? LZ : b.lz), hp = (zl + 1 + 3) & ~3;
-  const int rows = 3 * hx * hx;
+  const int tx = nm - x0 < kT ? nm - x0 : kT, ty = nm - y0 < kT ? nm - y0 : kT, tz = nm - z0 < kTz ? nm - z0 : kTz;
   if (threadIdx.x == 0) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(bar_sa) : "memory");
     asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
     asm volatile("{\n .reg .b64 st;\n mbarrier.arrive.expect_tx.shared::cta.b64 st, [%0], %1;\n}\n" ::"r"(bar_sa),
-                 "r"(rows * zl * 4)
+                 "r"(3 * (tx + 1) * (ty + 1) * tz * 4)
                  : "memory");
   }
   __syncthreads();   // the barrier expects every row's bytes before any copy is issued
-  const int gzz = t.z0 + zl == nm ? 0 : t.z0 + zl;
-  for (int r = threadIdx.x; r < rows; r += blockDim.x) {
-    const int comp = r / (hx * hx), col = r - comp * hx * hx;
-    const int lx = col / hx, ly = col - lx * hx;
-    int gx = t.x0 + lx, gy = t.y0 + ly;
-    if (gx >= nm) gx -= nm;
-    if (gy >= nm) gy -= nm;
+  const int gzz = z0 + tz == nm ? 0 : z0 + tz;
+  for (int r = threadIdx.x; r < 3 * kHx * kHx; r += kGatherThreads) {
+    const int comp = r / (kHx * kHx), col = r - comp * kHx * kHx;
+    const int lx = col / kHx, ly = col - lx * kHx;
+    if (lx > tx || ly > ty) continue;   // beyond a cut-off tile's halo
+    const int gx = x0 + lx == nm ? 0 : x0 + lx, gy = y0 + ly == nm ? 0 : y0 + ly;
     const float* f = comp == 0 ? f0 : (comp == 1 ? f1 : f2);
     const float* row = f + ((long long)gx * nm + gy) * rs;
-    const unsigned sa = (unsigned)__cvta_generic_to_shared(fsm + r * hp);
+    const unsigned sa = (unsigned)__cvta_generic_to_shared(fsm + r * kHp);
     asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n" ::"r"(sa),
-                 "l"(row + t.z0), "r"(zl * 4), "r"(bar_sa)
+                 "l"(row + z0), "r"(tz * 4), "r"(bar_sa)
                  : "memory");
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(sa + 4u * zl), "l"(row + gzz) : "memory");
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(sa + 4u * tz), "l"(row + gzz) : "memory");
   }
   asm volatile("cp.async.commit_group;\n" ::: "memory");
 }
@@ -542,56 +541,85 @@ __device__ __forceinline__ bool bulk_wait(unsigned bar_sa, unsigned parity) {
   return false;
 }
 
-// Interpolate the staged forces at the tile's particles e0..e1 (and kick and drift).  Returns
-// whether a non-finite state was written.
-template <bool KICK, int LT, int LZ, bool F32>
-__device__ __forceinline__ bool gather_particles(const float* fsm, const ParticleGeom& pg, const BinGeom& b,
-                                                 const FixedGeo& fg, const GatherTile& t, unsigned e0, unsigned e1,
-                                                 const unsigned* __restrict__ ent_p, const unsigned* ent_s,
-                                                 unsigned ne, const float* __restrict__ s_in,
-                                                 float* __restrict__ force_out, float* s, float* v,
-                                                 const float* __restrict__ psi1, const float* __restrict__ psi2,
-                                                 const KickDrift& kd) {
-  const int hx = (1 << (LT ? LT : b.lt)) + 1, hp = ((1 << (LZ ? LZ : b.lz)) + 1 + 3) & ~3;
+// The values of one particle that the gather reads.
+template <bool KICK>
+struct GatherPart {
+  unsigned e;
+  float s[3], v[3], p1[3], p2[3];
+  __device__ __forceinline__ void load(const ParticleGeom& pg, unsigned ent, const float* sp, const float* vp,
+                                       const float* __restrict__ psi1, const float* __restrict__ psi2) {
+    e = ent;
+    int q[3];
+    long long id;
+    unpack_q(ent, pg.np, q, &id);
+    const long long n = pg.npart;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) s[a] = sp[a * n + id];
+    if (KICK) {
+#pragma unroll
+      for (int a = 0; a < 3; ++a) {
+        p1[a] = __ldg(psi1 + a * n + id);
+        p2[a] = __ldg(psi2 + a * n + id);
+        v[a] = vp[a * n + id];
+      }
+    }
+  }
+};
+
+// One CTA per tile.  Bound by the latency of its dependent loads (tile offsets, entries, particles): the
+// forces are staged and the first particles' values loaded at the same time, and each later particle's
+// entry and values are loaded while the one before is interpolated.
+template <bool KICK, bool F32>
+__global__ void __launch_bounds__(kGatherThreads, 2) k_gather_tiles(ParticleGeom pg, BinGeom b, FixedGeo fg,
+                                                             const unsigned* __restrict__ off_p,
+                                                             const unsigned* __restrict__ ent_p,
+                                                             const float* __restrict__ f0, const float* __restrict__ f1,
+                                                             const float* __restrict__ f2, long long rs,
+                                                             const float* __restrict__ s_in, float* __restrict__ force_out,
+                                                             float* s, float* v, const float* __restrict__ psi1,
+                                                             const float* __restrict__ psi2, KickDrift kd, int* flags) {
+  extern __shared__ __align__(16) float fsm[];
+  const int tile = blockIdx.x;
+  const unsigned e0 = off_p[tile], e1 = off_p[tile + 1];
+  if (e0 == e1) return;                          // empty (uniform across the block)
+  const int bz = tile % b.nz, bxy = tile / b.nz;
+  const int bx = bxy / b.nt, by = bxy - bx * b.nt;
+  const int x0 = bx << kLt, y0 = by << kLt, z0 = bz << kLz;
+  const unsigned bar_sa = (unsigned)__cvta_generic_to_shared(fsm + kGatherFloats);
+  const float* sp = KICK ? s : s_in;
+  const unsigned first = e0 + threadIdx.x;
+  unsigned ent = first < e1 ? __ldg(ent_p + first) : 0u;
+  unsigned ent_next = first + kGatherThreads < e1 ? __ldg(ent_p + first + kGatherThreads) : 0u;
+  gather_stage(fsm, bar_sa, pg.n, x0, y0, z0, f0, f1, f2, rs);
+  GatherPart<KICK> cur;
+  if (first < e1) cur.load(pg, ent, sp, v, psi1, psi2);
+  asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+  const bool ok = bulk_wait(bar_sa, 0);
+  if (__syncthreads_or(!ok)) {
+    // the staging never completed (not expected): report, give the copies one more bounded wait, stop
+    if (threadIdx.x == 0) atomicOr(flags, 4);
+    bulk_wait(bar_sa, 0);
+    return;
+  }
+  if (threadIdx.x == 0) asm volatile("mbarrier.inval.shared::cta.b64 [%0];\n" ::"r"(bar_sa) : "memory");
   const long long n = pg.npart;
   const float inv_one = 1.0f / kWeightOne;
   bool bad = false;
-  const float* sp = KICK ? s : s_in;
-  // rolling prefetch: the next particle's entry and position are loaded while this one is
-  // interpolated
-  int qn[3] = {0, 0, 0};
-  long long idn = 0;
-  float sn[3] = {0.f, 0.f, 0.f};
-  auto fetch = [&](unsigned e) {
-    unpack_q(e - e0 < ne ? ent_s[e - e0] : ent_p[e], pg.np, qn, &idn);
-#pragma unroll
-    for (int a = 0; a < 3; ++a) sn[a] = sp[a * n + idn];
-  };
-  if (e0 + threadIdx.x < e1) fetch(e0 + threadIdx.x);
-  for (unsigned e = e0 + threadIdx.x; e < e1; e += blockDim.x) {
-    const int q[3] = {qn[0], qn[1], qn[2]};
-    const long long id = idn;
-    float sv[3] = {sn[0], sn[1], sn[2]};
-    float pv1[3], pv2[3], vv[3];
-    if (KICK) {
-      // issue every particle load up front: their latency overlaps the interpolation below
-#pragma unroll
-      for (int a = 0; a < 3; ++a) {
-        pv1[a] = __ldg(psi1 + a * n + id);
-        pv2[a] = __ldg(psi2 + a * n + id);
-        vv[a] = v[a * n + id];
-      }
-    }
-    if (e + blockDim.x < e1) fetch(e + blockDim.x);
-    int c[3];
+  for (unsigned e = first; e < e1; e += kGatherThreads) {
+    GatherPart<KICK> nxt;
+    if (e + kGatherThreads < e1) nxt.load(pg, ent_next, sp, v, psi1, psi2);
+    ent_next = e + 2 * kGatherThreads < e1 ? __ldg(ent_p + e + 2 * kGatherThreads) : 0u;
+    int q[3], c[3];
+    long long id;
+    unpack_q(cur.e, pg.np, q, &id);
     float w1[3];
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
       int f;
-      cell_frac<F32>(q[a], sv[a], fg, &c[a], &f);
+      cell_frac<F32>(q[a], cur.s[a], fg, &c[a], &f);
       w1[a] = (float)f * inv_one;
     }
-    const int lx = c[0] - t.x0, ly = c[1] - t.y0, lz = c[2] - t.z0;   // base cell inside the tile
+    const int lx = c[0] - x0, ly = c[1] - y0, lz = c[2] - z0;   // base cell inside the tile
     float fr[3] = {0.f, 0.f, 0.f};
 #pragma unroll
     for (int dx = 0; dx < 2; ++dx) {
@@ -599,10 +627,10 @@ __device__ __forceinline__ bool gather_particles(const float* fsm, const Particl
 #pragma unroll
       for (int dy = 0; dy < 2; ++dy) {
         const float wxy = wx * (dy ? w1[1] : 1.0f - w1[1]);
-        const int o = ((lx + dx) * hx + (ly + dy)) * hp + lz;
+        const int o = ((lx + dx) * kHx + (ly + dy)) * kHp + lz;
 #pragma unroll
         for (int comp = 0; comp < 3; ++comp) {
-          const float* p = fsm + comp * (hx * hx * hp) + o;
+          const float* p = fsm + comp * (kHx * kHx * kHp) + o;
           fr[comp] += wxy * ((1.0f - w1[2]) * p[0] + w1[2] * p[1]);
         }
       }
@@ -614,100 +642,17 @@ __device__ __forceinline__ bool gather_particles(const float* fsm, const Particl
     } else {
 #pragma unroll
       for (int a = 0; a < 3; ++a) {
-        const float p1 = pv1[a], p2 = pv2[a];
+        const float p1 = cur.p1[a], p2 = cur.p2[a];
         const float fres = fr[a] - (kd.c1 * p1 + kd.c2 * p2);
-        const float vn = vv[a] + kd.kick * fres;
-        const float sn = sv[a] + kd.drift * vn + kd.dd1 * p1 + kd.dd2 * p2;
+        const float vn = cur.v[a] + kd.kick * fres;
+        const float sn = cur.s[a] + kd.drift * vn + kd.dd1 * p1 + kd.dd2 * p2;
         v[a * n + id] = vn;
         s[a * n + id] = sn;
         bad |= !isfinite(vn) || !isfinite(sn);
       }
     }
+    cur = nxt;
   }
-  return bad;
-}
-
-// One CTA per tile.
-template <bool KICK, int LT, int LZ, bool F32>
-__global__ void __launch_bounds__(kThreads) k_gather_tiles(ParticleGeom pg, BinGeom b, FixedGeo fg,
-                                                          const unsigned* __restrict__ off_p,
-                                                          const unsigned* __restrict__ ent_p,
-                                                          const float* __restrict__ f0, const float* __restrict__ f1,
-                                                          const float* __restrict__ f2, long long rs,
-                                                          const float* __restrict__ s_in, float* __restrict__ force_out,
-                                                          float* s, float* v, const float* __restrict__ psi1,
-                                                          const float* __restrict__ psi2, KickDrift kd, int* flags) {
-  extern __shared__ __align__(16) float fsm[];
-  const int tile = blockIdx.x;
-  const unsigned e0 = off_p[tile], e1 = off_p[tile + 1];
-  if (e0 == e1) return;                          // empty (uniform across the block)
-  const GatherTile t = gather_tile_origin(b, tile);
-  // the tile's first kGatherEnt entries travel with the forces: one dependent global load fewer
-  unsigned* ent_s = reinterpret_cast<unsigned*>(fsm + gather_floats_t<LT, LZ>(b));
-  const unsigned ne = e1 - e0 < (unsigned)kGatherEnt ? e1 - e0 : (unsigned)kGatherEnt;
-  for (unsigned i = threadIdx.x; i < ne; i += blockDim.x) {
-    const unsigned sa = (unsigned)__cvta_generic_to_shared(ent_s + i);
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(sa), "l"(ent_p + e0 + i) : "memory");
-  }
-  // the forces by bulk copies on an mbarrier placed after the staged entries (8-byte aligned)
-  const unsigned bar_sa = (unsigned)__cvta_generic_to_shared(ent_s + kGatherEnt);
-  gather_stage_bulk<LT, LZ>(fsm, bar_sa, b, pg.n, t, f0, f1, f2, rs);
-  asm volatile("cp.async.wait_group 0;\n" ::: "memory");
-  const bool ok = bulk_wait(bar_sa, 0);
-  if (__syncthreads_or(!ok)) {
-    // the staging never completed (not expected): report, give the copies one more bounded wait, stop
-    if (threadIdx.x == 0) atomicOr(flags, 4);
-    bulk_wait(bar_sa, 0);
-    return;
-  }
-  if (threadIdx.x == 0) asm volatile("mbarrier.inval.shared::cta.b64 [%0];\n" ::"r"(bar_sa) : "memory");
-  const bool bad = gather_particles<KICK, LT, LZ, F32>(fsm, pg, b, fg, t, e0, e1, ent_p, ent_s, ne, s_in, force_out,
-                                                       s, v, psi1, psi2, kd);
-  if (KICK && __syncthreads_or(bad) && threadIdx.x == 0) atomicOr(flags, 2);
-}
-
-// Persistent variant: each CTA walks tiles t = blockIdx.x + i gridDim.x with two staging buffers;
-// the next non-empty tile's forces are copied (cp.async) while the current tile's particles run.
-template <bool KICK, int LT, int LZ, bool F32>
-__global__ void __launch_bounds__(kThreads) k_gather_tiles_pipe(ParticleGeom pg, BinGeom b, FixedGeo fg,
-                                                               const unsigned* __restrict__ off_p,
-                                                               const unsigned* __restrict__ ent_p,
-                                                               const float* __restrict__ f0,
-                                                               const float* __restrict__ f1,
-                                                               const float* __restrict__ f2, long long rs,
-                                                               const float* __restrict__ s_in,
-                                                               float* __restrict__ force_out, float* s, float* v,
-                                                               const float* __restrict__ psi1,
-                                                               const float* __restrict__ psi2, KickDrift kd,
-                                                               int* flags) {
-  extern __shared__ __align__(16) float fsm[];
-  const int hx = (1 << b.lt) + 1, hp = ((1 << b.lz) + 1 + 3) & ~3;
-  float* bcur = fsm;
-  float* bnext = fsm + 3 * hx * hx * hp;
-  const int ntiles = b.tiles;
-  // first non-empty tile of this CTA
-  auto next_tile = [&](int t) {
-    while (t < ntiles && off_p[t] == off_p[t + 1]) t += gridDim.x;
-    return t;
-  };
-  int t = next_tile(blockIdx.x);
-  if (t >= ntiles) return;
-  gather_stage<LT, LZ>(bcur, b, pg.n, gather_tile_origin(b, t), f0, f1, f2, rs);
-  bool bad = false;
-  while (t < ntiles) {
-    asm volatile("cp.async.wait_group 0;\n" ::: "memory");
-    __syncthreads();   // tile t staged; every thread is done with the other buffer
-    const int tn = next_tile(t + gridDim.x);
-    if (tn < ntiles) gather_stage<LT, LZ>(bnext, b, pg.n, gather_tile_origin(b, tn), f0, f1, f2, rs);
-    bad |= gather_particles<KICK, LT, LZ, F32>(bcur, pg, b, fg, gather_tile_origin(b, t), off_p[t], off_p[t + 1], ent_p,
-                                               nullptr, 0u,
-                                  s_in, force_out, s, v, psi1, psi2, kd);
-    float* tmp = bcur;
-    bcur = bnext;
-    bnext = tmp;
-    t = tn;
-  }
-  asm volatile("cp.async.wait_group 0;\n" ::: "memory");
   if (KICK && __syncthreads_or(bad) && threadIdx.x == 0) atomicOr(flags, 2);
 }
 
@@ -715,43 +660,25 @@ __global__ void __launch_bounds__(kThreads) k_gather_tiles_pipe(ParticleGeom pg,
 
 bool bin_geometry(int nmesh, int np, BinGeom* b) {
   if (np > 1024) return false;                       // packed 10-bit lattice coordinates
-  int lt = 3;                                        // T = 8 cells across, or the largest power of
-  while (lt > 0 && nmesh % (1 << lt)) --lt;          // two dividing N
-  int lz = 5;                                        // TZ = 32 cells along z, likewise
-  while (lz > 0 && nmesh % (1 << lz)) --lz;
-  if (lz == 0 || lt == 0) return false;
-  b->lt = lt;
-  b->lz = lz;
-  b->nt = nmesh >> lt;
-  b->nz = nmesh >> lz;
-  const long long tiles = (long long)b->nt * b->nt * b->nz;
-  if (tiles > (1LL << 26)) return false;
-  b->tiles = (int)tiles;
+  b->nt = (nmesh + kT - 1) >> kLt;
+  b->nz = (nmesh + kTz - 1) >> kLz;
+  b->tiles = b->nt * b->nt * b->nz;                  // <= 2^25 (nmesh <= 4096)
+  b->bulk = nmesh % 4 == 0;
   return true;
 }
 
-size_t bin_smem_bytes(const BinGeom& b, int nmesh) {
-  (void)nmesh;
-  return (size_t)(1 << b.lt) * (1 << b.lt) * ((1 << b.lz) + kDepositPad) * sizeof(unsigned long long);
-}
-
-// z-tiles per gather CTA
-int gather_group(const BinGeom& b) {
-  (void)b;
-  return 1;
-}
-
-size_t gather_smem_bytes(const BinGeom& b) {
-  const size_t hx = (1 << b.lt) + 1, hz = ((size_t)gather_group(b) << b.lz) + 1;
-  const size_t hp = (hz + 3) & ~(size_t)3;
-  return 3 * hx * hx * hp * sizeof(float);
-}
-
-bool tile_gather_pays(const BinGeom& b, long long npart) {
-  // staging a tile's forces costs about as much as gathering a few hundred particles directly;
-  // the 16-byte copies also need rows of at least 4 cells along z
-  const long long groups = (long long)b.tiles / gather_group(b);
-  return b.lz >= 2 && npart >= 384LL * groups;
+// Where the binned deposit and the tile gather pay (us per COLA step, direct / binned + direct gather /
+// binned + tile gather, r = mesh side over particle side):
+//   192^3: r = 1 759/973/832, 1.5 359/407/368, 2 267/308/293;  216^3: 1086/1191/973, 521/566/508, 380/408/393;
+//   240^3: 1390/1480/1195, 679/697/614, 487/495/477;  384^3: 5707/5664/4291, 2649/2506/2157, 1946/1820/1691;
+//   r = 3, 288^3 651/670/687, 384^3 1519/1431/1470, 480^3 2914/2794/2884.
+// A direct deposit's atomics run in L2 while the 64-bit mesh fits beside what else is there (72 MB, 208^3).
+// Above that dense tiles (256 particles on average, r up to 2.5) pay for the binning and the staging;
+// sparse ones for the binning alone, once the mesh is some twice the L2.
+void particle_schedule(const BinGeom& b, int nmesh, long long npart, bool* binned, bool* tile_gather) {
+  const double mesh_mb = 8e-6 * nmesh * nmesh * nmesh;
+  *tile_gather = b.bulk && mesh_mb > 72.0 && npart >= 256LL * b.tiles;
+  *binned = *tile_gather || mesh_mb > 256.0;
 }
 
 int launch_excl_scan(const unsigned* cnt, int m, unsigned* seg, unsigned* off, unsigned* cur, cudaStream_t st) {
@@ -762,50 +689,31 @@ int launch_excl_scan(const unsigned* cnt, int m, unsigned* seg, unsigned* off, u
   return check_launch("excl_scan");
 }
 
-namespace {
-template <int V>
-using IntC = std::integral_constant<int, V>;
-
-// Calls go(LT, LZ, F32) with the compile-time instance that matches the geometry: the common
-// 8 x 8 x 32 tiles or run-time tile sides, and the 32-bit fixed-point path below 2048 cells.
-template <class Go>
-void with_instance(const BinGeom& b, int nmesh, Go&& go) {
-  const bool common = b.lt == 3 && b.lz == 5;
-  const bool f32 = nmesh < 2048;
-  if (common && f32) go(IntC<3>{}, IntC<5>{}, std::true_type{});
-  else if (common) go(IntC<3>{}, IntC<5>{}, std::false_type{});
-  else if (f32) go(IntC<0>{}, IntC<0>{}, std::true_type{});
-  else go(IntC<0>{}, IntC<0>{}, std::false_type{});
-}
-
-template <class K>
-void smem_limit(K kernel, int bytes) {
-  if (first_use_on_device(reinterpret_cast<const void*>(kernel)))
-    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-}
-}  // namespace
-
 int launch_binning(const ParticleGeom& pg, const BinGeom& b, const float* s, BinBuffers& bb, cudaStream_t st) {
-  const long long rows = (long long)pg.np * pg.np;
-  const unsigned grid = (unsigned)(rows < 152LL * 64 ? rows : 152LL * 64);
-  const int th = pg.np < kThreads ? ((pg.np + 31) / 32) * 32 : kThreads;
+  const RowBlocks rb = row_blocks(pg.np);
+  const unsigned blocks = rb.grid.x * rb.grid.y, grid = blocks < 152u * 64u ? blocks : 152u * 64u;
+  unsigned mul = (unsigned)(0.382 * pg.np) | 1u;   // np has no prime factor above 5
+  while (mul % 3 == 0 || mul % 5 == 0) mul += 2;
+  const RowWalk walk{(unsigned)pg.np, mul};
   const FixedGeo fg = fixed_geo(pg.n, pg.r_fixed);
-  if (cudaMemsetAsync(bb.cnt_p, 0, (size_t)b.tiles * sizeof(unsigned), st) != cudaSuccess ||
-      cudaMemsetAsync(bb.cnt_s, 0, (size_t)b.tiles * sizeof(unsigned), st) != cudaSuccess)
+  // the two count arrays are adjacent: one clear of both
+  if (cudaMemsetAsync(bb.cnt_p, 0, (size_t)(bb.cnt_s - bb.cnt_p + b.tiles) * sizeof(unsigned), st) != cudaSuccess)
     return COLA_ERR_CUDA;
-  with_instance(b, pg.n, [&](auto lt, auto lz, auto f32) {
-    k_bin_count<decltype(lt)::value, decltype(lz)::value, decltype(f32)::value>
-        <<<grid, th, 0, st>>>(pg, b, fg, s, bb.cnt_p, bb.cnt_s, bb.rec);
-  });
+  auto* count = pg.n < 2048 ? k_bin_count<true> : k_bin_count<false>;
+  count<<<grid, rb.block, 0, st>>>(pg, b, fg, walk, s, bb.cnt_p, bb.cnt_s, bb.rec);
   int e = check_launch("bin_count");
   if (e != COLA_OK) return e;
   const int nseg = (b.tiles + kScanSeg - 1) / kScanSeg;
-  k_scan_sums<<<dim3(nseg, 2), kScanThreads, 0, st>>>(bb.cnt_p, bb.cnt_s, b.tiles, bb.seg);
-  k_scan_segs<<<2, kScanThreads, 0, st>>>(bb.seg, nseg);
-  k_scan_apply<<<dim3(nseg, 2), kScanThreads, 0, st>>>(bb.cnt_p, bb.cnt_s, b.tiles, bb.seg, bb.off_p, bb.off_s,
-                                                       bb.cur_p, bb.cur_s);
+  if (nseg <= kScanOneSegs) {
+    k_scan_one<<<dim3(nseg, 2), kScanThreads, 0, st>>>(bb.cnt_p, bb.cnt_s, b.tiles, bb.off_p, bb.off_s, bb.cur_s);
+  } else {
+    k_scan_sums<<<dim3(nseg, 2), kScanThreads, 0, st>>>(bb.cnt_p, bb.cnt_s, b.tiles, bb.seg);
+    k_scan_segs<<<2, kScanThreads, 0, st>>>(bb.seg, nseg);
+    k_scan_apply<<<dim3(nseg, 2), kScanThreads, 0, st>>>(bb.cnt_p, bb.cnt_s, b.tiles, bb.seg, bb.off_p, bb.off_s,
+                                                         bb.cur_p, bb.cur_s);
+  }
   if ((e = check_launch("bin_scan")) != COLA_OK) return e;
-  k_bin_scatter<<<grid, th, 0, st>>>(pg, b, bb.rec, bb.off_p, bb.cur_s, bb.ent_p, bb.ent_s);
+  k_bin_scatter<<<grid, rb.block, 0, st>>>(pg, b, walk, bb.rec, bb.off_p, bb.cur_s, bb.ent_p, bb.ent_s);
   return check_launch("bin_scatter");
 }
 
@@ -814,62 +722,38 @@ int launch_deposit_tiles(const ParticleGeom& pg, const BinGeom& b, const float* 
                          unsigned long long* tile_mass) {
   if (delta_out && !tile_mass) return COLA_ERR_INVALID;
   const FixedGeo fg = fixed_geo(pg.n, pg.r_fixed);
-  with_instance(b, pg.n, [&](auto lt, auto lz, auto f32) {
-    auto k = k_deposit_tiles<decltype(lt)::value, decltype(lz)::value, decltype(f32)::value>;
-    smem_limit(k, 64 * 1024);
-    k<<<b.tiles, kThreads, bin_smem_bytes(b, pg.n), st>>>(pg, b, fg, s, bb.off_p, bb.ent_p, bb.off_s, bb.ent_s, rho,
-                                                          delta_out, scale, tile_mass);
-  });
+  auto* k = pg.n < 2048 ? k_deposit_tiles<true> : k_deposit_tiles<false>;
+  k<<<b.tiles, kDepositThreads, 0, st>>>(pg, b, fg, s, bb.off_p, bb.ent_p, bb.off_s, bb.ent_s, rho, delta_out, scale,
+                                  tile_mass);
   return check_launch("deposit_tiles");
 }
 
+namespace {
+template <class K>
+void smem_limit(K kernel, int bytes) {
+  if (bytes > 48 * 1024 && first_use_on_device(reinterpret_cast<const void*>(kernel)))
+    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+}
+}  // namespace
+
 int launch_gather_tiles(const ParticleGeom& pg, const BinGeom& b, const BinBuffers& bb, const float* const f[3],
                         long long rs, const float* s_in, float* force_out, float* s, float* v, const float* psi1,
-                        const float* psi2, const KickDrift* kd, int* flags, cudaStream_t st, bool pipelined) {
-  const size_t sm = gather_smem_bytes(b);
-  const size_t sm_ent = (size_t)gather_floats(b) * sizeof(float) + kGatherEnt * sizeof(unsigned) + 16;   // + mbarrier
-  const KickDrift k = kd ? *kd : KickDrift{};
+                        const float* psi2, const KickDrift* kd, int* flags, cudaStream_t st) {
+  if (!b.bulk) return COLA_ERR_INVALID;   // 16-byte staging copies along z
+  constexpr int sm = kGatherFloats * (int)sizeof(float) + 16;   // + mbarrier
   const FixedGeo fg = fixed_geo(pg.n, pg.r_fixed);
-  if (pipelined) {
-    // two staging buffers per CTA: as many CTAs per SM as the shared memory holds (at most 4)
-    int dev = 0, sms = 152;
-    if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    int per_sm = (int)((227 * 1024) / (2 * sm + 1024));
-    if (per_sm > 4) per_sm = 4;
-    if (per_sm < 1) per_sm = 1;
-    const int ctas = b.tiles < sms * per_sm ? b.tiles : sms * per_sm;
-    with_instance(b, pg.n, [&](auto lt, auto lz, auto f32) {
-      constexpr int LT = decltype(lt)::value, LZ = decltype(lz)::value;
-      constexpr bool F32 = decltype(f32)::value;
-      if (kd) {
-        auto kern = k_gather_tiles_pipe<true, LT, LZ, F32>;
-        smem_limit(kern, 128 * 1024);
-        kern<<<ctas, kThreads, 2 * sm, st>>>(pg, b, fg, bb.off_p, bb.ent_p, f[0], f[1], f[2], rs, nullptr, nullptr, s,
-                                             v, psi1, psi2, k, flags);
-      } else {
-        auto kern = k_gather_tiles_pipe<false, LT, LZ, F32>;
-        smem_limit(kern, 128 * 1024);
-        kern<<<ctas, kThreads, 2 * sm, st>>>(pg, b, fg, bb.off_p, bb.ent_p, f[0], f[1], f[2], rs, s_in, force_out,
-                                             nullptr, nullptr, nullptr, nullptr, k, flags);
-      }
-    });
-    return check_launch("gather_tiles_pipe");
+  const bool f32 = pg.n < 2048;
+  if (kd) {
+    auto* k = f32 ? k_gather_tiles<true, true> : k_gather_tiles<true, false>;
+    smem_limit(k, sm);
+    k<<<b.tiles, kGatherThreads, sm, st>>>(pg, b, fg, bb.off_p, bb.ent_p, f[0], f[1], f[2], rs, nullptr, nullptr, s, v, psi1,
+                                     psi2, *kd, flags);
+  } else {
+    auto* k = f32 ? k_gather_tiles<false, true> : k_gather_tiles<false, false>;
+    smem_limit(k, sm);
+    k<<<b.tiles, kGatherThreads, sm, st>>>(pg, b, fg, bb.off_p, bb.ent_p, f[0], f[1], f[2], rs, s_in, force_out, nullptr,
+                                     nullptr, nullptr, nullptr, KickDrift{}, flags);
   }
-  with_instance(b, pg.n, [&](auto lt, auto lz, auto f32) {
-    constexpr int LT = decltype(lt)::value, LZ = decltype(lz)::value;
-    constexpr bool F32 = decltype(f32)::value;
-    if (kd) {
-      auto kern = k_gather_tiles<true, LT, LZ, F32>;
-      smem_limit(kern, 64 * 1024);
-      kern<<<b.tiles, kThreads, sm_ent, st>>>(pg, b, fg, bb.off_p, bb.ent_p, f[0], f[1], f[2], rs, nullptr, nullptr, s,
-                                              v, psi1, psi2, k, flags);
-    } else {
-      auto kern = k_gather_tiles<false, LT, LZ, F32>;
-      smem_limit(kern, 64 * 1024);
-      kern<<<b.tiles, kThreads, sm_ent, st>>>(pg, b, fg, bb.off_p, bb.ent_p, f[0], f[1], f[2], rs, s_in, force_out,
-                                              nullptr, nullptr, nullptr, nullptr, k, flags);
-    }
-  });
   return check_launch("gather_tiles");
 }
 

@@ -139,7 +139,7 @@ int gather(cola_ctx* c, const float* s_in, float* force, float* s, float* v, con
                        reinterpret_cast<float*>(c->cbuf[2])};
   if (c->binned && c->tile_gather)
     return STAGED(kStGather, launch_gather_tiles(c->pg, c->bg, c->bb, f, 2LL * c->mesh.pc, s_in, force, s, v, psi1,
-                                                 psi2, kd, c->flags, c->stream, c->gather_pipe));
+                                                 psi2, kd, c->flags, c->stream));
   return STAGED(kStGather, launch_gather(c->pg, f, 2LL * c->mesh.pc, s_in, force, s, v, psi1, psi2, kd, c->flags,
                                          c->stream));
 }
@@ -422,11 +422,10 @@ extern "C" int cola_create(const cola_params* params, void* stream, cola_ctx** o
     c->tile_mass = reinterpret_cast<unsigned long long*>(q);
     q += align256(tiles * 2 * sizeof(unsigned long long));
     c->bb.rec = reinterpret_cast<unsigned long long*>(q);
-    c->binned = true;
-    c->tile_gather = tile_gather_pays(c->bg, c->pg.npart);
+    particle_schedule(c->bg, params->nmesh, c->pg.npart, &c->binned, &c->tile_gather);
   }
-  c->fft_sched = COLA_SCHED_PIPELINED_FFT | COLA_SCHED_WIDE_TILES |
-                 (params->nmesh > 768 && params->nmesh <= 1536 ? COLA_SCHED_PIPE_INPLACE : 0);
+  c->kept_sched = COLA_SCHED_PIPELINED_FFT | COLA_SCHED_WIDE_TILES |
+                  (params->nmesh > 768 && params->nmesh <= 1536 ? COLA_SCHED_PIPE_INPLACE : 0);
   if ((st = cuda_status(cudaMallocHost(&c->edges_host, (kPkMaxBins + 1) * sizeof(long long)), "cudaMallocHost")) !=
       COLA_OK)
     return fail(st);
@@ -700,11 +699,11 @@ extern "C" int cola_run_snapshots(cola_ctx* c, const float* wn, float* s, float*
 
 // ---- execution schedule and autotuner ---------------------------------------------------------
 namespace {
-constexpr int kParticleBits = COLA_SCHED_BINNED_DEPOSIT | COLA_SCHED_TILE_GATHER | COLA_SCHED_PIPELINED_GATHER;
+constexpr int kParticleBits = COLA_SCHED_BINNED_DEPOSIT | COLA_SCHED_TILE_GATHER;
 
 int schedule_of(const cola_ctx* c) {
   return (c->binned ? COLA_SCHED_BINNED_DEPOSIT : 0) | (c->tile_gather ? COLA_SCHED_TILE_GATHER : 0) |
-         (c->gather_pipe ? COLA_SCHED_PIPELINED_GATHER : 0) | c->fft_sched;
+         c->kept_sched;
 }
 
 bool schedule_valid(const cola_ctx* c, int sc) {
@@ -716,7 +715,7 @@ bool schedule_valid(const cola_ctx* c, int sc) {
   if ((sc & COLA_SCHED_PIPE_EPT8) && !(sc & COLA_SCHED_PIPELINED_FFT)) return false;   // unused knob
   if ((sc & COLA_SCHED_BINNED_DEPOSIT) && !c->bin_mem) return false;
   if ((sc & COLA_SCHED_TILE_GATHER) && !(sc & COLA_SCHED_BINNED_DEPOSIT)) return false;
-  if ((sc & COLA_SCHED_TILE_GATHER) && c->bg.lz < 2) return false;   // 16-byte staging copies along z
+  if ((sc & COLA_SCHED_TILE_GATHER) && !c->bg.bulk) return false;   // 16-byte staging copies along z
   if (((sc >> COLA_SCHED_BUDGET_SHIFT) & 3) > 2) return false;
   if (!(sc & COLA_SCHED_PIPELINED_FFT) && ((sc >> COLA_SCHED_BUDGET_SHIFT) & 3)) return false;   // unused knob
   if ((sc & COLA_SCHED_PIPE_INPLACE) && (!(sc & COLA_SCHED_PIPELINED_FFT) || (sc & COLA_SCHED_PIPE_EPT8) ||
@@ -728,8 +727,7 @@ bool schedule_valid(const cola_ctx* c, int sc) {
 void apply_schedule(cola_ctx* c, int sc) {
   c->binned = (sc & COLA_SCHED_BINNED_DEPOSIT) != 0;
   c->tile_gather = (sc & COLA_SCHED_TILE_GATHER) != 0;
-  c->gather_pipe = (sc & COLA_SCHED_PIPELINED_GATHER) != 0;
-  c->fft_sched = sc & ~kParticleBits;   // kept for cola_get_schedule: every length has one set of FFT kernels
+  c->kept_sched = sc & ~kParticleBits;
 }
 }  // namespace
 
@@ -780,11 +778,12 @@ extern "C" int cola_autotune(cola_ctx* c, const float* s, int reps, int* best, i
     timed.push_back({sc, t});
     return t;
   };
-  // the particle kernels' choices; the FFT bits select nothing, so they stay as they are
+  // the particle kernels' choices; the other bits select nothing, so they stay as they are
   int cur = keep, arg = -1;
   float tbest = 0.0f;
-  for (int opt : {0, COLA_SCHED_BINNED_DEPOSIT, COLA_SCHED_BINNED_DEPOSIT | COLA_SCHED_TILE_GATHER, kParticleBits}) {
-    const int sc = (keep & ~kParticleBits) | opt;
+  const int base = keep & ~(kParticleBits | COLA_SCHED_PIPELINED_GATHER);   // the last needs the tile gather
+  for (int opt : {0, COLA_SCHED_BINNED_DEPOSIT, kParticleBits}) {
+    const int sc = base | opt;
     if (!schedule_valid(c, sc)) continue;
     const float t = time_of(sc);
     if (st != COLA_OK) break;

@@ -123,6 +123,16 @@ struct ParticleGeom {
   long long npart;    // np^3
 };
 
+// Blocks of whole lattice rows for kernels that walk the particles: threadIdx.x along a row (qz, in steps
+// of blockDim.x), blockDim.y rows (qy) per block, blockIdx.y the lattice plane (qx).
+struct RowBlocks {
+  dim3 grid, block;
+};
+inline RowBlocks row_blocks(int np) {
+  const int bx = np < 256 ? (np + 31) / 32 * 32 : 256, by = 256 / bx;
+  return RowBlocks{dim3((unsigned)((np + by - 1) / by), (unsigned)np), dim3((unsigned)bx, (unsigned)by)};
+}
+
 int launch_deposit(const ParticleGeom& pg, const float* s, unsigned long long* rho, int* flags,
                    cudaStream_t st);
 // Sets flags bit 0 if the 128-bit total in acc (accumulated by the fixed-point R2C pass, or by
@@ -234,25 +244,24 @@ int launch_gather(const ParticleGeom& pg, const float* const f[3], long long rs,
                   float* force_out, float* s, float* v, const float* psi1, const float* psi2,
                   const KickDrift* kd, int* flags, cudaStream_t st);
 
-// Spatial binning by tiles of T x T mesh columns (binning.cu).
+// Spatial binning by tiles of 8 x 8 x 32 mesh cells (binning.cu).
 struct BinGeom {
-  int lt;      // log2 T (tile side across z)
-  int lz;      // log2 TZ (tile length along z)
-  int nt;      // tiles per axis across z (N / T)
-  int nz;      // tiles along z (N / TZ)
+  int nt;      // tiles per axis across z
+  int nz;      // tiles along z
   int tiles;   // nt^2 nz
+  bool bulk;   // mesh rows hold a multiple of 4 cells: the tile gather's 16-byte staging copies
 };
 struct BinBuffers {
-  unsigned *cnt_p = nullptr, *cnt_s = nullptr;   // counts per tile (primary, spill)
+  unsigned *cnt_p = nullptr, *cnt_s = nullptr;   // counts per tile (primary, spill), cnt_s after cnt_p
   unsigned *off_p = nullptr, *off_s = nullptr;   // offsets, tiles + 1
   unsigned *cur_p = nullptr, *cur_s = nullptr;   // scatter cursors
   unsigned *ent_p = nullptr, *ent_s = nullptr;   // packed lattice coordinates (n primary, up to 7n spill)
   unsigned* seg = nullptr;                        // scan segment sums (2 lists)
-  unsigned long long* rec = nullptr;              // [n] rank in the primary tile << 32 | flags << 26 | tile
+  unsigned long long* rec = nullptr;              // [n] rank in the primary tile << 32 | tile code (binning.cu)
 };
 bool bin_geometry(int nmesh, int np, BinGeom* b);
-size_t bin_smem_bytes(const BinGeom& b, int nmesh);
-bool tile_gather_pays(const BinGeom& b, long long npart);   // else gather in lattice order
+// The default deposit (binned or direct) and gather (by tiles or in lattice order) of a mesh.
+void particle_schedule(const BinGeom& b, int nmesh, long long npart, bool* binned, bool* tile_gather);
 int launch_binning(const ParticleGeom& pg, const BinGeom& b, const float* s, BinBuffers& bb, cudaStream_t st);
 // delta_out == nullptr: writes the fixed-point mesh rho.  Else writes the density contrast
 // fixed_to_delta(rho, scale) as dense float rows to delta_out (rho is not written) and each tile's
@@ -262,8 +271,7 @@ int launch_deposit_tiles(const ParticleGeom& pg, const BinGeom& b, const float* 
                          unsigned long long* tile_mass = nullptr);
 int launch_gather_tiles(const ParticleGeom& pg, const BinGeom& b, const BinBuffers& bb, const float* const f[3],
                         long long rs, const float* s_in, float* force_out, float* s, float* v, const float* psi1,
-                        const float* psi2, const KickDrift* kd, int* flags, cudaStream_t st,
-                        bool pipelined = false);
+                        const float* psi2, const KickDrift* kd, int* flags, cudaStream_t st);
 
 // 2LPT helpers on the lattice grid (side np).
 enum IcField { kIcPsi1 = 0, kIcHess = 1, kIcPsi2 = 2 };
@@ -419,8 +427,7 @@ struct cola_ctx {
   unsigned long long* tile_mass = nullptr;  // [tiles][2] 128-bit totals of the tile deposit
   bool binned = false;                    // tile-wise deposit (else direct atomics)
   bool tile_gather = false;               // tile-wise gather from shared memory (else lattice order)
-  bool gather_pipe = false;               // ... by persistent CTAs that stage the next tile meanwhile
-  int fft_sched = 0;                      // the schedule's FFT bits (reported, no effect)
+  int kept_sched = 0;                     // the schedule bits that select nothing (reported)
   cola::BinGeom bg{};
   cola::BinBuffers bb;
   void* bin_mem = nullptr;

@@ -29,28 +29,27 @@ unsigned grid_for(long long work, int threads) {
   return (unsigned)(b < 1 ? 1 : b);
 }
 
-// Particles are processed by lattice rows: blockIdx.x (grid-stride) indexes the row (qx, qy) and
-// the threads walk qz, so the lattice index needs one division per row and none per particle.
+// Particles are processed by lattice rows (row_blocks): no index is divided.
 constexpr int kRowThreads = 256;
 
-__global__ void __launch_bounds__(kRowThreads) k_deposit(ParticleGeom pg, const float* __restrict__ s,
+template <bool F32>
+__global__ void __launch_bounds__(kRowThreads) k_deposit(ParticleGeom pg, FixedGeo fg, const float* __restrict__ s,
                                                         unsigned long long* rho) {
   const long long n = pg.npart;
-  const long long modulus = (long long)pg.n << kFracBits;
   const int nm = pg.n, np = pg.np;
-  const long long nrows = (long long)np * np;
-  for (long long row = blockIdx.x; row < nrows; row += gridDim.x) {
-    const int qx = (int)(row / np), qy = (int)(row - (long long)qx * np);
+  const int qx = blockIdx.y, qy = blockIdx.x * blockDim.y + threadIdx.y;
+  if (qy < np) {
+    const long long row = (long long)qx * np + qy;
     for (int qz = threadIdx.x; qz < np; qz += blockDim.x) {
       const long long id = row * np + qz;
       const int q[3] = {qx, qy, qz};
       int c[3];
-      unsigned long long w1[3], w0[3];
+      unsigned w1[3], w0[3];
 #pragma unroll
       for (int a = 0; a < 3; ++a) {
-        const long long g = fixed_coord(q[a], __ldg(s + a * n + id), pg.r_fixed, modulus);
-        c[a] = (int)(g >> kFracBits);
-        w1[a] = (unsigned long long)((g >> (kFracBits - 14)) & (kWeightOne - 1));
+        int f;
+        cell_frac<F32>(q[a], __ldg(s + a * n + id), fg, &c[a], &f);
+        w1[a] = (unsigned)f;
         w0[a] = kWeightOne - w1[a];
       }
 #pragma unroll
@@ -59,12 +58,12 @@ __global__ void __launch_bounds__(kRowThreads) k_deposit(ParticleGeom pg, const 
 #pragma unroll
         for (int dy = 0; dy < 2; ++dy) {
           const int iy = (c[1] + dy) == nm ? 0 : c[1] + dy;
-          const unsigned long long wxy = (dx ? w1[0] : w0[0]) * (dy ? w1[1] : w0[1]);
+          const unsigned wxy = (dx ? w1[0] : w0[0]) * (dy ? w1[1] : w0[1]);   // <= 2^28
           unsigned long long* rrow = rho + ((long long)ix * nm + iy) * nm;
 #pragma unroll
           for (int dz = 0; dz < 2; ++dz) {
             const int iz = (c[2] + dz) == nm ? 0 : c[2] + dz;
-            const unsigned long long w = wxy * (dz ? w1[2] : w0[2]);
+            const unsigned long long w = (unsigned long long)wxy * (dz ? w1[2] : w0[2]);
             if (w) atomicAdd(rrow + iz, w);   // result unused: compiles to a reduction (no return trip)
           }
         }
@@ -74,21 +73,20 @@ __global__ void __launch_bounds__(kRowThreads) k_deposit(ParticleGeom pg, const 
 }
 
 // CIC gather of the three force fields, optionally fused with the COLA kick and drift.
-template <bool KICK>
-__global__ void __launch_bounds__(kRowThreads) k_gather(ParticleGeom pg, const float* __restrict__ f0,
+template <bool KICK, bool F32>
+__global__ void __launch_bounds__(kRowThreads) k_gather(ParticleGeom pg, FixedGeo fg, const float* __restrict__ f0,
                                                        const float* __restrict__ f1, const float* __restrict__ f2,
                                                        long long rs, const float* __restrict__ s_in,
                                                        float* __restrict__ force_out, float* s, float* v,
                                                        const float* __restrict__ psi1,
                                                        const float* __restrict__ psi2, KickDrift kd, int* flags) {
   const long long n = pg.npart;
-  const long long modulus = (long long)pg.n << kFracBits;
   const int nm = pg.n, np = pg.np;
-  const long long nrows = (long long)np * np;
   const float inv_one = 1.0f / kWeightOne;
   bool bad = false;
-  for (long long row = blockIdx.x; row < nrows; row += gridDim.x) {
-    const int qx = (int)(row / np), qy = (int)(row - (long long)qx * np);
+  const int qx = blockIdx.y, qy = blockIdx.x * blockDim.y + threadIdx.y;
+  if (qy < np) {
+    const long long row = (long long)qx * np + qy;
 #pragma unroll 2
     for (int qz = threadIdx.x; qz < np; qz += blockDim.x) {
       const long long id = row * np + qz;
@@ -100,9 +98,9 @@ __global__ void __launch_bounds__(kRowThreads) k_gather(ParticleGeom pg, const f
 #pragma unroll
       for (int a = 0; a < 3; ++a) {
         sv[a] = sp[a * n + id];
-        const long long g = fixed_coord(q[a], sv[a], pg.r_fixed, modulus);
-        c[a] = (int)(g >> kFracBits);
-        w1[a] = (float)((int)(g >> (kFracBits - 14)) & (kWeightOne - 1)) * inv_one;
+        int f;
+        cell_frac<F32>(q[a], sv[a], fg, &c[a], &f);
+        w1[a] = (float)f * inv_one;
       }
       float fx = 0.f, fy = 0.f, fz = 0.f;
 #pragma unroll
@@ -140,7 +138,7 @@ __global__ void __launch_bounds__(kRowThreads) k_gather(ParticleGeom pg, const f
       }
     }
   }
-  if (KICK && __syncthreads_or(bad) && threadIdx.x == 0) atomicOr(flags, 2);
+  if (KICK && __syncthreads_or(bad) && threadIdx.x == 0 && threadIdx.y == 0) atomicOr(flags, 2);
 }
 
 // Exact overflow check of a fixed-point mesh: the 128-bit sum of the (possibly wrapped) cells
@@ -463,16 +461,12 @@ __global__ void k_dense_spectrum(int n, int pc, int nc, const float2* __restrict
 
 }  // namespace
 
-unsigned rows_grid(const ParticleGeom& pg) {
-  const long long rows = (long long)pg.np * pg.np;
-  const long long cap = 152LL * 64;
-  return (unsigned)(rows < cap ? rows : cap);
-}
-
 int launch_deposit(const ParticleGeom& pg, const float* s, unsigned long long* rho, int* flags, cudaStream_t st) {
   (void)flags;
-  const int th = pg.np < kRowThreads ? ((pg.np + 31) / 32) * 32 : kRowThreads;
-  k_deposit<<<rows_grid(pg), th, 0, st>>>(pg, s, rho);
+  const RowBlocks rb = row_blocks(pg.np);
+  const FixedGeo fg = fixed_geo(pg.n, pg.r_fixed);
+  if (pg.n < 2048) k_deposit<true><<<rb.grid, rb.block, 0, st>>>(pg, fg, s, rho);
+  else k_deposit<false><<<rb.grid, rb.block, 0, st>>>(pg, fg, s, rho);
   return check_launch("deposit");
 }
 
@@ -510,13 +504,16 @@ int launch_mass_check(const ParticleGeom& pg, const unsigned long long* rho, boo
 int launch_gather(const ParticleGeom& pg, const float* const f[3], long long rs, const float* s_in,
                   float* force_out, float* s, float* v, const float* psi1, const float* psi2,
                   const KickDrift* kd, int* flags, cudaStream_t st) {
-  const unsigned g = rows_grid(pg);
-  const int th = pg.np < kRowThreads ? ((pg.np + 31) / 32) * 32 : kRowThreads;
-  if (kd)
-    k_gather<true><<<g, th, 0, st>>>(pg, f[0], f[1], f[2], rs, nullptr, nullptr, s, v, psi1, psi2, *kd, flags);
-  else
-    k_gather<false><<<g, th, 0, st>>>(pg, f[0], f[1], f[2], rs, s_in, force_out, nullptr, nullptr, nullptr,
-                                      nullptr, KickDrift{}, flags);
+  const RowBlocks rb = row_blocks(pg.np);
+  const FixedGeo fg = fixed_geo(pg.n, pg.r_fixed);
+  if (kd) {
+    auto* k = pg.n < 2048 ? k_gather<true, true> : k_gather<true, false>;
+    k<<<rb.grid, rb.block, 0, st>>>(pg, fg, f[0], f[1], f[2], rs, nullptr, nullptr, s, v, psi1, psi2, *kd, flags);
+  } else {
+    auto* k = pg.n < 2048 ? k_gather<false, true> : k_gather<false, false>;
+    k<<<rb.grid, rb.block, 0, st>>>(pg, fg, f[0], f[1], f[2], rs, s_in, force_out, nullptr, nullptr, nullptr, nullptr,
+                                    KickDrift{}, flags);
+  }
   return check_launch("gather");
 }
 
