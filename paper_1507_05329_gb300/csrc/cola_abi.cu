@@ -462,8 +462,32 @@ extern "C" int cola_ic_2lpt(cola_ctx* c, const float* wn, float* s, float* v, fl
   for (int i = 0; i < 8; ++i) B[i] = reinterpret_cast<float2*>(static_cast<char*>(c->arena) + i * lbytes);
   const long long n = c->pg.npart;
   const float r = (float)c->p.nmesh / (float)c->p.np;   // lattice spacings -> mesh cells
-  // white noise -> W(k) -> delta_L(k) / np^3
-  COLA_TRY(noise_spectrum(c, wn, B[0]));
+  const float inv_n3 = (float)(1.0 / ((double)g.n * g.n * g.n));
+  const StepScalars& s0 = c->steps[0];
+  COLA_TRY(noise_spectrum(c, wn, B[0]));   // white noise -> W(k), z
+  if (ic_compiled(P)) {
+    // one x pass to delta_L / k^2 and its products with k_x, k_x^2; y passes to those with k_y, k_y^2; the
+    // row pass makes Psi1 and the second-order source of them (fft_ct.cuh); likewise Psi2 from the source
+    COLA_TRY(STAGED(kStFwdY, launch_pencils(P, g, 1, -1, &B[0], 1, c->stream)));
+    float2* const h[3] = {B[0], B[1], B[2]};
+    COLA_TRY(STAGED(kStFwdX, launch_ic_x(P, B[0], h, 3, 1.0f, c->amp_m2, c->stream)));
+    float2* const t0[3] = {B[0], B[3], B[4]};
+    COLA_TRY(STAGED(kStInvY, launch_ic_y(P, B[0], t0, 3, c->stream)));
+    float2* const t1[3] = {B[1], B[5], nullptr};
+    COLA_TRY(STAGED(kStInvY, launch_ic_y(P, B[1], t1, 2, c->stream)));
+    COLA_TRY(STAGED(kStInvY, launch_pencils(P, g, 1, +1, &B[2], 1, c->stream)));
+    float2* const t[6] = {B[0], B[3], B[4], B[1], B[5], B[2]};
+    COLA_TRY(STAGED(kStInvZ, launch_ic_z1(P, t, B[7], psi1, r, c->stream)));
+    COLA_TRY(STAGED(kStFwdY, launch_pencils(P, g, 1, -1, &B[7], 1, c->stream)));
+    float2* const hs[3] = {B[7], B[6], nullptr};
+    COLA_TRY(STAGED(kStFwdX, launch_ic_x(P, B[7], hs, 2, inv_n3, nullptr, c->stream)));
+    float2* const u[3] = {B[7], B[0], nullptr};
+    COLA_TRY(STAGED(kStInvY, launch_ic_y(P, B[7], u, 2, c->stream)));
+    COLA_TRY(STAGED(kStInvY, launch_pencils(P, g, 1, +1, &B[6], 1, c->stream)));
+    float2* const f[3] = {B[6], B[0], B[7]};
+    return STAGED(kStInvZ, launch_ic_z2(P, f, psi1, psi2, s, v, r, (float)s0.d1, (float)s0.d2, c->stream));
+  }
+  // delta_L(k) / np^3
   COLA_TRY(forward3d_yx(c, g, P, B[0]));
   COLA_TRY(STAGED(kStIc, launch_ic_amplitude(g, B[0], c->amp_m2, c->stream)));
   // Psi1 = i k delta_L / k^2
@@ -480,11 +504,9 @@ extern "C" int cola_ic_2lpt(cola_ctx* c, const float* wn, float* s, float* v, fl
   COLA_TRY(STAGED(kStFwdZ, launch_r2c_rows(P, g, kSrcFloat, B[7], 2LL * g.pc, 1.0f, B[7], c->stream)));
   COLA_TRY(forward3d_yx(c, g, P, B[7]));
   // Psi2 = -i k S(k) / k^2
-  const float inv_n3 = (float)(1.0 / ((double)g.n * g.n * g.n));
   for (int j = 0; j < 3; ++j) {
     COLA_TRY(inverse3d_mul(c, g, P, B[7], IcMul{kIcPsi2, j, 0, inv_n3}, B[1], r, psi2 + j * n));
   }
-  const StepScalars& s0 = c->steps[0];
   return STAGED(kStIc, launch_ic_positions(n, psi1, psi2, (float)s0.d1, (float)s0.d2, s, v, c->stream));
 }
 

@@ -103,6 +103,15 @@ struct IcMul;
 int launch_pencils_x_mul(const FftPlan& p, const Grid3& g, const float2* src, const IcMul& mul, float2* dst,
                          cudaStream_t st);
 inline bool fft_compiled(const FftPlan& p) { return p.ops != nullptr; }
+// The 2LPT passes of a compiled length up to 1024 (fft_ct.cuh): x and y passes that make `fields` (2 or 3)
+// spectra from one, the row passes from the spectra to Psi1 and the source, and to Psi2, s and v.
+bool ic_compiled(const FftPlan& p);
+int launch_ic_x(const FftPlan& p, const float2* in, float2* const* out, int fields, float scale, const float* amp_m2,
+                cudaStream_t st);
+int launch_ic_y(const FftPlan& p, const float2* in, float2* const* out, int fields, cudaStream_t st);
+int launch_ic_z1(const FftPlan& p, float2* const t[6], float2* src_k, float* psi1, float r_scale, cudaStream_t st);
+int launch_ic_z2(const FftPlan& p, float2* const f[3], const float* psi1, float* psi2, float* s, float* v,
+                 float r_scale, float d1, float d2, cudaStream_t st);
 // C2C along y (axis 1) or x (axis 0) of `fields` (1 to 3) complex grids; dir = -1 forward, +1 inverse.
 int launch_pencils(const FftPlan& p, const Grid3& g, int axis, int dir, float2* const* data, int fields,
                    cudaStream_t st);

@@ -149,6 +149,27 @@ int launch_c2r_rows_dense(const FftPlan& p, const Grid3&, const float2* data, fl
   return check_launch("c2r_dense");
 }
 
+bool ic_compiled(const FftPlan& p) { return p.ops && p.ops->ic_x; }
+
+int launch_ic_x(const FftPlan& p, const float2* in, float2* const* out, int fields, float scale, const float* amp_m2,
+                cudaStream_t st) {
+  p.ops->ic_x(in, out, fields, scale, amp_m2, p.tab, st);
+  return check_launch("ic_x");
+}
+int launch_ic_y(const FftPlan& p, const float2* in, float2* const* out, int fields, cudaStream_t st) {
+  p.ops->ic_y(in, out, fields, p.tab, st);
+  return check_launch("ic_y");
+}
+int launch_ic_z1(const FftPlan& p, float2* const t[6], float2* src_k, float* psi1, float r_scale, cudaStream_t st) {
+  p.ops->ic_z1(t, src_k, psi1, r_scale, p.tab, st);
+  return check_launch("ic_z1");
+}
+int launch_ic_z2(const FftPlan& p, float2* const f[3], const float* psi1, float* psi2, float* s, float* v,
+                 float r_scale, float d1, float d2, cudaStream_t st) {
+  p.ops->ic_z2(f, psi1, psi2, s, v, r_scale, d1, d2, p.tab, st);
+  return check_launch("ic_z2");
+}
+
 int launch_pencils(const FftPlan& p, const Grid3& g, int axis, int dir, float2* const* data, int fields,
                    cudaStream_t st) {
   if (p.ops) {

@@ -56,21 +56,57 @@ struct Launch {
   }
   static void green(const float2* in, float2* out_f, float2* out_h, const float* dtab, float g_scale,
                     const FftTables& t, float2* spec_out, cudaStream_t st) {
-    go(k_green<N>, dim3(C::chunks, N), C::T, PairCfg<N>::smem, st, in, out_f, out_h, dtab, g_scale, t.fwd, t.rev,
+    go(k_green<N>, dim3(C::chunks, N), C::T, MultiCfg<N, 2>::smem, st, in, out_f, out_h, dtab, g_scale, t.fwd, t.rev,
        spec_out);
   }
   static void pencils_yz(const float2* h, float2* out_y, float2* out_z, const float* dtab, const FftTables& t,
                          cudaStream_t st) {
-    go(k_pen_yz<N>, dim3(C::chunks, N), C::T, PairCfg<N>::smem, st, h, out_y, out_z, dtab, t.fwd);
+    go(k_pen_yz<N>, dim3(C::chunks, N), C::T, MultiCfg<N, 2>::smem, st, h, out_y, out_z, dtab, t.fwd);
+  }
+
+  // three tiles in a CTA: the lattices up to 1024
+  static constexpr bool kIc = MultiCfg<N, 3>::smem <= 227 * 1024;
+  static void ic_x(const float2* in, float2* const* out, int fields, float scale, const float* amp_m2,
+                   const FftTables& t, cudaStream_t st) {
+    if constexpr (kIc) {
+      const dim3 grid(C::chunks, N);
+      if (fields == 3)
+        go(k_ic_x<N, 3, true>, grid, C::T, MultiCfg<N, 3>::smem, st, in, Ptr3{{out[0], out[1], out[2]}}, scale, amp_m2,
+           t.fwd, t.rev);
+      else
+        go(k_ic_x<N, 2, false>, grid, C::T, MultiCfg<N, 2>::smem, st, in, Ptr3{{out[0], out[1], nullptr}}, scale,
+           (const float*)nullptr, t.fwd, t.rev);
+    }
+  }
+  static void ic_y(const float2* in, float2* const* out, int fields, const FftTables& t, cudaStream_t st) {
+    if constexpr (kIc) {
+      const dim3 grid(C::chunks, N);
+      if (fields == 3)
+        go(k_ic_y<N, 3>, grid, C::T, MultiCfg<N, 3>::smem, st, in, Ptr3{{out[0], out[1], out[2]}}, t.fwd);
+      else
+        go(k_ic_y<N, 2>, grid, C::T, MultiCfg<N, 2>::smem, st, in, Ptr3{{out[0], out[1], nullptr}}, t.fwd);
+    }
+  }
+  static void ic_z1(float2* const* f, float2* src_k, float* psi1, float r_scale, const FftTables& t, cudaStream_t st) {
+    if constexpr (kIc)
+      go(k_ic_z1<N>, kRowBlocks, R::T, IcRowCfg<N>::smem, st, IcRows{{f[0], f[1], f[2], f[3], f[4], f[5]}}, src_k, psi1,
+         (long long)N * N * N, r_scale, kPairs, t.fwd);
+  }
+  static void ic_z2(float2* const* f, const float* psi1, float* psi2, float* s, float* v, float r_scale, float d1,
+                    float d2, const FftTables& t, cudaStream_t st) {
+    if constexpr (kIc)
+      go(k_ic_z2<N>, dim3(kRowBlocks, 3), R::T, C2rCfg<N>::smem, st, Ptr3{{f[0], f[1], f[2]}}, psi1, psi2, s, v,
+         (long long)N * N * N, r_scale, d1, d2, kPairs, t.fwd);
   }
 };
 
-// whether part COLA_CT_PART holds size i, and the part's table
+// the launches of size I, and the table of this part's sizes
 template <int I>
 constexpr FftOps ops_of() {
   constexpr int N = kCtSizes[I];
   using L = Launch<N>;
-  return FftOps{N, L::r2c, L::c2r, L::c2r_dense, L::pencils, L::x_mul, L::green, L::pencils_yz};
+  return FftOps{N, L::r2c, L::c2r, L::c2r_dense, L::pencils, L::x_mul, L::green, L::kIc ? L::ic_x : nullptr, L::ic_y,
+                L::ic_z1, L::ic_z2, L::pencils_yz};
 }
 constexpr int kMine = (kCtCount - COLA_CT_PART + COLA_CT_PARTS - 1) / COLA_CT_PARTS;
 template <int... K>

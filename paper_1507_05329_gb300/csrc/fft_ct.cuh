@@ -248,30 +248,29 @@ __global__ void __launch_bounds__(PenCfg<N>::T, PenCfg<N>::minb) k_pen_mul(const
   pen_stage<N, false, PlanOf<N, false>::m - 1, +1, C::T>(TileR<N>{cur}, ColG<JS>{dst + (long long)y * C::PC + col, ok}, tw, tid);
 }
 
-// Two transforms of one tile from here on: middle groups in place in a and in b, last groups to da, db
-template <int N, bool REV, int DIR, int T, int G, class DA, class DB>
-__device__ __forceinline__ void pair_finish(float2* a, float2* b, const DA& da, const DB& db,
-                                            const float2* __restrict__ tw, int tid) {
+// NT transforms at once from here on, in the tiles s, s + tile, ...: middle groups in place, last groups
+// to d[0], d[1], ...
+template <int N, bool REV, int DIR, int T, int G, int NT, class D>
+__device__ __forceinline__ void multi_finish(float2* s, const D (&d)[NT], const float2* __restrict__ tw, int tid) {
   constexpr int M = PlanOf<N, REV>::m;
   if constexpr (G + 1 < M) {
-    pen_inplace<N, REV, G, DIR, T>(a, tw, tid);
-    pen_inplace<N, REV, G, DIR, T>(b, tw, tid);
+#pragma unroll
+    for (int i = 0; i < NT; ++i) pen_inplace<N, REV, G, DIR, T>(s + i * PenCfg<N>::tile, tw, tid);
     __syncthreads();
-    pair_finish<N, REV, DIR, T, G + 1>(a, b, da, db, tw, tid);
+    multi_finish<N, REV, DIR, T, G + 1>(s, d, tw, tid);
   } else {
-    pen_stage<N, REV, G, DIR, T>(TileR<N>{a}, da, tw, tid);
-    pen_stage<N, REV, G, DIR, T>(TileR<N>{b}, db, tw, tid);
+#pragma unroll
+    for (int i = 0; i < NT; ++i) pen_stage<N, REV, G, DIR, T>(TileR<N>{s + i * PenCfg<N>::tile}, d[i], tw, tid);
   }
 }
 
-// Configuration of the passes that hold two tiles
-template <int N>
-struct PairCfg {
+// Configuration of the passes that hold NT tiles
+template <int N, int NT>
+struct MultiCfg {
   using C = PenCfg<N>;
-  static constexpr int T = C::T;
-  static constexpr int smem = 2 * C::tile * 8;
+  static constexpr int smem = NT * C::tile * 8;
   static constexpr int regs = C::ept == 16 ? 80 : 64;
-  static constexpr int minb = imax(1, imin(imin(imax(1, imin(2048, 65536 / regs) / T), 16), (224 * 1024) / (smem + 1024)));
+  static constexpr int minb = imax(1, imin(imin(imax(1, imin(2048, 65536 / regs) / C::T), 16), (224 * 1024) / (smem + 1024)));
 };
 
 // Forward x pass, times g_scale / |m|^2 (H(k), the common factor of the force components
@@ -279,7 +278,7 @@ struct PairCfg {
 // with D constant along x: the y pass makes both from H).  out_h may be in.  spec_out (or null)
 // receives the forward spectrum.
 template <int N>
-__global__ void __launch_bounds__(PairCfg<N>::T, PairCfg<N>::minb) k_green(const float2* in, float2* out_f, float2* out_h,
+__global__ void __launch_bounds__(PenCfg<N>::T, MultiCfg<N, 2>::minb) k_green(const float2* in, float2* out_f, float2* out_h,
                                                                            const float* __restrict__ dtab, float g_scale,
                                                                            const float2* __restrict__ twf,
                                                                            const float2* __restrict__ twr,
@@ -345,13 +344,14 @@ __global__ void __launch_bounds__(PairCfg<N>::T, PairCfg<N>::minb) k_green(const
     }
   }
   __syncthreads();
-  pair_finish<N, true, +1, T, 1>(a, b, ColG<JS>{out_f + off, ok}, ColG<JS>{out_h + off, ok}, twr, tid);
+  const ColG<JS> d[2] = {{out_f + off, ok}, {out_h + off, ok}};
+  multi_finish<N, true, +1, T, 1>(sm, d, twr, tid);
 }
 
 // Inverse y pass of H into the y and z components: i D(k_y) H to out_y and i D(k_z) H to out_z (which
 // may be h: a tile is read whole before it is written)
 template <int N>
-__global__ void __launch_bounds__(PairCfg<N>::T, PairCfg<N>::minb) k_pen_yz(const float2* h, float2* out_y, float2* out_z,
+__global__ void __launch_bounds__(PenCfg<N>::T, MultiCfg<N, 2>::minb) k_pen_yz(const float2* h, float2* out_y, float2* out_z,
                                                                             const float* __restrict__ dtab,
                                                                             const float2* __restrict__ tw) {
   extern __shared__ float2 sm[];
@@ -391,7 +391,131 @@ __global__ void __launch_bounds__(PairCfg<N>::T, PairCfg<N>::minb) k_pen_yz(cons
     }
   }
   __syncthreads();
-  pair_finish<N, false, +1, T, 1>(a, b, ColG<JS>{out_y + off, ok}, ColG<JS>{out_z + off, ok}, tw, tid);
+  const ColG<JS> d[2] = {{out_y + off, ok}, {out_z + off, ok}};
+  multi_finish<N, false, +1, T, 1>(sm, d, tw, tid);
+}
+
+// ---- 2LPT (x and y passes) ----------------------------------------------------------------------
+// The 2LPT fields are delta_L(k) / k^2 times products of at most two wave numbers.  A wave number of an
+// axis is constant along the other axes' pencils, so one forward x pass makes the inverse x transforms of
+// delta/k^2 times 1, k_x and k_x^2, and each y pass those times 1, k_y and k_y^2 as far as they are
+// needed; k_z waits for the row pass.  3 x and 6 y transforms then serve the nine first-order fields,
+// where a transform of its own for each takes nine and nine (and a multiply each).  The factor of a single
+// derivative is 0 on its Nyquist plane, a square keeps it; factors i are left to the row pass.
+// With the row passes below (Hessians and source on chip, first positions written with Psi2) a call is 12
+// launches and moves 52 field-sized reads and writes where 45 launches moved 120: 256^3 lattice 1706 -> 917
+// us (0.51 ms for the 52 at the copy rate), 32^3 271 -> 82 us.
+
+// z times k^p, p = 0, 1, 2, k = 2 pi m / n of storage index j
+template <int N, int PW>
+__device__ __forceinline__ float2 times_k(float2 z, int j) {
+  constexpr float kf = 6.283185307179586f / N;
+  const int m = j < N / 2 ? j : j - N;
+  if constexpr (PW == 0) return z;
+  else if constexpr (PW == 1) return (2 * j == N ? 0.0f : m * kf) * z;
+  else return (m * kf) * (m * kf) * z;
+}
+// first group of the inverse transforms of v times 1, k, .., k^(NT-1) into the tiles s, s + tile, ..
+template <int N, bool REV, int NT, int PW = 0, int R>
+__device__ __forceinline__ void powers_stage(const float2 (&z)[R], int b, int w, float2* s, const float2* __restrict__ tw) {
+  if constexpr (PW < NT) {
+    using Q = Group<N, REV, 0, +1>;
+    static_assert(Q::R == R, "a first group's butterfly");
+    float2 v[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) v[r] = times_k<N, PW>(z[r], b + r * Q::NB);
+    Q::run(v, tw, 0);
+#pragma unroll
+    for (int r = 0; r < R; ++r) s[PW * PenCfg<N>::tile + ((b * R + r) << PenCfg<N>::lw) + w] = v[r];
+    powers_stage<N, REV, NT, PW + 1>(z, b, w, s, tw);
+  }
+}
+
+// Forward x transform of in, times scale / k^2 (and the amplitude amp_m2[|m|^2] when AMP), and the inverse
+// x transforms of that times 1, k_x, .. (NT of them) into out.p[0..NT-1]; out.p[0] may be in.
+template <int N, int NT, bool AMP>
+__global__ void __launch_bounds__(PenCfg<N>::T, MultiCfg<N, NT>::minb) k_ic_x(const float2* in, Ptr3 out, float scale,
+                                                                              const float* __restrict__ amp_m2,
+                                                                              const float2* __restrict__ twf,
+                                                                              const float2* __restrict__ twr) {
+  extern __shared__ float2 sm[];
+  using C = PenCfg<N>;
+  constexpr int T = C::T, M = PlanOf<N, false>::m;
+  constexpr long long JS = (long long)N * C::PC;
+  const int tid = threadIdx.x, col = blockIdx.x * C::W + (tid & (C::W - 1)), y = blockIdx.y;
+  const bool ok = col < C::NC;
+  const long long off = (long long)y * C::PC + col;
+  pen_stage<N, false, 0, -1, T>(ColG<JS>{const_cast<float2*>(in) + off, ok}, TileW<N>{sm}, twf, tid);
+  __syncthreads();
+  const float2* cur = pen_middle<N, false, -1, T, true>(sm, sm + C::tile, twf, tid);
+  using L = Group<N, false, M - 1, -1>;
+  constexpr int TOT = L::NB << C::lw, IT = (TOT + T - 1) / T;
+  constexpr float kf = 6.283185307179586f / N;
+  float2 spec[IT][L::R];
+  const int my = y < N / 2 ? y : y - N;
+#pragma unroll
+  for (int it = 0; it < IT; ++it) {
+    const int idx = tid + it * T;
+    if (TOT % T == 0 || idx < TOT) {
+      const int bb = idx >> C::lw;
+#pragma unroll
+      for (int r = 0; r < L::R; ++r) spec[it][r] = cur[idx + r * (L::NB << C::lw)];
+      L::run(spec[it], twf, bb);
+      const int myz = my * my + col * col;
+#pragma unroll
+      for (int r = 0; r < L::R; ++r) {
+        const int j = bb + r * L::NS;
+        const int mx = j < N / 2 ? j : j - N;
+        const int m2 = mx * mx + myz;
+        float g = m2 > 0 ? scale / ((float)m2 * kf * kf) : 0.0f;
+        if (AMP && ok) g *= __ldg(amp_m2 + m2);
+        spec[it][r] = g * spec[it][r];
+      }
+    }
+  }
+  __syncthreads();   // the forward's buffers are free
+#pragma unroll
+  for (int it = 0; it < IT; ++it) {
+    const int idx = tid + it * T;
+    if (TOT % T == 0 || idx < TOT) powers_stage<N, true, NT>(spec[it], idx >> C::lw, idx & (C::W - 1), sm, twr);
+  }
+  __syncthreads();
+  ColG<JS> d[NT];
+#pragma unroll
+  for (int i = 0; i < NT; ++i) d[i] = ColG<JS>{out.p[i] + off, ok};
+  multi_finish<N, true, +1, T, 1>(sm, d, twr, tid);
+}
+
+// Inverse y transforms of in times 1, k_y, .. (NT of them) into out.p[0..NT-1]; out.p[0] may be in.
+template <int N, int NT>
+__global__ void __launch_bounds__(PenCfg<N>::T, MultiCfg<N, NT>::minb) k_ic_y(const float2* in, Ptr3 out,
+                                                                              const float2* __restrict__ tw) {
+  extern __shared__ float2 sm[];
+  using C = PenCfg<N>;
+  using Q = Group<N, false, 0, +1>;
+  constexpr int T = C::T;
+  constexpr long long JS = C::PC, OS = (long long)N * C::PC;
+  const int tid = threadIdx.x, col = blockIdx.x * C::W + (tid & (C::W - 1));
+  const bool ok = col < C::NC;
+  const long long off = blockIdx.y * OS + col;
+  const ColG<JS> src{const_cast<float2*>(in) + off, ok};
+  constexpr int TOT = Q::NB << C::lw, IT = (TOT + T - 1) / T;
+#pragma unroll(IT <= 2 ? IT : 1)
+  for (int it = 0; it < IT; ++it) {
+    const int idx = tid + it * T;
+    if (TOT % T == 0 || idx < TOT) {
+      const int w = idx & (C::W - 1), bb = idx >> C::lw;
+      float2 z[Q::R];
+#pragma unroll
+      for (int r = 0; r < Q::R; ++r) z[r] = src(bb + r * Q::NB, w);
+      powers_stage<N, false, NT>(z, bb, w, sm, tw);
+    }
+  }
+  __syncthreads();
+  ColG<JS> d[NT];
+#pragma unroll
+  for (int i = 0; i < NT; ++i) d[i] = ColG<JS>{out.p[i] + off, ok};
+  multi_finish<N, false, +1, T, 1>(sm, d, tw, tid);
 }
 
 // ---- row pairs (the contiguous axis) -------------------------------------------------------------
@@ -505,6 +629,22 @@ struct RowPairLoad {
   }
 };
 
+// half rows of the two real rows that a transformed complex row holds
+template <int N>
+__device__ __forceinline__ void untangle_rows(const float2* res, float2* dst, long long pair0, long long npairs, int tid) {
+  using C = RowCfg<N>;
+  constexpr int NH = N / 2, TOT = C::pairs * (NH + 1);
+  for (int idx = tid; idx < TOT; idx += C::T) {
+    const int p = idx / (NH + 1), k = idx - p * (NH + 1);
+    if (pair0 + p >= npairs) break;
+    const float2 zk = res[p * C::RS + rpos(k)];
+    const float2 zn = res[p * C::RS + rpos(k == 0 ? 0 : N - k)];
+    float2* o = dst + 2 * (pair0 + p) * C::PC + k;
+    o[0] = make_float2(0.5f * (zk.x + zn.x), 0.5f * (zk.y - zn.y));
+    o[C::PC] = make_float2(0.5f * (zk.y + zn.y), -0.5f * (zk.x - zn.x));
+  }
+}
+
 template <int N>
 struct R2cCfg {
   static constexpr int bufs = 2;
@@ -531,16 +671,7 @@ __global__ void __launch_bounds__(RowCfg<N>::T, RowCfg<N>::minb(2)) k_r2c(const 
   float2* res = cur == a ? b : a;
   row_stage<N, PlanOf<N, false>::m - 1, -1>(RowSm<N>{cur}, RowSm<N>{res}, tw, tid);
   __syncthreads();
-  constexpr int NH = N / 2, TOT = C::pairs * (NH + 1);
-  for (int idx = tid; idx < TOT; idx += C::T) {
-    const int p = idx / (NH + 1), k = idx - p * (NH + 1);
-    if (pair0 + p >= npairs) break;
-    const float2 zk = res[p * C::RS + rpos(k)];
-    const float2 zn = res[p * C::RS + rpos(k == 0 ? 0 : N - k)];
-    float2* o = dst + 2 * (pair0 + p) * C::PC + k;
-    o[0] = make_float2(0.5f * (zk.x + zn.x), 0.5f * (zk.y - zn.y));
-    o[C::PC] = make_float2(0.5f * (zk.y + zn.y), -0.5f * (zk.x - zn.x));
-  }
+  untangle_rows<N>(res, dst, pair0, npairs, tid);
 }
 
 // C[k] = A[k] + i B[k] of two Hermitian half rows
@@ -609,6 +740,197 @@ __global__ void __launch_bounds__(RowCfg<N>::T, RowCfg<N>::minb(C2rCfg<N>::bufs)
   const RealPairStore<N, DENSE> o{DENSE ? out : reinterpret_cast<float*>(d), DENSE ? (long long)N : 2LL * C::PC, pair0,
                                   npairs, scale};
   row_stage<N, PlanOf<N, false>::m - 1, +1>(RowSm<N>{cur}, o, tw, tid);
+}
+
+// ---- 2LPT (row passes) ----------------------------------------------------------------------------
+// A Hermitian half row's entry kk times the factor of MODE: k^p (p = MODE & 3, as times_k) and i (MODE & 4).
+template <int N, int MODE>
+__device__ __forceinline__ float2 ic_entry(float2 z, int kk) {
+  z = times_k<N, MODE & 3>(z, kk);
+  return (MODE & 4) ? make_float2(-z.y, z.x) : z;
+}
+// Rows A and B (as complex rows A + i B after the transform) of two half rows per pair slot, with factors
+template <int N, int MA, int MB>
+struct FieldPairLoad {
+  const float2* a;   // row of slot 0
+  const float2* b;
+  long long stride;  // entries between slots' rows
+  int slots;         // valid slots
+  template <int STEP, bool, int R>
+  __device__ __forceinline__ void load(int p, int j0, float2 (&v)[R]) const {
+    constexpr int NH = N / 2;
+    const float2* ra = a + p * stride;
+    const float2* rb = b + p * stride;
+    const bool ok = p < slots;
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      const int k = j0 + r * STEP, kk = k <= NH ? k : N - k;
+      float2 A = make_float2(0.f, 0.f), B = make_float2(0.f, 0.f);
+      if (ok) {
+        A = ic_entry<N, MA>(ra[kk], kk);
+        B = ic_entry<N, MB>(rb[kk], kk);
+      }
+      if (kk == 0 || kk == NH) {
+        A.y = 0.f;
+        B.y = 0.f;
+      }
+      v[r] = k <= NH ? make_float2(A.x - B.y, A.y + B.x) : make_float2(A.x + B.y, B.x - A.y);
+    }
+  }
+};
+
+template <int N>
+struct IcRowCfg {
+  using C = RowCfg<N>;
+  static constexpr int smem = 3 * C::buf * 8;
+  static constexpr int regs = C::ept == 16 ? 128 : 96;
+  static constexpr int minb = imax(1, imin(imin(imax(1, imin(2048, 65536 / regs) / C::T), 16), (224 * 1024) / (smem + 1024)));
+};
+
+// all groups but the last of the inverse transform of src; returns the buffer the last group reads
+template <int N, class Src>
+__device__ __forceinline__ const float2* ic_row_inverse(const Src& src, float2* a, float2* b, const float2* __restrict__ tw,
+                                                        int tid) {
+  __syncthreads();   // the buffers' last readers are done
+  row_stage<N, 0, +1>(src, RowSm<N>{a}, tw, tid);
+  __syncthreads();
+  return row_middle<N, +1>(a, b, tw, tid);
+}
+// the last group of the rows in buf, each butterfly's values (at positions b + r NS of slot p) to f(it, p, b, v)
+template <int N, class F>
+__device__ __forceinline__ void ic_row_last(const float2* buf, const float2* __restrict__ tw, int tid, F&& f) {
+  using Q = Group<N, false, PlanOf<N, false>::m - 1, +1>;
+  using C = RowCfg<N>;
+  constexpr int TOT = C::pairs * Q::NB, IT = (TOT + C::T - 1) / C::T;
+#pragma unroll
+  for (int it = 0; it < IT; ++it) {
+    const int idx = tid + it * C::T;
+    if (TOT % C::T == 0 || idx < TOT) {
+      const int p = idx / Q::NB, b = idx - p * Q::NB;
+      float2 v[Q::R];
+      RowSm<N>{const_cast<float2*>(buf)}.template load<Q::NB, false>(p, b, v);
+      Q::run(v, tw, b);
+      f(it, p, b, v);
+    }
+  }
+}
+
+struct IcRows {
+  const float2* t[6];   // spectra over k_z: 1, k_y, k_y^2 (of the x transform), k_x, k_x k_y, k_x^2
+};
+
+// The first-order fields of row pairs: Psi1 (dense rows times r_scale into psi1, component stride npart),
+// the Hessians and from them the second-order source S = sum_{i<j} h_ii h_jj - h_ij^2, whose forward row
+// transform goes to src_k.  The Hessians and the source stay on chip.  Two Hessians of one row make one
+// complex transform, so that a thread meets both at the same site; Psi1_x and Psi1_y likewise, Psi1_z with
+// the other row's.
+template <int N>
+__global__ void __launch_bounds__(RowCfg<N>::T, IcRowCfg<N>::minb) k_ic_z1(IcRows f, float2* src_k, float* psi1,
+                                                                           long long npart, float r_scale, long long npairs,
+                                                                           const float2* __restrict__ tw) {
+  extern __shared__ float2 sm[];
+  using C = RowCfg<N>;
+  using Q = Group<N, false, PlanOf<N, false>::m - 1, +1>;
+  constexpr int TOT = C::pairs * Q::NB, IT = (TOT + C::T - 1) / C::T, NS = Q::NS;
+  const int tid = threadIdx.x;
+  const long long pair0 = (long long)blockIdx.x * C::pairs;
+  const int slots = npairs - pair0 < C::pairs ? (int)(npairs - pair0) : C::pairs;
+  float2* a = sm;
+  float2* b = sm + C::buf;
+  float* src = reinterpret_cast<float*>(sm + 2 * C::buf);   // the source: (row 2p, row 2p + 1) of a site as one complex
+#pragma unroll 1
+  for (int row = 0; row < 2; ++row) {
+    const long long o = (2 * pair0 + row) * C::PC, st = 2 * C::PC;
+    float s[IT][Q::R], sum[IT][Q::R];
+    ic_row_last<N>(ic_row_inverse<N>(FieldPairLoad<N, 0, 0>{f.t[5] + o, f.t[2] + o, st, slots}, a, b, tw, tid), tw, tid,
+                   [&](int it, int, int, float2(&v)[Q::R]) {   // h00, h11
+#pragma unroll
+                     for (int r = 0; r < Q::R; ++r) {
+                       s[it][r] = v[r].x * v[r].y;
+                       sum[it][r] = v[r].x + v[r].y;
+                     }
+                   });
+    ic_row_last<N>(ic_row_inverse<N>(FieldPairLoad<N, 2, 1>{f.t[0] + o, f.t[1] + o, st, slots}, a, b, tw, tid), tw, tid,
+                   [&](int it, int, int, float2(&v)[Q::R]) {   // h22, h12
+#pragma unroll
+                     for (int r = 0; r < Q::R; ++r) s[it][r] += sum[it][r] * v[r].x - v[r].y * v[r].y;
+                   });
+    ic_row_last<N>(ic_row_inverse<N>(FieldPairLoad<N, 0, 1>{f.t[4] + o, f.t[3] + o, st, slots}, a, b, tw, tid), tw, tid,
+                   [&](int it, int p, int bb, float2(&v)[Q::R]) {   // h01, h02
+#pragma unroll
+                     for (int r = 0; r < Q::R; ++r)
+                       src[2 * (p * C::RS + rpos(bb + r * NS)) + row] = s[it][r] - v[r].x * v[r].x - v[r].y * v[r].y;
+                   });
+    ic_row_last<N>(ic_row_inverse<N>(FieldPairLoad<N, 4, 4>{f.t[3] + o, f.t[1] + o, st, slots}, a, b, tw, tid), tw, tid,
+                   [&](int, int p, int bb, float2(&v)[Q::R]) {   // Psi1_x, Psi1_y
+                     if (p >= slots) return;
+                     float* q = psi1 + (2 * (pair0 + p) + row) * N + bb;
+#pragma unroll
+                     for (int r = 0; r < Q::R; ++r) {
+                       q[r * NS] = v[r].x * r_scale;
+                       q[npart + r * NS] = v[r].y * r_scale;
+                     }
+                   });
+  }
+  {
+    const long long o = 2 * pair0 * C::PC;
+    ic_row_last<N>(ic_row_inverse<N>(FieldPairLoad<N, 5, 5>{f.t[0] + o, f.t[0] + o + C::PC, 2 * C::PC, slots}, a, b, tw, tid),
+                   tw, tid, [&](int, int p, int bb, float2(&v)[Q::R]) {   // Psi1_z of both rows
+                     if (p >= slots) return;
+                     float* q = psi1 + 2 * npart + 2 * (pair0 + p) * N + bb;
+#pragma unroll
+                     for (int r = 0; r < Q::R; ++r) {
+                       q[r * NS] = v[r].x * r_scale;
+                       q[N + r * NS] = v[r].y * r_scale;
+                     }
+                   });
+  }
+  __syncthreads();
+  // the source's forward rows
+  row_stage<N, 0, -1>(RowSm<N>{sm + 2 * C::buf}, RowSm<N>{a}, tw, tid);
+  __syncthreads();
+  float2* cur = row_middle<N, -1>(a, b, tw, tid);
+  float2* res = cur == a ? b : a;
+  row_stage<N, PlanOf<N, false>::m - 1, -1>(RowSm<N>{cur}, RowSm<N>{res}, tw, tid);
+  __syncthreads();
+  untangle_rows<N>(res, src_k, pair0, npairs, tid);
+}
+
+// Psi2 (component blockIdx.y, factors -i k_j) of row pairs into dense rows times r_scale, and the first
+// positions s = d1 Psi1 + d2 Psi2 and velocities 0 of the same particles.
+template <int N>
+__global__ void __launch_bounds__(RowCfg<N>::T, RowCfg<N>::minb(C2rCfg<N>::bufs)) k_ic_z2(Ptr3 f, const float* __restrict__ psi1,
+                                                                                         float* psi2, float* s, float* v0,
+                                                                                         long long npart, float r_scale, float d1,
+                                                                                         float d2, long long npairs,
+                                                                                         const float2* __restrict__ tw) {
+  extern __shared__ float2 sm[];
+  using C = RowCfg<N>;
+  using Q = Group<N, false, PlanOf<N, false>::m - 1, +1>;
+  const int tid = threadIdx.x, comp = blockIdx.y;
+  const long long pair0 = (long long)blockIdx.x * C::pairs;
+  const int slots = npairs - pair0 < C::pairs ? (int)(npairs - pair0) : C::pairs;
+  const float2* row = f.p[comp] + 2 * pair0 * C::PC;
+  // i k_z for z, i for x and y (their k is in the spectrum); the sign of -i with the scale
+  if (comp == 2) row_stage<N, 0, +1>(FieldPairLoad<N, 5, 5>{row, row + C::PC, 2 * C::PC, slots}, RowSm<N>{sm}, tw, tid);
+  else row_stage<N, 0, +1>(FieldPairLoad<N, 4, 4>{row, row + C::PC, 2 * C::PC, slots}, RowSm<N>{sm}, tw, tid);
+  __syncthreads();
+  const float2* cur = row_middle<N, +1>(sm, sm + C::buf, tw, tid);
+  ic_row_last<N>(cur, tw, tid, [&](int, int p, int bb, float2(&v)[Q::R]) {
+    if (p >= slots) return;
+    const long long o = comp * npart + 2 * (pair0 + p) * N + bb;
+#pragma unroll
+    for (int r = 0; r < Q::R; ++r) {
+      const float p2[2] = {v[r].x * -r_scale, v[r].y * -r_scale};
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const long long i = o + h * N + r * Q::NS;
+        psi2[i] = p2[h];
+        s[i] = d1 * psi1[i] + d2 * p2[h];
+        v0[i] = 0.0f;
+      }
+    }
+  });
 }
 
 }  // namespace ct

@@ -19,6 +19,13 @@ struct FftOps {
   void (*x_mul)(const float2* src, const IcMul& mul, float2* dst, const FftTables&, cudaStream_t);
   void (*green)(const float2* in, float2* out_f, float2* out_h, const float* dtab, float g_scale, const FftTables&,
                 float2* spec_out, cudaStream_t);
+  // 2LPT fields (null where three tiles do not fit a CTA); see fft_ct.cuh
+  void (*ic_x)(const float2* in, float2* const* out, int fields, float scale, const float* amp_m2, const FftTables&,
+               cudaStream_t);
+  void (*ic_y)(const float2* in, float2* const* out, int fields, const FftTables&, cudaStream_t);
+  void (*ic_z1)(float2* const* t, float2* src_k, float* psi1, float r_scale, const FftTables&, cudaStream_t);
+  void (*ic_z2)(float2* const* f, const float* psi1, float* psi2, float* s, float* v, float r_scale, float d1, float d2,
+                const FftTables&, cudaStream_t);
   void (*pencils_yz)(const float2* h, float2* out_y, float2* out_z, const float* dtab, const FftTables&, cudaStream_t);
 };
 
