@@ -481,7 +481,7 @@ __global__ void __launch_bounds__(kDepositThreads, 4) k_deposit_tiles(ParticleGe
       tlo += wpart[2 * w];
       thi += wpart[2 * w + 1] + (tlo < wpart[2 * w]);
     }
-    tile_mass[2 * blockIdx.x] = tlo;   // one pair per tile, no atomics; launch_mass_reduce sums them
+    tile_mass[2 * blockIdx.x] = tlo;   // one pair per tile, no atomics; launch_mass_check sums them
     tile_mass[2 * blockIdx.x + 1] = thi;
   }
 }

@@ -152,7 +152,7 @@ int forward_yz(cola_ctx* c, const unsigned long long* rho, bool check_mass) {
   const float scale = (float)((double)n3 / ((double)c->pg.npart * 4398046511104.0));   // N^3 / (n 2^42)
   COLA_TRY(STAGED(kStFwdZ, launch_r2c_rows(c->mplan, g, kSrcFixedPoint, rho, g.n, scale, c->cbuf[2], c->stream,
                                            check_mass ? c->mass_acc : nullptr)));
-  if (check_mass) COLA_TRY(launch_mass_check(c->pg, nullptr, false, c->mass_acc, c->flags, c->stream));
+  if (check_mass) COLA_TRY(launch_mass_check(c->pg, nullptr, nullptr, 0, c->mass_acc, c->flags, c->stream));
   COLA_TRY(STAGED(kStFwdY, launch_pencils(c->mplan, g, 1, -1, &c->cbuf[2], 1, c->stream)));
   return COLA_OK;
 }
@@ -169,8 +169,7 @@ int deposit_and_forward_yz(cola_ctx* c, const float* s) {
     COLA_TRY(STAGED(kStDeposit, launch_deposit_tiles(c->pg, c->bg, s, c->bb, nullptr, c->stream, delta, scale,
                                                      c->tile_mass)));
     COLA_TRY(STAGED(kStFwdZ, launch_r2c_rows(c->mplan, g, kSrcFloat, delta, g.n, 1.0f, c->cbuf[2], c->stream)));
-    COLA_TRY(launch_mass_reduce(c->tile_mass, c->bg.tiles, c->mass_acc, c->stream));
-    COLA_TRY(launch_mass_check(c->pg, nullptr, false, c->mass_acc, c->flags, c->stream));
+    COLA_TRY(launch_mass_check(c->pg, nullptr, c->tile_mass, c->bg.tiles, c->mass_acc, c->flags, c->stream));
     return STAGED(kStFwdY, launch_pencils(c->mplan, g, 1, -1, &c->cbuf[2], 1, c->stream));
   }
   COLA_TRY(deposit_mesh(c, s, c->rho));
@@ -517,7 +516,7 @@ extern "C" int cola_deposit(cola_ctx* c, const float* s, unsigned long long* rho
   const size_t n3 = (size_t)c->mesh.n * c->mesh.n * c->mesh.n;
   (void)n3;
   COLA_TRY(deposit_mesh(c, s, rho));
-  return launch_mass_check(c->pg, rho, true, c->mass_acc, c->flags, c->stream);
+  return launch_mass_check(c->pg, rho, nullptr, 0, c->mass_acc, c->flags, c->stream);
 }
 
 extern "C" int cola_density_spectrum(cola_ctx* c, const float* s, float* delta_k) {

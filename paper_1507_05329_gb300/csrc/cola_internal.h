@@ -144,12 +144,10 @@ inline RowBlocks row_blocks(int np) {
 
 int launch_deposit(const ParticleGeom& pg, const float* s, unsigned long long* rho, int* flags,
                    cudaStream_t st);
-// Sets flags bit 0 if the 128-bit total in acc (accumulated by the fixed-point R2C pass, or by
-// summing rho here when sum_mesh) differs from n 2^42, i.e. if some cell wrapped; resets acc.
-int launch_mass_check(const ParticleGeom& pg, const unsigned long long* rho, bool sum_mesh, unsigned long long* acc,
-                      int* flags, cudaStream_t st);
-// Adds the 128-bit sum of m (lo, hi) pairs to the accumulator acc (kMassSlots pairs).
-int launch_mass_reduce(const unsigned long long* pairs, long long m, unsigned long long* acc, cudaStream_t st);
+// Sets flags bit 0 if the 128-bit total of acc (accumulated by the fixed-point R2C pass), of the cells of
+// rho (or null) and of m (lo, hi) pairs differs from n 2^42, i.e. if some cell wrapped; resets acc.
+int launch_mass_check(const ParticleGeom& pg, const unsigned long long* rho, const unsigned long long* pairs, long long m,
+                      unsigned long long* acc, int* flags, cudaStream_t st);
 
 // Fixed-point particle coordinates shared by the deposit, the gathers, the adjoint and FoF: a
 // particle at lattice index q (per axis) and displacement s (mesh cells) sits at
@@ -274,7 +272,7 @@ void particle_schedule(const BinGeom& b, int nmesh, long long npart, bool* binne
 int launch_binning(const ParticleGeom& pg, const BinGeom& b, const float* s, BinBuffers& bb, cudaStream_t st);
 // delta_out == nullptr: writes the fixed-point mesh rho.  Else writes the density contrast
 // fixed_to_delta(rho, scale) as dense float rows to delta_out (rho is not written) and each tile's
-// exact 128-bit total to tile_mass[2 tile .. 2 tile + 1] (for launch_mass_reduce).
+// exact 128-bit total to tile_mass[2 tile .. 2 tile + 1] (for launch_mass_check).
 int launch_deposit_tiles(const ParticleGeom& pg, const BinGeom& b, const float* s, const BinBuffers& bb,
                          unsigned long long* rho, cudaStream_t st, float* delta_out = nullptr, float scale = 0.0f,
                          unsigned long long* tile_mass = nullptr);

@@ -142,18 +142,38 @@ __global__ void __launch_bounds__(kRowThreads) k_gather(ParticleGeom pg, FixedGe
 }
 
 // Exact overflow check of a fixed-point mesh: the 128-bit sum of the (possibly wrapped) cells
-// equals n 2^42 exactly unless some cell wrapped past 2^64 (each wrap removes 2^64).
-__global__ void k_mass_check(const unsigned long long* __restrict__ acc, unsigned long long expect_lo,
-                             unsigned long long expect_hi, unsigned long long* acc_reset, int* flags) {
-  if (threadIdx.x == 0 && blockIdx.x == 0) {
-    unsigned long long lo = 0ULL, hi = 0ULL;
-    for (int k = 0; k < kMassSlots; ++k) {
-      const unsigned long long l = acc[2 * k];
-      lo += l;
-      hi += acc[2 * k + 1] + (lo < l);
-    }
-    if (lo != expect_lo || hi != expect_hi) atomicOr(flags, 1);
-    for (int k = 0; k < 2 * kMassSlots; ++k) acc_reset[k] = 0ULL;
+// equals n 2^42 exactly unless some cell wrapped past 2^64 (each wrap removes 2^64).  One block sums the
+// accumulator slots and m further (lo, hi) pairs (one thread over the 128 slots took 12 us a step).
+constexpr int kCheckThreads = 1024;
+__device__ __forceinline__ void add128(unsigned long long& lo, unsigned long long& hi, unsigned long long l,
+                                       unsigned long long h) {
+  lo += l;
+  hi += h + (lo < l);
+}
+__global__ void __launch_bounds__(kCheckThreads) k_mass_check(unsigned long long* acc, const unsigned long long* __restrict__ pairs,
+                                                              int m, unsigned long long expect_lo,
+                                                              unsigned long long expect_hi, int* flags) {
+  __shared__ unsigned long long part[2 * kCheckThreads / 32];
+  unsigned long long lo = 0ULL, hi = 0ULL;
+  if (threadIdx.x < kMassSlots) {
+    lo = acc[2 * threadIdx.x];
+    hi = acc[2 * threadIdx.x + 1];
+    acc[2 * threadIdx.x] = acc[2 * threadIdx.x + 1] = 0ULL;
+  }
+  for (int i = threadIdx.x; i < m; i += kCheckThreads) add128(lo, hi, pairs[2 * i], pairs[2 * i + 1]);
+  for (int off = 16; off > 0; off >>= 1)
+    add128(lo, hi, __shfl_down_sync(0xffffffffu, lo, off), __shfl_down_sync(0xffffffffu, hi, off));
+  if ((threadIdx.x & 31) == 0) {
+    part[threadIdx.x >> 5] = lo;
+    part[kCheckThreads / 32 + (threadIdx.x >> 5)] = hi;
+  }
+  __syncthreads();
+  if (threadIdx.x < 32) {
+    lo = part[threadIdx.x];
+    hi = part[kCheckThreads / 32 + threadIdx.x];
+    for (int off = 16; off > 0; off >>= 1)
+      add128(lo, hi, __shfl_down_sync(0xffffffffu, lo, off), __shfl_down_sync(0xffffffffu, hi, off));
+    if (threadIdx.x == 0 && (lo != expect_lo || hi != expect_hi)) atomicOr(flags, 1);
   }
 }
 
@@ -267,7 +287,8 @@ constexpr int kMaxBins = 128;
 // V / particles is subtracted from the bin mean.
 
 // bin of |m|^2 = m2 among edges[0..nbins] (edges[b] <= m2 < edges[b+1]), -1 outside
-__device__ __forceinline__ int pk_bin_of(long long m2, const long long* edges, int nbins) {
+template <class I>
+__device__ __forceinline__ int pk_bin_of(I m2, const I* edges, int nbins) {
   if (m2 < edges[0] || m2 >= edges[nbins]) return -1;
   int lo = 0, hi = nbins;
   while (hi - lo > 1) {
@@ -280,11 +301,19 @@ __device__ __forceinline__ int pk_bin_of(long long m2, const long long* edges, i
 // the half space of §3.3: {kz > 0} U {kz = 0, ky > 0} U {kz = ky = 0, kx > 0}
 __device__ __forceinline__ bool pk_half(int mx, int my, int kz) { return kz > 0 || my > 0 || (my == 0 && mx > 0); }
 
+// first lane of the run of equal bins that the lane is in, and whether it is the run's last
+__device__ __forceinline__ int pk_run(int bin, int lane, bool* last) {
+  const int before = __shfl_up_sync(0xffffffffu, bin, 1);
+  const unsigned heads = __ballot_sync(0xffffffffu, lane == 0 || before != bin);
+  *last = lane == 31 || (heads >> (lane + 1) & 1u);
+  return 31 - __clz(heads & (0xffffffffu >> (31 - lane)));
+}
+
 __global__ void __launch_bounds__(kPkThreads) k_pk_geometry(int n, int nc, const long long* __restrict__ edges_g,
                                                             int nbins, double* partials) {
   __shared__ long long edges[kMaxBins + 1];
   __shared__ double hk[kPkWarps][kMaxBins];
-  __shared__ long long hc[kPkWarps][kMaxBins];
+  __shared__ int hc[kPkWarps][kMaxBins];   // below 2^31 modes per warp: n^2 (n/2 + 1) / 9728
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   for (int i = threadIdx.x; i <= nbins; i += blockDim.x) edges[i] = edges_g[i];
   for (int i = threadIdx.x; i < kPkWarps * kMaxBins; i += blockDim.x) {
@@ -292,10 +321,9 @@ __global__ void __launch_bounds__(kPkThreads) k_pk_geometry(int n, int nc, const
     (&hc[0][0])[i] = 0;
   }
   __syncthreads();
-  const long long nrows = (long long)n * n;
-  for (long long row = (long long)blockIdx.x * kPkWarps + warp; row < nrows;
-       row += (long long)gridDim.x * kPkWarps) {
-    const int mx = signed_mode((int)(row / n), n), my = signed_mode((int)(row % n), n);
+  const int nrows = n * n;
+  for (int row = blockIdx.x * kPkWarps + warp; row < nrows; row += gridDim.x * kPkWarps) {
+    const int mx = signed_mode(row / n, n), my = signed_mode(row % n, n);
     for (int kz0 = 0; kz0 < nc; kz0 += 32) {
       const int kz = kz0 + lane;
       int bin = -1;
@@ -305,21 +333,16 @@ __global__ void __launch_bounds__(kPkThreads) k_pk_geometry(int n, int nc, const
         bin = pk_bin_of(m2, edges, nbins);
         if (bin >= 0) kk = sqrt((double)m2);
       }
-      long long c = bin >= 0 ? 1 : 0;
+      bool last;
+      const int head = pk_run(bin, lane, &last);
 #pragma unroll
       for (int d = 1; d < 32; d <<= 1) {
-        const int ob = __shfl_up_sync(0xffffffffu, bin, d);
         const double ok = __shfl_up_sync(0xffffffffu, kk, d);
-        const long long oc = __shfl_up_sync(0xffffffffu, c, d);
-        if (lane >= d && ob == bin) {
-          kk += ok;
-          c += oc;
-        }
+        if (lane - d >= head) kk += ok;
       }
-      const int nb_next = __shfl_down_sync(0xffffffffu, bin, 1);
-      if (bin >= 0 && (lane == 31 || nb_next != bin)) {
+      if (bin >= 0 && last) {
         hk[warp][bin] += kk;
-        hc[warp][bin] += c;
+        hc[warp][bin] += lane - head + 1;
       }
       __syncwarp();
     }
@@ -338,42 +361,53 @@ __global__ void __launch_bounds__(kPkThreads) k_pk_geometry(int n, int nc, const
   }
 }
 
+// Sum of column b of the nblocks rows of `cols` doubles, by a block of kPkSumThreads in a fixed order (one
+// thread per bin over 1216 rows took 113 us at any mesh size).  The result is thread 0's.
+constexpr int kPkSumThreads = 128;
+__device__ __forceinline__ double pk_column(const double* __restrict__ partials, int nblocks, int cols, int b) {
+  __shared__ double part[kPkSumThreads / 32];
+  double v = 0.0;
+  for (int i = threadIdx.x; i < nblocks; i += kPkSumThreads) v += partials[(size_t)i * cols + b];
+  for (int off = 16; off > 0; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);
+  __syncthreads();
+  if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = v;
+  __syncthreads();
+  v = 0.0;
+  for (int w = 0; w < kPkSumThreads / 32; ++w) v += part[w];
+  return v;
+}
+
 // geom[0..nbins) = sum of |m| per bin, geom[nbins..2 nbins) = mode count (exact in FP64)
-__global__ void k_pk_geometry_finish(const double* __restrict__ partials, int nblocks, int nbins, double* geom) {
-  for (int b = threadIdx.x; b < nbins; b += blockDim.x) {
-    double sk = 0.0, sc = 0.0;
-    for (int i = 0; i < nblocks; ++i) {
-      sk += partials[(size_t)i * 2 * nbins + b];
-      sc += partials[(size_t)i * 2 * nbins + nbins + b];
-    }
-    geom[b] = sk;
-    geom[nbins + b] = sc;
-  }
+__global__ void __launch_bounds__(kPkSumThreads) k_pk_geometry_finish(const double* __restrict__ partials, int nblocks,
+                                                                      int nbins, double* geom) {
+  const double v = pk_column(partials, nblocks, 2 * nbins, blockIdx.x);
+  if (threadIdx.x == 0) geom[blockIdx.x] = v;
 }
 
 constexpr int kPkUnroll = 4;   // k_z chunks of 32 whose loads a lane issues before scanning them
 
+// Bound by the instructions of the segmented scans: equal bins along a row are contiguous, so a run's
+// first lane comes from one ballot instead of a bin shuffle at every distance.
 __global__ void __launch_bounds__(kPkThreads) k_pk_power(int n, int pc, int nc, const float2* __restrict__ dk,
                                                          const long long* __restrict__ edges_g, int nbins,
                                                          int cic_correct, double* partials) {
-  __shared__ long long edges[kMaxBins + 1];
+  __shared__ int edges[kMaxBins + 1];   // |m|^2 <= 3 (n/2)^2 < 2^24
   __shared__ double hp[kPkWarps][kMaxBins];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  for (int i = threadIdx.x; i <= nbins; i += blockDim.x) edges[i] = edges_g[i];
+  for (int i = threadIdx.x; i <= nbins; i += blockDim.x) edges[i] = (int)edges_g[i];
   for (int i = threadIdx.x; i < kPkWarps * kMaxBins; i += blockDim.x) (&hp[0][0])[i] = 0.0;
   __syncthreads();
-  const long long nrows = (long long)n * n;
+  const int nrows = n * n;
   const float inv_n = 1.0f / (float)n;
-  for (long long row = (long long)blockIdx.x * kPkWarps + warp; row < nrows;
-       row += (long long)gridDim.x * kPkWarps) {
-    const int mx = signed_mode((int)(row / n), n), my = signed_mode((int)(row % n), n);
-    const long long mxy = (long long)mx * mx + (long long)my * my;
+  for (int row = blockIdx.x * kPkWarps + warp; row < nrows; row += gridDim.x * kPkWarps) {
+    const int mx = signed_mode(row / n, n), my = signed_mode(row % n, n);
+    const int mxy = mx * mx + my * my;
     float cxy = 1.0f;
     if (cic_correct) {
       const float sx = sinpif((float)mx * inv_n), sy = sinpif((float)my * inv_n);
       cxy = (1.0f - (2.0f / 3.0f) * sx * sx) * (1.0f - (2.0f / 3.0f) * sy * sy);
     }
-    const float2* rowp = dk + row * pc;
+    const float2* rowp = dk + (long long)row * pc;
     int bin = -2;   // the lane's current bin along the row (-2: not searched yet)
     for (int kz0 = 0; kz0 < nc; kz0 += 32 * kPkUnroll) {
       // the chunk's loads first (streaming: the spectrum is read once), then one scan per 32 modes
@@ -385,11 +419,12 @@ __global__ void __launch_bounds__(kPkThreads) k_pk_power(int n, int pc, int nc, 
       }
 #pragma unroll
       for (int u = 0; u < kPkUnroll; ++u) {
+        if (kz0 + 32 * u >= nc) break;
         const int kz = kz0 + 32 * u + lane;
         int b = -1;
         float p = 0.0f;
         if (kz < nc && pk_half(mx, my, kz)) {
-          const long long m2 = mxy + (long long)kz * kz;
+          const int m2 = mxy + kz * kz;
           // |m|^2 grows along the row: advance the previous bin instead of searching again
           if (bin < 0 || m2 < edges[bin]) bin = pk_bin_of(m2, edges, nbins);
           else
@@ -403,14 +438,14 @@ __global__ void __launch_bounds__(kPkThreads) k_pk_power(int n, int pc, int nc, 
             }
           }
         }
+        bool last;
+        const int head = pk_run(b, lane, &last);
 #pragma unroll
         for (int d = 1; d < 32; d <<= 1) {
-          const int ob = __shfl_up_sync(0xffffffffu, b, d);
           const float op = __shfl_up_sync(0xffffffffu, p, d);
-          if (lane >= d && ob == b) p += op;
+          if (lane - d >= head) p += op;
         }
-        const int nb_next = __shfl_down_sync(0xffffffffu, b, 1);
-        if (b >= 0 && (lane == 31 || nb_next != b)) hp[warp][b] += (double)p;
+        if (b >= 0 && last) hp[warp][b] += (double)p;
         __syncwarp();
       }
     }
@@ -423,17 +458,18 @@ __global__ void __launch_bounds__(kPkThreads) k_pk_power(int n, int pc, int nc, 
   }
 }
 
-// pk[0..nbins) = mean |k| (h/Mpc), pk[nbins..) = P = pscale * mean power - shot, pk[2 nbins..) = modes
-__global__ void k_pk_finish(const double* __restrict__ partials, int nblocks, int nbins,
-                            const double* __restrict__ geom, double kfund, double pscale, double shot, double* pk) {
-  for (int b = threadIdx.x; b < nbins; b += blockDim.x) {
-    double sp = 0.0;
-    for (int i = 0; i < nblocks; ++i) sp += partials[(size_t)i * nbins + b];
-    const double sk = geom[b], sc = geom[nbins + b];
-    pk[b] = sc > 0 ? sk / sc * kfund : 0.0;
-    pk[nbins + b] = sc > 0 ? pscale * sp / sc - shot : 0.0;
-    pk[2 * nbins + b] = sc;
-  }
+// pk[0..nbins) = mean |k| (h/Mpc), pk[nbins..) = P = pscale * mean power - shot, pk[2 nbins..) = modes;
+// a block per bin
+__global__ void __launch_bounds__(kPkSumThreads) k_pk_finish(const double* __restrict__ partials, int nblocks, int nbins,
+                                                             const double* __restrict__ geom, double kfund, double pscale,
+                                                             double shot, double* pk) {
+  const int b = blockIdx.x;
+  const double sp = pk_column(partials, nblocks, nbins, b);
+  if (threadIdx.x) return;
+  const double sk = geom[b], sc = geom[nbins + b];
+  pk[b] = sc > 0 ? sk / sc * kfund : 0.0;
+  pk[nbins + b] = sc > 0 ? pscale * sp / sc - shot : 0.0;
+  pk[2 * nbins + b] = sc;
 }
 
 // out[j m + i] = F_j at mesh cell cells[i] = (ix N + iy) N + iz of the real fields (rows of rs floats)
@@ -481,23 +517,24 @@ __global__ void k_mass_reduce(const unsigned long long* __restrict__ pairs, long
   mass_accumulate(lo, hi, mass_slot(acc));
 }
 
-int launch_mass_reduce(const unsigned long long* pairs, long long m, unsigned long long* acc, cudaStream_t st) {
-  k_mass_reduce<<<grid_for(m, 256), 256, 0, st>>>(pairs, m, acc);
-  return check_launch("mass_reduce");
-}
-
-int launch_mass_check(const ParticleGeom& pg, const unsigned long long* rho, bool sum_mesh, unsigned long long* acc,
-                      int* flags, cudaStream_t st) {
-  if (sum_mesh) {
+int launch_mass_check(const ParticleGeom& pg, const unsigned long long* rho, const unsigned long long* pairs, long long m,
+                      unsigned long long* acc, int* flags, cudaStream_t st) {
+  if (rho) {
     const long long cells = (long long)pg.n * pg.n * pg.n;
     k_mesh_sum<<<grid_for(cells, 256), 256, 0, st>>>(rho, cells, acc);
     const int e = check_launch("mesh_sum");
     if (e != COLA_OK) return e;
   }
+  if (m > 16 * kCheckThreads) {   // more than the one block of the check sums in a few turns
+    k_mass_reduce<<<grid_for(m, 256), 256, 0, st>>>(pairs, m, acc);
+    const int e = check_launch("mass_reduce");
+    if (e != COLA_OK) return e;
+    m = 0;
+  }
   // expected total: n 2^42 as a 128-bit number
   const unsigned long long n = (unsigned long long)pg.npart;
   const unsigned long long lo = n << 42, hi = n >> 22;
-  k_mass_check<<<1, 32, 0, st>>>(acc, lo, hi, acc, flags);
+  k_mass_check<<<1, kCheckThreads, 0, st>>>(acc, pairs, (int)m, lo, hi, flags);
   return check_launch("mass_check");
 }
 
@@ -559,7 +596,7 @@ int launch_snapshot(long long npart, const float* s, const float* v, const float
 int launch_pk_geometry(const Grid3& g, const long long* edges, int nbins, double* partials, int nblocks,
                        double* geom, cudaStream_t st) {
   k_pk_geometry<<<nblocks, kPkThreads, 0, st>>>(g.n, g.nc, edges, nbins, partials);
-  k_pk_geometry_finish<<<1, 128, 0, st>>>(partials, nblocks, nbins, geom);
+  k_pk_geometry_finish<<<2 * nbins, kPkSumThreads, 0, st>>>(partials, nblocks, nbins, geom);
   return check_launch("pk_geometry");
 }
 
@@ -571,7 +608,7 @@ int launch_pk_bins(const Grid3& g, const float2* dk, const long long* edges, int
 
 int launch_pk_finish(const double* partials, int nblocks, int nbins, const double* geom, double kfund, double pscale,
                      double shot, double* pk, cudaStream_t st) {
-  k_pk_finish<<<1, 128, 0, st>>>(partials, nblocks, nbins, geom, kfund, pscale, shot, pk);
+  k_pk_finish<<<nbins, kPkSumThreads, 0, st>>>(partials, nblocks, nbins, geom, kfund, pscale, shot, pk);
   return check_launch("pk_finish");
 }
 
