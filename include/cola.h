@@ -352,7 +352,7 @@ int cola_run_snapshots(cola_ctx* ctx, const float* white_noise, float* s, float*
  *                (groups of >= n_min members) are listed in increasing label order; only the first
  *                `capacity` are written.
  *   nhalo      : out, device int32: the number of haloes (may exceed capacity).
- * Work space (about 52 B per particle plus the search cells) is allocated on first use and kept
+ * Work space (about 56 B per particle plus the search cells) is allocated on first use and kept
  * until cola_destroy; requires np^3 < 2^31.  Asynchronous on the context's stream. */
 int cola_fof(cola_ctx* ctx, const float* s, double b, int n_min, int* label, int* size, int* halo_label,
              int* halo_size, double* halo_pos, int capacity, int* nhalo);

@@ -219,8 +219,10 @@ __global__ void __launch_bounds__(kThreads) k_bin_scatter(ParticleGeom pg, BinGe
   }
 }
 
-// Exclusive scan of the two per-tile count arrays into offsets (length m+1) and scatter cursors,
-// in three coalesced phases: per-segment sums, a scan of the segment sums, per-segment scans.
+// Exclusive scan of one or two count arrays (the tiles' primary and spill counts) into offsets (length
+// m+1) and, of the second, scatter cursors, in three coalesced phases: per-segment sums, a scan of the
+// segment sums, per-segment scans.  Counts and offsets are read and written 16 bytes at a time where the
+// arrays allow (they start on 256-byte boundaries).
 constexpr int kScanThreads = 512;
 constexpr int kScanSeg = kScanThreads * 8;   // counts per segment
 
@@ -249,15 +251,51 @@ __device__ __forceinline__ unsigned block_excl_scan(unsigned v, unsigned* total)
   return before + incl - v;
 }
 
+// counts base + 8 tid .. + 7 (0 beyond m)
+__device__ __forceinline__ void load8(const unsigned* __restrict__ cnt, int i0, int m, unsigned (&c)[8]) {
+  if (i0 + 8 <= m) {
+    const uint4 a = *reinterpret_cast<const uint4*>(cnt + i0), b = *reinterpret_cast<const uint4*>(cnt + i0 + 4);
+    c[0] = a.x, c[1] = a.y, c[2] = a.z, c[3] = a.w, c[4] = b.x, c[5] = b.y, c[6] = b.z, c[7] = b.w;
+  } else {
+#pragma unroll
+    for (int k = 0; k < 8; ++k) c[k] = i0 + k < m ? cnt[i0 + k] : 0u;
+  }
+}
+// offsets of the counts c at base.. from run on, to off (and cur), and off[m] after the last
+__device__ __forceinline__ void store8(unsigned run, const unsigned (&c)[8], int i0, int m, unsigned* off, unsigned* cur) {
+  unsigned o[8];
+#pragma unroll
+  for (int k = 0; k < 8; ++k) {
+    o[k] = run;
+    run += c[k];
+    if (i0 + k == m - 1) off[m] = run;
+  }
+  if (i0 + 8 <= m) {
+    const uint4 a = make_uint4(o[0], o[1], o[2], o[3]), b = make_uint4(o[4], o[5], o[6], o[7]);
+    *reinterpret_cast<uint4*>(off + i0) = a;
+    *reinterpret_cast<uint4*>(off + i0 + 4) = b;
+    if (cur) {
+      *reinterpret_cast<uint4*>(cur + i0) = a;
+      *reinterpret_cast<uint4*>(cur + i0 + 4) = b;
+    }
+  } else {
+#pragma unroll
+    for (int k = 0; k < 8; ++k)
+      if (i0 + k < m) {
+        off[i0 + k] = o[k];
+        if (cur) cur[i0 + k] = o[k];
+      }
+  }
+}
+
 __global__ void __launch_bounds__(kScanThreads) k_scan_sums(const unsigned* __restrict__ cnt_p,
                                                            const unsigned* __restrict__ cnt_s, int m,
                                                            unsigned* seg_sums) {
   const int list = blockIdx.y;
-  const unsigned* cnt = list ? cnt_s : cnt_p;
-  const int base = blockIdx.x * kScanSeg;
-  unsigned v = 0;
-  for (int i = threadIdx.x; i < kScanSeg; i += kScanThreads)
-    if (base + i < m) v += cnt[base + i];
+  unsigned c[8], v = 0;
+  load8(list ? cnt_s : cnt_p, blockIdx.x * kScanSeg + threadIdx.x * 8, m, c);
+#pragma unroll
+  for (int k = 0; k < 8; ++k) v += c[k];
   unsigned tot;
   block_excl_scan(v, &tot);
   if (threadIdx.x == 0) seg_sums[list * gridDim.x + blockIdx.x] = tot;
@@ -279,32 +317,15 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_segs(unsigned* seg_sums, 
 __global__ void __launch_bounds__(kScanThreads) k_scan_apply(const unsigned* __restrict__ cnt_p,
                                                             const unsigned* __restrict__ cnt_s, int m,
                                                             const unsigned* __restrict__ seg_sums, unsigned* off_p,
-                                                            unsigned* off_s, unsigned* cur_p, unsigned* cur_s) {
-  const int list = blockIdx.y;
-  const unsigned* cnt = list ? cnt_s : cnt_p;
-  unsigned* off = list ? off_s : off_p;
-  unsigned* cur = list ? cur_s : cur_p;
-  const int base = blockIdx.x * kScanSeg;
+                                                            unsigned* off_s, unsigned* cur_s) {
+  const int list = blockIdx.y, i0 = blockIdx.x * kScanSeg + threadIdx.x * 8;
   // each thread scans 8 consecutive counts; the thread totals are scanned across the block
-  unsigned c[8], v = 0;
+  unsigned c[8], v = 0, tot;
+  load8(list ? cnt_s : cnt_p, i0, m, c);
 #pragma unroll
-  for (int k = 0; k < 8; ++k) {
-    const int i = base + threadIdx.x * 8 + k;
-    c[k] = i < m ? cnt[i] : 0;
-    v += c[k];
-  }
-  unsigned tot;
-  unsigned run = seg_sums[list * gridDim.x + blockIdx.x] + block_excl_scan(v, &tot);
-#pragma unroll
-  for (int k = 0; k < 8; ++k) {
-    const int i = base + threadIdx.x * 8 + k;
-    if (i < m) {
-      off[i] = run;
-      cur[i] = run;
-    }
-    run += c[k];
-    if (i == m - 1) off[m] = run;
-  }
+  for (int k = 0; k < 8; ++k) v += c[k];
+  const unsigned run = seg_sums[list * gridDim.x + blockIdx.x] + block_excl_scan(v, &tot);
+  store8(run, c, i0, m, list ? off_s : off_p, list ? cur_s : nullptr);
 }
 
 // The scan in one launch for few segments: every block sums the counts before its segment itself (at
@@ -321,24 +342,12 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_one(const unsigned* __res
   for (int i = threadIdx.x; i < base; i += kScanThreads) v += cnt[i];
   block_excl_scan(v, &before);
   unsigned c[8];
+  load8(cnt, base + threadIdx.x * 8, m, c);
   v = 0;
 #pragma unroll
-  for (int k = 0; k < 8; ++k) {
-    const int i = base + threadIdx.x * 8 + k;
-    c[k] = i < m ? cnt[i] : 0;
-    v += c[k];
-  }
-  unsigned run = before + block_excl_scan(v, &tot);
-#pragma unroll
-  for (int k = 0; k < 8; ++k) {
-    const int i = base + threadIdx.x * 8 + k;
-    if (i < m) {
-      off[i] = run;
-      if (list) cur_s[i] = run;
-    }
-    run += c[k];
-    if (i == m - 1) off[m] = run;
-  }
+  for (int k = 0; k < 8; ++k) v += c[k];
+  const unsigned run = before + block_excl_scan(v, &tot);
+  store8(run, c, base + threadIdx.x * 8, m, off, list ? cur_s : nullptr);
 }
 
 // Tile-wise deposit.  The tile's primary and spill entries form one index range, so a CTA's threads run
@@ -681,11 +690,11 @@ void particle_schedule(const BinGeom& b, int nmesh, long long npart, bool* binne
   *binned = *tile_gather || mesh_mb > 256.0;
 }
 
-int launch_excl_scan(const unsigned* cnt, int m, unsigned* seg, unsigned* off, unsigned* cur, cudaStream_t st) {
+int launch_excl_scan(const unsigned* cnt, int m, unsigned* seg, unsigned* off, cudaStream_t st) {
   const int nseg = (m + kScanSeg - 1) / kScanSeg;
-  k_scan_sums<<<dim3(nseg, 1), kScanThreads, 0, st>>>(cnt, cnt, m, seg);
+  k_scan_sums<<<dim3(nseg, 1), kScanThreads, 0, st>>>(cnt, nullptr, m, seg);
   k_scan_segs<<<1, kScanThreads, 0, st>>>(seg, nseg);
-  k_scan_apply<<<dim3(nseg, 1), kScanThreads, 0, st>>>(cnt, cnt, m, seg, off, off, cur, cur);
+  k_scan_apply<<<dim3(nseg, 1), kScanThreads, 0, st>>>(cnt, nullptr, m, seg, off, nullptr, nullptr);
   return check_launch("excl_scan");
 }
 
@@ -710,7 +719,7 @@ int launch_binning(const ParticleGeom& pg, const BinGeom& b, const float* s, Bin
     k_scan_sums<<<dim3(nseg, 2), kScanThreads, 0, st>>>(bb.cnt_p, bb.cnt_s, b.tiles, bb.seg);
     k_scan_segs<<<2, kScanThreads, 0, st>>>(bb.seg, nseg);
     k_scan_apply<<<dim3(nseg, 2), kScanThreads, 0, st>>>(bb.cnt_p, bb.cnt_s, b.tiles, bb.seg, bb.off_p, bb.off_s,
-                                                         bb.cur_p, bb.cur_s);
+                                                         bb.cur_s);
   }
   if ((e = check_launch("bin_scan")) != COLA_OK) return e;
   k_bin_scatter<<<grid, rb.block, 0, st>>>(pg, b, walk, bb.rec, bb.off_p, bb.cur_s, bb.ent_p, bb.ent_s);

@@ -398,17 +398,17 @@ extern "C" int cola_create(const cola_params* params, void* stream, cola_ctx** o
     return fail(st);
   cudaMemset(c->flags, 0, sizeof(int));
   cudaMemset(c->mass_acc, 0, 2 * kMassSlots * sizeof(unsigned long long));
-  // tile binning buffers: 6 per-tile arrays, n primary entries and up to 7n spill entries
+  // tile binning buffers: 5 per-tile arrays, n primary entries and up to 7n spill entries
   if (bin_geometry(params->nmesh, params->np, &c->bg)) {
     const size_t tiles = (size_t)c->bg.tiles + 1;
     const size_t nseg = (tiles + 4095) / 4096 + 1;
-    const size_t bytes = 6 * align256(tiles * sizeof(unsigned)) + align256((size_t)c->pg.npart * 4) +
+    const size_t bytes = 5 * align256(tiles * sizeof(unsigned)) + align256((size_t)c->pg.npart * 4) +
                          align256((size_t)c->pg.npart * 28) + align256(2 * nseg * sizeof(unsigned)) +
                          align256(tiles * 2 * sizeof(unsigned long long)) + align256((size_t)c->pg.npart * 8);
     if ((st = cuda_status(cudaMalloc(&c->bin_mem, bytes), "cudaMalloc bins")) != COLA_OK) return fail(st);
     char* q = static_cast<char*>(c->bin_mem);
-    unsigned** arr[6] = {&c->bb.cnt_p, &c->bb.cnt_s, &c->bb.off_p, &c->bb.off_s, &c->bb.cur_p, &c->bb.cur_s};
-    for (int i = 0; i < 6; ++i) {
+    unsigned** arr[5] = {&c->bb.cnt_p, &c->bb.cnt_s, &c->bb.off_p, &c->bb.off_s, &c->bb.cur_s};
+    for (int i = 0; i < 5; ++i) {
       *arr[i] = reinterpret_cast<unsigned*>(q);
       q += align256(tiles * sizeof(unsigned));
     }
@@ -843,21 +843,23 @@ int fof_workspace(cola_ctx* c, const FofGeom& f, int capacity) {
       c->fof_mem = nullptr;
     }
     const long long nseg = ((n > f.ncells ? n : f.ncells) + 4095) / 4096 + 1;
-    const size_t b8 = align256((size_t)n * 8), b4 = align256((size_t)(n + 1) * 4);
+    const size_t b16 = align256((size_t)n * 16), b4 = align256((size_t)(n + 1) * 4);
     const size_t bc = align256((size_t)(f.ncells + 1) * 4);
-    const size_t bytes = 3 * b8 + 7 * b4 + 3 * bc + align256((size_t)nseg * 4);
+    const size_t bytes = b16 + 10 * b4 + 2 * bc + align256((size_t)nseg * 4);
     void* mem = nullptr;
     COLA_TRY(cuda_status(cudaMalloc(&mem, bytes), "cudaMalloc fof"));
     c->fof_mem = mem;
     c->fof_ncells = f.ncells;
     char* q = static_cast<char*>(mem);
-    for (int a = 0; a < 3; ++a, q += b8) c->fb.g[a] = reinterpret_cast<long long*>(q);
-    int** ints[3] = {&c->fb.key, &c->fb.sorted, &c->fb.parent};
-    for (int i = 0; i < 3; ++i, q += b4) *ints[i] = reinterpret_cast<int*>(q);
-    unsigned** uns[4] = {&c->fb.cnt, &c->fb.flag, &c->fb.hoff, &c->fb.hcur};
-    for (int i = 0; i < 4; ++i, q += b4) *uns[i] = reinterpret_cast<unsigned*>(q);
-    unsigned** cells[3] = {&c->fb.counts, &c->fb.off, &c->fb.cur};
-    for (int i = 0; i < 3; ++i, q += bc) *cells[i] = reinterpret_cast<unsigned*>(q);
+    c->fb.rec = reinterpret_cast<uint4*>(q);
+    q += b16;
+    for (int a = 0; a < 3; ++a, q += b4) c->fb.g[a] = reinterpret_cast<unsigned*>(q);
+    int** ints[4] = {&c->fb.key, &c->fb.ids, &c->fb.parent, &c->fb.min_id};
+    for (int i = 0; i < 4; ++i, q += b4) *ints[i] = reinterpret_cast<int*>(q);
+    unsigned** uns[3] = {&c->fb.cnt, &c->fb.flag, &c->fb.hoff};
+    for (int i = 0; i < 3; ++i, q += b4) *uns[i] = reinterpret_cast<unsigned*>(q);
+    unsigned** cells[2] = {&c->fb.counts, &c->fb.off};
+    for (int i = 0; i < 2; ++i, q += bc) *cells[i] = reinterpret_cast<unsigned*>(q);
     c->fb.seg = reinterpret_cast<unsigned*>(q);
   }
   if (capacity > c->fof_sums_cap) {

@@ -261,7 +261,7 @@ struct BinGeom {
 struct BinBuffers {
   unsigned *cnt_p = nullptr, *cnt_s = nullptr;   // counts per tile (primary, spill), cnt_s after cnt_p
   unsigned *off_p = nullptr, *off_s = nullptr;   // offsets, tiles + 1
-  unsigned *cur_p = nullptr, *cur_s = nullptr;   // scatter cursors
+  unsigned* cur_s = nullptr;                      // scatter cursors of the spill entries
   unsigned *ent_p = nullptr, *ent_s = nullptr;   // packed lattice coordinates (n primary, up to 7n spill)
   unsigned* seg = nullptr;                        // scan segment sums (2 lists)
   unsigned long long* rec = nullptr;              // [n] rank in the primary tile << 32 | tile code (binning.cu)
@@ -359,23 +359,24 @@ int launch_snapshot(long long npart, const float* s, const float* v, const float
 
 // Friends-of-friends (fof.cu): geometry of the cell search and work buffers.
 struct FofGeom {
-  long long modulus = 0;   // N 2^20
-  long long ell = 0;       // linking length in fixed-point units
-  long long ncells = 0;    // ncs^3
-  int ncs = 0;             // cells per axis, side >= ell
+  long long modulus = 0;        // N 2^20
+  long long ell = 0;            // linking length in fixed-point units
+  long long ncells = 0;         // ncs^3
+  unsigned long long inv = 0;   // floor(2^64 ncs / modulus)
+  int ncs = 0;                  // cells per axis, side > ell (1: one cell)
 };
 struct FofBuffers {
-  long long* g[3] = {nullptr, nullptr, nullptr};   // fixed-point coordinates [n] per axis
-  int* key = nullptr;                              // cell of each particle
-  int* sorted = nullptr;                           // particle ids sorted by cell
-  int* parent = nullptr;                           // union-find forest
+  unsigned* g[3] = {nullptr, nullptr, nullptr};    // fixed-point coordinates [n] per axis
+  uint4* rec = nullptr;                            // (coordinates, root after the first pass) sorted by cell
+  int* ids = nullptr;                              // particle of each record
+  int* key = nullptr;                              // cell of each particle, later root of each record
+  int* parent = nullptr;                           // union-find forest over the records
+  int* min_id = nullptr;                           // smallest particle id per root
   unsigned* cnt = nullptr;                         // members per root
-  unsigned* flag = nullptr;                        // 1 for roots of haloes
-  unsigned* hoff = nullptr;                        // [n + 1] halo index of each root
-  unsigned* hcur = nullptr;
+  unsigned* flag = nullptr;                        // 1 for the particles that label a halo
+  unsigned* hoff = nullptr;                        // [n + 1] halo index of each label
   unsigned* counts = nullptr;                      // [ncells] particles per cell
   unsigned* off = nullptr;                         // [ncells + 1]
-  unsigned* cur = nullptr;
   unsigned* seg = nullptr;                         // scan segment sums
   unsigned long long* sums = nullptr;              // [3][capacity] offset sums of the haloes
 };
@@ -383,9 +384,8 @@ bool fof_geometry(int nmesh, int np, double b, FofGeom* f);
 int launch_fof(const ParticleGeom& pg, const FofGeom& f, const float* s, const FofBuffers& fb, int n_min, int* label,
                int* size, int* halo_label, int* halo_size, double* halo_pos, int capacity, int* nhalo, int* flags,
                cudaStream_t st);
-// Exclusive scan of m counts into off[0..m] and a copy cur[0..m) (binning.cu); seg holds
-// ceil(m / 4096) partial sums.
-int launch_excl_scan(const unsigned* cnt, int m, unsigned* seg, unsigned* off, unsigned* cur, cudaStream_t st);
+// Exclusive scan of m counts into off[0..m] (binning.cu); seg holds ceil(m / 4096) partial sums.
+int launch_excl_scan(const unsigned* cnt, int m, unsigned* seg, unsigned* off, cudaStream_t st);
 
 // Power spectrum binning of a forward spectrum (side n).  launch_pk_geometry writes the bins' sum of
 // |m| and mode count (they depend only on n and the edges) to geom[2][nbins]; launch_pk_bins sums the
