@@ -34,25 +34,38 @@ unsigned grid_for(long long work, int threads) {
   return (unsigned)(b < 1 ? 1 : b);
 }
 
-__device__ __forceinline__ void lattice_of(long long id, int np, int* q) {
-  const long long np2 = (long long)np * np;
-  q[0] = (int)(id / np2);
-  const long long rem = id - (long long)q[0] * np2;
-  q[1] = (int)(rem / np);
-  q[2] = (int)(rem - (long long)q[1] * np);
-}
-
 // cell and weight of cell c+1 per axis, from the forward's fixed-point coordinate
-__device__ __forceinline__ void cic_cell(const ParticleGeom& pg, long long id, const float* s, long long n, int* c,
-                                         float* w1) {
-  int q[3];
-  lattice_of(id, pg.np, q);
-  const long long modulus = (long long)pg.n << kFracBits;
+template <bool F32>
+__device__ __forceinline__ void cic_cell(const FixedGeo& fg, const int (&q)[3], long long id, const float* __restrict__ s,
+                                         long long n, int* c, float* w1) {
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
-    const long long g = fixed_coord(q[a], s[a * n + id], pg.r_fixed, modulus);
-    c[a] = (int)(g >> kFracBits);
-    w1[a] = (float)((int)(g >> (kFracBits - 14)) & (kWeightOne - 1)) * (1.0f / kWeightOne);
+    int f;
+    cell_frac<F32>(q[a], __ldg(s + a * n + id), fg, &c[a], &f);
+    w1[a] = (float)f * (1.0f / kWeightOne);
+  }
+}
+
+// Particles are walked by lattice rows (row_blocks): no index is divided (two 64-bit divisions per particle
+// before).  Calls f(q, id) for the thread's particles.
+template <class F>
+__device__ __forceinline__ void for_particles(int np, F&& f) {
+  const int qx = blockIdx.y, qy = blockIdx.x * blockDim.y + threadIdx.y;
+  if (qy >= np) return;
+  const long long row = ((long long)qx * np + qy) * np;
+  for (int qz = threadIdx.x; qz < np; qz += blockDim.x) {
+    const int q[3] = {qx, qy, qz};
+    f(q, row + qz);
+  }
+}
+
+// adds v0 to p[0] and v1 to p[1], p + iz of an even-sided mesh: one 8-byte reduction where iz is even
+__device__ __forceinline__ void add_pair(float* row, int iz, int iz1, float v0, float v1) {
+  if ((iz & 1) == 0) {
+    asm volatile("red.global.add.v2.f32 [%0], {%1, %2};\n" ::"l"(row + iz), "f"(v0), "f"(v1) : "memory");
+  } else {
+    atomicAdd(row + iz, v0);
+    atomicAdd(row + iz1, v1);
   }
 }
 
@@ -71,16 +84,20 @@ __global__ void k_adj_step(long long n3, const float* __restrict__ lam_s, float*
   }
 }
 
-// deposit the three components of lam_f with CIC weights onto three real meshes (rows of rs)
-__global__ void k_adj_deposit(ParticleGeom pg, const float* __restrict__ s, const float* __restrict__ lam_f, float* m0,
-                              float* m1, float* m2, long long rs) {
+// deposit the three components of lam_f with CIC weights onto three real meshes (rows of rs); bound by the
+// rate of the atomics in L2
+template <bool F32>
+__global__ void __launch_bounds__(256) k_adj_deposit(ParticleGeom pg, FixedGeo fg, const float* __restrict__ s,
+                                                     const float* __restrict__ lam_f, float* m0, float* m1, float* m2,
+                                                     long long rs) {
   const long long n = pg.npart;
   const int nm = pg.n;
-  for (long long id = blockIdx.x * (long long)blockDim.x + threadIdx.x; id < n; id += (long long)gridDim.x * blockDim.x) {
+  for_particles(pg.np, [&](const int (&q)[3], long long id) {
     int c[3];
     float w1[3];
-    cic_cell(pg, id, s, n, c, w1);
+    cic_cell<F32>(fg, q, id, s, n, c, w1);
     const float l0 = lam_f[id], l1 = lam_f[n + id], l2 = lam_f[2 * n + id];
+    const int iz = c[2], iz1 = c[2] + 1 == nm ? 0 : c[2] + 1;
 #pragma unroll
     for (int dx = 0; dx < 2; ++dx) {
       const int ix = (c[0] + dx) == nm ? 0 : c[0] + dx;
@@ -90,17 +107,13 @@ __global__ void k_adj_deposit(ParticleGeom pg, const float* __restrict__ s, cons
         const int iy = (c[1] + dy) == nm ? 0 : c[1] + dy;
         const float wxy = wx * (dy ? w1[1] : 1.0f - w1[1]);
         const long long row = ((long long)ix * nm + iy) * rs;
-#pragma unroll
-        for (int dz = 0; dz < 2; ++dz) {
-          const int iz = (c[2] + dz) == nm ? 0 : c[2] + dz;
-          const float w = wxy * (dz ? w1[2] : 1.0f - w1[2]);
-          atomicAdd(m0 + row + iz, w * l0);
-          atomicAdd(m1 + row + iz, w * l1);
-          atomicAdd(m2 + row + iz, w * l2);
-        }
+        const float a = wxy * (1.0f - w1[2]), b = wxy * w1[2];
+        add_pair(m0 + row, iz, iz1, a * l0, b * l0);
+        add_pair(m1 + row, iz, iz1, a * l1, b * l1);
+        add_pair(m2 + row, iz, iz1, a * l2, b * l2);
       }
     }
-  }
+  });
 }
 
 // out(k) = sum_j conj(i D(m_j) g) L_j(k) = -i g sum_j D(m_j) L_j(k), g = g_scale / |m|^2; out may be L_0
@@ -124,15 +137,16 @@ __global__ void k_adj_combine(int n, int pc, int nc, const float2* l0, const flo
 }
 
 // lam_s += sum_c grad W(x - c) [lam_f . F_c + norm lam_delta_c]
-__global__ void k_adj_gather(ParticleGeom pg, const float* __restrict__ s, const float* __restrict__ lam_f,
+template <bool F32>
+__global__ void __launch_bounds__(256) k_adj_gather(ParticleGeom pg, FixedGeo fg, const float* __restrict__ s, const float* __restrict__ lam_f,
                              const float* __restrict__ f0, const float* __restrict__ f1, const float* __restrict__ f2,
                              const float* __restrict__ ld, long long rs, float norm, float* lam_s) {
   const long long n = pg.npart;
   const int nm = pg.n;
-  for (long long id = blockIdx.x * (long long)blockDim.x + threadIdx.x; id < n; id += (long long)gridDim.x * blockDim.x) {
+  for_particles(pg.np, [&](const int (&q)[3], long long id) {
     int c[3];
     float w1[3];
-    cic_cell(pg, id, s, n, c, w1);
+    cic_cell<F32>(fg, q, id, s, n, c, w1);
     const float l0 = lam_f[id], l1 = lam_f[n + id], l2 = lam_f[2 * n + id];
     float gxs = 0.f, gys = 0.f, gzs = 0.f;
 #pragma unroll
@@ -159,7 +173,7 @@ __global__ void k_adj_gather(ParticleGeom pg, const float* __restrict__ s, const
     lam_s[id] += gxs;
     lam_s[n + id] += gys;
     lam_s[2 * n + id] += gzs;
-  }
+  });
 }
 
 // lam_p1 += d1 lam_s; lam_p2 += d2 lam_s   (initial condition s_1 = D1 Psi1 + D2 Psi2)
@@ -199,10 +213,8 @@ __global__ void k_ic_source_adjoint(int n, int pc, const float* __restrict__ lam
 
 // ---- CIC density contrast of the loss grid (continuous weights) and its adjoint ---------------
 // grid coordinate y = (q N/np + s) ngrid / N, wrapped into [0, ngrid)
-__device__ __forceinline__ void grid_cell(const ParticleGeom& pg, long long id, const float* s, long long n, int ng,
-                                          double ratio, int* c, float* t) {
-  int q[3];
-  lattice_of(id, pg.np, q);
+__device__ __forceinline__ void grid_cell(const ParticleGeom& pg, const int (&q)[3], long long id,
+                                          const float* __restrict__ s, long long n, int ng, double ratio, int* c, float* t) {
   const double r = (double)pg.n / pg.np;
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
@@ -222,10 +234,10 @@ __device__ __forceinline__ void grid_cell(const ParticleGeom& pg, long long id, 
 __global__ void k_grid_deposit(ParticleGeom pg, const float* __restrict__ s, int ng, double ratio,
                                unsigned long long* rho) {
   const long long n = pg.npart;
-  for (long long id = blockIdx.x * (long long)blockDim.x + threadIdx.x; id < n; id += (long long)gridDim.x * blockDim.x) {
+  for_particles(pg.np, [&](const int (&q)[3], long long id) {
     int c[3];
     float t[3];
-    grid_cell(pg, id, s, n, ng, ratio, c, t);
+    grid_cell(pg, q, id, s, n, ng, ratio, c, t);
 #pragma unroll
     for (int dx = 0; dx < 2; ++dx) {
       const int ix = (c[0] + dx) == ng ? 0 : c[0] + dx;
@@ -238,12 +250,12 @@ __global__ void k_grid_deposit(ParticleGeom pg, const float* __restrict__ s, int
         for (int dz = 0; dz < 2; ++dz) {
           const int iz = (c[2] + dz) == ng ? 0 : c[2] + dz;
           const float w = wxy * (dz ? t[2] : 1.0f - t[2]);
-          const unsigned long long q = (unsigned long long)__double2ll_rn((double)w * 4294967296.0);
-          if (q) atomicAdd(rho + ((long long)ix * ng + iy) * ng + iz, q);
+          const unsigned long long u = (unsigned long long)__float2ll_rn(w * 4294967296.0f);   // the scaling is exact
+          if (u) atomicAdd(rho + ((long long)ix * ng + iy) * ng + iz, u);
         }
       }
     }
-  }
+  });
 }
 
 // delta = rho scale - 1, scale = ng^3 / (n 2^32), in FP64
@@ -256,10 +268,10 @@ __global__ void k_grid_finish(long long cells, const unsigned long long* __restr
 __global__ void k_grid_adjoint(ParticleGeom pg, const float* __restrict__ s, int ng, double ratio,
                                const float* __restrict__ lam_delta, float gscale, float* lam_s) {
   const long long n = pg.npart;
-  for (long long id = blockIdx.x * (long long)blockDim.x + threadIdx.x; id < n; id += (long long)gridDim.x * blockDim.x) {
+  for_particles(pg.np, [&](const int (&q)[3], long long id) {
     int c[3];
     float t[3];
-    grid_cell(pg, id, s, n, ng, ratio, c, t);
+    grid_cell(pg, q, id, s, n, ng, ratio, c, t);
     float g0 = 0.f, g1 = 0.f, g2 = 0.f;
 #pragma unroll
     for (int dx = 0; dx < 2; ++dx) {
@@ -283,7 +295,7 @@ __global__ void k_grid_adjoint(ParticleGeom pg, const float* __restrict__ s, int
     lam_s[id] = g0 * gscale;
     lam_s[n + id] = g1 * gscale;
     lam_s[2 * n + id] = g2 * gscale;
-  }
+  });
 }
 
 }  // namespace
@@ -298,7 +310,10 @@ int launch_adj_step(long long n3, const float* lam_s, float* lam_v, float* lam_p
 
 int launch_adj_deposit(const ParticleGeom& pg, const float* s, const float* lam_f, float* const m[3], long long rs,
                        cudaStream_t st) {
-  k_adj_deposit<<<grid_for(pg.npart, 256), 256, 0, st>>>(pg, s, lam_f, m[0], m[1], m[2], rs);
+  const RowBlocks rb = row_blocks(pg.np);
+  const FixedGeo fg = fixed_geo(pg.n, pg.r_fixed);
+  auto* k = pg.n < 2048 ? k_adj_deposit<true> : k_adj_deposit<false>;
+  k<<<rb.grid, rb.block, 0, st>>>(pg, fg, s, lam_f, m[0], m[1], m[2], rs);
   return check_launch("adj_deposit");
 }
 
@@ -311,7 +326,10 @@ int launch_adj_combine(const Grid3& g, float2* const l[3], const float* dtab, fl
 
 int launch_adj_gather(const ParticleGeom& pg, const float* s, const float* lam_f, const float* const f[3],
                       const float* lam_delta, long long rs, float norm, float* lam_s, cudaStream_t st) {
-  k_adj_gather<<<grid_for(pg.npart, 256), 256, 0, st>>>(pg, s, lam_f, f[0], f[1], f[2], lam_delta, rs, norm, lam_s);
+  const RowBlocks rb = row_blocks(pg.np);
+  const FixedGeo fg = fixed_geo(pg.n, pg.r_fixed);
+  auto* k = pg.n < 2048 ? k_adj_gather<true> : k_adj_gather<false>;
+  k<<<rb.grid, rb.block, 0, st>>>(pg, fg, s, lam_f, f[0], f[1], f[2], lam_delta, rs, norm, lam_s);
   return check_launch("adj_gather");
 }
 
@@ -331,7 +349,8 @@ int launch_grid_density(const ParticleGeom& pg, const float* s, int ngrid, unsig
   const long long cells = (long long)ngrid * ngrid * ngrid;
   if (cudaMemsetAsync(scratch, 0, cells * sizeof(unsigned long long), st) != cudaSuccess) return COLA_ERR_CUDA;
   const double ratio = (double)ngrid / pg.n;
-  k_grid_deposit<<<grid_for(pg.npart, 256), 256, 0, st>>>(pg, s, ngrid, ratio, scratch);
+  const RowBlocks rb = row_blocks(pg.np);
+  k_grid_deposit<<<rb.grid, rb.block, 0, st>>>(pg, s, ngrid, ratio, scratch);
   k_grid_finish<<<grid_for(cells, 256), 256, 0, st>>>(cells, scratch, (double)cells / ((double)pg.npart * 4294967296.0),
                                                       delta);
   return check_launch("grid_density");
@@ -349,7 +368,8 @@ int launch_grid_density_adjoint(const ParticleGeom& pg, const float* s, int ngri
                                 float* lam_s, cudaStream_t st) {
   const double ratio = (double)ngrid / pg.n;
   const double cells = (double)ngrid * ngrid * ngrid;
-  k_grid_adjoint<<<grid_for(pg.npart, 256), 256, 0, st>>>(pg, s, ngrid, ratio, lam_delta,
+  const RowBlocks rb = row_blocks(pg.np);
+  k_grid_adjoint<<<rb.grid, rb.block, 0, st>>>(pg, s, ngrid, ratio, lam_delta,
                                                           (float)(cells / (double)pg.npart * ratio), lam_s);
   return check_launch("grid_density_adjoint");
 }

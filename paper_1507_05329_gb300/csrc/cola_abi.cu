@@ -304,7 +304,7 @@ extern "C" void cola_destroy(cola_ctx* c) {
   if (c->edges_host) cudaFreeHost(c->edges_host);
   fft_plan_free(&c->mplan);
   fft_plan_free(&c->lplan);
-  void* bufs[] = {c->arena,    c->dtab,     c->amp_m2,  c->edges, c->pk_partials, c->pk_geom,
+  void* bufs[] = {c->arena,    c->dtab,     c->amp_m2,  c->ktab,   c->edges, c->pk_partials, c->pk_geom,
                   c->flags,    c->mass_acc, c->bin_mem, c->adj_mem,     c->fof_mem,  c->fof_sums};
   for (void* b : bufs)
     if (b) cudaFree(b);
@@ -371,6 +371,13 @@ extern "C" int cola_create(const cola_params* params, void* stream, cola_ctx** o
     }
     if ((st = cuda_status(cudaMalloc(&c->dtab, n * sizeof(float)), "cudaMalloc dtab")) != COLA_OK) return fail(st);
     cudaMemcpy(c->dtab, d.data(), n * sizeof(float), cudaMemcpyHostToDevice);
+  }
+  {
+    const int np = params->np;
+    std::vector<float> k(np);
+    for (int j = 0; j < np; ++j) k[j] = 2 * j == np ? 0.0f : (float)(2.0 * M_PI * (j < np / 2 ? j : j - np) / np);
+    if ((st = cuda_status(cudaMalloc(&c->ktab, np * sizeof(float)), "cudaMalloc ktab")) != COLA_OK) return fail(st);
+    cudaMemcpy(c->ktab, k.data(), np * sizeof(float), cudaMemcpyHostToDevice);
   }
   // sqrt(P(k) / V_cell) / np^3 per integer |m|^2 of the lattice, k = 2 pi |m| / L
   {
@@ -471,9 +478,9 @@ extern "C" int cola_ic_2lpt(cola_ctx* c, const float* wn, float* s, float* v, fl
     float2* const h[3] = {B[0], B[1], B[2]};
     COLA_TRY(STAGED(kStFwdX, launch_ic_x(P, B[0], h, 3, 1.0f, c->amp_m2, c->stream)));
     float2* const t0[3] = {B[0], B[3], B[4]};
-    COLA_TRY(STAGED(kStInvY, launch_ic_y(P, B[0], t0, 3, c->stream)));
+    COLA_TRY(STAGED(kStInvY, launch_ic_y(P, B[0], t0, 3, nullptr, c->stream)));
     float2* const t1[3] = {B[1], B[5], nullptr};
-    COLA_TRY(STAGED(kStInvY, launch_ic_y(P, B[1], t1, 2, c->stream)));
+    COLA_TRY(STAGED(kStInvY, launch_ic_y(P, B[1], t1, 2, nullptr, c->stream)));
     COLA_TRY(STAGED(kStInvY, launch_pencils(P, g, 1, +1, &B[2], 1, c->stream)));
     float2* const t[6] = {B[0], B[3], B[4], B[1], B[5], B[2]};
     COLA_TRY(STAGED(kStInvZ, launch_ic_z1(P, t, B[7], psi1, r, c->stream)));
@@ -481,7 +488,7 @@ extern "C" int cola_ic_2lpt(cola_ctx* c, const float* wn, float* s, float* v, fl
     float2* const hs[3] = {B[7], B[6], nullptr};
     COLA_TRY(STAGED(kStFwdX, launch_ic_x(P, B[7], hs, 2, inv_n3, nullptr, c->stream)));
     float2* const u[3] = {B[7], B[0], nullptr};
-    COLA_TRY(STAGED(kStInvY, launch_ic_y(P, B[7], u, 2, c->stream)));
+    COLA_TRY(STAGED(kStInvY, launch_ic_y(P, B[7], u, 2, nullptr, c->stream)));
     COLA_TRY(STAGED(kStInvY, launch_pencils(P, g, 1, +1, &B[6], 1, c->stream)));
     float2* const f[3] = {B[6], B[0], B[7]};
     return STAGED(kStInvZ, launch_ic_z2(P, f, psi1, psi2, s, v, r, (float)s0.d1, (float)s0.d2, c->stream));
@@ -926,16 +933,21 @@ int pm_force_adjoint(cola_ctx* c, const float* s_i, double force_scale) {
   float* const m[3] = {reinterpret_cast<float*>(c->adj_mesh[0]), reinterpret_cast<float*>(c->adj_mesh[1]),
                        reinterpret_cast<float*>(c->adj_mesh[2])};
   COLA_TRY(STAGED(kStAdjoint, launch_adj_deposit(c->pg, s_i, c->lam[4], m, 2LL * g.pc, c->stream)));
-  for (int j = 0; j < 3; ++j) {
-    COLA_TRY(STAGED(kStFwdZ, launch_r2c_rows(c->mplan, g, kSrcFloat, c->adj_mesh[j], 2LL * g.pc, 1.0f, c->adj_mesh[j],
-                                             c->stream)));
-    COLA_TRY(forward3d_yx(c, g, c->mplan, c->adj_mesh[j]));
-  }
+  COLA_TRY(STAGED(kStFwdZ, launch_r2c_rows(c->mplan, g, kSrcFloat, reinterpret_cast<const void* const*>(m), 3, 2LL * g.pc,
+                                           1.0f, c->adj_mesh, c->stream)));
+  COLA_TRY(STAGED(kStFwdY, launch_pencils(c->mplan, g, 1, -1, c->adj_mesh, 3, c->stream)));
   const double kf = 2.0 * M_PI / g.n;
   const double n3 = (double)g.n * g.n * g.n;
-  COLA_TRY(STAGED(kStAdjoint, launch_adj_combine(g, c->adj_mesh, c->dtab, (float)(force_scale / (kf * kf * n3)),
-                                                 c->adj_mesh[0], c->stream)));
-  COLA_TRY(inverse3d(c, g, c->mplan, c->adj_mesh[0]));
+  const float g_scale = (float)(force_scale / (kf * kf * n3));
+  if (fft_compiled(c->mplan)) {
+    COLA_TRY(STAGED(kStFwdX, launch_grad_adj(c->mplan, c->adj_mesh, c->adj_mesh[0], c->dtab, g_scale, c->stream)));
+    COLA_TRY(STAGED(kStInvY, launch_pencils(c->mplan, g, 1, +1, c->adj_mesh, 1, c->stream)));
+    COLA_TRY(STAGED(kStInvZ, launch_c2r_rows(c->mplan, g, c->adj_mesh, 1, c->stream)));
+  } else {
+    COLA_TRY(STAGED(kStFwdX, launch_pencils(c->mplan, g, 0, -1, c->adj_mesh, 3, c->stream)));
+    COLA_TRY(STAGED(kStAdjoint, launch_adj_combine(g, c->adj_mesh, c->dtab, g_scale, c->adj_mesh[0], c->stream)));
+    COLA_TRY(inverse3d(c, g, c->mplan, c->adj_mesh[0]));
+  }
   const float* f[3] = {reinterpret_cast<float*>(c->cbuf[0]), reinterpret_cast<float*>(c->cbuf[1]),
                        reinterpret_cast<float*>(c->cbuf[2])};
   return STAGED(kStAdjoint, launch_adj_gather(c->pg, s_i, c->lam[4], f, m[0], 2LL * g.pc,
@@ -953,6 +965,45 @@ int lpt_adjoint(cola_ctx* c, const float* wn, float* lam_wn) {
   const long long n = c->pg.npart;
   const float r = (float)c->p.nmesh / (float)c->p.np;
   const float inv_n3 = (float)(1.0 / ((double)g.n * g.n * g.n));
+  if (ic_compiled(P)) {
+    // lam_S = the inverse transform of sum_j i k_j / k^2 F(r lam_Psi2_j) / np^3 (the transpose of Psi2), in B[7]
+    const double kf = 2.0 * M_PI / g.n;
+    const void* l2[3] = {c->lam[3], c->lam[3] + n, c->lam[3] + 2 * n};
+    float2* const d2[3] = {B[7], B[6], B[5]};
+    COLA_TRY(STAGED(kStFwdZ, launch_r2c_rows(P, g, kSrcFloat, l2, 3, g.n, r, d2, c->stream)));
+    COLA_TRY(STAGED(kStFwdY, launch_pencils(P, g, 1, -1, d2, 3, c->stream)));
+    COLA_TRY(STAGED(kStFwdX, launch_grad_adj(P, d2, B[7], c->ktab, (float)(-(double)inv_n3 / (kf * kf)), c->stream)));
+    COLA_TRY(STAGED(kStInvY, launch_pencils(P, g, 1, +1, &B[7], 1, c->stream)));
+    COLA_TRY(STAGED(kStInvZ, launch_c2r_rows(P, g, &B[7], 1, c->stream)));
+    // the six Hessians: zz, yz, yy from one x transform, xz, xy from another, xx
+    COLA_TRY(noise_spectrum(c, wn, B[0]));
+    COLA_TRY(STAGED(kStFwdY, launch_pencils(P, g, 1, -1, &B[0], 1, c->stream)));
+    float2* const h3[3] = {B[0], B[1], B[2]};
+    COLA_TRY(STAGED(kStFwdX, launch_ic_x(P, B[0], h3, 3, 1.0f, c->amp_m2, c->stream)));
+    float2* const t0[3] = {B[0], B[3], B[4]};
+    const int z0[3] = {2, 1, 0}, z1[2] = {1, 0};
+    COLA_TRY(STAGED(kStInvY, launch_ic_y(P, B[0], t0, 3, z0, c->stream)));
+    float2* const t1[3] = {B[1], B[5], nullptr};
+    COLA_TRY(STAGED(kStInvY, launch_ic_y(P, B[1], t1, 2, z1, c->stream)));
+    COLA_TRY(STAGED(kStInvY, launch_pencils(P, g, 1, +1, &B[2], 1, c->stream)));
+    float2* const h[6] = {B[2], B[4], B[0], B[5], B[1], B[3]};   // xx, yy, zz, xy, xz, yz
+    COLA_TRY(STAGED(kStInvZ, launch_c2r_rows(P, g, h, 3, c->stream)));
+    COLA_TRY(STAGED(kStInvZ, launch_c2r_rows(P, g, h + 3, 3, c->stream)));
+    // lam_h = lam_S dS/dh in place, their spectra and those of lam_Psi1 (the ninth in the free lam_F)
+    COLA_TRY(STAGED(kStAdjoint, launch_ic_source_adjoint(g, B[7], h, c->stream)));
+    const void* l1[3] = {c->lam[2], c->lam[2] + n, c->lam[2] + 2 * n};
+    float2* const d1[3] = {B[6], B[7], reinterpret_cast<float2*>(c->lam[4])};
+    for (int q = 0; q < 6; q += 3) {
+      COLA_TRY(STAGED(kStFwdZ, launch_r2c_rows(P, g, kSrcFloat, reinterpret_cast<const void* const*>(h + q), 3, 2LL * g.pc,
+                                               1.0f, h + q, c->stream)));
+      COLA_TRY(STAGED(kStFwdY, launch_pencils(P, g, 1, -1, h + q, 3, c->stream)));
+    }
+    COLA_TRY(STAGED(kStFwdZ, launch_r2c_rows(P, g, kSrcFloat, l1, 3, g.n, 1.0f, d1, c->stream)));
+    COLA_TRY(STAGED(kStFwdY, launch_pencils(P, g, 1, -1, d1, 3, c->stream)));
+    COLA_TRY(STAGED(kStFwdX, launch_lpt_adj(P, h, d1, B[2], r, c->amp_m2, c->stream)));
+    COLA_TRY(STAGED(kStInvY, launch_pencils(P, g, 1, +1, &B[2], 1, c->stream)));
+    return STAGED(kStInvZ, launch_c2r_rows_dense(P, g, B[2], 1.0f, lam_wn, c->stream));
+  }
   // delta_L(k) / np^3 as in the forward
   COLA_TRY(noise_spectrum(c, wn, B[0]));
   COLA_TRY(forward3d_yx(c, g, P, B[0]));

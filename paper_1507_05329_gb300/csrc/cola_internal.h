@@ -85,11 +85,16 @@ struct Grid3 {
 enum RowSource { kSrcFixedPoint = 0, kSrcFloat = 1 };
 
 // Launchers (fft.cu).  All take the stream explicitly.
-// Forward R2C along z of n^2 rows; src is uint64 (scaled: value*scale - 1) or float rows with
-// the given row stride (floats or uint64 elements).  dst: complex grid rows of stride pc.
-int launch_r2c_rows(const FftPlan& p, const Grid3& g, RowSource kind, const void* src,
-                    long long src_row_stride, float scale, float2* dst, cudaStream_t st,
+// Forward R2C along z of the n^2 rows of `fields` (1 to 3) fields; src is uint64 (scaled: value*scale - 1)
+// or float rows (times scale) with the given row stride (floats or uint64 elements).  dst: complex grid rows
+// of stride pc, which may be the (padded) float rows themselves.
+int launch_r2c_rows(const FftPlan& p, const Grid3& g, RowSource kind, const void* const* src, int fields,
+                    long long src_row_stride, float scale, float2* const* dst, cudaStream_t st,
                     unsigned long long* mass_acc = nullptr);
+inline int launch_r2c_rows(const FftPlan& p, const Grid3& g, RowSource kind, const void* src, long long src_row_stride,
+                           float scale, float2* dst, cudaStream_t st, unsigned long long* mass_acc = nullptr) {
+  return launch_r2c_rows(p, g, kind, &src, 1, src_row_stride, scale, &dst, st, mass_acc);
+}
 // Inverse C2R along z, in place on `fields` (1 to 3) complex grids (real rows of stride 2*pc floats).
 int launch_c2r_rows(const FftPlan& p, const Grid3& g, float2* const* data, int fields, cudaStream_t st);
 // The C2R rows of data (not modified) written to out as dense rows of n floats times scale, where the
@@ -108,10 +113,17 @@ inline bool fft_compiled(const FftPlan& p) { return p.ops != nullptr; }
 bool ic_compiled(const FftPlan& p);
 int launch_ic_x(const FftPlan& p, const float2* in, float2* const* out, int fields, float scale, const float* amp_m2,
                 cudaStream_t st);
-int launch_ic_y(const FftPlan& p, const float2* in, float2* const* out, int fields, cudaStream_t st);
+int launch_ic_y(const FftPlan& p, const float2* in, float2* const* out, int fields, const int* zp, cudaStream_t st);
 int launch_ic_z1(const FftPlan& p, float2* const t[6], float2* src_k, float* psi1, float r_scale, cudaStream_t st);
 int launch_ic_z2(const FftPlan& p, float2* const f[3], const float* psi1, float* psi2, float* s, float* v,
                  float r_scale, float d1, float d2, cudaStream_t st);
+// The adjoint's x passes of a compiled length (any, and up to 1024): from three spectra over k_y, k_z the
+// inverse x transform of -i g_scale / |m|^2 sum_j D_j L_j, and from the nine cotangents of the first-order
+// 2LPT fields that of delta_L's.
+int launch_grad_adj(const FftPlan& p, float2* const l[3], float2* out, const float* dtab, float g_scale,
+                    cudaStream_t st);
+int launch_lpt_adj(const FftPlan& p, const float2* const h[6], const float2* const l[3], float2* out, float r_scale,
+                   const float* amp_m2, cudaStream_t st);
 // C2C along y (axis 1) or x (axis 0) of `fields` (1 to 3) complex grids; dir = -1 forward, +1 inverse.
 int launch_pencils(const FftPlan& p, const Grid3& g, int axis, int dir, float2* const* data, int fields,
                    cudaStream_t st);
@@ -421,6 +433,7 @@ struct cola_ctx {
   float2* cbuf[3] = {nullptr, nullptr, nullptr};   // complex N x N x pc each
   float* dtab = nullptr;                  // gradient kernel per storage index, N entries
   float* amp_m2 = nullptr;                // sqrt(P(k)/V_cell) per integer m^2 of the lattice
+  float* ktab = nullptr;                  // k in rad per lattice spacing per storage index, 0 at Nyquist, np entries
   long long* edges = nullptr;             // P(k) bin edges in m^2 (device), up to 129
   long long* edges_host = nullptr;        // pinned host copy of the current edges
   int edges_nbins = 0;

@@ -107,18 +107,19 @@ void fft_plan_free(FftPlan* plan) {
   plan->tw = nullptr;
 }
 
-int launch_r2c_rows(const FftPlan& p, const Grid3& g, RowSource kind, const void* src,
-                    long long src_row_stride, float scale, float2* dst, cudaStream_t st,
+int launch_r2c_rows(const FftPlan& p, const Grid3& g, RowSource kind, const void* const* src, int fields,
+                    long long src_row_stride, float scale, float2* const* dst, cudaStream_t st,
                     unsigned long long* mass_acc) {
   if (p.ops) {
-    p.ops->r2c(kind, src, src_row_stride, scale, dst, p.tab, mass_acc, st);
+    p.ops->r2c(kind, src, fields, src_row_stride, scale, dst, p.tab, mass_acc, st);
     return check_launch("r2c");
   }
   const long long nrows = (long long)g.rows();
   const TileShape t = tile_shape(g.n, 1 << 20);
   const unsigned blocks = (unsigned)((nrows + (2LL << t.lw) - 1) / (2LL << t.lw));
-  generic_r2c_launch(p.dev, t.lw, blocks, t.threads, t.smem, kind, src, src_row_stride, scale, dst, g.pc, nrows,
-                     kind == kSrcFixedPoint ? mass_acc : nullptr, st);
+  for (int i = 0; i < fields; ++i)
+    generic_r2c_launch(p.dev, t.lw, blocks, t.threads, t.smem, kind, src[i], src_row_stride, scale, dst[i], g.pc, nrows,
+                       kind == kSrcFixedPoint ? mass_acc : nullptr, st);
   return check_launch("r2c_rows");
 }
 
@@ -156,8 +157,8 @@ int launch_ic_x(const FftPlan& p, const float2* in, float2* const* out, int fiel
   p.ops->ic_x(in, out, fields, scale, amp_m2, p.tab, st);
   return check_launch("ic_x");
 }
-int launch_ic_y(const FftPlan& p, const float2* in, float2* const* out, int fields, cudaStream_t st) {
-  p.ops->ic_y(in, out, fields, p.tab, st);
+int launch_ic_y(const FftPlan& p, const float2* in, float2* const* out, int fields, const int* zp, cudaStream_t st) {
+  p.ops->ic_y(in, out, fields, zp, p.tab, st);
   return check_launch("ic_y");
 }
 int launch_ic_z1(const FftPlan& p, float2* const t[6], float2* src_k, float* psi1, float r_scale, cudaStream_t st) {
@@ -168,6 +169,17 @@ int launch_ic_z2(const FftPlan& p, float2* const f[3], const float* psi1, float*
                  float r_scale, float d1, float d2, cudaStream_t st) {
   p.ops->ic_z2(f, psi1, psi2, s, v, r_scale, d1, d2, p.tab, st);
   return check_launch("ic_z2");
+}
+
+int launch_lpt_adj(const FftPlan& p, const float2* const h[6], const float2* const l[3], float2* out, float r_scale,
+                   const float* amp_m2, cudaStream_t st) {
+  p.ops->lpt_adj(h, l, out, r_scale, amp_m2, p.tab, st);
+  return check_launch("lpt_adj");
+}
+int launch_grad_adj(const FftPlan& p, float2* const l[3], float2* out, const float* dtab, float g_scale,
+                    cudaStream_t st) {
+  p.ops->grad_adj(l, out, dtab, g_scale, p.tab, st);
+  return check_launch("grad_adj");
 }
 
 int launch_pencils(const FftPlan& p, const Grid3& g, int axis, int dir, float2* const* data, int fields,

@@ -22,12 +22,19 @@ struct Launch {
   static constexpr long long kPairs = (long long)N * N / 2;
   static constexpr unsigned kRowBlocks = (unsigned)((kPairs + R::pairs - 1) / R::pairs);
 
-  static void r2c(int kind, const void* src, long long rs, float scale, float2* dst, const FftTables& t,
-                  unsigned long long* acc, cudaStream_t st) {
+  static void r2c(int kind, const void* const* src, int fields, long long rs, float scale, float2* const* dst,
+                  const FftTables& t, unsigned long long* acc, cudaStream_t st) {
+    Src3 s{};
+    Ptr3 d{};
+    for (int i = 0; i < fields; ++i) {
+      s.p[i] = src[i];
+      d.p[i] = dst[i];
+    }
+    const dim3 grid(kRowBlocks, fields);
     if (kind == kSrcFixedPoint)
-      go(k_r2c<N, kSrcFixedPoint>, kRowBlocks, R::T, R2cCfg<N>::smem, st, src, rs, scale, dst, kPairs, t.fwd, acc);
+      go(k_r2c<N, kSrcFixedPoint>, grid, R::T, R2cCfg<N>::smem, st, s, rs, scale, d, kPairs, t.fwd, acc);
     else
-      go(k_r2c<N, kSrcFloat>, kRowBlocks, R::T, R2cCfg<N>::smem, st, src, rs, scale, dst, kPairs, t.fwd,
+      go(k_r2c<N, kSrcFloat>, grid, R::T, R2cCfg<N>::smem, st, s, rs, scale, d, kPairs, t.fwd,
          (unsigned long long*)nullptr);
   }
   static void c2r(float2* const* data, int fields, const FftTables& t, cudaStream_t st) {
@@ -78,13 +85,18 @@ struct Launch {
            (const float*)nullptr, t.fwd, t.rev);
     }
   }
-  static void ic_y(const float2* in, float2* const* out, int fields, const FftTables& t, cudaStream_t st) {
+  static void ic_y(const float2* in, float2* const* out, int fields, const int* zp, const FftTables& t,
+                   cudaStream_t st) {
     if constexpr (kIc) {
       const dim3 grid(C::chunks, N);
+      Pow3 z{};
+      for (int i = 0; zp && i < fields; ++i) z.p[i] = zp[i];
       if (fields == 3)
-        go(k_ic_y<N, 3>, grid, C::T, MultiCfg<N, 3>::smem, st, in, Ptr3{{out[0], out[1], out[2]}}, t.fwd);
+        go(k_ic_y<N, 3>, grid, C::T, MultiCfg<N, 3>::smem, st, in, Ptr3{{out[0], out[1], out[2]}}, z,
+           t.fwd);
       else
-        go(k_ic_y<N, 2>, grid, C::T, MultiCfg<N, 2>::smem, st, in, Ptr3{{out[0], out[1], nullptr}}, t.fwd);
+        go(k_ic_y<N, 2>, grid, C::T, MultiCfg<N, 2>::smem, st, in, Ptr3{{out[0], out[1], nullptr}}, z,
+           t.fwd);
     }
   }
   static void ic_z1(float2* const* f, float2* src_k, float* psi1, float r_scale, const FftTables& t, cudaStream_t st) {
@@ -98,6 +110,17 @@ struct Launch {
       go(k_ic_z2<N>, dim3(kRowBlocks, 3), R::T, C2rCfg<N>::smem, st, Ptr3{{f[0], f[1], f[2]}}, psi1, psi2, s, v,
          (long long)N * N * N, r_scale, d1, d2, kPairs, t.fwd);
   }
+  static void lpt_adj(const float2* const* h, const float2* const* p, float2* out, float r_scale, const float* amp_m2,
+                      const FftTables& t, cudaStream_t st) {
+    if constexpr (kIc)
+      go(k_lpt_adj<N>, dim3(C::chunks, N), C::T, MultiCfg<N, 3>::smem, st,
+         Lpt9{{h[0], h[1], h[2], h[3], h[4], h[5]}, {p[0], p[1], p[2]}}, out, r_scale, amp_m2, t.fwd, t.rev);
+  }
+  static void grad_adj(float2* const* l, float2* out, const float* dtab, float g_scale, const FftTables& t,
+                       cudaStream_t st) {
+    go(k_grad_adj<N>, dim3(C::chunks, N), C::T, MultiCfg<N, 2>::smem, st, (const float2*)l[0], (const float2*)l[1],
+       (const float2*)l[2], out, dtab, g_scale, t.fwd, t.rev);
+  }
 };
 
 // the launches of size I, and the table of this part's sizes
@@ -106,7 +129,7 @@ constexpr FftOps ops_of() {
   constexpr int N = kCtSizes[I];
   using L = Launch<N>;
   return FftOps{N, L::r2c, L::c2r, L::c2r_dense, L::pencils, L::x_mul, L::green, L::kIc ? L::ic_x : nullptr, L::ic_y,
-                L::ic_z1, L::ic_z2, L::pencils_yz};
+                L::ic_z1, L::ic_z2, L::lpt_adj, L::grad_adj, L::pencils_yz};
 }
 constexpr int kMine = (kCtCount - COLA_CT_PART + COLA_CT_PARTS - 1) / COLA_CT_PARTS;
 template <int... K>

@@ -205,6 +205,9 @@ __device__ __forceinline__ float2* pen_middle(float2* a, float2* b, const float2
 struct Ptr3 {
   float2* p[3];
 };
+struct Src3 {
+  const void* p[3];
+};
 
 // C2C along y (AXIS 1) or x (AXIS 0), in place, of the fields data.p[blockIdx.z]
 template <int N, int AXIS, int DIR>
@@ -486,9 +489,21 @@ __global__ void __launch_bounds__(PenCfg<N>::T, MultiCfg<N, NT>::minb) k_ic_x(co
   multi_finish<N, true, +1, T, 1>(sm, d, twr, tid);
 }
 
-// Inverse y transforms of in times 1, k_y, .. (NT of them) into out.p[0..NT-1]; out.p[0] may be in.
+struct Pow3 {
+  int p[3];   // powers 0, 1, 2
+};
+// column store times a factor
+template <long long JS>
+struct ColScaled {
+  ColG<JS> g;
+  float f;
+  __device__ __forceinline__ void operator()(int j, int w, float2 v) const { g(j, w, f * v); }
+};
+
+// Inverse y transforms of in times 1, k_y, .. (NT of them), times k_z^zp.p[i], into out.p[0..NT-1];
+// out.p[0] may be in.
 template <int N, int NT>
-__global__ void __launch_bounds__(PenCfg<N>::T, MultiCfg<N, NT>::minb) k_ic_y(const float2* in, Ptr3 out,
+__global__ void __launch_bounds__(PenCfg<N>::T, MultiCfg<N, NT>::minb) k_ic_y(const float2* in, Ptr3 out, Pow3 zp,
                                                                               const float2* __restrict__ tw) {
   extern __shared__ float2 sm[];
   using C = PenCfg<N>;
@@ -512,10 +527,224 @@ __global__ void __launch_bounds__(PenCfg<N>::T, MultiCfg<N, NT>::minb) k_ic_y(co
     }
   }
   __syncthreads();
-  ColG<JS> d[NT];
+  constexpr float kf = 6.283185307179586f / N;
+  const float kz = col * kf, kz_odd = 2 * col == N ? 0.0f : kz;
+  ColScaled<JS> d[NT];
 #pragma unroll
-  for (int i = 0; i < NT; ++i) d[i] = ColG<JS>{out.p[i] + off, ok};
+  for (int i = 0; i < NT; ++i)
+    d[i] = ColScaled<JS>{{out.p[i] + off, ok}, zp.p[i] == 0 ? 1.0f : (zp.p[i] == 1 ? kz_odd : kz * kz)};
   multi_finish<N, false, +1, T, 1>(sm, d, tw, tid);
+}
+
+// ---- transposed gradients (the adjoint's x passes) ------------------------------------------------
+// NT forward transforms of the tiles s, s + tile, .. whose first groups are done, but for the last groups
+template <int N, int T, int NT, int G = 1>
+__device__ __forceinline__ void multi_forward(float2* s, const float2* __restrict__ tw, int tid) {
+  if constexpr (G + 1 < PlanOf<N, false>::m) {
+#pragma unroll
+    for (int i = 0; i < NT; ++i) pen_inplace<N, false, G, -1, T>(s + i * PenCfg<N>::tile, tw, tid);
+    __syncthreads();
+    multi_forward<N, T, NT, G + 1>(s, tw, tid);
+  }
+}
+
+// The inverse x transform of -i g sum_j D(k_j) L_j(k), g = g_scale / |m|^2, of three spectra over k_y, k_z
+// (x still in real space); out may be one of them.  D(k_y) and D(k_z) are constant along x, so two forward
+// transforms serve the three components.
+template <int N>
+__global__ void __launch_bounds__(PenCfg<N>::T, MultiCfg<N, 2>::minb) k_grad_adj(const float2* l0, const float2* l1,
+                                                                                 const float2* l2, float2* out,
+                                                                                 const float* __restrict__ dtab, float g_scale,
+                                                                                 const float2* __restrict__ twf,
+                                                                                 const float2* __restrict__ twr) {
+  extern __shared__ float2 sm[];
+  using C = PenCfg<N>;
+  using A = Group<N, false, 0, -1>;
+  using L = Group<N, false, PlanOf<N, false>::m - 1, -1>;
+  using F = Group<N, true, 0, +1>;
+  constexpr int T = C::T;
+  constexpr long long JS = (long long)N * C::PC;
+  const int tid = threadIdx.x, col = blockIdx.x * C::W + (tid & (C::W - 1)), y = blockIdx.y;
+  const bool ok = col < C::NC;
+  const long long off = (long long)y * C::PC + col;
+  const float dy = __ldg(dtab + y), dz = ok ? __ldg(dtab + col) : 0.0f;
+  {
+    constexpr int TOT = A::NB << C::lw, IT = (TOT + T - 1) / T;
+#pragma unroll(IT <= 2 ? IT : 1)
+    for (int it = 0; it < IT; ++it) {
+      const int idx = tid + it * T;
+      if (TOT % T == 0 || idx < TOT) {
+        const int w = idx & (C::W - 1), bb = idx >> C::lw;
+        float2 v[A::R], u[A::R];
+#pragma unroll
+        for (int r = 0; r < A::R; ++r) {
+          const long long e = off + (bb + r * A::NB) * JS;
+          v[r] = u[r] = make_float2(0.f, 0.f);
+          if (ok) {
+            v[r] = l0[e];
+            u[r] = dy * l1[e] + dz * l2[e];
+          }
+        }
+        A::run(v, twf, 0);
+        A::run(u, twf, 0);
+#pragma unroll
+        for (int r = 0; r < A::R; ++r) {
+          sm[((bb * A::R + r) << C::lw) + w] = v[r];
+          sm[C::tile + ((bb * A::R + r) << C::lw) + w] = u[r];
+        }
+      }
+    }
+  }
+  __syncthreads();
+  multi_forward<N, T, 2>(sm, twf, tid);
+  constexpr int TOT = L::NB << C::lw, IT = (TOT + T - 1) / T;
+  float2 spec[IT][L::R];
+  const int my = y < N / 2 ? y : y - N;
+#pragma unroll
+  for (int it = 0; it < IT; ++it) {
+    const int idx = tid + it * T;
+    if (TOT % T == 0 || idx < TOT) {
+      const int bb = idx >> C::lw;
+      float2 v[L::R], u[L::R];
+#pragma unroll
+      for (int r = 0; r < L::R; ++r) {
+        v[r] = sm[idx + r * (L::NB << C::lw)];
+        u[r] = sm[C::tile + idx + r * (L::NB << C::lw)];
+      }
+      L::run(v, twf, bb);
+      L::run(u, twf, bb);
+      const int myz = my * my + col * col;
+#pragma unroll
+      for (int r = 0; r < L::R; ++r) {
+        const int j = bb + r * L::NS, mx = j < N / 2 ? j : j - N, m2 = mx * mx + myz;
+        const float g = m2 > 0 ? g_scale / (float)m2 : 0.0f, dx = __ldg(dtab + j);
+        const float2 z = dx * v[r] + u[r];
+        spec[it][r] = make_float2(g * z.y, -g * z.x);
+      }
+    }
+  }
+  __syncthreads();   // the forward's tiles are free
+#pragma unroll
+  for (int it = 0; it < IT; ++it) {
+    const int idx = tid + it * T;
+    if (TOT % T == 0 || idx < TOT) {
+      const int w = idx & (C::W - 1), bb = idx >> C::lw;
+      F::run(spec[it], twr, 0);
+#pragma unroll
+      for (int r = 0; r < L::R; ++r) sm[((bb * L::R + r) << C::lw) + w] = spec[it][r];
+    }
+  }
+  __syncthreads();
+  const ColG<JS> d[1] = {{out + off, ok}};
+  multi_finish<N, true, +1, T, 1>(sm, d, twr, tid);
+}
+
+// Transpose of the first-order 2LPT maps: the inverse x transform of
+//   amp(|m|^2) / k^2 [ sum_ij k_i k_j h_ij - i r sum_j k_j p_j ]
+// of the six Hessian cotangents h (xx, yy, zz, xy, xz, yz) and the three displacement cotangents p, all
+// spectra over k_y, k_z with x in real space; out may be one of them.  Powers of k_y and k_z are constant
+// along x: three forward transforms, of the factors of 1, k_x and k_x^2, serve all nine.
+struct Lpt9 {
+  const float2* h[6];
+  const float2* p[3];
+};
+template <int N>
+__global__ void __launch_bounds__(PenCfg<N>::T, MultiCfg<N, 3>::minb) k_lpt_adj(Lpt9 in, float2* out, float r_scale,
+                                                                               const float* __restrict__ amp_m2,
+                                                                               const float2* __restrict__ twf,
+                                                                               const float2* __restrict__ twr) {
+  extern __shared__ float2 sm[];
+  using C = PenCfg<N>;
+  using A = Group<N, false, 0, -1>;
+  using L = Group<N, false, PlanOf<N, false>::m - 1, -1>;
+  using F = Group<N, true, 0, +1>;
+  constexpr int T = C::T;
+  constexpr long long JS = (long long)N * C::PC;
+  constexpr float kf = 6.283185307179586f / N;
+  const int tid = threadIdx.x, col = blockIdx.x * C::W + (tid & (C::W - 1)), y = blockIdx.y;
+  const bool ok = col < C::NC;
+  const long long off = (long long)y * C::PC + col;
+  const int my = y < N / 2 ? y : y - N;
+  const float ky = my * kf, kz = col * kf, oy = 2 * y == N ? 0.0f : ky, oz = 2 * col == N ? 0.0f : kz;
+  {
+    constexpr int TOT = A::NB << C::lw, IT = (TOT + T - 1) / T;
+#pragma unroll 1
+    for (int it = 0; it < IT; ++it) {
+      const int idx = tid + it * T;
+      if (TOT % T == 0 || idx < TOT) {
+        const int w = idx & (C::W - 1), bb = idx >> C::lw;
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {   // factors of 1, k_x, k_x^2
+          float2 v[A::R];
+#pragma unroll
+          for (int r = 0; r < A::R; ++r) {
+            const long long e = off + (bb + r * A::NB) * JS;
+            v[r] = make_float2(0.f, 0.f);
+            if (ok) {
+              if (q == 0) {
+                const float2 g = r_scale * (oy * in.p[1][e] + oz * in.p[2][e]);
+                v[r] = (ky * ky) * in.h[1][e] + (kz * kz) * in.h[2][e] + (oy * oz) * in.h[5][e] + make_float2(g.y, -g.x);
+              } else if (q == 1) {
+                const float2 g = r_scale * in.p[0][e];
+                v[r] = oy * in.h[3][e] + oz * in.h[4][e] + make_float2(g.y, -g.x);
+              } else {
+                v[r] = in.h[0][e];
+              }
+            }
+          }
+          A::run(v, twf, 0);
+#pragma unroll
+          for (int r = 0; r < A::R; ++r) sm[q * C::tile + ((bb * A::R + r) << C::lw) + w] = v[r];
+        }
+      }
+    }
+  }
+  __syncthreads();
+  multi_forward<N, T, 3>(sm, twf, tid);
+  constexpr int TOT = L::NB << C::lw, IT = (TOT + T - 1) / T;
+  float2 spec[IT][L::R];
+#pragma unroll
+  for (int it = 0; it < IT; ++it) {
+    const int idx = tid + it * T;
+    if (TOT % T == 0 || idx < TOT) {
+      const int bb = idx >> C::lw;
+#pragma unroll
+      for (int q = 0; q < 3; ++q) {
+        float2 v[L::R];
+#pragma unroll
+        for (int r = 0; r < L::R; ++r) v[r] = sm[q * C::tile + idx + r * (L::NB << C::lw)];
+        L::run(v, twf, bb);
+#pragma unroll
+        for (int r = 0; r < L::R; ++r) {
+          const int j = bb + r * L::NS, mx = j < N / 2 ? j : j - N;
+          const float kx = mx * kf;
+          const float f = q == 0 ? 1.0f : (q == 1 ? (2 * j == N ? 0.0f : kx) : kx * kx);
+          spec[it][r] = q == 0 ? v[r] : spec[it][r] + f * v[r];
+        }
+      }
+      const int myz = my * my + col * col;
+#pragma unroll
+      for (int r = 0; r < L::R; ++r) {
+        const int j = bb + r * L::NS, mx = j < N / 2 ? j : j - N, m2 = mx * mx + myz;
+        const float g = m2 > 0 && ok ? __ldg(amp_m2 + m2) / ((float)m2 * kf * kf) : 0.0f;
+        spec[it][r] = g * spec[it][r];
+      }
+    }
+  }
+  __syncthreads();   // the forward's tiles are free
+#pragma unroll
+  for (int it = 0; it < IT; ++it) {
+    const int idx = tid + it * T;
+    if (TOT % T == 0 || idx < TOT) {
+      const int w = idx & (C::W - 1), bb = idx >> C::lw;
+      F::run(spec[it], twr, 0);
+#pragma unroll
+      for (int r = 0; r < L::R; ++r) sm[((bb * L::R + r) << C::lw) + w] = spec[it][r];
+    }
+  }
+  __syncthreads();
+  const ColG<JS> d[1] = {{out + off, ok}};
+  multi_finish<N, true, +1, T, 1>(sm, d, twr, tid);
 }
 
 // ---- row pairs (the contiguous axis) -------------------------------------------------------------
@@ -652,16 +881,17 @@ struct R2cCfg {
 };
 
 // Forward R2C of the row pairs (in place when src is dst's own rows: a CTA reads its rows whole first)
+// of the fields src.p[blockIdx.y] into dst.p[blockIdx.y]
 template <int N, int SRC>
-__global__ void __launch_bounds__(RowCfg<N>::T, RowCfg<N>::minb(2)) k_r2c(const void* src, long long rs, float scale,
-                                                                          float2* dst, long long npairs,
+__global__ void __launch_bounds__(RowCfg<N>::T, RowCfg<N>::minb(2)) k_r2c(Src3 src, long long rs, float scale,
+                                                                          Ptr3 dst, long long npairs,
                                                                           const float2* __restrict__ tw,
                                                                           unsigned long long* mass_acc) {
   extern __shared__ float2 sm[];
   using C = RowCfg<N>;
   const int tid = threadIdx.x;
   const long long pair0 = (long long)blockIdx.x * C::pairs;
-  const RowPairLoad<SRC> g{src, rs, pair0, npairs, scale};
+  const RowPairLoad<SRC> g{src.p[blockIdx.y], rs, pair0, npairs, scale};
   float2* a = sm;
   float2* b = sm + C::buf;
   row_stage<N, 0, -1>(g, RowSm<N>{a}, tw, tid);
@@ -671,7 +901,7 @@ __global__ void __launch_bounds__(RowCfg<N>::T, RowCfg<N>::minb(2)) k_r2c(const 
   float2* res = cur == a ? b : a;
   row_stage<N, PlanOf<N, false>::m - 1, -1>(RowSm<N>{cur}, RowSm<N>{res}, tw, tid);
   __syncthreads();
-  untangle_rows<N>(res, dst, pair0, npairs, tid);
+  untangle_rows<N>(res, dst.p[blockIdx.y], pair0, npairs, tid);
 }
 
 // C[k] = A[k] + i B[k] of two Hermitian half rows

@@ -11,8 +11,8 @@ namespace cola {
 // Every launch covers a whole n^3 field (rows of pc complex entries); see fft_ct.cuh for the passes.
 struct FftOps {
   int n;
-  void (*r2c)(int kind, const void* src, long long rs, float scale, float2* dst, const FftTables&,
-              unsigned long long* mass_acc, cudaStream_t);
+  void (*r2c)(int kind, const void* const* src, int fields, long long rs, float scale, float2* const* dst,
+              const FftTables&, unsigned long long* mass_acc, cudaStream_t);
   void (*c2r)(float2* const* data, int fields, const FftTables&, cudaStream_t);
   void (*c2r_dense)(const float2* data, float scale, float* out, const FftTables&, cudaStream_t);
   void (*pencils)(int axis, int dir, float2* const* data, int fields, const FftTables&, cudaStream_t);
@@ -22,10 +22,13 @@ struct FftOps {
   // 2LPT fields (null where three tiles do not fit a CTA); see fft_ct.cuh
   void (*ic_x)(const float2* in, float2* const* out, int fields, float scale, const float* amp_m2, const FftTables&,
                cudaStream_t);
-  void (*ic_y)(const float2* in, float2* const* out, int fields, const FftTables&, cudaStream_t);
+  void (*ic_y)(const float2* in, float2* const* out, int fields, const int* zp, const FftTables&, cudaStream_t);
   void (*ic_z1)(float2* const* t, float2* src_k, float* psi1, float r_scale, const FftTables&, cudaStream_t);
   void (*ic_z2)(float2* const* f, const float* psi1, float* psi2, float* s, float* v, float r_scale, float d1, float d2,
                 const FftTables&, cudaStream_t);
+  void (*lpt_adj)(const float2* const* h, const float2* const* p, float2* out, float r_scale, const float* amp_m2,
+                  const FftTables&, cudaStream_t);
+  void (*grad_adj)(float2* const* l, float2* out, const float* dtab, float g_scale, const FftTables&, cudaStream_t);
   void (*pencils_yz)(const float2* h, float2* out_y, float2* out_z, const float* dtab, const FftTables&, cudaStream_t);
 };
 
