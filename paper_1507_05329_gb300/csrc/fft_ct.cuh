@@ -39,46 +39,64 @@ struct Group {
     return w;
   }
   __device__ __forceinline__ static void run(float2 (&v)[R], const float2* __restrict__ table, int k) {
+    run(reinterpret_cast<float2(&)[1][R]>(v), table, k);
+  }
+  // NV butterflies of the same index (adjacent columns)
+  template <int NV>
+  __device__ __forceinline__ static void run(float2 (&v)[NV][R], const float2* __restrict__ table, int k) {
     const float2* t1 = table + O1 + k;
-    if constexpr (R2 == 1) {
-      if constexpr (NS > 1) {
+    if constexpr (NS > 1) {
 #pragma unroll
-        for (int r = 1; r < R1; ++r) v[r] = cmul(v[r], tw(t1 + (r - 1) * NS));
+      for (int r = 1; r < R1; ++r) {
+        const float2 t = tw(t1 + (r - 1) * NS);
+#pragma unroll
+        for (int c = 0; c < NV; ++c)
+#pragma unroll
+          for (int i = 0; i < R2; ++i) v[c][i + r * R2] = cmul(v[c][i + r * R2], t);
       }
-      Dft<R1, DIR>::run(v);
+    }
+    if constexpr (R2 == 1) {
+#pragma unroll
+      for (int c = 0; c < NV; ++c) Dft<R1, DIR>::run(v[c]);
     } else {
       // stage r1 on the R2 sub-butterflies b + i N/R, then stage r2 on the R1 butterflies their
       // outputs r share
 #pragma unroll
-      for (int i = 0; i < R2; ++i) {
-        float2 t[R1];
+      for (int c = 0; c < NV; ++c)
 #pragma unroll
-        for (int r = 0; r < R1; ++r) t[r] = v[i + r * R2];
-        if constexpr (NS > 1) {
+        for (int i = 0; i < R2; ++i) {
+          float2 t[R1];
 #pragma unroll
-          for (int r = 1; r < R1; ++r) t[r] = cmul(t[r], tw(t1 + (r - 1) * NS));
+          for (int r = 0; r < R1; ++r) t[r] = v[c][i + r * R2];
+          Dft<R1, DIR>::run(t);
+#pragma unroll
+          for (int r = 0; r < R1; ++r) v[c][i + r * R2] = t[r];
         }
-        Dft<R1, DIR>::run(t);
-#pragma unroll
-        for (int r = 0; r < R1; ++r) v[i + r * R2] = t[r];
-      }
       const float2* t2 = table + O2 + k;
-      float2 o[R];
 #pragma unroll
-      for (int r = 0; r < R1; ++r) {
-        float2 u[R2];
+      for (int r = 0; r < R1; ++r)
 #pragma unroll
-        for (int i = 0; i < R2; ++i) u[i] = v[i + r * R2];
-        if (NS > 1 || r > 0) {
+        for (int i = 1; i < R2; ++i)
+          if (NS > 1 || r > 0) {
+            const float2 t = tw(t2 + (i - 1) * NS * R1 + r * NS);
 #pragma unroll
-          for (int i = 1; i < R2; ++i) u[i] = cmul(u[i], tw(t2 + (i - 1) * NS * R1 + r * NS));
+            for (int c = 0; c < NV; ++c) v[c][i + r * R2] = cmul(v[c][i + r * R2], t);
+          }
+#pragma unroll
+      for (int c = 0; c < NV; ++c) {
+        float2 o[R];
+#pragma unroll
+        for (int r = 0; r < R1; ++r) {
+          float2 u[R2];
+#pragma unroll
+          for (int i = 0; i < R2; ++i) u[i] = v[c][i + r * R2];
+          Dft<R2, DIR>::run(u);
+#pragma unroll
+          for (int i = 0; i < R2; ++i) o[r + i * R1] = u[i];
         }
-        Dft<R2, DIR>::run(u);
 #pragma unroll
-        for (int i = 0; i < R2; ++i) o[r + i * R1] = u[i];
+        for (int r = 0; r < R; ++r) v[c][r] = o[r];
       }
-#pragma unroll
-      for (int r = 0; r < R; ++r) v[r] = o[r];
     }
   }
   __device__ __forceinline__ static int k_of(int b) {
@@ -90,22 +108,29 @@ struct Group {
 };
 
 // ---- tiles of W columns (strided passes) ---------------------------------------------------------
-// element (j, w) at (j << LW) + w.  Rows are 64 bytes: only the stores of a first group of even radix
+// element (j, w) at (j << lw) + w.  Rows are 64 bytes: only the stores of a first group of even radix
 // meet two rows on the same banks (a pair of wavefronts for one), which costs less than a padded index.
+//
+// Groups up to radix kPairR run on two adjacent columns per thread: every access moves 16 bytes and a
+// twiddle serves both.  On single columns the passes waited on the load/store queue (mio_throttle 13 of 30
+// warp cycles per instruction, L1 at 73%, DRAM at 52%; now 7, 81% and 62%).  ms, before -> after: 512^3 y
+// 0.254 -> 0.214, Green 0.554 -> 0.505, inverse y 0.617 -> 0.580; 384^3 inverse y 0.268 -> 0.247.  A column beyond the row's valid entries may be the
+// row's pad entry (rows hold an even number): it is transformed like the others and never used.
+constexpr int kPairR = 10;
+
 template <int N>
 struct PenCfg {
   static constexpr int lw = N <= 1536 ? 3 : 2;             // two tiles (the Green pass) fit a CTA
   static constexpr int W = 1 << lw;
   static constexpr Groups P = make_groups(N, false);
-  static constexpr int ept = P.max_radix > 10 ? 16 : 8;   // values a thread holds in a group
-  static constexpr int T = imin(1024, round_up((N * W + ept - 1) / ept, 32));
+  static constexpr int T = imin(1024, round_up((N * W + 15) / 16, 32));   // 16 values per thread
   static constexpr int PC = ((N / 2 + 1) + 1) & ~1;
   static constexpr int NC = N / 2 + 1;
   static constexpr int chunks = (NC + W - 1) / W;
   static constexpr int tile = N * W;                       // complex elements
   // one work buffer that the middle groups overwrite (each thread's values in registers over a barrier);
   // two where two still leave as many CTAs per SM as the registers do
-  static constexpr int regs = ept == 16 ? 64 : 40;
+  static constexpr int regs = 64;
   static constexpr int by_regs = imax(1, imin(2048, 65536 / regs) / T);
   static constexpr bool pp = P.m > 2 && 2 * tile * 8 * by_regs <= 220 * 1024;
   static constexpr int bufs = pp ? 2 : 1;
@@ -113,89 +138,147 @@ struct PenCfg {
   static constexpr int minb = imax(1, imin(imin(by_regs, 24), (224 * 1024) / (smem + 1024)));
 };
 
-template <int N>
-struct TileR {
-  const float2* s;
-  __device__ __forceinline__ float2 operator()(int j, int w) const { return s[(j << PenCfg<N>::lw) + w]; }
-};
-template <int N>
-struct TileW {
-  float2* s;
-  __device__ __forceinline__ void operator()(int j, int w, float2 v) const { s[(j << PenCfg<N>::lw) + w] = v; }
+// The butterflies of a radix-R group over a tile: columns per task and task idx's columns w.. and butterfly
+template <int N, int R>
+struct PenTask {
+  using C = PenCfg<N>;
+  static constexpr int NV = R <= kPairR ? 2 : 1;
+  static constexpr int TOT = ((N / R) << C::lw) / NV, IT = (TOT + C::T - 1) / C::T;
+  __device__ __forceinline__ static bool live(int idx) { return TOT % C::T == 0 || idx < TOT; }
+  __device__ __forceinline__ static int w(int idx) { return (idx & (C::W / NV - 1)) * NV; }
+  __device__ __forceinline__ static int b(int idx) { return idx / (C::W / NV); }
 };
 
-// W adjacent columns of a strided pencil of row stride JS; columns beyond the row's valid entries read 0
-template <long long JS>
-struct ColG {
-  float2* base;   // column col0 + w of row 0
-  bool ok;        // the thread's column exists
-  __device__ __forceinline__ float2 operator()(int j, int) const { return ok ? base[j * JS] : make_float2(0.f, 0.f); }
-  __device__ __forceinline__ void operator()(int j, int, float2 v) const {
-    if (ok) base[j * JS] = v;
+// rows j0 + r STEP of columns w.. of a tile in shared memory
+template <int N>
+struct Tile {
+  float2* s;
+  template <int STEP, int NV, int R>
+  __device__ __forceinline__ void load(int j0, int w, float2 (&v)[NV][R]) const {
+    const float2* q = s + (j0 << PenCfg<N>::lw) + w;
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      if constexpr (NV == 2) {
+        const float4 t = *reinterpret_cast<const float4*>(q + r * (STEP << PenCfg<N>::lw));
+        v[0][r] = make_float2(t.x, t.y);
+        v[1][r] = make_float2(t.z, t.w);
+      } else {
+        v[0][r] = q[r * (STEP << PenCfg<N>::lw)];
+      }
+    }
+  }
+  template <int STEP, int NV, int R>
+  __device__ __forceinline__ void store(int j0, int w, const float2 (&v)[NV][R]) const {
+    float2* q = s + (j0 << PenCfg<N>::lw) + w;
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      if constexpr (NV == 2)
+        *reinterpret_cast<float4*>(q + r * (STEP << PenCfg<N>::lw)) = make_float4(v[0][r].x, v[0][r].y, v[1][r].x, v[1][r].y);
+      else q[r * (STEP << PenCfg<N>::lw)] = v[0][r];
+    }
   }
 };
 
-template <int N, bool REV, int G, int DIR, int T, class Src, class Dst>
+// the same of a strided pencil in global memory (row stride JS); columns from `left` on read 0
+template <long long JS>
+struct ColG {
+  float2* base;   // column 0 of the tile, row 0
+  int left;       // valid columns
+  template <int STEP, int NV, int R>
+  __device__ __forceinline__ void load(int j0, int w, float2 (&v)[NV][R]) const {
+    const float2* q = base + j0 * JS + w;
+    const bool ok = w < left;
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      if constexpr (NV == 2) {
+        const float4 t = ok ? *reinterpret_cast<const float4*>(q + r * (STEP * JS)) : make_float4(0.f, 0.f, 0.f, 0.f);
+        v[0][r] = make_float2(t.x, t.y);
+        v[1][r] = make_float2(t.z, t.w);
+      } else {
+        v[0][r] = ok ? q[r * (STEP * JS)] : make_float2(0.f, 0.f);
+      }
+    }
+  }
+  template <int STEP, int NV, int R>
+  __device__ __forceinline__ void store(int j0, int w, const float2 (&v)[NV][R]) const {
+    if (w >= left) return;
+    float2* q = base + j0 * JS + w;
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      if constexpr (NV == 2)
+        *reinterpret_cast<float4*>(q + r * (STEP * JS)) = make_float4(v[0][r].x, v[0][r].y, v[1][r].x, v[1][r].y);
+      else q[r * (STEP * JS)] = v[0][r];
+    }
+  }
+};
+// where the tile of this block lies in a grid: AXIS 1 (y pencils of plane blockIdx.y) or 0 (x pencils of row)
+template <int N, int AXIS>
+struct PenPlace {
+  using C = PenCfg<N>;
+  static constexpr long long JS = AXIS == 1 ? C::PC : (long long)N * C::PC, OS = AXIS == 1 ? (long long)N * C::PC : C::PC;
+  int col0, left;
+  long long off;
+  __device__ __forceinline__ PenPlace() {
+    col0 = blockIdx.x * C::W;
+    left = C::NC - col0;
+    off = blockIdx.y * OS + col0;
+  }
+  __device__ __forceinline__ ColG<JS> of(const float2* p) const { return ColG<JS>{const_cast<float2*>(p) + off, left}; }
+};
+
+template <int N, bool REV, int G, int DIR, class Src, class Dst>
 __device__ __forceinline__ void pen_stage(const Src& src, const Dst& dst, const float2* __restrict__ tw, int tid) {
   using Q = Group<N, REV, G, DIR>;
-  constexpr int TOT = Q::NB << PenCfg<N>::lw, IT = (TOT + T - 1) / T;
-#pragma unroll(IT <= 2 ? IT : 1)
-  for (int it = 0; it < IT; ++it) {
-    const int idx = tid + it * T;
-    if (TOT % T == 0 || idx < TOT) {
-      const int w = idx & (PenCfg<N>::W - 1), b = idx >> PenCfg<N>::lw, k = Q::k_of(b);
-      float2 v[Q::R];
-#pragma unroll
-      for (int r = 0; r < Q::R; ++r) v[r] = src(b + r * Q::NB, w);
+  using K = PenTask<N, Q::R>;
+#pragma unroll(K::IT <= 2 ? K::IT : 1)
+  for (int it = 0; it < K::IT; ++it) {
+    const int idx = tid + it * PenCfg<N>::T;
+    if (K::live(idx)) {
+      const int w = K::w(idx), b = K::b(idx), k = Q::k_of(b);
+      float2 v[K::NV][Q::R];
+      src.template load<Q::NB>(b, w, v);
       Q::run(v, tw, k);
-      const int o = Q::out_row(b, k);
-#pragma unroll
-      for (int r = 0; r < Q::R; ++r) dst(o + r * Q::NS, w, v[r]);
+      dst.template store<Q::NS>(Q::out_row(b, k), w, v);
     }
   }
 }
 
 // a middle group that overwrites its buffer; the caller synchronises before the next group reads
-template <int N, bool REV, int G, int DIR, int T>
+template <int N, bool REV, int G, int DIR>
 __device__ __forceinline__ void pen_inplace(float2* buf, const float2* __restrict__ tw, int tid) {
   using Q = Group<N, REV, G, DIR>;
-  constexpr int TOT = Q::NB << PenCfg<N>::lw, IT = (TOT + T - 1) / T;
-  float2 v[IT][Q::R];
+  using K = PenTask<N, Q::R>;
+  float2 v[K::IT][K::NV][Q::R];
 #pragma unroll
-  for (int it = 0; it < IT; ++it) {
-    const int idx = tid + it * T;
-    if (TOT % T == 0 || idx < TOT) {
-#pragma unroll
-      for (int r = 0; r < Q::R; ++r) v[it][r] = buf[idx + r * (Q::NB << PenCfg<N>::lw)];
-    }
+  for (int it = 0; it < K::IT; ++it) {
+    const int idx = tid + it * PenCfg<N>::T;
+    if (K::live(idx)) Tile<N>{buf}.template load<Q::NB>(K::b(idx), K::w(idx), v[it]);
   }
   __syncthreads();
 #pragma unroll
-  for (int it = 0; it < IT; ++it) {
-    const int idx = tid + it * T;
-    if (TOT % T == 0 || idx < TOT) {
-      const int w = idx & (PenCfg<N>::W - 1), b = idx >> PenCfg<N>::lw, k = Q::k_of(b);
+  for (int it = 0; it < K::IT; ++it) {
+    const int idx = tid + it * PenCfg<N>::T;
+    if (K::live(idx)) {
+      const int b = K::b(idx), k = Q::k_of(b);
       Q::run(v[it], tw, k);
-      const int o = (Q::out_row(b, k) << PenCfg<N>::lw) + w;
-#pragma unroll
-      for (int r = 0; r < Q::R; ++r) buf[o + r * (Q::NS << PenCfg<N>::lw)] = v[it][r];
+      Tile<N>{buf}.template store<Q::NS>(Q::out_row(b, k), K::w(idx), v[it]);
     }
   }
 }
 
 // groups 1 .. m-2 from a (ping-pong with b, or in place); returns the buffer that holds the result,
 // synchronised
-template <int N, bool REV, int DIR, int T, bool PP, int G = 1>
+template <int N, bool REV, int DIR, bool PP, int G = 1>
 __device__ __forceinline__ float2* pen_middle(float2* a, float2* b, const float2* __restrict__ tw, int tid) {
   if constexpr (G + 1 < PlanOf<N, REV>::m) {
     if constexpr (PP) {
-      pen_stage<N, REV, G, DIR, T>(TileR<N>{a}, TileW<N>{b}, tw, tid);
+      pen_stage<N, REV, G, DIR>(Tile<N>{a}, Tile<N>{b}, tw, tid);
       __syncthreads();
-      return pen_middle<N, REV, DIR, T, PP, G + 1>(b, a, tw, tid);
+      return pen_middle<N, REV, DIR, PP, G + 1>(b, a, tw, tid);
     } else {
-      pen_inplace<N, REV, G, DIR, T>(a, tw, tid);
+      pen_inplace<N, REV, G, DIR>(a, tw, tid);
       __syncthreads();
-      return pen_middle<N, REV, DIR, T, PP, G + 1>(a, b, tw, tid);
+      return pen_middle<N, REV, DIR, PP, G + 1>(a, b, tw, tid);
     }
   } else {
     return a;
@@ -212,58 +295,71 @@ struct Src3 {
 // C2C along y (AXIS 1) or x (AXIS 0), in place, of the fields data.p[blockIdx.z]
 template <int N, int AXIS, int DIR>
 __global__ void __launch_bounds__(PenCfg<N>::T, PenCfg<N>::minb) k_pen(Ptr3 data, const float2* __restrict__ tw) {
-  extern __shared__ float2 sm[];
+  extern __shared__ __align__(16) float2 sm[];
   using C = PenCfg<N>;
-  constexpr long long JS = AXIS == 1 ? C::PC : (long long)N * C::PC, OS = AXIS == 1 ? (long long)N * C::PC : C::PC;
-  const int tid = threadIdx.x, col = blockIdx.x * PenCfg<N>::W + (tid & (PenCfg<N>::W - 1));
-  const ColG<JS> g{data.p[blockIdx.z] + blockIdx.y * OS + col, col < C::NC};
-  pen_stage<N, false, 0, DIR, C::T>(g, TileW<N>{sm}, tw, tid);
+  const int tid = threadIdx.x;
+  const auto g = PenPlace<N, AXIS>().of(data.p[blockIdx.z]);
+  pen_stage<N, false, 0, DIR>(g, Tile<N>{sm}, tw, tid);
   __syncthreads();
-  float2* cur = pen_middle<N, false, DIR, C::T, C::pp>(sm, sm + C::tile, tw, tid);
-  pen_stage<N, false, PlanOf<N, false>::m - 1, DIR, C::T>(TileR<N>{cur}, g, tw, tid);
+  float2* cur = pen_middle<N, false, DIR, C::pp>(sm, sm + C::tile, tw, tid);
+  pen_stage<N, false, PlanOf<N, false>::m - 1, DIR>(Tile<N>{cur}, g, tw, tid);
 }
 
 // The inverse x pass of the 2LPT multiplier mp times the lattice spectrum src, into dst
-template <long long JS>
+template <int N, long long JS>
 struct ColMul {
-  const float2* base;
-  bool ok;
-  int n, my, mz;
+  ColG<JS> g;
+  int my, col0;
   IcMul mp;
-  __device__ __forceinline__ float2 operator()(int j, int) const {
-    if (!ok) return make_float2(0.f, 0.f);
-    const int m[3] = {signed_mode(j, n), my, mz};
-    return ic_multiply_mode(base[j * JS], m, n, mp);
+  template <int STEP, int NV, int R>
+  __device__ __forceinline__ void load(int j0, int w, float2 (&v)[NV][R]) const {
+    g.template load<STEP>(j0, w, v);
+#pragma unroll
+    for (int c = 0; c < NV; ++c)
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        const int m[3] = {signed_mode(j0 + r * STEP, N), my, col0 + w + c};
+        v[c][r] = ic_multiply_mode(v[c][r], m, N, mp);
+      }
   }
 };
 template <int N>
-__global__ void __launch_bounds__(PenCfg<N>::T, PenCfg<N>::minb) k_pen_mul(const float2* __restrict__ src, float2* dst,
+__global__ void __launch_bounds__(PenCfg<N>::T, PenCfg<N>::minb) k_pen_mul(const float2* src, float2* dst,
                                                                            IcMul mp, const float2* __restrict__ tw) {
-  extern __shared__ float2 sm[];
+  extern __shared__ __align__(16) float2 sm[];
   using C = PenCfg<N>;
-  constexpr long long JS = (long long)N * C::PC;
-  const int tid = threadIdx.x, col = blockIdx.x * PenCfg<N>::W + (tid & (PenCfg<N>::W - 1)), y = blockIdx.y;
-  const bool ok = col < C::NC;
-  const ColMul<JS> g{src + (long long)y * C::PC + col, ok, N, signed_mode(y, N), col, mp};
-  pen_stage<N, false, 0, +1, C::T>(g, TileW<N>{sm}, tw, tid);
+  const int tid = threadIdx.x;
+  const PenPlace<N, 0> at;
+  const ColMul<N, PenPlace<N, 0>::JS> g{at.of(src), signed_mode(blockIdx.y, N), at.col0, mp};
+  pen_stage<N, false, 0, +1>(g, Tile<N>{sm}, tw, tid);
   __syncthreads();
-  float2* cur = pen_middle<N, false, +1, C::T, C::pp>(sm, sm + C::tile, tw, tid);
-  pen_stage<N, false, PlanOf<N, false>::m - 1, +1, C::T>(TileR<N>{cur}, ColG<JS>{dst + (long long)y * C::PC + col, ok}, tw, tid);
+  float2* cur = pen_middle<N, false, +1, C::pp>(sm, sm + C::tile, tw, tid);
+  pen_stage<N, false, PlanOf<N, false>::m - 1, +1>(Tile<N>{cur}, at.of(dst), tw, tid);
 }
 
 // NT transforms at once from here on, in the tiles s, s + tile, ...: middle groups in place, last groups
 // to d[0], d[1], ...
-template <int N, bool REV, int DIR, int T, int G, int NT, class D>
+template <int N, bool REV, int DIR, int G, int NT, class D>
 __device__ __forceinline__ void multi_finish(float2* s, const D (&d)[NT], const float2* __restrict__ tw, int tid) {
-  constexpr int M = PlanOf<N, REV>::m;
-  if constexpr (G + 1 < M) {
+  if constexpr (G + 1 < PlanOf<N, REV>::m) {
 #pragma unroll
-    for (int i = 0; i < NT; ++i) pen_inplace<N, REV, G, DIR, T>(s + i * PenCfg<N>::tile, tw, tid);
+    for (int i = 0; i < NT; ++i) pen_inplace<N, REV, G, DIR>(s + i * PenCfg<N>::tile, tw, tid);
     __syncthreads();
-    multi_finish<N, REV, DIR, T, G + 1>(s, d, tw, tid);
+    multi_finish<N, REV, DIR, G + 1>(s, d, tw, tid);
   } else {
 #pragma unroll
-    for (int i = 0; i < NT; ++i) pen_stage<N, REV, G, DIR, T>(TileR<N>{s + i * PenCfg<N>::tile}, d[i], tw, tid);
+    for (int i = 0; i < NT; ++i) pen_stage<N, REV, G, DIR>(Tile<N>{s + i * PenCfg<N>::tile}, d[i], tw, tid);
+  }
+}
+
+// NT forward transforms of the tiles s, s + tile, .. whose first groups are done, but for the last groups
+template <int N, int NT, int G = 1>
+__device__ __forceinline__ void multi_forward(float2* s, const float2* __restrict__ tw, int tid) {
+  if constexpr (G + 1 < PlanOf<N, false>::m) {
+#pragma unroll
+    for (int i = 0; i < NT; ++i) pen_inplace<N, false, G, -1>(s + i * PenCfg<N>::tile, tw, tid);
+    __syncthreads();
+    multi_forward<N, NT, G + 1>(s, tw, tid);
   }
 }
 
@@ -272,8 +368,27 @@ template <int N, int NT>
 struct MultiCfg {
   using C = PenCfg<N>;
   static constexpr int smem = NT * C::tile * 8;
-  static constexpr int regs = C::ept == 16 ? 80 : 64;
+  static constexpr int regs = NT == 2 ? 80 : 96;
   static constexpr int minb = imax(1, imin(imin(imax(1, imin(2048, 65536 / regs) / C::T), 16), (224 * 1024) / (smem + 1024)));
+};
+
+// Last group of a forward x transform (L) and first of the inverse (F): the same butterflies on the same
+// registers
+template <int N>
+struct Turn {
+  using L = Group<N, false, PlanOf<N, false>::m - 1, -1>;
+  using F = Group<N, true, 0, +1>;
+  using K = PenTask<N, L::R>;
+  static_assert(L::R == F::R && L::NS == L::NB && F::NS == 1, "the inverse starts from the forward's registers");
+  float2 spec[K::IT][K::NV][L::R];   // values at rows b + r NS of the task's columns
+  // f(value, x row, column) of every value
+  template <class Fn>
+  __device__ __forceinline__ void each(int it, int idx, int col0, Fn&& f) {
+#pragma unroll
+    for (int c = 0; c < K::NV; ++c)
+#pragma unroll
+      for (int r = 0; r < L::R; ++r) f(spec[it][c][r], K::b(idx) + r * L::NS, col0 + K::w(idx) + c);
+  }
 };
 
 // Forward x pass, times g_scale / |m|^2 (H(k), the common factor of the force components
@@ -282,120 +397,100 @@ struct MultiCfg {
 // receives the forward spectrum.
 template <int N>
 __global__ void __launch_bounds__(PenCfg<N>::T, MultiCfg<N, 2>::minb) k_green(const float2* in, float2* out_f, float2* out_h,
-                                                                           const float* __restrict__ dtab, float g_scale,
-                                                                           const float2* __restrict__ twf,
-                                                                           const float2* __restrict__ twr,
-                                                                           float2* spec_out) {
-  extern __shared__ float2 sm[];
+                                                                              const float* __restrict__ dtab, float g_scale,
+                                                                              const float2* __restrict__ twf,
+                                                                              const float2* __restrict__ twr,
+                                                                              float2* spec_out) {
+  extern __shared__ __align__(16) float2 sm[];
   using C = PenCfg<N>;
-  constexpr int T = C::T, M = PlanOf<N, false>::m;
-  constexpr long long JS = (long long)N * C::PC;
-  const int tid = threadIdx.x, col = blockIdx.x * PenCfg<N>::W + (tid & (PenCfg<N>::W - 1)), y = blockIdx.y;
-  const bool ok = col < C::NC;
-  const long long off = (long long)y * C::PC + col;
-  float2* a = sm;
-  float2* b = sm + C::tile;
-  pen_stage<N, false, 0, -1, T>(ColG<JS>{const_cast<float2*>(in) + off, ok}, TileW<N>{a}, twf, tid);
+  using X = Turn<N>;
+  using K = typename X::K;
+  constexpr long long JS = PenPlace<N, 0>::JS;
+  const int tid = threadIdx.x, y = blockIdx.y;
+  const PenPlace<N, 0> at;
+  pen_stage<N, false, 0, -1>(at.of(in), Tile<N>{sm}, twf, tid);
   __syncthreads();
-  const float2* cur = pen_middle<N, false, -1, T, true>(a, b, twf, tid);
-  using L = Group<N, false, M - 1, -1>;
-  using F = Group<N, true, 0, +1>;
-  static_assert(L::R == F::R && L::NS == L::NB && F::NS == 1, "the inverse starts from the forward's registers");
-  constexpr int TOT = L::NB << PenCfg<N>::lw, IT = (TOT + T - 1) / T;
-  float2 spec[IT][L::R];
+  float2* cur = pen_middle<N, false, -1, true>(sm, sm + C::tile, twf, tid);
+  X x;
   const int my = y < N / 2 ? y : y - N;
 #pragma unroll
-  for (int it = 0; it < IT; ++it) {
-    const int idx = tid + it * T;
-    if (TOT % T == 0 || idx < TOT) {
-      const int bb = idx >> PenCfg<N>::lw;
-#pragma unroll
-      for (int r = 0; r < L::R; ++r) spec[it][r] = cur[idx + r * (L::NB << PenCfg<N>::lw)];
-      L::run(spec[it], twf, bb);
-      if (spec_out && ok) {
-#pragma unroll
-        for (int r = 0; r < L::R; ++r) spec_out[off + (bb + r * L::NS) * JS] = spec[it][r];
-      }
-      const int myz = my * my + col * col;
-#pragma unroll
-      for (int r = 0; r < L::R; ++r) {
-        const int j = bb + r * L::NS;
+  for (int it = 0; it < K::IT; ++it) {
+    const int idx = tid + it * C::T;
+    if (K::live(idx)) {
+      Tile<N>{cur}.template load<X::L::NB>(K::b(idx), K::w(idx), x.spec[it]);
+      X::L::run(x.spec[it], twf, K::b(idx));
+      if (spec_out) at.of(spec_out).template store<X::L::NS>(K::b(idx), K::w(idx), x.spec[it]);
+      x.each(it, idx, at.col0, [&](float2& z, int j, int col) {
         const int mx = j < N / 2 ? j : j - N;
-        const int m2 = mx * mx + myz;
-        spec[it][r] = (m2 > 0 ? g_scale / (float)m2 : 0.0f) * spec[it][r];
-      }
+        const int m2 = mx * mx + (my * my + col * col);
+        z = (m2 > 0 ? g_scale / (float)m2 : 0.0f) * z;
+      });
     }
   }
   __syncthreads();   // the forward's buffers are free
 #pragma unroll
-  for (int it = 0; it < IT; ++it) {
-    const int idx = tid + it * T;
-    if (TOT % T == 0 || idx < TOT) {
-      const int w = idx & (PenCfg<N>::W - 1), bb = idx >> PenCfg<N>::lw;
-      float2 v[L::R];
+  for (int it = 0; it < K::IT; ++it) {
+    const int idx = tid + it * C::T;
+    if (K::live(idx)) {
+      const int b = K::b(idx), w = K::w(idx);
+      float2 v[K::NV][X::L::R];
 #pragma unroll
-      for (int r = 0; r < L::R; ++r) {
-        const float d = __ldg(dtab + bb + r * L::NS);
-        v[r] = make_float2(-d * spec[it][r].y, d * spec[it][r].x);   // i D H
+      for (int r = 0; r < X::L::R; ++r) {
+        const float d = __ldg(dtab + b + r * X::L::NS);
+#pragma unroll
+        for (int c = 0; c < K::NV; ++c) v[c][r] = make_float2(-d * x.spec[it][c][r].y, d * x.spec[it][c][r].x);   // i D H
       }
-      F::run(v, twr, 0);
-#pragma unroll
-      for (int r = 0; r < L::R; ++r) a[((bb * L::R + r) << PenCfg<N>::lw) + w] = v[r];
-      F::run(spec[it], twr, 0);
-#pragma unroll
-      for (int r = 0; r < L::R; ++r) b[((bb * L::R + r) << PenCfg<N>::lw) + w] = spec[it][r];
+      X::F::run(v, twr, 0);
+      Tile<N>{sm}.template store<1>(b * X::L::R, w, v);
+      X::F::run(x.spec[it], twr, 0);
+      Tile<N>{sm + C::tile}.template store<1>(b * X::L::R, w, x.spec[it]);
     }
   }
   __syncthreads();
-  const ColG<JS> d[2] = {{out_f + off, ok}, {out_h + off, ok}};
-  multi_finish<N, true, +1, T, 1>(sm, d, twr, tid);
+  const ColG<JS> d[2] = {at.of(out_f), at.of(out_h)};
+  multi_finish<N, true, +1, 1>(sm, d, twr, tid);
 }
 
 // Inverse y pass of H into the y and z components: i D(k_y) H to out_y and i D(k_z) H to out_z (which
 // may be h: a tile is read whole before it is written)
 template <int N>
 __global__ void __launch_bounds__(PenCfg<N>::T, MultiCfg<N, 2>::minb) k_pen_yz(const float2* h, float2* out_y, float2* out_z,
-                                                                            const float* __restrict__ dtab,
-                                                                            const float2* __restrict__ tw) {
-  extern __shared__ float2 sm[];
+                                                                               const float* __restrict__ dtab,
+                                                                               const float2* __restrict__ tw) {
+  extern __shared__ __align__(16) float2 sm[];
   using C = PenCfg<N>;
-  constexpr int T = C::T;
-  constexpr long long JS = C::PC, OS = (long long)N * C::PC;
-  const int tid = threadIdx.x, col = blockIdx.x * PenCfg<N>::W + (tid & (PenCfg<N>::W - 1));
-  const bool ok = col < C::NC;
-  const long long off = blockIdx.y * OS + col;
-  float2* a = sm;
-  float2* b = sm + C::tile;
-  const ColG<JS> src{const_cast<float2*>(h) + off, ok};
-  const float dz = ok ? __ldg(dtab + col) : 0.0f;
   using Q = Group<N, false, 0, +1>;
-  constexpr int TOT = Q::NB << PenCfg<N>::lw, IT = (TOT + T - 1) / T;
-#pragma unroll(IT <= 2 ? IT : 1)
-  for (int it = 0; it < IT; ++it) {
-    const int idx = tid + it * T;
-    if (TOT % T == 0 || idx < TOT) {
-      const int w = idx & (PenCfg<N>::W - 1), bb = idx >> PenCfg<N>::lw;
-      float2 z[Q::R], v[Q::R];
-#pragma unroll
-      for (int r = 0; r < Q::R; ++r) z[r] = src(bb + r * Q::NB, w);
+  using K = PenTask<N, Q::R>;
+  const int tid = threadIdx.x;
+  const PenPlace<N, 1> at;
+#pragma unroll(K::IT <= 2 ? K::IT : 1)
+  for (int it = 0; it < K::IT; ++it) {
+    const int idx = tid + it * C::T;
+    if (K::live(idx)) {
+      const int w = K::w(idx), b = K::b(idx);
+      float2 z[K::NV][Q::R], v[K::NV][Q::R];
+      at.of(h).template load<Q::NB>(b, w, z);
 #pragma unroll
       for (int r = 0; r < Q::R; ++r) {
-        const float d = __ldg(dtab + bb + r * Q::NB);
-        v[r] = make_float2(-d * z[r].y, d * z[r].x);
+        const float d = __ldg(dtab + b + r * Q::NB);
+#pragma unroll
+        for (int c = 0; c < K::NV; ++c) v[c][r] = make_float2(-d * z[c][r].y, d * z[c][r].x);
       }
       Q::run(v, tw, 0);
+      Tile<N>{sm}.template store<1>(b * Q::R, w, v);
 #pragma unroll
-      for (int r = 0; r < Q::R; ++r) a[((bb * Q::R + r) << PenCfg<N>::lw) + w] = v[r];
+      for (int c = 0; c < K::NV; ++c) {
+        const float d = w + c < at.left ? __ldg(dtab + at.col0 + w + c) : 0.0f;
 #pragma unroll
-      for (int r = 0; r < Q::R; ++r) z[r] = make_float2(-dz * z[r].y, dz * z[r].x);
+        for (int r = 0; r < Q::R; ++r) z[c][r] = make_float2(-d * z[c][r].y, d * z[c][r].x);
+      }
       Q::run(z, tw, 0);
-#pragma unroll
-      for (int r = 0; r < Q::R; ++r) b[((bb * Q::R + r) << PenCfg<N>::lw) + w] = z[r];
+      Tile<N>{sm + C::tile}.template store<1>(b * Q::R, w, z);
     }
   }
   __syncthreads();
-  const ColG<JS> d[2] = {{out_y + off, ok}, {out_z + off, ok}};
-  multi_finish<N, false, +1, T, 1>(sm, d, tw, tid);
+  const ColG<PenPlace<N, 1>::JS> d[2] = {at.of(out_y), at.of(out_z)};
+  multi_finish<N, false, +1, 1>(sm, d, tw, tid);
 }
 
 // ---- 2LPT (x and y passes) ----------------------------------------------------------------------
@@ -409,27 +504,32 @@ __global__ void __launch_bounds__(PenCfg<N>::T, MultiCfg<N, 2>::minb) k_pen_yz(c
 // launches and moves 52 field-sized reads and writes where 45 launches moved 120: 256^3 lattice 1706 -> 917
 // us (0.51 ms for the 52 at the copy rate), 32^3 271 -> 82 us.
 
-// z times k^p, p = 0, 1, 2, k = 2 pi m / n of storage index j
+// factor k^p, p = 0, 1, 2, k = 2 pi m / n of storage index j
+template <int N>
+__device__ __forceinline__ float k_power(int p, int j) {
+  constexpr float kf = 6.283185307179586f / N;
+  const float k = (j < N / 2 ? j : j - N) * kf;
+  return p == 0 ? 1.0f : (p == 1 ? (2 * j == N ? 0.0f : k) : k * k);
+}
+// z times k^p of storage index j
 template <int N, int PW>
 __device__ __forceinline__ float2 times_k(float2 z, int j) {
-  constexpr float kf = 6.283185307179586f / N;
-  const int m = j < N / 2 ? j : j - N;
   if constexpr (PW == 0) return z;
-  else if constexpr (PW == 1) return (2 * j == N ? 0.0f : m * kf) * z;
-  else return (m * kf) * (m * kf) * z;
+  else return k_power<N>(PW, j) * z;
 }
-// first group of the inverse transforms of v times 1, k, .., k^(NT-1) into the tiles s, s + tile, ..
-template <int N, bool REV, int NT, int PW = 0, int R>
-__device__ __forceinline__ void powers_stage(const float2 (&z)[R], int b, int w, float2* s, const float2* __restrict__ tw) {
+// first group of the inverse transforms of z times 1, k, .., k^(NT-1) into the tiles s, s + tile, ..
+template <int N, bool REV, int NT, int PW = 0, int NV, int R>
+__device__ __forceinline__ void powers_stage(const float2 (&z)[NV][R], int b, int w, float2* s, const float2* __restrict__ tw) {
   if constexpr (PW < NT) {
     using Q = Group<N, REV, 0, +1>;
     static_assert(Q::R == R, "a first group's butterfly");
-    float2 v[R];
+    float2 v[NV][R];
 #pragma unroll
-    for (int r = 0; r < R; ++r) v[r] = times_k<N, PW>(z[r], b + r * Q::NB);
+    for (int r = 0; r < R; ++r)
+#pragma unroll
+      for (int c = 0; c < NV; ++c) v[c][r] = times_k<N, PW>(z[c][r], b + r * Q::NB);
     Q::run(v, tw, 0);
-#pragma unroll
-    for (int r = 0; r < R; ++r) s[PW * PenCfg<N>::tile + ((b * R + r) << PenCfg<N>::lw) + w] = v[r];
+    Tile<N>{s + PW * PenCfg<N>::tile}.template store<1>(b * R, w, v);
     powers_stage<N, REV, NT, PW + 1>(z, b, w, s, tw);
   }
 }
@@ -441,63 +541,65 @@ __global__ void __launch_bounds__(PenCfg<N>::T, MultiCfg<N, NT>::minb) k_ic_x(co
                                                                               const float* __restrict__ amp_m2,
                                                                               const float2* __restrict__ twf,
                                                                               const float2* __restrict__ twr) {
-  extern __shared__ float2 sm[];
+  extern __shared__ __align__(16) float2 sm[];
   using C = PenCfg<N>;
-  constexpr int T = C::T, M = PlanOf<N, false>::m;
-  constexpr long long JS = (long long)N * C::PC;
-  const int tid = threadIdx.x, col = blockIdx.x * C::W + (tid & (C::W - 1)), y = blockIdx.y;
-  const bool ok = col < C::NC;
-  const long long off = (long long)y * C::PC + col;
-  pen_stage<N, false, 0, -1, T>(ColG<JS>{const_cast<float2*>(in) + off, ok}, TileW<N>{sm}, twf, tid);
-  __syncthreads();
-  const float2* cur = pen_middle<N, false, -1, T, true>(sm, sm + C::tile, twf, tid);
-  using L = Group<N, false, M - 1, -1>;
-  constexpr int TOT = L::NB << C::lw, IT = (TOT + T - 1) / T;
+  using X = Turn<N>;
+  using K = typename X::K;
   constexpr float kf = 6.283185307179586f / N;
-  float2 spec[IT][L::R];
+  const int tid = threadIdx.x, y = blockIdx.y;
+  const PenPlace<N, 0> at;
+  pen_stage<N, false, 0, -1>(at.of(in), Tile<N>{sm}, twf, tid);
+  __syncthreads();
+  float2* cur = pen_middle<N, false, -1, true>(sm, sm + C::tile, twf, tid);
+  X x;
   const int my = y < N / 2 ? y : y - N;
 #pragma unroll
-  for (int it = 0; it < IT; ++it) {
-    const int idx = tid + it * T;
-    if (TOT % T == 0 || idx < TOT) {
-      const int bb = idx >> C::lw;
-#pragma unroll
-      for (int r = 0; r < L::R; ++r) spec[it][r] = cur[idx + r * (L::NB << C::lw)];
-      L::run(spec[it], twf, bb);
-      const int myz = my * my + col * col;
-#pragma unroll
-      for (int r = 0; r < L::R; ++r) {
-        const int j = bb + r * L::NS;
+  for (int it = 0; it < K::IT; ++it) {
+    const int idx = tid + it * C::T;
+    if (K::live(idx)) {
+      Tile<N>{cur}.template load<X::L::NB>(K::b(idx), K::w(idx), x.spec[it]);
+      X::L::run(x.spec[it], twf, K::b(idx));
+      x.each(it, idx, at.col0, [&](float2& z, int j, int col) {
         const int mx = j < N / 2 ? j : j - N;
-        const int m2 = mx * mx + myz;
+        const int m2 = mx * mx + (my * my + col * col);
         float g = m2 > 0 ? scale / ((float)m2 * kf * kf) : 0.0f;
-        if (AMP && ok) g *= __ldg(amp_m2 + m2);
-        spec[it][r] = g * spec[it][r];
-      }
+        if (AMP && col < C::NC) g *= __ldg(amp_m2 + m2);
+        z = g * z;
+      });
     }
   }
   __syncthreads();   // the forward's buffers are free
 #pragma unroll
-  for (int it = 0; it < IT; ++it) {
-    const int idx = tid + it * T;
-    if (TOT % T == 0 || idx < TOT) powers_stage<N, true, NT>(spec[it], idx >> C::lw, idx & (C::W - 1), sm, twr);
+  for (int it = 0; it < K::IT; ++it) {
+    const int idx = tid + it * C::T;
+    if (K::live(idx)) powers_stage<N, true, NT>(x.spec[it], K::b(idx), K::w(idx), sm, twr);
   }
   __syncthreads();
-  ColG<JS> d[NT];
+  ColG<PenPlace<N, 0>::JS> d[NT];
 #pragma unroll
-  for (int i = 0; i < NT; ++i) d[i] = ColG<JS>{out.p[i] + off, ok};
-  multi_finish<N, true, +1, T, 1>(sm, d, twr, tid);
+  for (int i = 0; i < NT; ++i) d[i] = at.of(out.p[i]);
+  multi_finish<N, true, +1, 1>(sm, d, twr, tid);
 }
 
 struct Pow3 {
   int p[3];   // powers 0, 1, 2
 };
-// column store times a factor
-template <long long JS>
-struct ColScaled {
+// column store times k_z^p
+template <int N, long long JS>
+struct ColPow {
   ColG<JS> g;
-  float f;
-  __device__ __forceinline__ void operator()(int j, int w, float2 v) const { g(j, w, f * v); }
+  int p, col0;
+  template <int STEP, int NV, int R>
+  __device__ __forceinline__ void store(int j0, int w, const float2 (&v)[NV][R]) const {
+    float2 u[NV][R];
+#pragma unroll
+    for (int c = 0; c < NV; ++c) {
+      const float f = k_power<N>(p, col0 + w + c);   // k_z <= N/2: the Nyquist entry's square is the same
+#pragma unroll
+      for (int r = 0; r < R; ++r) u[c][r] = f * v[c][r];
+    }
+    g.template store<STEP>(j0, w, u);
+  }
 };
 
 // Inverse y transforms of in times 1, k_y, .. (NT of them), times k_z^zp.p[i], into out.p[0..NT-1];
@@ -505,47 +607,47 @@ struct ColScaled {
 template <int N, int NT>
 __global__ void __launch_bounds__(PenCfg<N>::T, MultiCfg<N, NT>::minb) k_ic_y(const float2* in, Ptr3 out, Pow3 zp,
                                                                               const float2* __restrict__ tw) {
-  extern __shared__ float2 sm[];
+  extern __shared__ __align__(16) float2 sm[];
   using C = PenCfg<N>;
   using Q = Group<N, false, 0, +1>;
-  constexpr int T = C::T;
-  constexpr long long JS = C::PC, OS = (long long)N * C::PC;
-  const int tid = threadIdx.x, col = blockIdx.x * C::W + (tid & (C::W - 1));
-  const bool ok = col < C::NC;
-  const long long off = blockIdx.y * OS + col;
-  const ColG<JS> src{const_cast<float2*>(in) + off, ok};
-  constexpr int TOT = Q::NB << C::lw, IT = (TOT + T - 1) / T;
-#pragma unroll(IT <= 2 ? IT : 1)
-  for (int it = 0; it < IT; ++it) {
-    const int idx = tid + it * T;
-    if (TOT % T == 0 || idx < TOT) {
-      const int w = idx & (C::W - 1), bb = idx >> C::lw;
-      float2 z[Q::R];
-#pragma unroll
-      for (int r = 0; r < Q::R; ++r) z[r] = src(bb + r * Q::NB, w);
-      powers_stage<N, false, NT>(z, bb, w, sm, tw);
+  using K = PenTask<N, Q::R>;
+  constexpr long long JS = PenPlace<N, 1>::JS;
+  const int tid = threadIdx.x;
+  const PenPlace<N, 1> at;
+#pragma unroll(K::IT <= 2 ? K::IT : 1)
+  for (int it = 0; it < K::IT; ++it) {
+    const int idx = tid + it * C::T;
+    if (K::live(idx)) {
+      float2 z[K::NV][Q::R];
+      at.of(in).template load<Q::NB>(K::b(idx), K::w(idx), z);
+      powers_stage<N, false, NT>(z, K::b(idx), K::w(idx), sm, tw);
     }
   }
   __syncthreads();
-  constexpr float kf = 6.283185307179586f / N;
-  const float kz = col * kf, kz_odd = 2 * col == N ? 0.0f : kz;
-  ColScaled<JS> d[NT];
+  ColPow<N, JS> d[NT];
 #pragma unroll
-  for (int i = 0; i < NT; ++i)
-    d[i] = ColScaled<JS>{{out.p[i] + off, ok}, zp.p[i] == 0 ? 1.0f : (zp.p[i] == 1 ? kz_odd : kz * kz)};
-  multi_finish<N, false, +1, T, 1>(sm, d, tw, tid);
+  for (int i = 0; i < NT; ++i) d[i] = ColPow<N, JS>{at.of(out.p[i]), zp.p[i], at.col0};
+  multi_finish<N, false, +1, 1>(sm, d, tw, tid);
 }
 
 // ---- transposed gradients (the adjoint's x passes) ------------------------------------------------
-// NT forward transforms of the tiles s, s + tile, .. whose first groups are done, but for the last groups
-template <int N, int T, int NT, int G = 1>
-__device__ __forceinline__ void multi_forward(float2* s, const float2* __restrict__ tw, int tid) {
-  if constexpr (G + 1 < PlanOf<N, false>::m) {
+// inverse x transform of the values of x, from the tile s, to d
+template <int N, class D>
+__device__ __forceinline__ void turn_back(Turn<N>& x, float2* s, const D& d, const float2* __restrict__ twr, int tid) {
+  using X = Turn<N>;
+  using K = typename X::K;
+  __syncthreads();   // the forward's tiles are free
 #pragma unroll
-    for (int i = 0; i < NT; ++i) pen_inplace<N, false, G, -1, T>(s + i * PenCfg<N>::tile, tw, tid);
-    __syncthreads();
-    multi_forward<N, T, NT, G + 1>(s, tw, tid);
+  for (int it = 0; it < K::IT; ++it) {
+    const int idx = tid + it * PenCfg<N>::T;
+    if (K::live(idx)) {
+      X::F::run(x.spec[it], twr, 0);
+      Tile<N>{s}.template store<1>(K::b(idx) * X::L::R, K::w(idx), x.spec[it]);
+    }
   }
+  __syncthreads();
+  const D ds[1] = {d};
+  multi_finish<N, true, +1, 1>(s, ds, twr, tid);
 }
 
 // The inverse x transform of -i g sum_j D(k_j) L_j(k), g = g_scale / |m|^2, of three spectra over k_y, k_z
@@ -557,86 +659,64 @@ __global__ void __launch_bounds__(PenCfg<N>::T, MultiCfg<N, 2>::minb) k_grad_adj
                                                                                  const float* __restrict__ dtab, float g_scale,
                                                                                  const float2* __restrict__ twf,
                                                                                  const float2* __restrict__ twr) {
-  extern __shared__ float2 sm[];
+  extern __shared__ __align__(16) float2 sm[];
   using C = PenCfg<N>;
   using A = Group<N, false, 0, -1>;
-  using L = Group<N, false, PlanOf<N, false>::m - 1, -1>;
-  using F = Group<N, true, 0, +1>;
-  constexpr int T = C::T;
-  constexpr long long JS = (long long)N * C::PC;
-  const int tid = threadIdx.x, col = blockIdx.x * C::W + (tid & (C::W - 1)), y = blockIdx.y;
-  const bool ok = col < C::NC;
-  const long long off = (long long)y * C::PC + col;
-  const float dy = __ldg(dtab + y), dz = ok ? __ldg(dtab + col) : 0.0f;
-  {
-    constexpr int TOT = A::NB << C::lw, IT = (TOT + T - 1) / T;
-#pragma unroll(IT <= 2 ? IT : 1)
-    for (int it = 0; it < IT; ++it) {
-      const int idx = tid + it * T;
-      if (TOT % T == 0 || idx < TOT) {
-        const int w = idx & (C::W - 1), bb = idx >> C::lw;
-        float2 v[A::R], u[A::R];
+  using KA = PenTask<N, A::R>;
+  using X = Turn<N>;
+  using K = typename X::K;
+  const int tid = threadIdx.x, y = blockIdx.y;
+  const PenPlace<N, 0> at;
+  const float dy = __ldg(dtab + y);
+#pragma unroll(KA::IT <= 2 ? KA::IT : 1)
+  for (int it = 0; it < KA::IT; ++it) {
+    const int idx = tid + it * C::T;
+    if (KA::live(idx)) {
+      const int w = KA::w(idx), b = KA::b(idx);
+      float2 v[KA::NV][A::R], u[KA::NV][A::R];
+      at.of(l0).template load<A::NB>(b, w, v);
+      A::run(v, twf, 0);
+      Tile<N>{sm}.template store<1>(b * A::R, w, v);
+      at.of(l1).template load<A::NB>(b, w, v);
+      at.of(l2).template load<A::NB>(b, w, u);
 #pragma unroll
-        for (int r = 0; r < A::R; ++r) {
-          const long long e = off + (bb + r * A::NB) * JS;
-          v[r] = u[r] = make_float2(0.f, 0.f);
-          if (ok) {
-            v[r] = l0[e];
-            u[r] = dy * l1[e] + dz * l2[e];
-          }
-        }
-        A::run(v, twf, 0);
-        A::run(u, twf, 0);
+      for (int c = 0; c < KA::NV; ++c) {
+        const float dz = w + c < at.left ? __ldg(dtab + at.col0 + w + c) : 0.0f;
 #pragma unroll
-        for (int r = 0; r < A::R; ++r) {
-          sm[((bb * A::R + r) << C::lw) + w] = v[r];
-          sm[C::tile + ((bb * A::R + r) << C::lw) + w] = u[r];
-        }
+        for (int r = 0; r < A::R; ++r) u[c][r] = dy * v[c][r] + dz * u[c][r];
       }
+      A::run(u, twf, 0);
+      Tile<N>{sm + C::tile}.template store<1>(b * A::R, w, u);
     }
   }
   __syncthreads();
-  multi_forward<N, T, 2>(sm, twf, tid);
-  constexpr int TOT = L::NB << C::lw, IT = (TOT + T - 1) / T;
-  float2 spec[IT][L::R];
+  multi_forward<N, 2>(sm, twf, tid);
+  X x;
   const int my = y < N / 2 ? y : y - N;
 #pragma unroll
-  for (int it = 0; it < IT; ++it) {
-    const int idx = tid + it * T;
-    if (TOT % T == 0 || idx < TOT) {
-      const int bb = idx >> C::lw;
-      float2 v[L::R], u[L::R];
+  for (int it = 0; it < K::IT; ++it) {
+    const int idx = tid + it * C::T;
+    if (K::live(idx)) {
+      const int b = K::b(idx);
+      float2 u[K::NV][X::L::R];
+      Tile<N>{sm}.template load<X::L::NB>(b, K::w(idx), x.spec[it]);
+      X::L::run(x.spec[it], twf, b);
+      Tile<N>{sm + C::tile}.template load<X::L::NB>(b, K::w(idx), u);
+      X::L::run(u, twf, b);
 #pragma unroll
-      for (int r = 0; r < L::R; ++r) {
-        v[r] = sm[idx + r * (L::NB << C::lw)];
-        u[r] = sm[C::tile + idx + r * (L::NB << C::lw)];
-      }
-      L::run(v, twf, bb);
-      L::run(u, twf, bb);
-      const int myz = my * my + col * col;
+      for (int r = 0; r < X::L::R; ++r) {
+        const float dx = __ldg(dtab + b + r * X::L::NS);
 #pragma unroll
-      for (int r = 0; r < L::R; ++r) {
-        const int j = bb + r * L::NS, mx = j < N / 2 ? j : j - N, m2 = mx * mx + myz;
-        const float g = m2 > 0 ? g_scale / (float)m2 : 0.0f, dx = __ldg(dtab + j);
-        const float2 z = dx * v[r] + u[r];
-        spec[it][r] = make_float2(g * z.y, -g * z.x);
+        for (int c = 0; c < K::NV; ++c) x.spec[it][c][r] = dx * x.spec[it][c][r] + u[c][r];
       }
+      x.each(it, idx, at.col0, [&](float2& z, int j, int col) {
+        const int mx = j < N / 2 ? j : j - N, m2 = mx * mx + (my * my + col * col);
+        const float g = m2 > 0 ? g_scale / (float)m2 : 0.0f;
+        z = make_float2(g * z.y, -g * z.x);
+      });
     }
   }
-  __syncthreads();   // the forward's tiles are free
-#pragma unroll
-  for (int it = 0; it < IT; ++it) {
-    const int idx = tid + it * T;
-    if (TOT % T == 0 || idx < TOT) {
-      const int w = idx & (C::W - 1), bb = idx >> C::lw;
-      F::run(spec[it], twr, 0);
-#pragma unroll
-      for (int r = 0; r < L::R; ++r) sm[((bb * L::R + r) << C::lw) + w] = spec[it][r];
-    }
-  }
-  __syncthreads();
-  const ColG<JS> d[1] = {{out + off, ok}};
-  multi_finish<N, true, +1, T, 1>(sm, d, twr, tid);
+  turn_back<N>(x, sm, at.of(out), twr, tid);
 }
 
 // Transpose of the first-order 2LPT maps: the inverse x transform of
@@ -653,98 +733,92 @@ __global__ void __launch_bounds__(PenCfg<N>::T, MultiCfg<N, 3>::minb) k_lpt_adj(
                                                                                const float* __restrict__ amp_m2,
                                                                                const float2* __restrict__ twf,
                                                                                const float2* __restrict__ twr) {
-  extern __shared__ float2 sm[];
+  extern __shared__ __align__(16) float2 sm[];
   using C = PenCfg<N>;
   using A = Group<N, false, 0, -1>;
-  using L = Group<N, false, PlanOf<N, false>::m - 1, -1>;
-  using F = Group<N, true, 0, +1>;
-  constexpr int T = C::T;
-  constexpr long long JS = (long long)N * C::PC;
+  using KA = PenTask<N, A::R>;
+  using X = Turn<N>;
+  using K = typename X::K;
   constexpr float kf = 6.283185307179586f / N;
-  const int tid = threadIdx.x, col = blockIdx.x * C::W + (tid & (C::W - 1)), y = blockIdx.y;
-  const bool ok = col < C::NC;
-  const long long off = (long long)y * C::PC + col;
+  const int tid = threadIdx.x, y = blockIdx.y;
+  const PenPlace<N, 0> at;
   const int my = y < N / 2 ? y : y - N;
-  const float ky = my * kf, kz = col * kf, oy = 2 * y == N ? 0.0f : ky, oz = 2 * col == N ? 0.0f : kz;
-  {
-    constexpr int TOT = A::NB << C::lw, IT = (TOT + T - 1) / T;
+  const float ky2 = k_power<N>(2, y), oy = k_power<N>(1, y);
 #pragma unroll 1
-    for (int it = 0; it < IT; ++it) {
-      const int idx = tid + it * T;
-      if (TOT % T == 0 || idx < TOT) {
-        const int w = idx & (C::W - 1), bb = idx >> C::lw;
+  for (int it = 0; it < KA::IT; ++it) {
+    const int idx = tid + it * C::T;
+    if (KA::live(idx)) {
+      const int w = KA::w(idx), b = KA::b(idx);
+      float2 v[KA::NV][A::R], u[KA::NV][A::R];
+      // v += f(column) u, u = rows of p; IMAG: times -i
+      auto add = [&](const float2* p, auto&& f, bool imag) {
+        at.of(p).template load<A::NB>(b, w, u);
 #pragma unroll
-        for (int q = 0; q < 3; ++q) {   // factors of 1, k_x, k_x^2
-          float2 v[A::R];
+        for (int c = 0; c < KA::NV; ++c) {
+          const float g = f(at.col0 + w + c);
 #pragma unroll
           for (int r = 0; r < A::R; ++r) {
-            const long long e = off + (bb + r * A::NB) * JS;
-            v[r] = make_float2(0.f, 0.f);
-            if (ok) {
-              if (q == 0) {
-                const float2 g = r_scale * (oy * in.p[1][e] + oz * in.p[2][e]);
-                v[r] = (ky * ky) * in.h[1][e] + (kz * kz) * in.h[2][e] + (oy * oz) * in.h[5][e] + make_float2(g.y, -g.x);
-              } else if (q == 1) {
-                const float2 g = r_scale * in.p[0][e];
-                v[r] = oy * in.h[3][e] + oz * in.h[4][e] + make_float2(g.y, -g.x);
-              } else {
-                v[r] = in.h[0][e];
-              }
-            }
+            const float2 z = g * u[c][r];
+            v[c][r] = v[c][r] + (imag ? make_float2(z.y, -z.x) : z);
           }
-          A::run(v, twf, 0);
-#pragma unroll
-          for (int r = 0; r < A::R; ++r) sm[q * C::tile + ((bb * A::R + r) << C::lw) + w] = v[r];
         }
-      }
+      };
+      auto put = [&](int q) {
+        A::run(v, twf, 0);
+        Tile<N>{sm + q * C::tile}.template store<1>(b * A::R, w, v);
+      };
+      auto clear = [&]() {
+#pragma unroll
+        for (int c = 0; c < KA::NV; ++c)
+#pragma unroll
+          for (int r = 0; r < A::R; ++r) v[c][r] = make_float2(0.f, 0.f);
+      };
+      clear();
+      add(in.h[1], [&](int) { return ky2; }, false);
+      add(in.h[2], [&](int col) { return k_power<N>(2, col); }, false);
+      add(in.h[5], [&](int col) { return oy * k_power<N>(1, col); }, false);
+      add(in.p[1], [&](int) { return r_scale * oy; }, true);
+      add(in.p[2], [&](int col) { return r_scale * k_power<N>(1, col); }, true);
+      put(0);
+      clear();
+      add(in.h[3], [&](int) { return oy; }, false);
+      add(in.h[4], [&](int col) { return k_power<N>(1, col); }, false);
+      add(in.p[0], [&](int) { return r_scale; }, true);
+      put(1);
+      at.of(in.h[0]).template load<A::NB>(b, w, v);
+      put(2);
     }
   }
   __syncthreads();
-  multi_forward<N, T, 3>(sm, twf, tid);
-  constexpr int TOT = L::NB << C::lw, IT = (TOT + T - 1) / T;
-  float2 spec[IT][L::R];
+  multi_forward<N, 3>(sm, twf, tid);
+  X x;
 #pragma unroll
-  for (int it = 0; it < IT; ++it) {
-    const int idx = tid + it * T;
-    if (TOT % T == 0 || idx < TOT) {
-      const int bb = idx >> C::lw;
+  for (int it = 0; it < K::IT; ++it) {
+    const int idx = tid + it * C::T;
+    if (K::live(idx)) {
+      const int b = K::b(idx);
+      Tile<N>{sm}.template load<X::L::NB>(b, K::w(idx), x.spec[it]);
+      X::L::run(x.spec[it], twf, b);
 #pragma unroll
-      for (int q = 0; q < 3; ++q) {
-        float2 v[L::R];
+      for (int q = 1; q < 3; ++q) {
+        float2 u[K::NV][X::L::R];
+        Tile<N>{sm + q * C::tile}.template load<X::L::NB>(b, K::w(idx), u);
+        X::L::run(u, twf, b);
 #pragma unroll
-        for (int r = 0; r < L::R; ++r) v[r] = sm[q * C::tile + idx + r * (L::NB << C::lw)];
-        L::run(v, twf, bb);
+        for (int r = 0; r < X::L::R; ++r) {
+          const float f = k_power<N>(q, b + r * X::L::NS);
 #pragma unroll
-        for (int r = 0; r < L::R; ++r) {
-          const int j = bb + r * L::NS, mx = j < N / 2 ? j : j - N;
-          const float kx = mx * kf;
-          const float f = q == 0 ? 1.0f : (q == 1 ? (2 * j == N ? 0.0f : kx) : kx * kx);
-          spec[it][r] = q == 0 ? v[r] : spec[it][r] + f * v[r];
+          for (int c = 0; c < K::NV; ++c) x.spec[it][c][r] = x.spec[it][c][r] + f * u[c][r];
         }
       }
-      const int myz = my * my + col * col;
-#pragma unroll
-      for (int r = 0; r < L::R; ++r) {
-        const int j = bb + r * L::NS, mx = j < N / 2 ? j : j - N, m2 = mx * mx + myz;
-        const float g = m2 > 0 && ok ? __ldg(amp_m2 + m2) / ((float)m2 * kf * kf) : 0.0f;
-        spec[it][r] = g * spec[it][r];
-      }
+      x.each(it, idx, at.col0, [&](float2& z, int j, int col) {
+        const int mx = j < N / 2 ? j : j - N, m2 = mx * mx + (my * my + col * col);
+        const float g = m2 > 0 && col < C::NC ? __ldg(amp_m2 + m2) / ((float)m2 * kf * kf) : 0.0f;
+        z = g * z;
+      });
     }
   }
-  __syncthreads();   // the forward's tiles are free
-#pragma unroll
-  for (int it = 0; it < IT; ++it) {
-    const int idx = tid + it * T;
-    if (TOT % T == 0 || idx < TOT) {
-      const int w = idx & (C::W - 1), bb = idx >> C::lw;
-      F::run(spec[it], twr, 0);
-#pragma unroll
-      for (int r = 0; r < L::R; ++r) sm[((bb * L::R + r) << C::lw) + w] = spec[it][r];
-    }
-  }
-  __syncthreads();
-  const ColG<JS> d[1] = {{out + off, ok}};
-  multi_finish<N, true, +1, T, 1>(sm, d, twr, tid);
+  turn_back<N>(x, sm, at.of(out), twr, tid);
 }
 
 // ---- row pairs (the contiguous axis) -------------------------------------------------------------
@@ -1129,7 +1203,7 @@ __global__ void __launch_bounds__(RowCfg<N>::T, IcRowCfg<N>::minb) k_ic_z1(IcRow
 // Psi2 (component blockIdx.y, factors -i k_j) of row pairs into dense rows times r_scale, and the first
 // positions s = d1 Psi1 + d2 Psi2 and velocities 0 of the same particles.
 template <int N>
-__global__ void __launch_bounds__(RowCfg<N>::T, RowCfg<N>::minb(C2rCfg<N>::bufs)) k_ic_z2(Ptr3 f, const float* __restrict__ psi1,
+__global__ void __launch_bounds__(RowCfg<N>::T, RowCfg<N>::minb(C2rCfg<N>::bufs)) k_ic_z2(Ptr3 f, const float* psi1,
                                                                                          float* psi2, float* s, float* v0,
                                                                                          long long npart, float r_scale, float d1,
                                                                                          float d2, long long npairs,
@@ -1150,13 +1224,16 @@ __global__ void __launch_bounds__(RowCfg<N>::T, RowCfg<N>::minb(C2rCfg<N>::bufs)
     if (p >= slots) return;
     const long long o = comp * npart + 2 * (pair0 + p) * N + bb;
 #pragma unroll
-    for (int r = 0; r < Q::R; ++r) {
-      const float p2[2] = {v[r].x * -r_scale, v[r].y * -r_scale};
+    for (int h = 0; h < 2; ++h) {
+      float p1[Q::R];   // every load of a row before its stores, which may alias as far as the compiler knows
 #pragma unroll
-      for (int h = 0; h < 2; ++h) {
+      for (int r = 0; r < Q::R; ++r) p1[r] = psi1[o + h * N + r * Q::NS];
+#pragma unroll
+      for (int r = 0; r < Q::R; ++r) {
         const long long i = o + h * N + r * Q::NS;
-        psi2[i] = p2[h];
-        s[i] = d1 * psi1[i] + d2 * p2[h];
+        const float p2 = (h ? v[r].y : v[r].x) * -r_scale;
+        psi2[i] = p2;
+        s[i] = d1 * p1[r] + d2 * p2;
         v0[i] = 0.0f;
       }
     }
