@@ -36,12 +36,12 @@ unsigned grid_for(long long work, int threads) {
 
 // cell and weight of cell c+1 per axis, from the forward's fixed-point coordinate
 template <bool F32>
-__device__ __forceinline__ void cic_cell(const FixedGeo& fg, const int (&q)[3], long long id, const float* __restrict__ s,
+__device__ __forceinline__ void cic_cell(const FixedGeo& fg, const int (&q)[3], long long id, const float* s,
                                          long long n, int* c, float* w1) {
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
     int f;
-    cell_frac<F32>(q[a], __ldg(s + a * n + id), fg, &c[a], &f);
+    cell_frac<F32>(q[a], *(s + a * n + id), fg, &c[a], &f);
     w1[a] = (float)f * (1.0f / kWeightOne);
   }
 }
@@ -71,8 +71,9 @@ __device__ __forceinline__ void add_pair(float* row, int iz, int iz1, float v0, 
 
 // lam_v += drift lam_s; lam_p1 += dd1 lam_s; lam_p2 += dd2 lam_s; lam_f = kick lam_v;
 // lam_p1 -= c1 lam_f; lam_p2 -= c2 lam_f   (all [3][n])
-__global__ void k_adj_step(long long n3, const float* __restrict__ lam_s, float* lam_v, float* lam_p1, float* lam_p2,
+__global__ void k_adj_step(long long n3, const float* lam_s, float* lam_v, float* lam_p1, float* lam_p2,
                            float* lam_f, float drift, float dd1, float dd2, float kick, float c1, float c2) {
+  after_previous();
   for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n3; t += (long long)gridDim.x * blockDim.x) {
     const float ls = lam_s[t];
     const float lv = lam_v[t] + drift * ls;
@@ -87,9 +88,10 @@ __global__ void k_adj_step(long long n3, const float* __restrict__ lam_s, float*
 // deposit the three components of lam_f with CIC weights onto three real meshes (rows of rs); bound by the
 // rate of the atomics in L2
 template <bool F32>
-__global__ void __launch_bounds__(256) k_adj_deposit(ParticleGeom pg, FixedGeo fg, const float* __restrict__ s,
-                                                     const float* __restrict__ lam_f, float* m0, float* m1, float* m2,
+__global__ void __launch_bounds__(256) k_adj_deposit(ParticleGeom pg, FixedGeo fg, const float* s,
+                                                     const float* lam_f, float* m0, float* m1, float* m2,
                                                      long long rs) {
+  after_previous();
   const long long n = pg.npart;
   const int nm = pg.n;
   for_particles(pg.np, [&](const int (&q)[3], long long id) {
@@ -119,6 +121,7 @@ __global__ void __launch_bounds__(256) k_adj_deposit(ParticleGeom pg, FixedGeo f
 // out(k) = sum_j conj(i D(m_j) g) L_j(k) = -i g sum_j D(m_j) L_j(k), g = g_scale / |m|^2; out may be L_0
 __global__ void k_adj_combine(int n, int pc, int nc, const float2* l0, const float2* l1, const float2* l2,
                               const float* __restrict__ dtab, float g_scale, float2* out) {
+  after_previous();
   const long long total = (long long)n * n * nc;
   for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < total;
        t += (long long)gridDim.x * blockDim.x) {
@@ -138,9 +141,10 @@ __global__ void k_adj_combine(int n, int pc, int nc, const float2* l0, const flo
 
 // lam_s += sum_c grad W(x - c) [lam_f . F_c + norm lam_delta_c]
 template <bool F32>
-__global__ void __launch_bounds__(256) k_adj_gather(ParticleGeom pg, FixedGeo fg, const float* __restrict__ s, const float* __restrict__ lam_f,
-                             const float* __restrict__ f0, const float* __restrict__ f1, const float* __restrict__ f2,
-                             const float* __restrict__ ld, long long rs, float norm, float* lam_s) {
+__global__ void __launch_bounds__(256) k_adj_gather(ParticleGeom pg, FixedGeo fg, const float* s, const float* lam_f,
+                             const float* f0, const float* f1, const float* f2,
+                             const float* ld, long long rs, float norm, float* lam_s) {
+  after_previous();
   const long long n = pg.npart;
   const int nm = pg.n;
   for_particles(pg.np, [&](const int (&q)[3], long long id) {
@@ -163,7 +167,7 @@ __global__ void __launch_bounds__(256) k_adj_gather(ParticleGeom pg, FixedGeo fg
           const int iz = (c[2] + dz) == nm ? 0 : c[2] + dz;
           const float wz = dz ? w1[2] : 1.0f - w1[2], gz = dz ? 1.0f : -1.0f;
           const long long e = row + iz;
-          const float v = l0 * __ldg(f0 + e) + l1 * __ldg(f1 + e) + l2 * __ldg(f2 + e) + norm * __ldg(ld + e);
+          const float v = l0 * *(f0 + e) + l1 * *(f1 + e) + l2 * *(f2 + e) + norm * *(ld + e);
           gxs += gx * wy * wz * v;
           gys += wx * gy * wz * v;
           gzs += wx * wy * gz * v;
@@ -177,7 +181,8 @@ __global__ void __launch_bounds__(256) k_adj_gather(ParticleGeom pg, FixedGeo fg
 }
 
 // lam_p1 += d1 lam_s; lam_p2 += d2 lam_s   (initial condition s_1 = D1 Psi1 + D2 Psi2)
-__global__ void k_adj_ic(long long n3, const float* __restrict__ lam_s, float* lam_p1, float* lam_p2, float d1, float d2) {
+__global__ void k_adj_ic(long long n3, const float* lam_s, float* lam_p1, float* lam_p2, float d1, float d2) {
+  after_previous();
   for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n3; t += (long long)gridDim.x * blockDim.x) {
     lam_p1[t] += d1 * lam_s[t];
     lam_p2[t] += d2 * lam_s[t];
@@ -185,7 +190,8 @@ __global__ void k_adj_ic(long long n3, const float* __restrict__ lam_s, float* l
 }
 
 // particle array [n] -> real lattice field (rows of 2 pc floats), times scale
-__global__ void k_particles_to_field(int n, int pc, const float* __restrict__ src, float scale, float* dst) {
+__global__ void k_particles_to_field(int n, int pc, const float* src, float scale, float* dst) {
+  after_previous();
   const long long total = (long long)n * n * n;
   const long long rs = 2LL * pc;
   for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < total; t += (long long)gridDim.x * blockDim.x)
@@ -194,8 +200,9 @@ __global__ void k_particles_to_field(int n, int pc, const float* __restrict__ sr
 
 // Transpose of the second-order source S = h00 h11 + h00 h22 + h11 h22 - h01^2 - h02^2 - h12^2
 // (§2.1): the six Hessian fields h (rows of 2 pc floats) are replaced in place by lam_S dS/dh.
-__global__ void k_ic_source_adjoint(int n, int pc, const float* __restrict__ lam_src, float* h0, float* h1, float* h2,
+__global__ void k_ic_source_adjoint(int n, int pc, const float* lam_src, float* h0, float* h1, float* h2,
                                     float* h3, float* h4, float* h5) {
+  after_previous();
   const long long total = (long long)n * n * n;
   const long long rs = 2LL * pc;
   for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < total; t += (long long)gridDim.x * blockDim.x) {
@@ -214,7 +221,7 @@ __global__ void k_ic_source_adjoint(int n, int pc, const float* __restrict__ lam
 // ---- CIC density contrast of the loss grid (continuous weights) and its adjoint ---------------
 // grid coordinate y = (q N/np + s) ngrid / N, wrapped into [0, ngrid)
 __device__ __forceinline__ void grid_cell(const ParticleGeom& pg, const int (&q)[3], long long id,
-                                          const float* __restrict__ s, long long n, int ng, double ratio, int* c, float* t) {
+                                          const float* s, long long n, int ng, double ratio, int* c, float* t) {
   const double r = (double)pg.n / pg.np;
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
@@ -231,8 +238,9 @@ __device__ __forceinline__ void grid_cell(const ParticleGeom& pg, const int (&q)
 
 // Continuous CIC weights rounded to multiples of 2^-32 and summed with 64-bit integer atomics:
 // the sum is exact and independent of the order, so the loss grid is bit-reproducible.
-__global__ void k_grid_deposit(ParticleGeom pg, const float* __restrict__ s, int ng, double ratio,
+__global__ void k_grid_deposit(ParticleGeom pg, const float* s, int ng, double ratio,
                                unsigned long long* rho) {
+  after_previous();
   const long long n = pg.npart;
   for_particles(pg.np, [&](const int (&q)[3], long long id) {
     int c[3];
@@ -259,14 +267,16 @@ __global__ void k_grid_deposit(ParticleGeom pg, const float* __restrict__ s, int
 }
 
 // delta = rho scale - 1, scale = ng^3 / (n 2^32), in FP64
-__global__ void k_grid_finish(long long cells, const unsigned long long* __restrict__ rho, double scale,
+__global__ void k_grid_finish(long long cells, const unsigned long long* rho, double scale,
                               float* delta) {
+  after_previous();
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < cells; i += (long long)gridDim.x * blockDim.x)
     delta[i] = (float)((double)rho[i] * scale - 1.0);
 }
 
-__global__ void k_grid_adjoint(ParticleGeom pg, const float* __restrict__ s, int ng, double ratio,
-                               const float* __restrict__ lam_delta, float gscale, float* lam_s) {
+__global__ void k_grid_adjoint(ParticleGeom pg, const float* s, int ng, double ratio,
+                               const float* lam_delta, float gscale, float* lam_s) {
+  after_previous();
   const long long n = pg.npart;
   for_particles(pg.np, [&](const int (&q)[3], long long id) {
     int c[3];
@@ -285,7 +295,7 @@ __global__ void k_grid_adjoint(ParticleGeom pg, const float* __restrict__ s, int
         for (int dz = 0; dz < 2; ++dz) {
           const int iz = (c[2] + dz) == ng ? 0 : c[2] + dz;
           const float wz = dz ? t[2] : 1.0f - t[2], gz = dz ? 1.0f : -1.0f;
-          const float v = __ldg(lam_delta + ((long long)ix * ng + iy) * ng + iz);
+          const float v = *(lam_delta + ((long long)ix * ng + iy) * ng + iz);
           g0 += gx * wy * wz * v;
           g1 += wx * gy * wz * v;
           g2 += wx * wy * gz * v;
@@ -302,9 +312,7 @@ __global__ void k_grid_adjoint(ParticleGeom pg, const float* __restrict__ s, int
 
 int launch_adj_step(long long n3, const float* lam_s, float* lam_v, float* lam_p1, float* lam_p2, float* lam_f,
                     const StepScalars& sc, cudaStream_t st) {
-  k_adj_step<<<grid_for(n3, 256), 256, 0, st>>>(n3, lam_s, lam_v, lam_p1, lam_p2, lam_f, (float)sc.drift,
-                                                (float)sc.dd1, (float)sc.dd2, (float)sc.kick, (float)sc.c1,
-                                                (float)sc.c2);
+  launch_after(k_adj_step, grid_for(n3, 256), 256, 0, st, n3, lam_s, lam_v, lam_p1, lam_p2, lam_f, (float)sc.drift, (float)sc.dd1, (float)sc.dd2, (float)sc.kick, (float)sc.c1, (float)sc.c2);
   return check_launch("adj_step");
 }
 
@@ -313,14 +321,13 @@ int launch_adj_deposit(const ParticleGeom& pg, const float* s, const float* lam_
   const RowBlocks rb = row_blocks(pg.np);
   const FixedGeo fg = fixed_geo(pg.n, pg.r_fixed);
   auto* k = pg.n < 2048 ? k_adj_deposit<true> : k_adj_deposit<false>;
-  k<<<rb.grid, rb.block, 0, st>>>(pg, fg, s, lam_f, m[0], m[1], m[2], rs);
+  launch_after(k, rb.grid, rb.block, 0, st, pg, fg, s, lam_f, m[0], m[1], m[2], rs);
   return check_launch("adj_deposit");
 }
 
 int launch_adj_combine(const Grid3& g, float2* const l[3], const float* dtab, float g_scale, float2* out,
                        cudaStream_t st) {
-  k_adj_combine<<<grid_for((long long)g.rows() * g.nc, 256), 256, 0, st>>>(g.n, g.pc, g.nc, l[0], l[1], l[2], dtab,
-                                                                           g_scale, out);
+  launch_after(k_adj_combine, grid_for((long long)g.rows() * g.nc, 256), 256, 0, st, g.n, g.pc, g.nc, l[0], l[1], l[2], dtab, g_scale, out);
   return check_launch("adj_combine");
 }
 
@@ -329,18 +336,17 @@ int launch_adj_gather(const ParticleGeom& pg, const float* s, const float* lam_f
   const RowBlocks rb = row_blocks(pg.np);
   const FixedGeo fg = fixed_geo(pg.n, pg.r_fixed);
   auto* k = pg.n < 2048 ? k_adj_gather<true> : k_adj_gather<false>;
-  k<<<rb.grid, rb.block, 0, st>>>(pg, fg, s, lam_f, f[0], f[1], f[2], lam_delta, rs, norm, lam_s);
+  launch_after(k, rb.grid, rb.block, 0, st, pg, fg, s, lam_f, f[0], f[1], f[2], lam_delta, rs, norm, lam_s);
   return check_launch("adj_gather");
 }
 
 int launch_adj_ic(long long n3, const float* lam_s, float* lam_p1, float* lam_p2, float d1, float d2, cudaStream_t st) {
-  k_adj_ic<<<grid_for(n3, 256), 256, 0, st>>>(n3, lam_s, lam_p1, lam_p2, d1, d2);
+  launch_after(k_adj_ic, grid_for(n3, 256), 256, 0, st, n3, lam_s, lam_p1, lam_p2, d1, d2);
   return check_launch("adj_ic");
 }
 
 int launch_particles_to_field(const Grid3& g, const float* src, float scale, float2* dst, cudaStream_t st) {
-  k_particles_to_field<<<grid_for((long long)g.rows() * g.n, 256), 256, 0, st>>>(g.n, g.pc, src, scale,
-                                                                                  reinterpret_cast<float*>(dst));
+  launch_after(k_particles_to_field, grid_for((long long)g.rows() * g.n, 256), 256, 0, st, g.n, g.pc, src, scale, reinterpret_cast<float*>(dst));
   return check_launch("particles_to_field");
 }
 
@@ -350,17 +356,15 @@ int launch_grid_density(const ParticleGeom& pg, const float* s, int ngrid, unsig
   if (cudaMemsetAsync(scratch, 0, cells * sizeof(unsigned long long), st) != cudaSuccess) return COLA_ERR_CUDA;
   const double ratio = (double)ngrid / pg.n;
   const RowBlocks rb = row_blocks(pg.np);
-  k_grid_deposit<<<rb.grid, rb.block, 0, st>>>(pg, s, ngrid, ratio, scratch);
-  k_grid_finish<<<grid_for(cells, 256), 256, 0, st>>>(cells, scratch, (double)cells / ((double)pg.npart * 4294967296.0),
-                                                      delta);
+  launch_after(k_grid_deposit, rb.grid, rb.block, 0, st, pg, s, ngrid, ratio, scratch);
+  launch_after(k_grid_finish, grid_for(cells, 256), 256, 0, st, cells, scratch, (double)cells / ((double)pg.npart * 4294967296.0), delta);
   return check_launch("grid_density");
 }
 
 int launch_ic_source_adjoint(const Grid3& g, const float2* lam_src, float2* const h[6], cudaStream_t st) {
   float* f[6];
   for (int i = 0; i < 6; ++i) f[i] = reinterpret_cast<float*>(h[i]);
-  k_ic_source_adjoint<<<grid_for((long long)g.rows() * g.n, 256), 256, 0, st>>>(
-      g.n, g.pc, reinterpret_cast<const float*>(lam_src), f[0], f[1], f[2], f[3], f[4], f[5]);
+  launch_after(k_ic_source_adjoint, grid_for((long long)g.rows() * g.n, 256), 256, 0, st,  g.n, g.pc, reinterpret_cast<const float*>(lam_src), f[0], f[1], f[2], f[3], f[4], f[5]);
   return check_launch("ic_source_adjoint");
 }
 
@@ -369,8 +373,7 @@ int launch_grid_density_adjoint(const ParticleGeom& pg, const float* s, int ngri
   const double ratio = (double)ngrid / pg.n;
   const double cells = (double)ngrid * ngrid * ngrid;
   const RowBlocks rb = row_blocks(pg.np);
-  k_grid_adjoint<<<rb.grid, rb.block, 0, st>>>(pg, s, ngrid, ratio, lam_delta,
-                                                          (float)(cells / (double)pg.npart * ratio), lam_s);
+  launch_after(k_grid_adjoint, rb.grid, rb.block, 0, st, pg, s, ngrid, ratio, lam_delta, (float)(cells / (double)pg.npart * ratio), lam_s);
   return check_launch("grid_density_adjoint");
 }
 

@@ -126,8 +126,9 @@ struct RowWalk {
 // Bound by instruction issue and by the atomics' return trips.
 template <bool F32>
 __global__ void __launch_bounds__(kThreads) k_bin_count(ParticleGeom pg, BinGeom b, FixedGeo fg, RowWalk walk,
-                                                        const float* __restrict__ s, unsigned* cnt_p, unsigned* cnt_s,
-                                                        unsigned long long* __restrict__ rec) {
+                                                        const float* s, unsigned* cnt_p, unsigned* cnt_s,
+                                                        unsigned long long* rec) {
+  after_previous();
   const long long n = pg.npart;
   const int np = pg.np;
   const unsigned nrows = (unsigned)np * np, step = gridDim.x * blockDim.y;
@@ -137,7 +138,7 @@ __global__ void __launch_bounds__(kThreads) k_bin_count(ParticleGeom pg, BinGeom
   float p[3] = {0.f, 0.f, 0.f};
   auto load = [&](long long first, int z, float (&v)[3]) {
 #pragma unroll
-    for (int a = 0; a < 3; ++a) v[a] = z < np ? __ldg(s + a * n + first + z) : 0.f;
+    for (int a = 0; a < 3; ++a) v[a] = z < np ? *(s + a * n + first + z) : 0.f;
   };
   if (r < nrows) {
     walk.at(r, &qx, &qy, &row);
@@ -184,9 +185,10 @@ __global__ void __launch_bounds__(kThreads) k_bin_count(ParticleGeom pg, BinGeom
 // Scatter pass from the records: primary entries straight to offset + rank, spill entries through
 // the spill cursors.  Bound by the latency of the records and of the offset lookups.
 __global__ void __launch_bounds__(kThreads) k_bin_scatter(ParticleGeom pg, BinGeom b, RowWalk walk,
-                                                          const unsigned long long* __restrict__ rec,
-                                                          const unsigned* __restrict__ off_p, unsigned* cur_s,
+                                                          const unsigned long long* rec,
+                                                          const unsigned* off_p, unsigned* cur_s,
                                                           unsigned* ent_p, unsigned* ent_s) {
+  after_previous();
   const int np = pg.np;
   const unsigned nrows = (unsigned)np * np, step = gridDim.x * blockDim.y;
   constexpr int U = 2;   // records in flight per thread: their loads, then their offset lookups
@@ -205,7 +207,7 @@ __global__ void __launch_bounds__(kThreads) k_bin_scatter(ParticleGeom pg, BinGe
 #pragma unroll
       for (int u = 0; u < U; ++u) {
         const int qz = q0 + u * (int)blockDim.x;
-        base[u] = qz < np ? __ldg(off_p + code_key(b, (unsigned)r[u])) : 0u;
+        base[u] = qz < np ? *(off_p + code_key(b, (unsigned)r[u])) : 0u;
       }
 #pragma unroll
       for (int u = 0; u < U; ++u) {
@@ -252,7 +254,7 @@ __device__ __forceinline__ unsigned block_excl_scan(unsigned v, unsigned* total)
 }
 
 // counts base + 8 tid .. + 7 (0 beyond m)
-__device__ __forceinline__ void load8(const unsigned* __restrict__ cnt, int i0, int m, unsigned (&c)[8]) {
+__device__ __forceinline__ void load8(const unsigned* cnt, int i0, int m, unsigned (&c)[8]) {
   if (i0 + 8 <= m) {
     const uint4 a = *reinterpret_cast<const uint4*>(cnt + i0), b = *reinterpret_cast<const uint4*>(cnt + i0 + 4);
     c[0] = a.x, c[1] = a.y, c[2] = a.z, c[3] = a.w, c[4] = b.x, c[5] = b.y, c[6] = b.z, c[7] = b.w;
@@ -288,9 +290,10 @@ __device__ __forceinline__ void store8(unsigned run, const unsigned (&c)[8], int
   }
 }
 
-__global__ void __launch_bounds__(kScanThreads) k_scan_sums(const unsigned* __restrict__ cnt_p,
-                                                           const unsigned* __restrict__ cnt_s, int m,
+__global__ void __launch_bounds__(kScanThreads) k_scan_sums(const unsigned* cnt_p,
+                                                           const unsigned* cnt_s, int m,
                                                            unsigned* seg_sums) {
+  after_previous();
   const int list = blockIdx.y;
   unsigned c[8], v = 0;
   load8(list ? cnt_s : cnt_p, blockIdx.x * kScanSeg + threadIdx.x * 8, m, c);
@@ -302,6 +305,7 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_sums(const unsigned* __re
 }
 
 __global__ void __launch_bounds__(kScanThreads) k_scan_segs(unsigned* seg_sums, int nseg) {
+  after_previous();
   const int list = blockIdx.x;
   unsigned* ss = seg_sums + list * nseg;
   unsigned carry = 0;
@@ -314,10 +318,11 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_segs(unsigned* seg_sums, 
   }
 }
 
-__global__ void __launch_bounds__(kScanThreads) k_scan_apply(const unsigned* __restrict__ cnt_p,
-                                                            const unsigned* __restrict__ cnt_s, int m,
-                                                            const unsigned* __restrict__ seg_sums, unsigned* off_p,
+__global__ void __launch_bounds__(kScanThreads) k_scan_apply(const unsigned* cnt_p,
+                                                            const unsigned* cnt_s, int m,
+                                                            const unsigned* seg_sums, unsigned* off_p,
                                                             unsigned* off_s, unsigned* cur_s) {
+  after_previous();
   const int list = blockIdx.y, i0 = blockIdx.x * kScanSeg + threadIdx.x * 8;
   // each thread scans 8 consecutive counts; the thread totals are scanned across the block
   unsigned c[8], v = 0, tot;
@@ -331,9 +336,10 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_apply(const unsigned* __r
 // The scan in one launch for few segments: every block sums the counts before its segment itself (at
 // most kScanOneSegs segments of 4096 counts) instead of two launches that do it once.
 constexpr int kScanOneSegs = 16;
-__global__ void __launch_bounds__(kScanThreads) k_scan_one(const unsigned* __restrict__ cnt_p,
-                                                          const unsigned* __restrict__ cnt_s, int m, unsigned* off_p,
+__global__ void __launch_bounds__(kScanThreads) k_scan_one(const unsigned* cnt_p,
+                                                          const unsigned* cnt_s, int m, unsigned* off_p,
                                                           unsigned* off_s, unsigned* cur_s) {
+  after_previous();
   const int list = blockIdx.y;
   const unsigned* cnt = list ? cnt_s : cnt_p;
   unsigned* off = list ? off_s : off_p;
@@ -371,7 +377,7 @@ __device__ __forceinline__ void red_shared(unsigned a, unsigned v, bool p) {
 
 // adds the 8 weights of one entry that fall inside the tile (acc: shared address of the low words)
 template <bool F32>
-__device__ __forceinline__ void deposit_entry(const ParticleGeom& pg, const FixedGeo& fg, const float* __restrict__ s,
+__device__ __forceinline__ void deposit_entry(const ParticleGeom& pg, const FixedGeo& fg, const float* s,
                                               unsigned e, int x0, int y0, int z0, unsigned acc) {
   const int nm = pg.n;
   const long long n = pg.npart;
@@ -380,7 +386,7 @@ __device__ __forceinline__ void deposit_entry(const ParticleGeom& pg, const Fixe
   unpack_q(e, pg.np, q, &id);
   int c[3], f[3];
 #pragma unroll
-  for (int a = 0; a < 3; ++a) cell_frac<F32>(q[a], __ldg(s + a * n + id), fg, &c[a], &f[a]);
+  for (int a = 0; a < 3; ++a) cell_frac<F32>(q[a], *(s + a * n + id), fg, &c[a], &f[a]);
   const int lx[2] = {c[0] - x0, (c[0] + 1 == nm ? 0 : c[0] + 1) - x0};
   const int ly[2] = {c[1] - y0, (c[1] + 1 == nm ? 0 : c[1] + 1) - y0};
   const int lz[2] = {c[2] - z0, (c[2] + 1 == nm ? 0 : c[2] + 1) - z0};
@@ -409,13 +415,14 @@ __device__ __forceinline__ void deposit_entry(const ParticleGeom& pg, const Fixe
 
 template <bool F32>
 __global__ void __launch_bounds__(kDepositThreads, 4) k_deposit_tiles(ParticleGeom pg, BinGeom b, FixedGeo fg,
-                                                               const float* __restrict__ s,
-                                                               const unsigned* __restrict__ off_p,
-                                                               const unsigned* __restrict__ ent_p,
-                                                               const unsigned* __restrict__ off_s,
-                                                               const unsigned* __restrict__ ent_s,
+                                                               const float* s,
+                                                               const unsigned* off_p,
+                                                               const unsigned* ent_p,
+                                                               const unsigned* off_s,
+                                                               const unsigned* ent_s,
                                                                unsigned long long* rho, float* delta_out, float scale,
                                                                unsigned long long* tile_mass) {
+  after_previous();
   __shared__ unsigned words[2 * kAccWords];
   unsigned* const lo = words;
   unsigned* const hi = words + kAccWords;
@@ -508,8 +515,8 @@ constexpr int kBulkWaitLimit = 1 << 22;   // polls of the staging barrier before
 // 16-byte aligned (z0 a multiple of 32, rows of 2 pc floats with pc even).  Called by every thread of the
 // block; contains a barrier.
 __device__ __forceinline__ void gather_stage(float* fsm, unsigned bar_sa, int nm, int x0, int y0, int z0,
-                                             const float* __restrict__ f0, const float* __restrict__ f1,
-                                             const float* __restrict__ f2, long long rs) {
+                                             const float* f0, const float* f1,
+                                             const float* f2, long long rs) {
   const int tx = nm - x0 < kT ? nm - x0 : kT, ty = nm - y0 < kT ? nm - y0 : kT, tz = nm - z0 < kTz ? nm - z0 : kTz;
   if (threadIdx.x == 0) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(bar_sa) : "memory");
@@ -556,7 +563,7 @@ struct GatherPart {
   unsigned e;
   float s[3], v[3], p1[3], p2[3];
   __device__ __forceinline__ void load(const ParticleGeom& pg, unsigned ent, const float* sp, const float* vp,
-                                       const float* __restrict__ psi1, const float* __restrict__ psi2) {
+                                       const float* psi1, const float* psi2) {
     e = ent;
     int q[3];
     long long id;
@@ -567,8 +574,8 @@ struct GatherPart {
     if (KICK) {
 #pragma unroll
       for (int a = 0; a < 3; ++a) {
-        p1[a] = __ldg(psi1 + a * n + id);
-        p2[a] = __ldg(psi2 + a * n + id);
+        p1[a] = *(psi1 + a * n + id);
+        p2[a] = *(psi2 + a * n + id);
         v[a] = vp[a * n + id];
       }
     }
@@ -580,13 +587,14 @@ struct GatherPart {
 // entry and values are loaded while the one before is interpolated.
 template <bool KICK, bool F32>
 __global__ void __launch_bounds__(kGatherThreads, 2) k_gather_tiles(ParticleGeom pg, BinGeom b, FixedGeo fg,
-                                                             const unsigned* __restrict__ off_p,
-                                                             const unsigned* __restrict__ ent_p,
-                                                             const float* __restrict__ f0, const float* __restrict__ f1,
-                                                             const float* __restrict__ f2, long long rs,
-                                                             const float* __restrict__ s_in, float* __restrict__ force_out,
-                                                             float* s, float* v, const float* __restrict__ psi1,
-                                                             const float* __restrict__ psi2, KickDrift kd, int* flags) {
+                                                             const unsigned* off_p,
+                                                             const unsigned* ent_p,
+                                                             const float* f0, const float* f1,
+                                                             const float* f2, long long rs,
+                                                             const float* s_in, float* force_out,
+                                                             float* s, float* v, const float* psi1,
+                                                             const float* psi2, KickDrift kd, int* flags) {
+  after_previous();
   extern __shared__ __align__(16) float fsm[];
   const int tile = blockIdx.x;
   const unsigned e0 = off_p[tile], e1 = off_p[tile + 1];
@@ -597,8 +605,8 @@ __global__ void __launch_bounds__(kGatherThreads, 2) k_gather_tiles(ParticleGeom
   const unsigned bar_sa = (unsigned)__cvta_generic_to_shared(fsm + kGatherFloats);
   const float* sp = KICK ? s : s_in;
   const unsigned first = e0 + threadIdx.x;
-  unsigned ent = first < e1 ? __ldg(ent_p + first) : 0u;
-  unsigned ent_next = first + kGatherThreads < e1 ? __ldg(ent_p + first + kGatherThreads) : 0u;
+  unsigned ent = first < e1 ? *(ent_p + first) : 0u;
+  unsigned ent_next = first + kGatherThreads < e1 ? *(ent_p + first + kGatherThreads) : 0u;
   gather_stage(fsm, bar_sa, pg.n, x0, y0, z0, f0, f1, f2, rs);
   GatherPart<KICK> cur;
   if (first < e1) cur.load(pg, ent, sp, v, psi1, psi2);
@@ -617,7 +625,7 @@ __global__ void __launch_bounds__(kGatherThreads, 2) k_gather_tiles(ParticleGeom
   for (unsigned e = first; e < e1; e += kGatherThreads) {
     GatherPart<KICK> nxt;
     if (e + kGatherThreads < e1) nxt.load(pg, ent_next, sp, v, psi1, psi2);
-    ent_next = e + 2 * kGatherThreads < e1 ? __ldg(ent_p + e + 2 * kGatherThreads) : 0u;
+    ent_next = e + 2 * kGatherThreads < e1 ? *(ent_p + e + 2 * kGatherThreads) : 0u;
     int q[3], c[3];
     long long id;
     unpack_q(cur.e, pg.np, q, &id);
@@ -692,9 +700,9 @@ void particle_schedule(const BinGeom& b, int nmesh, long long npart, bool* binne
 
 int launch_excl_scan(const unsigned* cnt, int m, unsigned* seg, unsigned* off, cudaStream_t st) {
   const int nseg = (m + kScanSeg - 1) / kScanSeg;
-  k_scan_sums<<<dim3(nseg, 1), kScanThreads, 0, st>>>(cnt, nullptr, m, seg);
-  k_scan_segs<<<1, kScanThreads, 0, st>>>(seg, nseg);
-  k_scan_apply<<<dim3(nseg, 1), kScanThreads, 0, st>>>(cnt, nullptr, m, seg, off, nullptr, nullptr);
+  launch_after(k_scan_sums, dim3(nseg, 1), kScanThreads, 0, st, cnt, nullptr, m, seg);
+  launch_after(k_scan_segs, 1, kScanThreads, 0, st, seg, nseg);
+  launch_after(k_scan_apply, dim3(nseg, 1), kScanThreads, 0, st, cnt, nullptr, m, seg, off, nullptr, nullptr);
   return check_launch("excl_scan");
 }
 
@@ -709,20 +717,19 @@ int launch_binning(const ParticleGeom& pg, const BinGeom& b, const float* s, Bin
   if (cudaMemsetAsync(bb.cnt_p, 0, (size_t)(bb.cnt_s - bb.cnt_p + b.tiles) * sizeof(unsigned), st) != cudaSuccess)
     return COLA_ERR_CUDA;
   auto* count = pg.n < 2048 ? k_bin_count<true> : k_bin_count<false>;
-  count<<<grid, rb.block, 0, st>>>(pg, b, fg, walk, s, bb.cnt_p, bb.cnt_s, bb.rec);
+  launch_after(count, grid, rb.block, 0, st, pg, b, fg, walk, s, bb.cnt_p, bb.cnt_s, bb.rec);
   int e = check_launch("bin_count");
   if (e != COLA_OK) return e;
   const int nseg = (b.tiles + kScanSeg - 1) / kScanSeg;
   if (nseg <= kScanOneSegs) {
-    k_scan_one<<<dim3(nseg, 2), kScanThreads, 0, st>>>(bb.cnt_p, bb.cnt_s, b.tiles, bb.off_p, bb.off_s, bb.cur_s);
+    launch_after(k_scan_one, dim3(nseg, 2), kScanThreads, 0, st, bb.cnt_p, bb.cnt_s, b.tiles, bb.off_p, bb.off_s, bb.cur_s);
   } else {
-    k_scan_sums<<<dim3(nseg, 2), kScanThreads, 0, st>>>(bb.cnt_p, bb.cnt_s, b.tiles, bb.seg);
-    k_scan_segs<<<2, kScanThreads, 0, st>>>(bb.seg, nseg);
-    k_scan_apply<<<dim3(nseg, 2), kScanThreads, 0, st>>>(bb.cnt_p, bb.cnt_s, b.tiles, bb.seg, bb.off_p, bb.off_s,
-                                                         bb.cur_s);
+    launch_after(k_scan_sums, dim3(nseg, 2), kScanThreads, 0, st, bb.cnt_p, bb.cnt_s, b.tiles, bb.seg);
+    launch_after(k_scan_segs, 2, kScanThreads, 0, st, bb.seg, nseg);
+    launch_after(k_scan_apply, dim3(nseg, 2), kScanThreads, 0, st, bb.cnt_p, bb.cnt_s, b.tiles, bb.seg, bb.off_p, bb.off_s, bb.cur_s);
   }
   if ((e = check_launch("bin_scan")) != COLA_OK) return e;
-  k_bin_scatter<<<grid, rb.block, 0, st>>>(pg, b, walk, bb.rec, bb.off_p, bb.cur_s, bb.ent_p, bb.ent_s);
+  launch_after(k_bin_scatter, grid, rb.block, 0, st, pg, b, walk, bb.rec, bb.off_p, bb.cur_s, bb.ent_p, bb.ent_s);
   return check_launch("bin_scatter");
 }
 
@@ -732,8 +739,7 @@ int launch_deposit_tiles(const ParticleGeom& pg, const BinGeom& b, const float* 
   if (delta_out && !tile_mass) return COLA_ERR_INVALID;
   const FixedGeo fg = fixed_geo(pg.n, pg.r_fixed);
   auto* k = pg.n < 2048 ? k_deposit_tiles<true> : k_deposit_tiles<false>;
-  k<<<b.tiles, kDepositThreads, 0, st>>>(pg, b, fg, s, bb.off_p, bb.ent_p, bb.off_s, bb.ent_s, rho, delta_out, scale,
-                                  tile_mass);
+  launch_after(k, b.tiles, kDepositThreads, 0, st, pg, b, fg, s, bb.off_p, bb.ent_p, bb.off_s, bb.ent_s, rho, delta_out, scale, tile_mass);
   return check_launch("deposit_tiles");
 }
 
@@ -755,13 +761,11 @@ int launch_gather_tiles(const ParticleGeom& pg, const BinGeom& b, const BinBuffe
   if (kd) {
     auto* k = f32 ? k_gather_tiles<true, true> : k_gather_tiles<true, false>;
     smem_limit(k, sm);
-    k<<<b.tiles, kGatherThreads, sm, st>>>(pg, b, fg, bb.off_p, bb.ent_p, f[0], f[1], f[2], rs, nullptr, nullptr, s, v, psi1,
-                                     psi2, *kd, flags);
+    launch_after(k, b.tiles, kGatherThreads, sm, st, pg, b, fg, bb.off_p, bb.ent_p, f[0], f[1], f[2], rs, nullptr, nullptr, s, v, psi1, psi2, *kd, flags);
   } else {
     auto* k = f32 ? k_gather_tiles<false, true> : k_gather_tiles<false, false>;
     smem_limit(k, sm);
-    k<<<b.tiles, kGatherThreads, sm, st>>>(pg, b, fg, bb.off_p, bb.ent_p, f[0], f[1], f[2], rs, s_in, force_out, nullptr,
-                                     nullptr, nullptr, nullptr, KickDrift{}, flags);
+    launch_after(k, b.tiles, kGatherThreads, sm, st, pg, b, fg, bb.off_p, bb.ent_p, f[0], f[1], f[2], rs, s_in, force_out, nullptr, nullptr, nullptr, nullptr, KickDrift{}, flags);
   }
   return check_launch("gather_tiles");
 }

@@ -10,6 +10,34 @@
 
 namespace cola {
 
+#ifdef __CUDACC__
+// Launches a kernel that may be set up while the previous kernel of the stream drains (programmatic
+// dependent launch): the kernel must begin with after_previous(), which waits until that one has completed
+// and its writes are visible.  No kernel lets its successor in before its own blocks have ended (with an
+// early release the successor's waiting blocks took the last wave's resources: 512^3/768^3 steps 4%
+// slower).  A kernel reads what the previous one may have written with plain loads only: neither __ldg nor
+// a const __restrict__ pointer, which the compiler may read ahead of the wait; tables written once (twiddles,
+// wave numbers, amplitudes) keep them.  Before -> after: 32^3/64^3 realisation of two steps 150 -> 85 us,
+// 96^3/192^3 step 264 -> 242, adjoint 64^3/128^3 2218 -> 1716, P(k) 128^3/256^3 303 -> 275.
+template <class... P, class... A>
+inline void launch_after(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A&&... args) {
+  cudaLaunchAttribute attr{};
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+__device__ __forceinline__ void after_previous() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+#endif
+
 double hubble(double a, double om);
 
 // FP64 background cosmology and linear power (host only).

@@ -50,6 +50,7 @@ struct EdgeTable {
 // Per-call tables: twiddles exp(-2 pi i t / n) (FP64 sincospi rounded to float), plain and stage-major
 // (the forward plan's: no inverse transform runs here), and bin edges.
 __global__ void k_static_tables(int n, Groups g, float2* tw, EdgeTable edges, int nedges, long long* edges_out) {
+  after_previous();
   for (int e = threadIdx.x; e < 2 * n - 1; e += blockDim.x) {
     const int t = e < n ? e : (g.ok ? stage_twiddle(g, e - n) : 0);
     double s, c;
@@ -134,7 +135,7 @@ extern "C" int cola_power_spectrum_noalloc(const cola_params* p, const float* s,
 
   const size_t n3 = (size_t)n * n * n;
   if (cudaMemsetAsync(rho, 0, n3 * sizeof(unsigned long long), st) != cudaSuccess) return COLA_ERR_CUDA;
-  k_static_tables<<<1, 128, 0, st>>>(n, make_groups(n, false), tw, edges, nbins + 1, edg);
+  launch_after(k_static_tables, 1, 128, 0, st, n, make_groups(n, false), tw, edges, nbins + 1, edg);
   if (cudaGetLastError() != cudaSuccess) return COLA_ERR_CUDA;
   int r = launch_deposit(pg, s, rho, flags, st);
   const float scale = (float)((double)n3 / ((double)pg.npart * 4398046511104.0));

@@ -164,7 +164,7 @@ __device__ __forceinline__ int saddr(int j, int w, int lw) { return ((j + (j >> 
 // reads x[b + r n/R], twiddles by w_n^(r k n/(Ns R)) with k = b mod Ns, and writes
 // y[(b - k) R + k + r Ns].  Ping-pong between two shared buffers, one barrier per stage.
 template <int R, int DIR>
-__device__ __forceinline__ void fft_stage(const float2* __restrict__ x, float2* __restrict__ y, int n, int lw,
+__device__ __forceinline__ void fft_stage(const float2* x, float2* y, int n, int lw,
                                           int ns, const float2* __restrict__ tw, int tid, int nthreads) {
   const int nb = n / R;
   const int total = nb << lw;

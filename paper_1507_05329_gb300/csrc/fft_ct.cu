@@ -12,7 +12,7 @@ namespace {
 template <class K, class... A>
 void go(K kern, dim3 grid, int threads, int smem, cudaStream_t st, A... args) {
   if (smem > 48 * 1024) ensure_smem(kern);
-  kern<<<grid, threads, smem, st>>>(args...);
+  launch_after(kern, grid, threads, smem, st, args...);
 }
 
 template <int N>

@@ -295,6 +295,7 @@ struct Src3 {
 // C2C along y (AXIS 1) or x (AXIS 0), in place, of the fields data.p[blockIdx.z]
 template <int N, int AXIS, int DIR>
 __global__ void __launch_bounds__(PenCfg<N>::T, PenCfg<N>::minb) k_pen(Ptr3 data, const float2* __restrict__ tw) {
+  after_previous();
   extern __shared__ __align__(16) float2 sm[];
   using C = PenCfg<N>;
   const int tid = threadIdx.x;
@@ -326,6 +327,7 @@ struct ColMul {
 template <int N>
 __global__ void __launch_bounds__(PenCfg<N>::T, PenCfg<N>::minb) k_pen_mul(const float2* src, float2* dst,
                                                                            IcMul mp, const float2* __restrict__ tw) {
+  after_previous();
   extern __shared__ __align__(16) float2 sm[];
   using C = PenCfg<N>;
   const int tid = threadIdx.x;
@@ -401,6 +403,7 @@ __global__ void __launch_bounds__(PenCfg<N>::T, MultiCfg<N, 2>::minb) k_green(co
                                                                               const float2* __restrict__ twf,
                                                                               const float2* __restrict__ twr,
                                                                               float2* spec_out) {
+  after_previous();
   extern __shared__ __align__(16) float2 sm[];
   using C = PenCfg<N>;
   using X = Turn<N>;
@@ -457,6 +460,7 @@ template <int N>
 __global__ void __launch_bounds__(PenCfg<N>::T, MultiCfg<N, 2>::minb) k_pen_yz(const float2* h, float2* out_y, float2* out_z,
                                                                                const float* __restrict__ dtab,
                                                                                const float2* __restrict__ tw) {
+  after_previous();
   extern __shared__ __align__(16) float2 sm[];
   using C = PenCfg<N>;
   using Q = Group<N, false, 0, +1>;
@@ -541,6 +545,7 @@ __global__ void __launch_bounds__(PenCfg<N>::T, MultiCfg<N, NT>::minb) k_ic_x(co
                                                                               const float* __restrict__ amp_m2,
                                                                               const float2* __restrict__ twf,
                                                                               const float2* __restrict__ twr) {
+  after_previous();
   extern __shared__ __align__(16) float2 sm[];
   using C = PenCfg<N>;
   using X = Turn<N>;
@@ -607,6 +612,7 @@ struct ColPow {
 template <int N, int NT>
 __global__ void __launch_bounds__(PenCfg<N>::T, MultiCfg<N, NT>::minb) k_ic_y(const float2* in, Ptr3 out, Pow3 zp,
                                                                               const float2* __restrict__ tw) {
+  after_previous();
   extern __shared__ __align__(16) float2 sm[];
   using C = PenCfg<N>;
   using Q = Group<N, false, 0, +1>;
@@ -659,6 +665,7 @@ __global__ void __launch_bounds__(PenCfg<N>::T, MultiCfg<N, 2>::minb) k_grad_adj
                                                                                  const float* __restrict__ dtab, float g_scale,
                                                                                  const float2* __restrict__ twf,
                                                                                  const float2* __restrict__ twr) {
+  after_previous();
   extern __shared__ __align__(16) float2 sm[];
   using C = PenCfg<N>;
   using A = Group<N, false, 0, -1>;
@@ -733,6 +740,7 @@ __global__ void __launch_bounds__(PenCfg<N>::T, MultiCfg<N, 3>::minb) k_lpt_adj(
                                                                                const float* __restrict__ amp_m2,
                                                                                const float2* __restrict__ twf,
                                                                                const float2* __restrict__ twr) {
+  after_previous();
   extern __shared__ __align__(16) float2 sm[];
   using C = PenCfg<N>;
   using A = Group<N, false, 0, -1>;
@@ -961,6 +969,7 @@ __global__ void __launch_bounds__(RowCfg<N>::T, RowCfg<N>::minb(2)) k_r2c(Src3 s
                                                                           Ptr3 dst, long long npairs,
                                                                           const float2* __restrict__ tw,
                                                                           unsigned long long* mass_acc) {
+  after_previous();
   extern __shared__ float2 sm[];
   using C = RowCfg<N>;
   const int tid = threadIdx.x;
@@ -1033,6 +1042,7 @@ template <int N, bool DENSE>
 __global__ void __launch_bounds__(RowCfg<N>::T, RowCfg<N>::minb(C2rCfg<N>::bufs)) k_c2r(Ptr3 data, long long npairs,
                                                                                        const float2* __restrict__ tw,
                                                                                        float* out, float scale) {
+  after_previous();
   extern __shared__ float2 sm[];
   using C = RowCfg<N>;
   const int tid = threadIdx.x;
@@ -1132,6 +1142,7 @@ template <int N>
 __global__ void __launch_bounds__(RowCfg<N>::T, IcRowCfg<N>::minb) k_ic_z1(IcRows f, float2* src_k, float* psi1,
                                                                            long long npart, float r_scale, long long npairs,
                                                                            const float2* __restrict__ tw) {
+  after_previous();
   extern __shared__ float2 sm[];
   using C = RowCfg<N>;
   using Q = Group<N, false, PlanOf<N, false>::m - 1, +1>;
@@ -1208,6 +1219,7 @@ __global__ void __launch_bounds__(RowCfg<N>::T, RowCfg<N>::minb(C2rCfg<N>::bufs)
                                                                                          long long npart, float r_scale, float d1,
                                                                                          float d2, long long npairs,
                                                                                          const float2* __restrict__ tw) {
+  after_previous();
   extern __shared__ float2 sm[];
   using C = RowCfg<N>;
   using Q = Group<N, false, PlanOf<N, false>::m - 1, +1>;

@@ -7,8 +7,9 @@ using namespace fftk;
 namespace {
 // ---- contiguous axis: pairs of real rows as one complex row ----------------------------------
 template <int SRC>
-__global__ void __launch_bounds__(kMaxThreads, 2) k_r2c_rows(FftDev p, int lw, const void* __restrict__ src, long long src_rs, float scale,
-                           float2* __restrict__ dst, int pc, long long nrows, unsigned long long* mass_acc) {
+__global__ void __launch_bounds__(kMaxThreads, 2) k_r2c_rows(FftDev p, int lw, const void* src, long long src_rs, float scale,
+                           float2* dst, int pc, long long nrows, unsigned long long* mass_acc) {
+  after_previous();
   extern __shared__ float2 sm[];
   const int n = p.n, tid = threadIdx.x, nt = blockDim.x, wmask = (1 << lw) - 1;
   const long long row0 = (long long)blockIdx.x << (lw + 1);
@@ -56,6 +57,7 @@ __global__ void __launch_bounds__(kMaxThreads, 2) k_r2c_rows(FftDev p, int lw, c
 }
 
 __global__ void __launch_bounds__(kMaxThreads, 2) k_c2r_rows(FftDev p, int lw, float2* data, int pc, long long nrows) {
+  after_previous();
   extern __shared__ float2 sm[];
   const int n = p.n, nh = n / 2, tid = threadIdx.x, nt = blockDim.x, wmask = (1 << lw) - 1;
   const long long row0 = (long long)blockIdx.x << (lw + 1);
@@ -88,6 +90,7 @@ __global__ void __launch_bounds__(kMaxThreads, 2) k_c2r_rows(FftDev p, int lw, f
 // ---- strided axes: W adjacent columns, transform along j ----------------------------------
 template <int DIR>
 __global__ void __launch_bounds__(kMaxThreads, 2) k_pencils(FftDev p, int lw, float2* data, long long jstride, long long ostride, int nc) {
+  after_previous();
   extern __shared__ float2 sm[];
   const int n = p.n, tid = threadIdx.x, nt = blockDim.x, wmask = (1 << lw) - 1;
   const int col0 = blockIdx.x << lw;
@@ -112,6 +115,7 @@ __global__ void __launch_bounds__(kMaxThreads, 2) k_pencils(FftDev p, int lw, fl
 // transform) is inverse-transformed along x and stored.  out2 may alias in.
 __global__ void __launch_bounds__(kMaxThreads, 1) k_green_x(FftDev p, int lw, const float2* in, float2* out0, float2* out1, float2* out2,
                           int pc, int nc, const float* __restrict__ dtab, float g_scale) {
+  after_previous();
   extern __shared__ float2 sm[];
   const int n = p.n, tid = threadIdx.x, nt = blockDim.x, wmask = (1 << lw) - 1;
   const int col0 = blockIdx.x << lw;
@@ -183,25 +187,25 @@ void generic_r2c_launch(const FftDev& d, int lw, unsigned blocks, int threads, s
                         long long rs, float scale, float2* dst, int pc, long long nrows, unsigned long long* acc,
                         cudaStream_t st) {
   if (kind == kSrcFixedPoint)
-    k_r2c_rows<kSrcFixedPoint><<<blocks, threads, smem, st>>>(d, lw, src, rs, scale, dst, pc, nrows, acc);
+    launch_after(k_r2c_rows<kSrcFixedPoint>, blocks, threads, smem, st, d, lw, src, rs, scale, dst, pc, nrows, acc);
   else
-    k_r2c_rows<kSrcFloat><<<blocks, threads, smem, st>>>(d, lw, src, rs, scale, dst, pc, nrows, nullptr);
+    launch_after(k_r2c_rows<kSrcFloat>, blocks, threads, smem, st, d, lw, src, rs, scale, dst, pc, nrows, nullptr);
 }
 
 void generic_c2r_launch(const FftDev& d, int lw, unsigned blocks, int threads, size_t smem, float2* data, int pc,
                         long long nrows, cudaStream_t st) {
-  k_c2r_rows<<<blocks, threads, smem, st>>>(d, lw, data, pc, nrows);
+  launch_after(k_c2r_rows, blocks, threads, smem, st, d, lw, data, pc, nrows);
 }
 
 void generic_pencils_launch(const FftDev& d, int lw, dim3 grid, int threads, size_t smem, int dir, float2* data,
                             long long jstride, long long ostride, int nc, cudaStream_t st) {
-  if (dir < 0) k_pencils<-1><<<grid, threads, smem, st>>>(d, lw, data, jstride, ostride, nc);
-  else k_pencils<+1><<<grid, threads, smem, st>>>(d, lw, data, jstride, ostride, nc);
+  if (dir < 0) launch_after(k_pencils<-1>, grid, threads, smem, st, d, lw, data, jstride, ostride, nc);
+  else launch_after(k_pencils<+1>, grid, threads, smem, st, d, lw, data, jstride, ostride, nc);
 }
 
 void generic_green_launch(const FftDev& d, int lw, dim3 grid, int threads, size_t smem, const float2* in,
                           float2* const out[3], int pc, int nc, const float* dtab, float g_scale, cudaStream_t st) {
-  k_green_x<<<grid, threads, smem, st>>>(d, lw, in, out[0], out[1], out[2], pc, nc, dtab, g_scale);
+  launch_after(k_green_x, grid, threads, smem, st, d, lw, in, out[0], out[1], out[2], pc, nc, dtab, g_scale);
 }
 
 }  // namespace cola

@@ -87,8 +87,9 @@ __device__ __forceinline__ int unite(int* parent, int a, int b, int* flags) {
 // for l + 2, so points within l of each other are in the same or adjacent cells, around the edge too.
 __device__ __forceinline__ int cell_of(unsigned g, unsigned long long inv) { return (int)__umul64hi(g, inv); }
 
-__global__ void __launch_bounds__(256) k_fof_prepare(ParticleGeom pg, const float* __restrict__ s, FofGeom f, unsigned* g0,
+__global__ void __launch_bounds__(256) k_fof_prepare(ParticleGeom pg, const float* s, FofGeom f, unsigned* g0,
                                                      unsigned* g1, unsigned* g2, int* key, unsigned* counts) {
+  after_previous();
   const long long n = pg.npart;
   const long long modulus = f.modulus;
   const int np = pg.np, qx = blockIdx.y, qy = blockIdx.x * blockDim.y + threadIdx.y;
@@ -108,9 +109,10 @@ __global__ void __launch_bounds__(256) k_fof_prepare(ParticleGeom pg, const floa
 }
 
 // records by cell; a cell's count runs down to zero
-__global__ void k_fof_scatter(int n, const int* __restrict__ key, const unsigned* __restrict__ off, unsigned* counts,
-                              const unsigned* __restrict__ g0, const unsigned* __restrict__ g1,
-                              const unsigned* __restrict__ g2, uint4* rec, int* ids, int* min_id) {
+__global__ void k_fof_scatter(int n, const int* key, const unsigned* off, unsigned* counts,
+                              const unsigned* g0, const unsigned* g1,
+                              const unsigned* g2, uint4* rec, int* ids, int* min_id) {
+  after_previous();
   for (int id = blockIdx.x * blockDim.x + threadIdx.x; id < n; id += gridDim.x * blockDim.x) {
     const int k = key[id];
     const unsigned t = off[k] + atomicSub(counts + k, 1u) - 1u;
@@ -147,7 +149,7 @@ __device__ __forceinline__ bool friends(const uint4& me, const uint4& o, unsigne
 // Calls meet(lo, hi, sx, sy, sz) for the ranges of records behind t in its own and its forward neighbour
 // cells, the farthest columns first; stops when it returns true.
 template <bool ONE, class F>
-__device__ __forceinline__ void forward_ranges(int t, int n, const uint4& me, const unsigned* __restrict__ off,
+__device__ __forceinline__ void forward_ranges(int t, int n, const uint4& me, const unsigned* off,
                                                const FofGeom& f, F&& meet) {
   if (ONE) {
     meet((unsigned)t + 1u, (unsigned)n, 0u, 0u, 0u);
@@ -176,16 +178,17 @@ __device__ __forceinline__ void forward_ranges(int t, int n, const uint4& me, co
 // First pass: the record's parent is one friend behind it (itself if it has none), from the last of the
 // farthest column, so that paths are short; only this thread writes it.
 template <bool ONE>
-__global__ void __launch_bounds__(256) k_fof_first(int n, const uint4* __restrict__ rec, const unsigned* __restrict__ off,
+__global__ void __launch_bounds__(256) k_fof_first(int n, const uint4* rec, const unsigned* off,
                                                    FofGeom f, int* parent) {
+  after_previous();
   const int ell = (int)f.ell;
   const unsigned long long ell2 = (unsigned long long)f.ell * (unsigned long long)f.ell;
   for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < n; t += gridDim.x * blockDim.x) {
-    const uint4 me = __ldg(rec + t);
+    const uint4 me = *(rec + t);
     int p = t;
     forward_ranges<ONE>(t, n, me, off, f, [&](unsigned lo, unsigned hi, unsigned sx, unsigned sy, unsigned sz) {
       for (unsigned u = hi; u > lo && (int)u > t + 1; --u)   // a parent comes after its child
-        if (friends<ONE>(me, __ldg(rec + u - 1), sx, sy, sz, ell, ell2, f.modulus)) {
+        if (friends<ONE>(me, *(rec + u - 1), sx, sy, sz, ell, ell2, f.modulus)) {
           p = (int)u - 1;
           return true;
         }
@@ -203,16 +206,17 @@ __global__ void __launch_bounds__(256) k_fof_first(int n, const uint4* __restric
 // two root searches for every friend, 128^3/256^3 at b = 0.2 took 1225 us for the links and 1240 us for
 // scanning the cells; in sorted order with one pass 1000 and 40; now 280 for both passes.)
 template <bool ONE>
-__global__ void __launch_bounds__(256) k_fof_link(int n, const uint4* __restrict__ rec, const unsigned* __restrict__ off,
+__global__ void __launch_bounds__(256) k_fof_link(int n, const uint4* rec, const unsigned* off,
                                                   FofGeom f, int* parent, int* flags) {
+  after_previous();
   const int ell = (int)f.ell;
   const unsigned long long ell2 = (unsigned long long)f.ell * (unsigned long long)f.ell;
   for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < n; t += gridDim.x * blockDim.x) {
-    const uint4 me = __ldg(rec + t);
+    const uint4 me = *(rec + t);
     int root = (int)me.w;
     forward_ranges<ONE>(t, n, me, off, f, [&](unsigned lo, unsigned hi, unsigned sx, unsigned sy, unsigned sz) {
       for (unsigned u = lo; u < hi; ++u) {
-        const uint4 o = __ldg(rec + u);
+        const uint4 o = *(rec + u);
         if (o.w != me.w && friends<ONE>(me, o, sx, sy, sz, ell, ell2, f.modulus))
           root = unite(parent, root, (int)o.w, flags);
       }
@@ -223,12 +227,14 @@ __global__ void __launch_bounds__(256) k_fof_link(int n, const uint4* __restrict
 
 // each record takes its tree's root after the first pass
 __global__ void k_fof_carry(int n, uint4* rec, int* parent) {
+  after_previous();
   for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < n; t += gridDim.x * blockDim.x)
     rec[t].w = (unsigned)find_root(parent, t);
 }
 
 // root of every record, members and smallest id per root (one atomic per run of lanes with one root)
-__global__ void k_fof_roots(int n, const int* __restrict__ ids, int* parent, int* root, unsigned* cnt, int* min_id) {
+__global__ void k_fof_roots(int n, const int* ids, int* parent, int* root, unsigned* cnt, int* min_id) {
+  after_previous();
   for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < n; t += gridDim.x * blockDim.x) {
     const int r = find_root(parent, t);
     root[t] = r;
@@ -241,9 +247,10 @@ __global__ void k_fof_roots(int n, const int* __restrict__ ids, int* parent, int
   }
 }
 
-__global__ void k_fof_label(int n, const int* __restrict__ ids, const int* __restrict__ root,
-                            const unsigned* __restrict__ cnt, const int* __restrict__ min_id, int n_min, int* label,
+__global__ void k_fof_label(int n, const int* ids, const int* root,
+                            const unsigned* cnt, const int* min_id, int n_min, int* label,
                             int* size, unsigned* halo_flag) {
+  after_previous();
   for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < n; t += gridDim.x * blockDim.x) {
     const int id = ids[t], r = root[t], l = min_id[r];
     const unsigned c = cnt[r];
@@ -253,11 +260,12 @@ __global__ void k_fof_label(int n, const int* __restrict__ ids, const int* __res
   }
 }
 
-__global__ void k_fof_halo_sums(int n, const uint4* __restrict__ rec, const int* __restrict__ root,
-                                const unsigned* __restrict__ cnt, const int* __restrict__ min_id, int n_min,
-                                const unsigned* __restrict__ hoff, const unsigned* __restrict__ g0,
-                                const unsigned* __restrict__ g1, const unsigned* __restrict__ g2, long long modulus,
+__global__ void k_fof_halo_sums(int n, const uint4* rec, const int* root,
+                                const unsigned* cnt, const int* min_id, int n_min,
+                                const unsigned* hoff, const unsigned* g0,
+                                const unsigned* g1, const unsigned* g2, long long modulus,
                                 int capacity, unsigned long long* sums) {
+  after_previous();
   for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < n; t += gridDim.x * blockDim.x) {
     const int r = root[t];
     if (cnt[r] < (unsigned)n_min) continue;
@@ -282,11 +290,12 @@ __global__ void k_fof_halo_sums(int n, const uint4* __restrict__ rec, const int*
   }
 }
 
-__global__ void k_fof_halo_finish(int n, const unsigned* __restrict__ halo_flag, const int* __restrict__ size,
-                                  const unsigned* __restrict__ hoff, const unsigned* __restrict__ g0,
-                                  const unsigned* __restrict__ g1, const unsigned* __restrict__ g2, long long modulus,
-                                  int capacity, const unsigned long long* __restrict__ sums, int* halo_label,
+__global__ void k_fof_halo_finish(int n, const unsigned* halo_flag, const int* size,
+                                  const unsigned* hoff, const unsigned* g0,
+                                  const unsigned* g1, const unsigned* g2, long long modulus,
+                                  int capacity, const unsigned long long* sums, int* halo_label,
                                   int* halo_size, double* halo_pos, int* nhalo) {
+  after_previous();
   for (int id = blockIdx.x * blockDim.x + threadIdx.x; id < n; id += gridDim.x * blockDim.x) {
     if (id == 0) *nhalo = (int)hoff[n];
     if (!halo_flag[id]) continue;
@@ -340,29 +349,26 @@ int launch_fof(const ParticleGeom& pg, const FofGeom& f, const float* s, const F
     return COLA_ERR_CUDA;
   const unsigned gp = grid_for(n, 256);
   const RowBlocks rb = row_blocks(pg.np);
-  k_fof_prepare<<<rb.grid, rb.block, 0, st>>>(pg, s, f, fb.g[0], fb.g[1], fb.g[2], fb.key, fb.counts);
+  launch_after(k_fof_prepare, rb.grid, rb.block, 0, st, pg, s, f, fb.g[0], fb.g[1], fb.g[2], fb.key, fb.counts);
   if ((e = check_launch("fof_prepare")) != COLA_OK) return e;
   if ((e = launch_excl_scan(fb.counts, (int)f.ncells, fb.seg, fb.off, st)) != COLA_OK) return e;
-  k_fof_scatter<<<gp, 256, 0, st>>>(n, fb.key, fb.off, fb.counts, fb.g[0], fb.g[1], fb.g[2], fb.rec, fb.ids,
-                                    fb.min_id);
+  launch_after(k_fof_scatter, gp, 256, 0, st, n, fb.key, fb.off, fb.counts, fb.g[0], fb.g[1], fb.g[2], fb.rec, fb.ids, fb.min_id);
   const unsigned gl = (unsigned)((n + 255LL) / 256);   // one record per thread: their work differs most
-  if (f.ncs == 1) k_fof_first<true><<<gl, 256, 0, st>>>(n, fb.rec, fb.off, f, fb.parent);
-  else k_fof_first<false><<<gl, 256, 0, st>>>(n, fb.rec, fb.off, f, fb.parent);
-  k_fof_carry<<<gp, 256, 0, st>>>(n, fb.rec, fb.parent);
-  if (f.ncs == 1) k_fof_link<true><<<gl, 256, 0, st>>>(n, fb.rec, fb.off, f, fb.parent, flags);
-  else k_fof_link<false><<<gl, 256, 0, st>>>(n, fb.rec, fb.off, f, fb.parent, flags);
-  k_fof_roots<<<gp, 256, 0, st>>>(n, fb.ids, fb.parent, fb.key, fb.cnt, fb.min_id);   // key: the roots from here on
-  k_fof_label<<<gp, 256, 0, st>>>(n, fb.ids, fb.key, fb.cnt, fb.min_id, n_min, label, size, fb.flag);
+  if (f.ncs == 1) launch_after(k_fof_first<true>, gl, 256, 0, st, n, fb.rec, fb.off, f, fb.parent);
+  else launch_after(k_fof_first<false>, gl, 256, 0, st, n, fb.rec, fb.off, f, fb.parent);
+  launch_after(k_fof_carry, gp, 256, 0, st, n, fb.rec, fb.parent);
+  if (f.ncs == 1) launch_after(k_fof_link<true>, gl, 256, 0, st, n, fb.rec, fb.off, f, fb.parent, flags);
+  else launch_after(k_fof_link<false>, gl, 256, 0, st, n, fb.rec, fb.off, f, fb.parent, flags);
+  launch_after(k_fof_roots, gp, 256, 0, st, n, fb.ids, fb.parent, fb.key, fb.cnt, fb.min_id);   // key: the roots from here on
+  launch_after(k_fof_label, gp, 256, 0, st, n, fb.ids, fb.key, fb.cnt, fb.min_id, n_min, label, size, fb.flag);
   if ((e = check_launch("fof_link")) != COLA_OK) return e;
   if ((e = launch_excl_scan(fb.flag, n, fb.seg, fb.hoff, st)) != COLA_OK) return e;
   const int cap = capacity > 0 ? capacity : 0;
   if (cap > 0 && halo_pos) {
     if (cudaMemsetAsync(fb.sums, 0, 3ULL * cap * sizeof(unsigned long long), st) != cudaSuccess) return COLA_ERR_CUDA;
-    k_fof_halo_sums<<<gp, 256, 0, st>>>(n, fb.rec, fb.key, fb.cnt, fb.min_id, n_min, fb.hoff, fb.g[0], fb.g[1], fb.g[2],
-                                        f.modulus, cap, fb.sums);
+    launch_after(k_fof_halo_sums, gp, 256, 0, st, n, fb.rec, fb.key, fb.cnt, fb.min_id, n_min, fb.hoff, fb.g[0], fb.g[1], fb.g[2], f.modulus, cap, fb.sums);
   }
-  k_fof_halo_finish<<<gp, 256, 0, st>>>(n, fb.flag, size, fb.hoff, fb.g[0], fb.g[1], fb.g[2], f.modulus, cap, fb.sums,
-                                        halo_label, halo_size, cap > 0 ? halo_pos : nullptr, nhalo);
+  launch_after(k_fof_halo_finish, gp, 256, 0, st, n, fb.flag, size, fb.hoff, fb.g[0], fb.g[1], fb.g[2], f.modulus, cap, fb.sums, halo_label, halo_size, cap > 0 ? halo_pos : nullptr, nhalo);
   return check_launch("fof_halos");
 }
 

@@ -33,8 +33,9 @@ unsigned grid_for(long long work, int threads) {
 constexpr int kRowThreads = 256;
 
 template <bool F32>
-__global__ void __launch_bounds__(kRowThreads) k_deposit(ParticleGeom pg, FixedGeo fg, const float* __restrict__ s,
+__global__ void __launch_bounds__(kRowThreads) k_deposit(ParticleGeom pg, FixedGeo fg, const float* s,
                                                         unsigned long long* rho) {
+  after_previous();
   const long long n = pg.npart;
   const int nm = pg.n, np = pg.np;
   const int qx = blockIdx.y, qy = blockIdx.x * blockDim.y + threadIdx.y;
@@ -48,7 +49,7 @@ __global__ void __launch_bounds__(kRowThreads) k_deposit(ParticleGeom pg, FixedG
 #pragma unroll
       for (int a = 0; a < 3; ++a) {
         int f;
-        cell_frac<F32>(q[a], __ldg(s + a * n + id), fg, &c[a], &f);
+        cell_frac<F32>(q[a], *(s + a * n + id), fg, &c[a], &f);
         w1[a] = (unsigned)f;
         w0[a] = kWeightOne - w1[a];
       }
@@ -74,12 +75,13 @@ __global__ void __launch_bounds__(kRowThreads) k_deposit(ParticleGeom pg, FixedG
 
 // CIC gather of the three force fields, optionally fused with the COLA kick and drift.
 template <bool KICK, bool F32>
-__global__ void __launch_bounds__(kRowThreads) k_gather(ParticleGeom pg, FixedGeo fg, const float* __restrict__ f0,
-                                                       const float* __restrict__ f1, const float* __restrict__ f2,
-                                                       long long rs, const float* __restrict__ s_in,
-                                                       float* __restrict__ force_out, float* s, float* v,
-                                                       const float* __restrict__ psi1,
-                                                       const float* __restrict__ psi2, KickDrift kd, int* flags) {
+__global__ void __launch_bounds__(kRowThreads) k_gather(ParticleGeom pg, FixedGeo fg, const float* f0,
+                                                       const float* f1, const float* f2,
+                                                       long long rs, const float* s_in,
+                                                       float* force_out, float* s, float* v,
+                                                       const float* psi1,
+                                                       const float* psi2, KickDrift kd, int* flags) {
+  after_previous();
   const long long n = pg.npart;
   const int nm = pg.n, np = pg.np;
   const float inv_one = 1.0f / kWeightOne;
@@ -114,9 +116,9 @@ __global__ void __launch_bounds__(kRowThreads) k_gather(ParticleGeom pg, FixedGe
           const long long rbase = ((long long)ix * nm + iy) * rs;
           const int iz0 = c[2], iz1 = (c[2] + 1) == nm ? 0 : c[2] + 1;
           const float wz1 = w1[2], wz0 = 1.0f - w1[2];
-          fx += wxy * (wz0 * __ldg(f0 + rbase + iz0) + wz1 * __ldg(f0 + rbase + iz1));
-          fy += wxy * (wz0 * __ldg(f1 + rbase + iz0) + wz1 * __ldg(f1 + rbase + iz1));
-          fz += wxy * (wz0 * __ldg(f2 + rbase + iz0) + wz1 * __ldg(f2 + rbase + iz1));
+          fx += wxy * (wz0 * *(f0 + rbase + iz0) + wz1 * *(f0 + rbase + iz1));
+          fy += wxy * (wz0 * *(f1 + rbase + iz0) + wz1 * *(f1 + rbase + iz1));
+          fz += wxy * (wz0 * *(f2 + rbase + iz0) + wz1 * *(f2 + rbase + iz1));
         }
       }
       if (!KICK) {
@@ -127,7 +129,7 @@ __global__ void __launch_bounds__(kRowThreads) k_gather(ParticleGeom pg, FixedGe
         const float fp[3] = {fx, fy, fz};
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
-          const float p1 = __ldg(psi1 + a * n + id), p2 = __ldg(psi2 + a * n + id);
+          const float p1 = *(psi1 + a * n + id), p2 = *(psi2 + a * n + id);
           const float fres = fp[a] - (kd.c1 * p1 + kd.c2 * p2);
           const float vn = v[a * n + id] + kd.kick * fres;
           const float sn = sv[a] + kd.drift * vn + kd.dd1 * p1 + kd.dd2 * p2;
@@ -150,9 +152,10 @@ __device__ __forceinline__ void add128(unsigned long long& lo, unsigned long lon
   lo += l;
   hi += h + (lo < l);
 }
-__global__ void __launch_bounds__(kCheckThreads) k_mass_check(unsigned long long* acc, const unsigned long long* __restrict__ pairs,
+__global__ void __launch_bounds__(kCheckThreads) k_mass_check(unsigned long long* acc, const unsigned long long* pairs,
                                                               int m, unsigned long long expect_lo,
                                                               unsigned long long expect_hi, int* flags) {
+  after_previous();
   __shared__ unsigned long long part[2 * kCheckThreads / 32];
   unsigned long long lo = 0ULL, hi = 0ULL;
   if (threadIdx.x < kMassSlots) {
@@ -177,7 +180,8 @@ __global__ void __launch_bounds__(kCheckThreads) k_mass_check(unsigned long long
   }
 }
 
-__global__ void k_mesh_sum(const unsigned long long* __restrict__ rho, long long cells, unsigned long long* acc) {
+__global__ void k_mesh_sum(const unsigned long long* rho, long long cells, unsigned long long* acc) {
+  after_previous();
   unsigned long long lo = 0, hi = 0;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < cells; i += (long long)gridDim.x * blockDim.x) {
     const unsigned long long v = rho[i];
@@ -190,6 +194,7 @@ __global__ void k_mesh_sum(const unsigned long long* __restrict__ rho, long long
 // ---- 2LPT helpers on the lattice grid (side n = np, half spectrum rows of pc) --------------
 
 __global__ void k_ic_amplitude(int n, int pc, int nc, float2* wk, const float* __restrict__ amp_m2) {
+  after_previous();
   const long long total = (long long)n * n * nc;
   for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < total;
        t += (long long)gridDim.x * blockDim.x) {
@@ -206,8 +211,9 @@ __global__ void k_ic_amplitude(int n, int pc, int nc, float2* wk, const float* _
 // dst(k) = M(k) src(k): Psi1 component i: i kodd_i / k^2; Hessian (i, j): k_i k_j / k^2 (diagonal
 // uses the full k_i, off-diagonal the Nyquist-zeroed kodd); Psi2 component i: -i kodd_i / k^2.
 // k in radians per lattice spacing, times 'scale'.
-__global__ void k_ic_multiply(int n, int pc, int nc, const float2* __restrict__ src, float2* dst, IcMul mp,
+__global__ void k_ic_multiply(int n, int pc, int nc, const float2* src, float2* dst, IcMul mp,
                               int accumulate) {
+  after_previous();
   const long long total = (long long)n * n * nc;
   for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < total;
        t += (long long)gridDim.x * blockDim.x) {
@@ -224,9 +230,10 @@ __global__ void k_ic_multiply(int n, int pc, int nc, const float2* __restrict__ 
 }
 
 // S = h00 h11 + h00 h22 + h11 h22 - h01^2 - h02^2 - h12^2 on real rows of stride 2 pc.
-__global__ void k_ic_source(int n, int pc, const float* __restrict__ h0, const float* __restrict__ h1,
-                            const float* __restrict__ h2, const float* __restrict__ h3,
-                            const float* __restrict__ h4, const float* __restrict__ h5, float* dst) {
+__global__ void k_ic_source(int n, int pc, const float* h0, const float* h1,
+                            const float* h2, const float* h3,
+                            const float* h4, const float* h5, float* dst) {
+  after_previous();
   const long long total = (long long)n * n * n;
   const long long rs = 2LL * pc;
   for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < total;
@@ -237,7 +244,8 @@ __global__ void k_ic_source(int n, int pc, const float* __restrict__ h0, const f
   }
 }
 
-__global__ void k_ic_to_particles(int n, int pc, const float* __restrict__ field, float scale, float* dst) {
+__global__ void k_ic_to_particles(int n, int pc, const float* field, float scale, float* dst) {
+  after_previous();
   const long long total = (long long)n * n * n;
   const long long rs = 2LL * pc;
   for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < total;
@@ -245,8 +253,9 @@ __global__ void k_ic_to_particles(int n, int pc, const float* __restrict__ field
     dst[t] = field[(t / n) * rs + (t % n)] * scale;
 }
 
-__global__ void k_ic_positions(long long n3, const float* __restrict__ psi1, const float* __restrict__ psi2,
+__global__ void k_ic_positions(long long n3, const float* psi1, const float* psi2,
                                float d1, float d2, float* s, float* v) {
+  after_previous();
   for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n3;
        t += (long long)gridDim.x * blockDim.x) {
     s[t] = d1 * psi1[t] + d2 * psi2[t];
@@ -255,9 +264,10 @@ __global__ void k_ic_positions(long long n3, const float* __restrict__ psi1, con
 }
 
 // s_out = s + alpha v + b1 psi1 + b2 psi2;  v_out = v + g1 psi1 + g2 psi2   (all [3][n])
-__global__ void k_snapshot(long long n3, const float* __restrict__ s, const float* __restrict__ v,
-                           const float* __restrict__ psi1, const float* __restrict__ psi2, float alpha, float b1,
+__global__ void k_snapshot(long long n3, const float* s, const float* v,
+                           const float* psi1, const float* psi2, float alpha, float b1,
                            float b2, float g1, float g2, float* s_out, float* v_out) {
+  after_previous();
   for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n3;
        t += (long long)gridDim.x * blockDim.x) {
     const float p1 = psi1[t], p2 = psi2[t], vv = v[t];
@@ -309,8 +319,9 @@ __device__ __forceinline__ int pk_run(int bin, int lane, bool* last) {
   return 31 - __clz(heads & (0xffffffffu >> (31 - lane)));
 }
 
-__global__ void __launch_bounds__(kPkThreads) k_pk_geometry(int n, int nc, const long long* __restrict__ edges_g,
+__global__ void __launch_bounds__(kPkThreads) k_pk_geometry(int n, int nc, const long long* edges_g,
                                                             int nbins, double* partials) {
+  after_previous();
   __shared__ long long edges[kMaxBins + 1];
   __shared__ double hk[kPkWarps][kMaxBins];
   __shared__ int hc[kPkWarps][kMaxBins];   // below 2^31 modes per warp: n^2 (n/2 + 1) / 9728
@@ -364,7 +375,7 @@ __global__ void __launch_bounds__(kPkThreads) k_pk_geometry(int n, int nc, const
 // Sum of column b of the nblocks rows of `cols` doubles, by a block of kPkSumThreads in a fixed order (one
 // thread per bin over 1216 rows took 113 us at any mesh size).  The result is thread 0's.
 constexpr int kPkSumThreads = 128;
-__device__ __forceinline__ double pk_column(const double* __restrict__ partials, int nblocks, int cols, int b) {
+__device__ __forceinline__ double pk_column(const double* partials, int nblocks, int cols, int b) {
   __shared__ double part[kPkSumThreads / 32];
   double v = 0.0;
   for (int i = threadIdx.x; i < nblocks; i += kPkSumThreads) v += partials[(size_t)i * cols + b];
@@ -378,8 +389,9 @@ __device__ __forceinline__ double pk_column(const double* __restrict__ partials,
 }
 
 // geom[0..nbins) = sum of |m| per bin, geom[nbins..2 nbins) = mode count (exact in FP64)
-__global__ void __launch_bounds__(kPkSumThreads) k_pk_geometry_finish(const double* __restrict__ partials, int nblocks,
+__global__ void __launch_bounds__(kPkSumThreads) k_pk_geometry_finish(const double* partials, int nblocks,
                                                                       int nbins, double* geom) {
+  after_previous();
   const double v = pk_column(partials, nblocks, 2 * nbins, blockIdx.x);
   if (threadIdx.x == 0) geom[blockIdx.x] = v;
 }
@@ -388,9 +400,10 @@ constexpr int kPkUnroll = 4;   // k_z chunks of 32 whose loads a lane issues bef
 
 // Bound by the instructions of the segmented scans: equal bins along a row are contiguous, so a run's
 // first lane comes from one ballot instead of a bin shuffle at every distance.
-__global__ void __launch_bounds__(kPkThreads) k_pk_power(int n, int pc, int nc, const float2* __restrict__ dk,
-                                                         const long long* __restrict__ edges_g, int nbins,
+__global__ void __launch_bounds__(kPkThreads) k_pk_power(int n, int pc, int nc, const float2* dk,
+                                                         const long long* edges_g, int nbins,
                                                          int cic_correct, double* partials) {
+  after_previous();
   __shared__ int edges[kMaxBins + 1];   // |m|^2 <= 3 (n/2)^2 < 2^24
   __shared__ double hp[kPkWarps][kMaxBins];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -460,9 +473,10 @@ __global__ void __launch_bounds__(kPkThreads) k_pk_power(int n, int pc, int nc, 
 
 // pk[0..nbins) = mean |k| (h/Mpc), pk[nbins..) = P = pscale * mean power - shot, pk[2 nbins..) = modes;
 // a block per bin
-__global__ void __launch_bounds__(kPkSumThreads) k_pk_finish(const double* __restrict__ partials, int nblocks, int nbins,
-                                                             const double* __restrict__ geom, double kfund, double pscale,
+__global__ void __launch_bounds__(kPkSumThreads) k_pk_finish(const double* partials, int nblocks, int nbins,
+                                                             const double* geom, double kfund, double pscale,
                                                              double shot, double* pk) {
+  after_previous();
   const int b = blockIdx.x;
   const double sp = pk_column(partials, nblocks, nbins, b);
   if (threadIdx.x) return;
@@ -473,9 +487,10 @@ __global__ void __launch_bounds__(kPkSumThreads) k_pk_finish(const double* __res
 }
 
 // out[j m + i] = F_j at mesh cell cells[i] = (ix N + iy) N + iz of the real fields (rows of rs floats)
-__global__ void k_sample_mesh(int n, long long rs, const float* __restrict__ f0, const float* __restrict__ f1,
-                              const float* __restrict__ f2, const long long* __restrict__ cells, long long m,
-                              float* __restrict__ out) {
+__global__ void k_sample_mesh(int n, long long rs, const float* f0, const float* f1,
+                              const float* f2, const long long* cells, long long m,
+                              float* out) {
+  after_previous();
   const long long n3 = (long long)n * n * n;
   for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < m; t += (long long)gridDim.x * blockDim.x) {
     long long c = cells[t];
@@ -488,7 +503,8 @@ __global__ void k_sample_mesh(int n, long long rs, const float* __restrict__ f0,
   }
 }
 
-__global__ void k_dense_spectrum(int n, int pc, int nc, const float2* __restrict__ src, float2* dst) {
+__global__ void k_dense_spectrum(int n, int pc, int nc, const float2* src, float2* dst) {
+  after_previous();
   const long long total = (long long)n * n * nc;
   for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < total;
        t += (long long)gridDim.x * blockDim.x)
@@ -501,13 +517,14 @@ int launch_deposit(const ParticleGeom& pg, const float* s, unsigned long long* r
   (void)flags;
   const RowBlocks rb = row_blocks(pg.np);
   const FixedGeo fg = fixed_geo(pg.n, pg.r_fixed);
-  if (pg.n < 2048) k_deposit<true><<<rb.grid, rb.block, 0, st>>>(pg, fg, s, rho);
-  else k_deposit<false><<<rb.grid, rb.block, 0, st>>>(pg, fg, s, rho);
+  if (pg.n < 2048) launch_after(k_deposit<true>, rb.grid, rb.block, 0, st, pg, fg, s, rho);
+  else launch_after(k_deposit<false>, rb.grid, rb.block, 0, st, pg, fg, s, rho);
   return check_launch("deposit");
 }
 
 // 128-bit sum of m (lo, hi) pairs into the accumulator slots
-__global__ void k_mass_reduce(const unsigned long long* __restrict__ pairs, long long m, unsigned long long* acc) {
+__global__ void k_mass_reduce(const unsigned long long* pairs, long long m, unsigned long long* acc) {
+  after_previous();
   unsigned long long lo = 0, hi = 0;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < m; i += (long long)gridDim.x * blockDim.x) {
     const unsigned long long l = pairs[2 * i];
@@ -521,12 +538,12 @@ int launch_mass_check(const ParticleGeom& pg, const unsigned long long* rho, con
                       unsigned long long* acc, int* flags, cudaStream_t st) {
   if (rho) {
     const long long cells = (long long)pg.n * pg.n * pg.n;
-    k_mesh_sum<<<grid_for(cells, 256), 256, 0, st>>>(rho, cells, acc);
+    launch_after(k_mesh_sum, grid_for(cells, 256), 256, 0, st, rho, cells, acc);
     const int e = check_launch("mesh_sum");
     if (e != COLA_OK) return e;
   }
   if (m > 16 * kCheckThreads) {   // more than the one block of the check sums in a few turns
-    k_mass_reduce<<<grid_for(m, 256), 256, 0, st>>>(pairs, m, acc);
+    launch_after(k_mass_reduce, grid_for(m, 256), 256, 0, st, pairs, m, acc);
     const int e = check_launch("mass_reduce");
     if (e != COLA_OK) return e;
     m = 0;
@@ -534,7 +551,7 @@ int launch_mass_check(const ParticleGeom& pg, const unsigned long long* rho, con
   // expected total: n 2^42 as a 128-bit number
   const unsigned long long n = (unsigned long long)pg.npart;
   const unsigned long long lo = n << 42, hi = n >> 22;
-  k_mass_check<<<1, kCheckThreads, 0, st>>>(acc, pairs, (int)m, lo, hi, flags);
+  launch_after(k_mass_check, 1, kCheckThreads, 0, st, acc, pairs, (int)m, lo, hi, flags);
   return check_launch("mass_check");
 }
 
@@ -545,83 +562,76 @@ int launch_gather(const ParticleGeom& pg, const float* const f[3], long long rs,
   const FixedGeo fg = fixed_geo(pg.n, pg.r_fixed);
   if (kd) {
     auto* k = pg.n < 2048 ? k_gather<true, true> : k_gather<true, false>;
-    k<<<rb.grid, rb.block, 0, st>>>(pg, fg, f[0], f[1], f[2], rs, nullptr, nullptr, s, v, psi1, psi2, *kd, flags);
+    launch_after(k, rb.grid, rb.block, 0, st, pg, fg, f[0], f[1], f[2], rs, nullptr, nullptr, s, v, psi1, psi2, *kd, flags);
   } else {
     auto* k = pg.n < 2048 ? k_gather<false, true> : k_gather<false, false>;
-    k<<<rb.grid, rb.block, 0, st>>>(pg, fg, f[0], f[1], f[2], rs, s_in, force_out, nullptr, nullptr, nullptr, nullptr,
-                                    KickDrift{}, flags);
+    launch_after(k, rb.grid, rb.block, 0, st, pg, fg, f[0], f[1], f[2], rs, s_in, force_out, nullptr, nullptr, nullptr, nullptr, KickDrift{}, flags);
   }
   return check_launch("gather");
 }
 
 int launch_ic_amplitude(const Grid3& g, float2* wk, const float* amp_m2, cudaStream_t st) {
-  k_ic_amplitude<<<grid_for((long long)g.rows() * g.nc, 256), 256, 0, st>>>(g.n, g.pc, g.nc, wk, amp_m2);
+  launch_after(k_ic_amplitude, grid_for((long long)g.rows() * g.nc, 256), 256, 0, st, g.n, g.pc, g.nc, wk, amp_m2);
   return check_launch("ic_amplitude");
 }
 
 int launch_ic_multiply(const Grid3& g, const float2* src, float2* dst, IcField kind, int i, int j, float scale,
                        cudaStream_t st, bool accumulate) {
-  k_ic_multiply<<<grid_for((long long)g.rows() * g.nc, 256), 256, 0, st>>>(g.n, g.pc, g.nc, src, dst,
-                                                                           IcMul{(int)kind, i, j, scale},
-                                                                           accumulate ? 1 : 0);
+  launch_after(k_ic_multiply, grid_for((long long)g.rows() * g.nc, 256), 256, 0, st, g.n, g.pc, g.nc, src, dst, IcMul{(int)kind, i, j, scale}, accumulate ? 1 : 0);
   return check_launch("ic_multiply");
 }
 
 int launch_ic_source(const Grid3& g, float2* const h[6], float2* dst, cudaStream_t st) {
   auto f = [](float2* p) { return reinterpret_cast<const float*>(p); };
-  k_ic_source<<<grid_for((long long)g.rows() * g.n, 256), 256, 0, st>>>(
-      g.n, g.pc, f(h[0]), f(h[1]), f(h[2]), f(h[3]), f(h[4]), f(h[5]), reinterpret_cast<float*>(dst));
+  launch_after(k_ic_source, grid_for((long long)g.rows() * g.n, 256), 256, 0, st,  g.n, g.pc, f(h[0]), f(h[1]), f(h[2]), f(h[3]), f(h[4]), f(h[5]), reinterpret_cast<float*>(dst));
   return check_launch("ic_source");
 }
 
 int launch_ic_to_particles(const Grid3& g, const float2* field, float scale, float* dst, cudaStream_t st) {
-  k_ic_to_particles<<<grid_for((long long)g.rows() * g.n, 256), 256, 0, st>>>(
-      g.n, g.pc, reinterpret_cast<const float*>(field), scale, dst);
+  launch_after(k_ic_to_particles, grid_for((long long)g.rows() * g.n, 256), 256, 0, st,  g.n, g.pc, reinterpret_cast<const float*>(field), scale, dst);
   return check_launch("ic_to_particles");
 }
 
 int launch_ic_positions(long long npart, const float* psi1, const float* psi2, float d1, float d2, float* s,
                         float* v, cudaStream_t st) {
-  k_ic_positions<<<grid_for(3 * npart, 256), 256, 0, st>>>(3 * npart, psi1, psi2, d1, d2, s, v);
+  launch_after(k_ic_positions, grid_for(3 * npart, 256), 256, 0, st, 3 * npart, psi1, psi2, d1, d2, s, v);
   return check_launch("ic_positions");
 }
 
 int launch_snapshot(long long npart, const float* s, const float* v, const float* psi1, const float* psi2, float alpha,
                     float b1, float b2, float g1, float g2, float* s_out, float* v_out, cudaStream_t st) {
-  k_snapshot<<<grid_for(3 * npart, 256), 256, 0, st>>>(3 * npart, s, v, psi1, psi2, alpha, b1, b2, g1, g2, s_out,
-                                                       v_out);
+  launch_after(k_snapshot, grid_for(3 * npart, 256), 256, 0, st, 3 * npart, s, v, psi1, psi2, alpha, b1, b2, g1, g2, s_out, v_out);
   return check_launch("snapshot");
 }
 
 int launch_pk_geometry(const Grid3& g, const long long* edges, int nbins, double* partials, int nblocks,
                        double* geom, cudaStream_t st) {
-  k_pk_geometry<<<nblocks, kPkThreads, 0, st>>>(g.n, g.nc, edges, nbins, partials);
-  k_pk_geometry_finish<<<2 * nbins, kPkSumThreads, 0, st>>>(partials, nblocks, nbins, geom);
+  launch_after(k_pk_geometry, nblocks, kPkThreads, 0, st, g.n, g.nc, edges, nbins, partials);
+  launch_after(k_pk_geometry_finish, 2 * nbins, kPkSumThreads, 0, st, partials, nblocks, nbins, geom);
   return check_launch("pk_geometry");
 }
 
 int launch_pk_bins(const Grid3& g, const float2* dk, const long long* edges, int nbins, int cic_correct,
                    double* partials, int nblocks, cudaStream_t st) {
-  k_pk_power<<<nblocks, kPkThreads, 0, st>>>(g.n, g.pc, g.nc, dk, edges, nbins, cic_correct, partials);
+  launch_after(k_pk_power, nblocks, kPkThreads, 0, st, g.n, g.pc, g.nc, dk, edges, nbins, cic_correct, partials);
   return check_launch("pk_bins");
 }
 
 int launch_pk_finish(const double* partials, int nblocks, int nbins, const double* geom, double kfund, double pscale,
                      double shot, double* pk, cudaStream_t st) {
-  k_pk_finish<<<nbins, kPkSumThreads, 0, st>>>(partials, nblocks, nbins, geom, kfund, pscale, shot, pk);
+  launch_after(k_pk_finish, nbins, kPkSumThreads, 0, st, partials, nblocks, nbins, geom, kfund, pscale, shot, pk);
   return check_launch("pk_finish");
 }
 
 int launch_sample_mesh(const Grid3& g, const float* const f[3], const long long* cells, long long m, float* out,
                        cudaStream_t st) {
   if (m <= 0) return COLA_OK;
-  k_sample_mesh<<<grid_for(m, 256), 256, 0, st>>>(g.n, 2LL * g.pc, f[0], f[1], f[2], cells, m, out);
+  launch_after(k_sample_mesh, grid_for(m, 256), 256, 0, st, g.n, 2LL * g.pc, f[0], f[1], f[2], cells, m, out);
   return check_launch("sample_mesh");
 }
 
 int launch_dense_spectrum(const Grid3& g, const float2* src, float* dst, cudaStream_t st) {
-  k_dense_spectrum<<<grid_for((long long)g.rows() * g.nc, 256), 256, 0, st>>>(g.n, g.pc, g.nc, src,
-                                                                              reinterpret_cast<float2*>(dst));
+  launch_after(k_dense_spectrum, grid_for((long long)g.rows() * g.nc, 256), 256, 0, st, g.n, g.pc, g.nc, src, reinterpret_cast<float2*>(dst));
   return check_launch("dense_spectrum");
 }
 

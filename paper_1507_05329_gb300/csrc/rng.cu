@@ -53,7 +53,8 @@ __device__ __forceinline__ void box_muller(unsigned a, unsigned b, float* z0, fl
 }
 
 // out: real rows of the lattice (site i = row * np + iz at row * rs + iz)
-__global__ void k_white_noise(unsigned k0, unsigned k1, long long n, int np, long long rs, float* __restrict__ out) {
+__global__ void k_white_noise(unsigned k0, unsigned k1, long long n, int np, long long rs, float* out) {
+  after_previous();
   const long long m = (n + 3) >> 2;
   for (long long j = blockIdx.x * (long long)blockDim.x + threadIdx.x; j < m; j += (long long)gridDim.x * blockDim.x) {
     const Words4 w = philox4x32_10((unsigned)j, (unsigned)(j >> 32), 0u, 0u, k0, k1);
@@ -71,7 +72,8 @@ __global__ void k_white_noise(unsigned k0, unsigned k1, long long n, int np, lon
   }
 }
 
-__global__ void k_philox_words(unsigned k0, unsigned k1, long long first, long long count, unsigned* __restrict__ out) {
+__global__ void k_philox_words(unsigned k0, unsigned k1, long long first, long long count, unsigned* out) {
+  after_previous();
   for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < count;
        t += (long long)gridDim.x * blockDim.x) {
     const long long j = first + t;
@@ -90,7 +92,7 @@ unsigned grid_of(long long work) {
 
 int launch_white_noise(unsigned long long seed, int np, long long row_stride, float* out, cudaStream_t st) {
   const long long n = (long long)np * np * np;
-  k_white_noise<<<grid_of((n + 3) / 4), 256, 0, st>>>((unsigned)seed, (unsigned)(seed >> 32), n, np, row_stride, out);
+  launch_after(k_white_noise, grid_of((n + 3) / 4), 256, 0, st, (unsigned)seed, (unsigned)(seed >> 32), n, np, row_stride, out);
   const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) {
     std::fprintf(stderr, "cola: launch of white_noise failed: %s\n", cudaGetErrorString(e));
@@ -100,7 +102,7 @@ int launch_white_noise(unsigned long long seed, int np, long long row_stride, fl
 }
 
 int launch_philox_words(unsigned long long seed, long long first, long long count, unsigned* out, cudaStream_t st) {
-  k_philox_words<<<grid_of(count), 256, 0, st>>>((unsigned)seed, (unsigned)(seed >> 32), first, count, out);
+  launch_after(k_philox_words, grid_of(count), 256, 0, st, (unsigned)seed, (unsigned)(seed >> 32), first, count, out);
   const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) {
     std::fprintf(stderr, "cola: launch of philox_words failed: %s\n", cudaGetErrorString(e));
