@@ -108,8 +108,7 @@ struct Group {
 };
 
 // ---- tiles of W columns (strided passes) ---------------------------------------------------------
-// element (j, w) at (j << lw) + w.  Rows are 64 bytes: only the stores of a first group of even radix
-// meet two rows on the same banks (a pair of wavefronts for one), which costs less than a padded index.
+// element (j, w) at (j << lw) + w (Tile).
 //
 // Groups up to radix kPairR run on two adjacent columns per thread: every access moves 16 bytes and a
 // twiddle serves both.  On single columns the passes waited on the load/store queue (mio_throttle 13 of 30
@@ -120,7 +119,11 @@ constexpr int kPairR = 10;
 
 template <int N>
 struct PenCfg {
-  static constexpr int lw = N <= 1536 ? 3 : 2;             // two tiles (the Green pass) fit a CTA
+  // 16 columns where two tiles still leave two CTAs per SM and the last, partly empty chunk of columns is
+  // small beside the rest; 4 where two tiles of 8 would not fit a CTA.  us of y / Green / inverse y with 8
+  // and 16: 192^3 16.6/32.3/39.8 and 16.2/28.9/33.3, 320^3 57/142/176 and 55/120/133, 360^3 78/175/207 and
+  // 92/195/221, 120^3 8.1/12.4/14.9 and 8.2/12.5/13.7; 4 columns at 1024^3 1976/7846/5692 for 1854/5074/5546.
+  static constexpr int lw = N > 1536 ? 2 : (N >= 144 && N <= 320 ? 4 : 3);
   static constexpr int W = 1 << lw;
   static constexpr Groups P = make_groups(N, false);
   static constexpr int T = imin(1024, round_up((N * W + 15) / 16, 32));   // 16 values per thread
@@ -149,32 +152,58 @@ struct PenTask {
   __device__ __forceinline__ static int b(int idx) { return idx / (C::W / NV); }
 };
 
-// rows j0 + r STEP of columns w.. of a tile in shared memory
-template <int N>
+// Rows j0 + r STEP of columns w.. of a tile in shared memory, in the transforms of the plan or (REV) the
+// reversed plan.  With 64-byte rows, row j of a first group of even radix S lies at slot j ^ (j/S & 1): its
+// stores, S rows apart in neighbouring threads, then meet both halves of the banks.  Every later stride is a
+// multiple of S, so a butterfly's slots are two pointers plus multiples of the stride.  (768^3 inverse y 2.24
+// -> 2.11 ms, y 0.903 -> 0.871; 512^3 y 0.213 -> 0.204; 1024^3 inverse y 5.55 -> 5.42.)
+template <int N, bool REV>
 struct Tile {
+  static constexpr int R0 = Group<N, REV, 0, 1>::R;
+  static constexpr int S = PenCfg<N>::W == 8 && R0 % 2 == 0 ? R0 : 0;
   float2* s;
+  // pointers of the rows of even and odd r (STEP 1: j0 is a multiple of S; else STEP is)
+  template <int STEP>
+  __device__ __forceinline__ void places(int j0, int w, float2** even, float2** odd) const {
+    constexpr int lw = PenCfg<N>::lw;
+    if constexpr (S == 0) {
+      *even = *odd = s + (j0 << lw) + w;
+    } else if constexpr (STEP == 1) {
+      const int t = j0 / S & 1;
+      *even = s + ((j0 + t) << lw) + w;
+      *odd = s + ((j0 - t) << lw) + w;
+    } else {
+      static_assert(STEP % S == 0, "strides after the first group");
+      const int t = j0 / S & 1;
+      *even = s + ((j0 ^ t) << lw) + w;
+      *odd = s + ((j0 ^ t ^ (STEP / S & 1)) << lw) + w;
+    }
+  }
   template <int STEP, int NV, int R>
   __device__ __forceinline__ void load(int j0, int w, float2 (&v)[NV][R]) const {
-    const float2* q = s + (j0 << PenCfg<N>::lw) + w;
+    float2 *even, *odd;
+    places<STEP>(j0, w, &even, &odd);
 #pragma unroll
     for (int r = 0; r < R; ++r) {
+      const float2* q = (r & 1 ? odd : even) + r * (STEP << PenCfg<N>::lw);
       if constexpr (NV == 2) {
-        const float4 t = *reinterpret_cast<const float4*>(q + r * (STEP << PenCfg<N>::lw));
+        const float4 t = *reinterpret_cast<const float4*>(q);
         v[0][r] = make_float2(t.x, t.y);
         v[1][r] = make_float2(t.z, t.w);
       } else {
-        v[0][r] = q[r * (STEP << PenCfg<N>::lw)];
+        v[0][r] = *q;
       }
     }
   }
   template <int STEP, int NV, int R>
   __device__ __forceinline__ void store(int j0, int w, const float2 (&v)[NV][R]) const {
-    float2* q = s + (j0 << PenCfg<N>::lw) + w;
+    float2 *even, *odd;
+    places<STEP>(j0, w, &even, &odd);
 #pragma unroll
     for (int r = 0; r < R; ++r) {
-      if constexpr (NV == 2)
-        *reinterpret_cast<float4*>(q + r * (STEP << PenCfg<N>::lw)) = make_float4(v[0][r].x, v[0][r].y, v[1][r].x, v[1][r].y);
-      else q[r * (STEP << PenCfg<N>::lw)] = v[0][r];
+      float2* q = (r & 1 ? odd : even) + r * (STEP << PenCfg<N>::lw);
+      if constexpr (NV == 2) *reinterpret_cast<float4*>(q) = make_float4(v[0][r].x, v[0][r].y, v[1][r].x, v[1][r].y);
+      else *q = v[0][r];
     }
   }
 };
@@ -252,7 +281,7 @@ __device__ __forceinline__ void pen_inplace(float2* buf, const float2* __restric
 #pragma unroll
   for (int it = 0; it < K::IT; ++it) {
     const int idx = tid + it * PenCfg<N>::T;
-    if (K::live(idx)) Tile<N>{buf}.template load<Q::NB>(K::b(idx), K::w(idx), v[it]);
+    if (K::live(idx)) Tile<N, REV>{buf}.template load<Q::NB>(K::b(idx), K::w(idx), v[it]);
   }
   __syncthreads();
 #pragma unroll
@@ -261,7 +290,7 @@ __device__ __forceinline__ void pen_inplace(float2* buf, const float2* __restric
     if (K::live(idx)) {
       const int b = K::b(idx), k = Q::k_of(b);
       Q::run(v[it], tw, k);
-      Tile<N>{buf}.template store<Q::NS>(Q::out_row(b, k), K::w(idx), v[it]);
+      Tile<N, REV>{buf}.template store<Q::NS>(Q::out_row(b, k), K::w(idx), v[it]);
     }
   }
 }
@@ -272,7 +301,7 @@ template <int N, bool REV, int DIR, bool PP, int G = 1>
 __device__ __forceinline__ float2* pen_middle(float2* a, float2* b, const float2* __restrict__ tw, int tid) {
   if constexpr (G + 1 < PlanOf<N, REV>::m) {
     if constexpr (PP) {
-      pen_stage<N, REV, G, DIR>(Tile<N>{a}, Tile<N>{b}, tw, tid);
+      pen_stage<N, REV, G, DIR>(Tile<N, REV>{a}, Tile<N, REV>{b}, tw, tid);
       __syncthreads();
       return pen_middle<N, REV, DIR, PP, G + 1>(b, a, tw, tid);
     } else {
@@ -300,10 +329,10 @@ __global__ void __launch_bounds__(PenCfg<N>::T, PenCfg<N>::minb) k_pen(Ptr3 data
   using C = PenCfg<N>;
   const int tid = threadIdx.x;
   const auto g = PenPlace<N, AXIS>().of(data.p[blockIdx.z]);
-  pen_stage<N, false, 0, DIR>(g, Tile<N>{sm}, tw, tid);
+  pen_stage<N, false, 0, DIR>(g, Tile<N, false>{sm}, tw, tid);
   __syncthreads();
   float2* cur = pen_middle<N, false, DIR, C::pp>(sm, sm + C::tile, tw, tid);
-  pen_stage<N, false, PlanOf<N, false>::m - 1, DIR>(Tile<N>{cur}, g, tw, tid);
+  pen_stage<N, false, PlanOf<N, false>::m - 1, DIR>(Tile<N, false>{cur}, g, tw, tid);
 }
 
 // The inverse x pass of the 2LPT multiplier mp times the lattice spectrum src, into dst
@@ -333,10 +362,10 @@ __global__ void __launch_bounds__(PenCfg<N>::T, PenCfg<N>::minb) k_pen_mul(const
   const int tid = threadIdx.x;
   const PenPlace<N, 0> at;
   const ColMul<N, PenPlace<N, 0>::JS> g{at.of(src), signed_mode(blockIdx.y, N), at.col0, mp};
-  pen_stage<N, false, 0, +1>(g, Tile<N>{sm}, tw, tid);
+  pen_stage<N, false, 0, +1>(g, Tile<N, false>{sm}, tw, tid);
   __syncthreads();
   float2* cur = pen_middle<N, false, +1, C::pp>(sm, sm + C::tile, tw, tid);
-  pen_stage<N, false, PlanOf<N, false>::m - 1, +1>(Tile<N>{cur}, at.of(dst), tw, tid);
+  pen_stage<N, false, PlanOf<N, false>::m - 1, +1>(Tile<N, false>{cur}, at.of(dst), tw, tid);
 }
 
 // NT transforms at once from here on, in the tiles s, s + tile, ...: middle groups in place, last groups
@@ -350,7 +379,7 @@ __device__ __forceinline__ void multi_finish(float2* s, const D (&d)[NT], const 
     multi_finish<N, REV, DIR, G + 1>(s, d, tw, tid);
   } else {
 #pragma unroll
-    for (int i = 0; i < NT; ++i) pen_stage<N, REV, G, DIR>(Tile<N>{s + i * PenCfg<N>::tile}, d[i], tw, tid);
+    for (int i = 0; i < NT; ++i) pen_stage<N, REV, G, DIR>(Tile<N, REV>{s + i * PenCfg<N>::tile}, d[i], tw, tid);
   }
 }
 
@@ -411,7 +440,7 @@ __global__ void __launch_bounds__(PenCfg<N>::T, MultiCfg<N, 2>::minb) k_green(co
   constexpr long long JS = PenPlace<N, 0>::JS;
   const int tid = threadIdx.x, y = blockIdx.y;
   const PenPlace<N, 0> at;
-  pen_stage<N, false, 0, -1>(at.of(in), Tile<N>{sm}, twf, tid);
+  pen_stage<N, false, 0, -1>(at.of(in), Tile<N, false>{sm}, twf, tid);
   __syncthreads();
   float2* cur = pen_middle<N, false, -1, true>(sm, sm + C::tile, twf, tid);
   X x;
@@ -420,7 +449,7 @@ __global__ void __launch_bounds__(PenCfg<N>::T, MultiCfg<N, 2>::minb) k_green(co
   for (int it = 0; it < K::IT; ++it) {
     const int idx = tid + it * C::T;
     if (K::live(idx)) {
-      Tile<N>{cur}.template load<X::L::NB>(K::b(idx), K::w(idx), x.spec[it]);
+      Tile<N, false>{cur}.template load<X::L::NB>(K::b(idx), K::w(idx), x.spec[it]);
       X::L::run(x.spec[it], twf, K::b(idx));
       if (spec_out) at.of(spec_out).template store<X::L::NS>(K::b(idx), K::w(idx), x.spec[it]);
       x.each(it, idx, at.col0, [&](float2& z, int j, int col) {
@@ -444,9 +473,9 @@ __global__ void __launch_bounds__(PenCfg<N>::T, MultiCfg<N, 2>::minb) k_green(co
         for (int c = 0; c < K::NV; ++c) v[c][r] = make_float2(-d * x.spec[it][c][r].y, d * x.spec[it][c][r].x);   // i D H
       }
       X::F::run(v, twr, 0);
-      Tile<N>{sm}.template store<1>(b * X::L::R, w, v);
+      Tile<N, true>{sm}.template store<1>(b * X::L::R, w, v);
       X::F::run(x.spec[it], twr, 0);
-      Tile<N>{sm + C::tile}.template store<1>(b * X::L::R, w, x.spec[it]);
+      Tile<N, true>{sm + C::tile}.template store<1>(b * X::L::R, w, x.spec[it]);
     }
   }
   __syncthreads();
@@ -481,7 +510,7 @@ __global__ void __launch_bounds__(PenCfg<N>::T, MultiCfg<N, 2>::minb) k_pen_yz(c
         for (int c = 0; c < K::NV; ++c) v[c][r] = make_float2(-d * z[c][r].y, d * z[c][r].x);
       }
       Q::run(v, tw, 0);
-      Tile<N>{sm}.template store<1>(b * Q::R, w, v);
+      Tile<N, false>{sm}.template store<1>(b * Q::R, w, v);
 #pragma unroll
       for (int c = 0; c < K::NV; ++c) {
         const float d = w + c < at.left ? __ldg(dtab + at.col0 + w + c) : 0.0f;
@@ -489,7 +518,7 @@ __global__ void __launch_bounds__(PenCfg<N>::T, MultiCfg<N, 2>::minb) k_pen_yz(c
         for (int r = 0; r < Q::R; ++r) z[c][r] = make_float2(-d * z[c][r].y, d * z[c][r].x);
       }
       Q::run(z, tw, 0);
-      Tile<N>{sm + C::tile}.template store<1>(b * Q::R, w, z);
+      Tile<N, false>{sm + C::tile}.template store<1>(b * Q::R, w, z);
     }
   }
   __syncthreads();
@@ -533,7 +562,7 @@ __device__ __forceinline__ void powers_stage(const float2 (&z)[NV][R], int b, in
 #pragma unroll
       for (int c = 0; c < NV; ++c) v[c][r] = times_k<N, PW>(z[c][r], b + r * Q::NB);
     Q::run(v, tw, 0);
-    Tile<N>{s + PW * PenCfg<N>::tile}.template store<1>(b * R, w, v);
+    Tile<N, REV>{s + PW * PenCfg<N>::tile}.template store<1>(b * R, w, v);
     powers_stage<N, REV, NT, PW + 1>(z, b, w, s, tw);
   }
 }
@@ -553,7 +582,7 @@ __global__ void __launch_bounds__(PenCfg<N>::T, MultiCfg<N, NT>::minb) k_ic_x(co
   constexpr float kf = 6.283185307179586f / N;
   const int tid = threadIdx.x, y = blockIdx.y;
   const PenPlace<N, 0> at;
-  pen_stage<N, false, 0, -1>(at.of(in), Tile<N>{sm}, twf, tid);
+  pen_stage<N, false, 0, -1>(at.of(in), Tile<N, false>{sm}, twf, tid);
   __syncthreads();
   float2* cur = pen_middle<N, false, -1, true>(sm, sm + C::tile, twf, tid);
   X x;
@@ -562,7 +591,7 @@ __global__ void __launch_bounds__(PenCfg<N>::T, MultiCfg<N, NT>::minb) k_ic_x(co
   for (int it = 0; it < K::IT; ++it) {
     const int idx = tid + it * C::T;
     if (K::live(idx)) {
-      Tile<N>{cur}.template load<X::L::NB>(K::b(idx), K::w(idx), x.spec[it]);
+      Tile<N, false>{cur}.template load<X::L::NB>(K::b(idx), K::w(idx), x.spec[it]);
       X::L::run(x.spec[it], twf, K::b(idx));
       x.each(it, idx, at.col0, [&](float2& z, int j, int col) {
         const int mx = j < N / 2 ? j : j - N;
@@ -648,7 +677,7 @@ __device__ __forceinline__ void turn_back(Turn<N>& x, float2* s, const D& d, con
     const int idx = tid + it * PenCfg<N>::T;
     if (K::live(idx)) {
       X::F::run(x.spec[it], twr, 0);
-      Tile<N>{s}.template store<1>(K::b(idx) * X::L::R, K::w(idx), x.spec[it]);
+      Tile<N, true>{s}.template store<1>(K::b(idx) * X::L::R, K::w(idx), x.spec[it]);
     }
   }
   __syncthreads();
@@ -683,7 +712,7 @@ __global__ void __launch_bounds__(PenCfg<N>::T, MultiCfg<N, 2>::minb) k_grad_adj
       float2 v[KA::NV][A::R], u[KA::NV][A::R];
       at.of(l0).template load<A::NB>(b, w, v);
       A::run(v, twf, 0);
-      Tile<N>{sm}.template store<1>(b * A::R, w, v);
+      Tile<N, false>{sm}.template store<1>(b * A::R, w, v);
       at.of(l1).template load<A::NB>(b, w, v);
       at.of(l2).template load<A::NB>(b, w, u);
 #pragma unroll
@@ -693,7 +722,7 @@ __global__ void __launch_bounds__(PenCfg<N>::T, MultiCfg<N, 2>::minb) k_grad_adj
         for (int r = 0; r < A::R; ++r) u[c][r] = dy * v[c][r] + dz * u[c][r];
       }
       A::run(u, twf, 0);
-      Tile<N>{sm + C::tile}.template store<1>(b * A::R, w, u);
+      Tile<N, false>{sm + C::tile}.template store<1>(b * A::R, w, u);
     }
   }
   __syncthreads();
@@ -706,9 +735,9 @@ __global__ void __launch_bounds__(PenCfg<N>::T, MultiCfg<N, 2>::minb) k_grad_adj
     if (K::live(idx)) {
       const int b = K::b(idx);
       float2 u[K::NV][X::L::R];
-      Tile<N>{sm}.template load<X::L::NB>(b, K::w(idx), x.spec[it]);
+      Tile<N, false>{sm}.template load<X::L::NB>(b, K::w(idx), x.spec[it]);
       X::L::run(x.spec[it], twf, b);
-      Tile<N>{sm + C::tile}.template load<X::L::NB>(b, K::w(idx), u);
+      Tile<N, false>{sm + C::tile}.template load<X::L::NB>(b, K::w(idx), u);
       X::L::run(u, twf, b);
 #pragma unroll
       for (int r = 0; r < X::L::R; ++r) {
@@ -773,7 +802,7 @@ __global__ void __launch_bounds__(PenCfg<N>::T, MultiCfg<N, 3>::minb) k_lpt_adj(
       };
       auto put = [&](int q) {
         A::run(v, twf, 0);
-        Tile<N>{sm + q * C::tile}.template store<1>(b * A::R, w, v);
+        Tile<N, false>{sm + q * C::tile}.template store<1>(b * A::R, w, v);
       };
       auto clear = [&]() {
 #pragma unroll
@@ -805,12 +834,12 @@ __global__ void __launch_bounds__(PenCfg<N>::T, MultiCfg<N, 3>::minb) k_lpt_adj(
     const int idx = tid + it * C::T;
     if (K::live(idx)) {
       const int b = K::b(idx);
-      Tile<N>{sm}.template load<X::L::NB>(b, K::w(idx), x.spec[it]);
+      Tile<N, false>{sm}.template load<X::L::NB>(b, K::w(idx), x.spec[it]);
       X::L::run(x.spec[it], twf, b);
 #pragma unroll
       for (int q = 1; q < 3; ++q) {
         float2 u[K::NV][X::L::R];
-        Tile<N>{sm + q * C::tile}.template load<X::L::NB>(b, K::w(idx), u);
+        Tile<N, false>{sm + q * C::tile}.template load<X::L::NB>(b, K::w(idx), u);
         X::L::run(u, twf, b);
 #pragma unroll
         for (int r = 0; r < X::L::R; ++r) {
