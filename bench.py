@@ -89,9 +89,9 @@ def stage_bytes(n_mesh: int, n_part: int, binned: bool = True) -> dict:
         "deposit": 12.0 * n_part + mesh,
         "fwd_z_r2c": mesh + cplx,
         "fwd_y": 2 * cplx,
-        "green_x": cplx + 3 * cplx,
-        "inv_y": 2 * cplx,
-        "inv_z_c2r": cplx + real,
+        "green_x": cplx + 2 * cplx,              # F_x, and H for both F_y and F_z
+        "inv_y": 2 * cplx + 3 * cplx,            # all components in one stage call
+        "inv_z_c2r": 3 * (cplx + real),
         "gather_kick_drift": 3 * real + 48.0 * n_part + 24.0 * n_part,
     }
 
@@ -378,7 +378,7 @@ def run_reference(args):
 # ---- our arm -------------------------------------------------------------------------------------
 def source_digest() -> str:
     h = hashlib.sha256()
-    for f in ("fft.cu", "fft_core.cuh", "fft_fast.inc", "particles.cu", "binning.cu"):   # the PM-step kernels
+    for f in ("fft.cu", "fft_core.cuh", "fft_ct.cuh", "fft_plan.h", "particles.cu", "binning.cu"):   # the PM-step kernels
         with open(os.path.join(ROOT, "paper_1507_05329_gb300", "csrc", f), "rb") as fh:
             h.update(fh.read())
     return h.hexdigest()[:16]
