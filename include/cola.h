@@ -268,9 +268,11 @@ int cola_grid_density(cola_ctx* ctx, const float* s, int ngrid, float* delta);
 int cola_grid_density_adjoint(cola_ctx* ctx, const float* s, int ngrid, const float* lam_delta, float* lam_s);
 
 /* ---- Batched realisations in one CUDA graph (the paper's many mock catalogues, §3) ----------
- * A batch owns one context per realisation and `nstreams` non-blocking lanes.  Realisations are
- * assigned to lanes longest-first (cost ~ particles + mesh cells x log N) and run back to back on
- * their lane; lanes run concurrently.  cola_batch_run enqueues cola_run (2LPT + n_step PM steps +
+ * A batch owns one context per realisation and `nstreams` non-blocking lanes.  As many realisations
+ * run side by side as fit the L2 together (lanes beyond that would slow each other down), the
+ * largest meshes first; among members of the same number of lanes, realisations are assigned to
+ * lanes longest-first (cost ~ particles + mesh cells x log N) and run back to back on their lane.
+ * cola_batch_run enqueues cola_run (2LPT + n_step PM steps +
  * P(k) in nbins bins) of every realisation, forked from and joined back into `stream`:
  *   use_graph = 0 : plain launches;
  *   use_graph = 1 : the first call runs once eagerly (warm-up, then synchronises), captures the

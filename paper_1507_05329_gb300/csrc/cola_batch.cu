@@ -31,6 +31,19 @@ double realisation_cost(const cola_params& p) {
   return p.nstep * (84.0 * n + 104.0 * m * (1.0 + std::log2((double)p.nmesh) / 16.0));
 }
 
+// How many realisations of a mesh of n^3 cells run side by side, of at most `lanes`: as many as fit the L2
+// together (about 7 fields of 4 n^3 bytes each: density, spectra, forces and the particles of the usual n/2
+// lattice), at least one.  A kernel of a large mesh fills the chip by itself, and a second realisation only
+// throws the first one's fields out of the L2; small ones leave most of the chip idle, and overlap well.
+// Eight equal members of two steps in a graph, microseconds with 1 / 2 / 4 / 8 lanes (126 MB of L2):
+// 64^3 723 / 422 / 290 / 216, 96^3 1294 / 828 / 647 / 703, 128^3 1764 / 1399 / 1500 / 1691,
+// 192^3 4647 / 5144 / 5795 / 5855, 256^3 9199 / 8737 / 9604 / 9843, 320^3 18259 / 17986 / 19685 / 20126;
+// four of 192^3 with 192^3 particles 7315 / 10097 / 10211.
+int lane_width(int n, int l2_bytes, int lanes) {
+  const double fit = (double)l2_bytes / (28.0 * n * n * n);
+  return (int)std::min((double)lanes, std::max(1.0, std::floor(fit)));
+}
+
 }  // namespace
 
 struct cola_batch {
@@ -41,10 +54,17 @@ struct cola_batch {
   cudaEvent_t start = nullptr, done = nullptr;
   std::vector<cudaStream_t> streams;    // owned
   std::vector<int> lane;                // member -> stream index
+  // members in the order they are enqueued; phases of equal width, a phase after the one before it
+  std::vector<int> order;
+  struct Phase {
+    int first, last;   // members order[first, last)
+    int width;         // on streams [0, width)
+  };
+  std::vector<Phase> phases;
   std::vector<cola_ctx*> ctx;           // owned
   std::vector<cola_batch_io> io;
   cudaEvent_t fork = nullptr;
-  std::vector<cudaEvent_t> join;
+  std::vector<cudaEvent_t> join;        // one per stream: its last member of the phase has run
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t exec = nullptr;
   bool warmed = false;
@@ -56,9 +76,18 @@ namespace {
 int enqueue(cola_batch* b, cudaStream_t on) {
   BATCH_TRY(cuda_status(cudaEventRecord(b->fork, on), "fork"));
   for (cudaStream_t s : b->streams) BATCH_TRY(cuda_status(cudaStreamWaitEvent(s, b->fork, 0), "fork wait"));
-  for (int i = 0; i < b->count; ++i) {
-    const cola_batch_io& o = b->io[i];
-    BATCH_TRY(cola_run(b->ctx[i], o.white_noise, o.s, o.v, o.psi1, o.psi2, o.pk, b->nbins));
+  int before = 0;   // streams of the phase before
+  for (const cola_batch::Phase& ph : b->phases) {
+    for (int l = 0; l < before; ++l) BATCH_TRY(cuda_status(cudaEventRecord(b->join[l], b->streams[l]), "phase"));
+    for (int l = 0; l < ph.width; ++l)
+      for (int k = 0; k < before; ++k)
+        if (k != l) BATCH_TRY(cuda_status(cudaStreamWaitEvent(b->streams[l], b->join[k], 0), "phase wait"));
+    before = ph.width;
+    for (int m = ph.first; m < ph.last; ++m) {
+      const int i = b->order[m];
+      const cola_batch_io& o = b->io[i];
+      BATCH_TRY(cola_run(b->ctx[i], o.white_noise, o.s, o.v, o.psi1, o.psi2, o.pk, b->nbins));
+    }
   }
   for (size_t l = 0; l < b->streams.size(); ++l) {
     BATCH_TRY(cuda_status(cudaEventRecord(b->join[l], b->streams[l]), "join"));
@@ -127,17 +156,31 @@ extern "C" int cola_batch_create(const cola_params* params, const cola_batch_io*
   if (st == COLA_OK) st = cuda_status(cudaEventCreateWithFlags(&b->done, cudaEventDisableTiming), "event");
   if (st == COLA_OK) st = cuda_status(cudaStreamCreateWithFlags(&b->origin, cudaStreamNonBlocking), "stream");
   if (st != COLA_OK) return fail(st);
-  // longest-processing-time-first: the costliest realisation goes to the least loaded lane
-  std::vector<int> order(count);
-  std::iota(order.begin(), order.end(), 0);
-  std::stable_sort(order.begin(), order.end(),
-                   [&](int a, int c) { return realisation_cost(params[a]) > realisation_cost(params[c]); });
-  std::vector<double> load(lanes, 0.0);
+  // The largest meshes first, in phases of members that may run side by side; within a phase the costliest
+  // realisation goes to the least loaded lane.
+  int dev = 0, l2 = 0;
+  st = cuda_status(cudaGetDevice(&dev), "device");
+  if (st == COLA_OK) st = cuda_status(cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, dev), "L2 size");
+  if (st != COLA_OK) return fail(st);
+  auto width = [&](int i) { return lane_width(params[i].nmesh, l2, lanes); };
+  b->order.resize(count);
+  std::iota(b->order.begin(), b->order.end(), 0);
+  std::stable_sort(b->order.begin(), b->order.end(), [&](int a, int c) {
+    return width(a) != width(c) ? width(a) < width(c) : realisation_cost(params[a]) > realisation_cost(params[c]);
+  });
   b->lane.assign(count, 0);
-  for (int i : order) {
-    const int l = (int)(std::min_element(load.begin(), load.end()) - load.begin());
-    b->lane[i] = l;
-    load[l] += realisation_cost(params[i]);
+  for (int first = 0; first < count;) {
+    const int w = width(b->order[first]);
+    std::vector<double> load(w, 0.0);
+    int last = first;
+    for (; last < count && width(b->order[last]) == w; ++last) {
+      const int i = b->order[last];
+      const int l = (int)(std::min_element(load.begin(), load.end()) - load.begin());
+      b->lane[i] = l;
+      load[l] += realisation_cost(params[i]);
+    }
+    b->phases.push_back({first, last, w});
+    first = last;
   }
   b->ctx.assign(count, nullptr);
   for (int i = 0; i < count; ++i) {
