@@ -534,7 +534,7 @@ __global__ void __launch_bounds__(PenCfg<N>::T, MultiCfg<N, 2>::minb) k_pen_yz(c
 // where a transform of its own for each takes nine and nine (and a multiply each).  The factor of a single
 // derivative is 0 on its Nyquist plane, a square keeps it; factors i are left to the row pass.
 // With the row passes below (Hessians and source on chip, first positions written with Psi2) a call is 12
-// launches and moves 52 field-sized reads and writes where 45 launches moved 120: 256^3 lattice 1706 -> 917
+// launches and moves 52 field-sized reads and writes where 45 launches moved 120: 256^3 lattice 1706 -> 833
 // us (0.51 ms for the 52 at the copy rate), 32^3 271 -> 82 us.
 
 // factor k^p, p = 0, 1, 2, k = 2 pi m / n of storage index j
