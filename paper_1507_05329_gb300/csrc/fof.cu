@@ -113,12 +113,12 @@ __global__ void k_fof_scatter(int n, const int* key, const unsigned* off, unsign
                               const unsigned* g0, const unsigned* g1,
                               const unsigned* g2, uint4* rec, int* ids, int* min_id) {
   after_previous();
-  for (int id = blockIdx.x * blockDim.x + threadIdx.x; id < n; id += gridDim.x * blockDim.x) {
+  for (long long id = blockIdx.x * (long long)blockDim.x + threadIdx.x; id < n; id += (long long)gridDim.x * blockDim.x) {
     const int k = key[id];
     const unsigned t = off[k] + atomicSub(counts + k, 1u) - 1u;
     rec[t] = make_uint4(g0[id], g1[id], g2[id], t);
-    ids[t] = id;
-    min_id[t] = id;
+    ids[t] = (int)id;
+    min_id[t] = (int)id;
   }
 }
 
@@ -176,26 +176,28 @@ __device__ __forceinline__ void forward_ranges(int t, int n, const uint4& me, co
 }
 
 // First pass: the record's parent is one friend behind it (itself if it has none), from the last of the
-// farthest column, so that paths are short; only this thread writes it.
+// farthest column, so that paths are short; only this thread writes it.  Element counts come near 2^31, so
+// here and below the index of a walk, and its step of a whole grid above all, has 64 bits.
 template <bool ONE>
 __global__ void __launch_bounds__(256) k_fof_first(int n, const uint4* rec, const unsigned* off,
                                                    FofGeom f, int* parent) {
   after_previous();
   const int ell = (int)f.ell;
   const unsigned long long ell2 = (unsigned long long)f.ell * (unsigned long long)f.ell;
-  for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < n; t += gridDim.x * blockDim.x) {
-    const uint4 me = *(rec + t);
-    int p = t;
-    forward_ranges<ONE>(t, n, me, off, f, [&](unsigned lo, unsigned hi, unsigned sx, unsigned sy, unsigned sz) {
-      for (unsigned u = hi; u > lo && (int)u > t + 1; --u)   // a parent comes after its child
-        if (friends<ONE>(me, *(rec + u - 1), sx, sy, sz, ell, ell2, f.modulus)) {
-          p = (int)u - 1;
-          return true;
-        }
-      return false;
-    });
-    parent[t] = p;
-  }
+  const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  const int t = (int)i;
+  const uint4 me = *(rec + t);
+  int p = t;
+  forward_ranges<ONE>(t, n, me, off, f, [&](unsigned lo, unsigned hi, unsigned sx, unsigned sy, unsigned sz) {
+    for (unsigned u = hi; u > lo && (int)u > t + 1; --u)   // a parent comes after its child
+      if (friends<ONE>(me, *(rec + u - 1), sx, sy, sz, ell, ell2, f.modulus)) {
+        p = (int)u - 1;
+        return true;
+      }
+    return false;
+  });
+  parent[t] = p;
 }
 
 // Second pass: joins record t with its friends behind it of another tree than its own after the first
@@ -211,32 +213,33 @@ __global__ void __launch_bounds__(256) k_fof_link(int n, const uint4* rec, const
   after_previous();
   const int ell = (int)f.ell;
   const unsigned long long ell2 = (unsigned long long)f.ell * (unsigned long long)f.ell;
-  for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < n; t += gridDim.x * blockDim.x) {
-    const uint4 me = *(rec + t);
-    int root = (int)me.w;
-    forward_ranges<ONE>(t, n, me, off, f, [&](unsigned lo, unsigned hi, unsigned sx, unsigned sy, unsigned sz) {
-      for (unsigned u = lo; u < hi; ++u) {
-        const uint4 o = *(rec + u);
-        if (o.w != me.w && friends<ONE>(me, o, sx, sy, sz, ell, ell2, f.modulus))
-          root = unite(parent, root, (int)o.w, flags);
-      }
-      return false;
-    });
-  }
+  const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  const int t = (int)i;
+  const uint4 me = *(rec + t);
+  int root = (int)me.w;
+  forward_ranges<ONE>(t, n, me, off, f, [&](unsigned lo, unsigned hi, unsigned sx, unsigned sy, unsigned sz) {
+    for (unsigned u = lo; u < hi; ++u) {
+      const uint4 o = *(rec + u);
+      if (o.w != me.w && friends<ONE>(me, o, sx, sy, sz, ell, ell2, f.modulus))
+        root = unite(parent, root, (int)o.w, flags);
+    }
+    return false;
+  });
 }
 
 // each record takes its tree's root after the first pass
 __global__ void k_fof_carry(int n, uint4* rec, int* parent) {
   after_previous();
-  for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < n; t += gridDim.x * blockDim.x)
-    rec[t].w = (unsigned)find_root(parent, t);
+  for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n; t += (long long)gridDim.x * blockDim.x)
+    rec[t].w = (unsigned)find_root(parent, (int)t);
 }
 
 // root of every record, members and smallest id per root (one atomic per run of lanes with one root)
 __global__ void k_fof_roots(int n, const int* ids, int* parent, int* root, unsigned* cnt, int* min_id) {
   after_previous();
-  for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < n; t += gridDim.x * blockDim.x) {
-    const int r = find_root(parent, t);
+  for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n; t += (long long)gridDim.x * blockDim.x) {
+    const int r = find_root(parent, (int)t);
     root[t] = r;
     const unsigned grp = __match_any_sync(__activemask(), r);
     const int least = __reduce_min_sync(grp, ids[t]);
@@ -251,7 +254,7 @@ __global__ void k_fof_label(int n, const int* ids, const int* root,
                             const unsigned* cnt, const int* min_id, int n_min, int* label,
                             int* size, unsigned* halo_flag) {
   after_previous();
-  for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < n; t += gridDim.x * blockDim.x) {
+  for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n; t += (long long)gridDim.x * blockDim.x) {
     const int id = ids[t], r = root[t], l = min_id[r];
     const unsigned c = cnt[r];
     label[id] = l;
@@ -266,7 +269,7 @@ __global__ void k_fof_halo_sums(int n, const uint4* rec, const int* root,
                                 const unsigned* g1, const unsigned* g2, long long modulus,
                                 int capacity, unsigned long long* sums) {
   after_previous();
-  for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < n; t += gridDim.x * blockDim.x) {
+  for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n; t += (long long)gridDim.x * blockDim.x) {
     const int r = root[t];
     if (cnt[r] < (unsigned)n_min) continue;
     const int l = min_id[r];
@@ -296,13 +299,13 @@ __global__ void k_fof_halo_finish(int n, const unsigned* halo_flag, const int* s
                                   int capacity, const unsigned long long* sums, int* halo_label,
                                   int* halo_size, double* halo_pos, int* nhalo) {
   after_previous();
-  for (int id = blockIdx.x * blockDim.x + threadIdx.x; id < n; id += gridDim.x * blockDim.x) {
+  for (long long id = blockIdx.x * (long long)blockDim.x + threadIdx.x; id < n; id += (long long)gridDim.x * blockDim.x) {
     if (id == 0) *nhalo = (int)hoff[n];
     if (!halo_flag[id]) continue;
     const unsigned h = hoff[id];
     if (h >= (unsigned)capacity) continue;
     const unsigned c = (unsigned)size[id];
-    if (halo_label) halo_label[h] = id;
+    if (halo_label) halo_label[h] = (int)id;
     if (halo_size) halo_size[h] = (int)c;
     if (halo_pos) {
       const unsigned g[3] = {g0[id], g1[id], g2[id]};
