@@ -597,7 +597,10 @@ int pk_from_spectrum(cola_ctx* c, const float2* dk, double* pk, int nbins, int f
   if (c->pk_geom_nbins != nbins) {   // once per bin count: mode counts and mean |k| of the bins
     COLA_TRY(STAGED(kStPk, launch_pk_geometry(c->mesh, c->edges, nbins, c->pk_partials, c->pk_blocks, c->pk_geom,
                                               c->stream)));
-    c->pk_geom_nbins = nbins;
+    // a captured pass has not run, and may never: later calls cannot rely on it
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    COLA_TRY(cuda_status(cudaStreamIsCapturing(c->stream, &capture), "capture status"));
+    c->pk_geom_nbins = capture == cudaStreamCaptureStatusNone ? nbins : 0;
   }
   COLA_TRY(STAGED(kStPk, launch_pk_bins(c->mesh, dk, c->edges, nbins, corr, c->pk_partials, c->pk_blocks,
                                         c->stream)));
