@@ -744,10 +744,12 @@ int launch_deposit_tiles(const ParticleGeom& pg, const BinGeom& b, const float* 
 }
 
 namespace {
+constexpr int kGatherSmem = kGatherFloats * (int)sizeof(float) + 16;   // + mbarrier
 template <class K>
-void smem_limit(K kernel, int bytes) {
-  if (bytes > 48 * 1024 && first_use_on_device(reinterpret_cast<const void*>(kernel)))
-    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+void gather_smem_limit(K kernel) {
+  once_on_device(reinterpret_cast<const void*>(kernel), [](const void* k) {
+    cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kGatherSmem);
+  });
 }
 }  // namespace
 
@@ -755,17 +757,16 @@ int launch_gather_tiles(const ParticleGeom& pg, const BinGeom& b, const BinBuffe
                         long long rs, const float* s_in, float* force_out, float* s, float* v, const float* psi1,
                         const float* psi2, const KickDrift* kd, int* flags, cudaStream_t st) {
   if (!b.bulk) return COLA_ERR_INVALID;   // 16-byte staging copies along z
-  constexpr int sm = kGatherFloats * (int)sizeof(float) + 16;   // + mbarrier
   const FixedGeo fg = fixed_geo(pg.n, pg.r_fixed);
   const bool f32 = pg.n < 2048;
   if (kd) {
     auto* k = f32 ? k_gather_tiles<true, true> : k_gather_tiles<true, false>;
-    smem_limit(k, sm);
-    launch_after(k, b.tiles, kGatherThreads, sm, st, pg, b, fg, bb.off_p, bb.ent_p, f[0], f[1], f[2], rs, nullptr, nullptr, s, v, psi1, psi2, *kd, flags);
+    gather_smem_limit(k);
+    launch_after(k, b.tiles, kGatherThreads, kGatherSmem, st, pg, b, fg, bb.off_p, bb.ent_p, f[0], f[1], f[2], rs, nullptr, nullptr, s, v, psi1, psi2, *kd, flags);
   } else {
     auto* k = f32 ? k_gather_tiles<false, true> : k_gather_tiles<false, false>;
-    smem_limit(k, sm);
-    launch_after(k, b.tiles, kGatherThreads, sm, st, pg, b, fg, bb.off_p, bb.ent_p, f[0], f[1], f[2], rs, s_in, force_out, nullptr, nullptr, nullptr, nullptr, KickDrift{}, flags);
+    gather_smem_limit(k);
+    launch_after(k, b.tiles, kGatherThreads, kGatherSmem, st, pg, b, fg, bb.off_p, bb.ent_p, f[0], f[1], f[2], rs, s_in, force_out, nullptr, nullptr, nullptr, nullptr, KickDrift{}, flags);
   }
   return check_launch("gather_tiles");
 }

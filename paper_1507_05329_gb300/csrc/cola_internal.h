@@ -95,9 +95,10 @@ int fft_plan_init(FftPlan* plan, int n);   // allocates and fills the twiddle ta
 void fft_plan_free(FftPlan* plan);
 void fft_set_smem_limits();                // raise the dynamic shared-memory limit of the run-time FFT kernels
 
-// True the first time it is called for `key` on the current device (thread safe).  Kernel attributes
-// (the dynamic shared-memory limit) are per device, so every setter is keyed by (device, kernel).
-bool first_use_on_device(const void* key);
+// Calls set(key) the first time it is called for `key` on the current device.  A thread that asks for the
+// same key meanwhile returns only after that call has ended, so none launches a kernel whose attributes
+// another thread is about to set.  Kernel attributes (the dynamic shared-memory limit) are per device.
+void once_on_device(const void* key, void (*set)(const void* key));
 
 // Geometry of a 3D field of side n in the in-place real-to-complex layout:
 // complex rows of pc = (n/2+1 rounded up to even) entries, real rows of 2*pc floats.

@@ -87,17 +87,17 @@ int fft_plan_init(FftPlan* plan, int n) {
   if (cudaMemcpy(plan->tw, h.data(), total * sizeof(float2), cudaMemcpyHostToDevice) != cudaSuccess)
     return COLA_ERR_CUDA;
   fft_plan_set(plan, n, plan->tw);
-  if (first_use_on_device(reinterpret_cast<const void*>(&generic_set_smem_limits))) generic_set_smem_limits();
+  once_on_device(reinterpret_cast<const void*>(&generic_set_smem_limits), [](const void*) { generic_set_smem_limits(); });
   return COLA_OK;
 }
 
-bool first_use_on_device(const void* key) {
+void once_on_device(const void* key, void (*set)(const void* key)) {
   static std::mutex mu;
   static std::set<std::pair<int, const void*>> done;
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) dev = -1;
-  std::lock_guard<std::mutex> lock(mu);
-  return done.insert({dev, key}).second;
+  std::lock_guard<std::mutex> lock(mu);   // held over set
+  if (done.insert({dev, key}).second) set(key);
 }
 
 void fft_set_smem_limits() { generic_set_smem_limits(); }

@@ -221,8 +221,9 @@ __device__ __forceinline__ int tile_elems(int n, int lw) { return (n + n / 16 + 
 // device (host side; the attribute is per device).
 template <class K>
 inline void ensure_smem(K kernel) {
-  if (first_use_on_device(reinterpret_cast<const void*>(kernel)))
-    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+  once_on_device(reinterpret_cast<const void*>(kernel), [](const void* k) {
+    cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+  });
 }
 
 }  // namespace fftk
