@@ -206,7 +206,7 @@ int inverse3d(cola_ctx* c, const Grid3& g, const FftPlan& p, float2* b) {
 // inverse pass and the last pass writes the particle layout itself; else separate kernels do.
 int inverse3d_mul(cola_ctx* c, const Grid3& g, const FftPlan& p, const float2* src, const IcMul& mul, float2* dst,
                   float scale = 1.0f, float* particles = nullptr) {
-  if (fft_compiled(p)) {
+  if (x_mul_compiled(p)) {
     COLA_TRY(STAGED(kStFwdX, launch_pencils_x_mul(p, g, src, mul, dst, c->stream)));
   } else {
     COLA_TRY(STAGED(kStIc, launch_ic_multiply(g, src, dst, (IcField)mul.kind, mul.ci, mul.cj, mul.scale, c->stream)));
@@ -520,8 +520,6 @@ extern "C" int cola_deposit(cola_ctx* c, const float* s, unsigned long long* rho
   if (!c) return COLA_ERR_INVALID;
   COLA_TRY(check_ptr(s));
   COLA_TRY(check_ptr(rho));
-  const size_t n3 = (size_t)c->mesh.n * c->mesh.n * c->mesh.n;
-  (void)n3;
   COLA_TRY(deposit_mesh(c, s, rho));
   return launch_mass_check(c->pg, rho, nullptr, 0, c->mass_acc, c->flags, c->stream);
 }

@@ -131,9 +131,10 @@ int launch_c2r_rows(const FftPlan& p, const Grid3& g, float2* const* data, int f
 // launch_ic_to_particles.
 int launch_c2r_rows_dense(const FftPlan& p, const Grid3& g, const float2* data, float scale, float* out,
                           cudaStream_t st);
-// The inverse x pass of mul times the lattice spectrum src into dst (src unchanged) where the length has
-// compiled kernels; the same floats as launch_ic_multiply followed by launch_pencils(axis 0, +1).
+// The inverse x pass of mul times the lattice spectrum src into dst (src unchanged), of compiled lengths above
+// 1024; the same floats as launch_ic_multiply followed by launch_pencils(axis 0, +1).
 struct IcMul;
+bool x_mul_compiled(const FftPlan& p);
 int launch_pencils_x_mul(const FftPlan& p, const Grid3& g, const float2* src, const IcMul& mul, float2* dst,
                          cudaStream_t st);
 inline bool fft_compiled(const FftPlan& p) { return p.ops != nullptr; }

@@ -136,9 +136,12 @@ int launch_c2r_rows(const FftPlan& p, const Grid3& g, float2* const* data, int f
   return check_launch("c2r_rows");
 }
 
+bool ic_compiled(const FftPlan& p) { return p.ops && p.ops->ic_x; }
+bool x_mul_compiled(const FftPlan& p) { return p.ops && p.ops->x_mul; }
+
 int launch_pencils_x_mul(const FftPlan& p, const Grid3&, const float2* src, const IcMul& mul, float2* dst,
                          cudaStream_t st) {
-  if (!p.ops) return COLA_ERR_INVALID;
+  if (!x_mul_compiled(p)) return COLA_ERR_INVALID;
   p.ops->x_mul(src, mul, dst, p.tab, st);
   return check_launch("pencils_x_mul");
 }
@@ -150,7 +153,6 @@ int launch_c2r_rows_dense(const FftPlan& p, const Grid3&, const float2* data, fl
   return check_launch("c2r_dense");
 }
 
-bool ic_compiled(const FftPlan& p) { return p.ops && p.ops->ic_x; }
 
 int launch_ic_x(const FftPlan& p, const float2* in, float2* const* out, int fields, float scale, const float* amp_m2,
                 cudaStream_t st) {

@@ -58,8 +58,11 @@ struct Launch {
       else go(k_pen<N, 0, +1>, grid, C::T, C::smem, st, p, t.fwd);
     }
   }
+  // lattices up to 1024 (three tiles fit a CTA) have the fused 2LPT passes; only longer ones multiply field by field
+  static constexpr bool kIc = N <= 1024;
+  static_assert(!kIc || MultiCfg<N, 3>::smem <= 227 * 1024, "three tiles in a CTA");
   static void x_mul(const float2* src, const IcMul& mul, float2* dst, const FftTables& t, cudaStream_t st) {
-    go(k_pen_mul<N>, dim3(C::chunks, N), C::T, C::smem, st, src, dst, mul, t.fwd);
+    if constexpr (!kIc) go(k_pen_mul<N>, dim3(C::chunks, N), C::T, C::smem, st, src, dst, mul, t.fwd);
   }
   static void green(const float2* in, float2* out_f, float2* out_h, const float* dtab, float g_scale,
                     const FftTables& t, float2* spec_out, cudaStream_t st) {
@@ -71,8 +74,6 @@ struct Launch {
     go(k_pen_yz<N>, dim3(C::chunks, N), C::T, MultiCfg<N, 2>::smem, st, h, out_y, out_z, dtab, t.fwd);
   }
 
-  // three tiles in a CTA: the lattices up to 1024
-  static constexpr bool kIc = MultiCfg<N, 3>::smem <= 227 * 1024;
   static void ic_x(const float2* in, float2* const* out, int fields, float scale, const float* amp_m2,
                    const FftTables& t, cudaStream_t st) {
     if constexpr (kIc) {
@@ -128,8 +129,8 @@ template <int I>
 constexpr FftOps ops_of() {
   constexpr int N = kCtSizes[I];
   using L = Launch<N>;
-  return FftOps{N, L::r2c, L::c2r, L::c2r_dense, L::pencils, L::x_mul, L::green, L::kIc ? L::ic_x : nullptr, L::ic_y,
-                L::ic_z1, L::ic_z2, L::lpt_adj, L::grad_adj, L::pencils_yz};
+  return FftOps{N, L::r2c, L::c2r, L::c2r_dense, L::pencils, L::kIc ? nullptr : L::x_mul, L::green,
+                L::kIc ? L::ic_x : nullptr, L::ic_y, L::ic_z1, L::ic_z2, L::lpt_adj, L::grad_adj, L::pencils_yz};
 }
 constexpr int kMine = (kCtCount - COLA_CT_PART + COLA_CT_PARTS - 1) / COLA_CT_PARTS;
 template <int... K>

@@ -16,10 +16,10 @@ struct FftOps {
   void (*c2r)(float2* const* data, int fields, const FftTables&, cudaStream_t);
   void (*c2r_dense)(const float2* data, float scale, float* out, const FftTables&, cudaStream_t);
   void (*pencils)(int axis, int dir, float2* const* data, int fields, const FftTables&, cudaStream_t);
-  void (*x_mul)(const float2* src, const IcMul& mul, float2* dst, const FftTables&, cudaStream_t);
+  void (*x_mul)(const float2* src, const IcMul& mul, float2* dst, const FftTables&, cudaStream_t);   // null where ic_x is not
   void (*green)(const float2* in, float2* out_f, float2* out_h, const float* dtab, float g_scale, const FftTables&,
                 float2* spec_out, cudaStream_t);
-  // 2LPT fields (null where three tiles do not fit a CTA); see fft_ct.cuh
+  // 2LPT fields (ic_x is null, and none of these is called, above 1024); see fft_ct.cuh
   void (*ic_x)(const float2* in, float2* const* out, int fields, float scale, const float* amp_m2, const FftTables&,
                cudaStream_t);
   void (*ic_y)(const float2* in, float2* const* out, int fields, const int* zp, const FftTables&, cudaStream_t);
