@@ -196,16 +196,15 @@ int cola_power_spectrum(cola_ctx* ctx, const float* s, double* pk, int nbins);
  *                               _TILE_GATHER; _PIPE_INPLACE excludes _PIPE_EPT8 and a budget), kept and
  *                               reported, and select nothing.
  * cola_create picks a schedule from the sizes (the binned deposit and tile gather where the mesh is too
- * large for the direct deposit's atomics to stay in L2 and the tiles are dense enough); cola_get_schedule reads it and cola_set_schedule replaces it (COLA_ERR_INVALID for an
- * unavailable or malformed schedule).
+ * large for the direct deposit's atomics to stay in L2 and the tiles are dense enough); cola_get_schedule
+ * reads it and cola_set_schedule replaces it (COLA_ERR_INVALID for an unavailable or malformed schedule).
  * cola_autotune times `reps` PM force evaluations (deposit, FFTs, Poisson + gradient, gather) at
  * displacements s (device float32 [3][np^3]; an evolved state is representative, a lattice is not)
- * for the deposit/gather choices, the other bits unchanged.  It keeps the fastest, writes it to *best
- * (may be NULL), and writes the
- * schedules it timed and their milliseconds per evaluation, in timing order, to
- * scheds[0..max_candidates) and ms[0..max_candidates) (either may be NULL).  Returns the number of
- * schedules timed, or minus a cola_status.  It synchronises the stream and allocates a temporary
- * force array: call it outside graph capture. */
+ * for the deposit/gather choices, _PIPELINED_GATHER cleared and the other bits unchanged.  It keeps the
+ * fastest, writes it to *best (may be NULL), and writes the schedules it timed and their milliseconds
+ * per evaluation, in timing order, to scheds[0..max_candidates) and ms[0..max_candidates) (either may
+ * be NULL).  Returns the number of schedules timed, or minus a cola_status.  It synchronises the stream
+ * and allocates a temporary force array: call it outside graph capture. */
 #define COLA_SCHED_BINNED_DEPOSIT 1
 #define COLA_SCHED_TILE_GATHER 2
 #define COLA_SCHED_PIPELINED_FFT 4
@@ -272,8 +271,8 @@ int cola_grid_density_adjoint(cola_ctx* ctx, const float* s, int ngrid, const fl
  * run side by side as fit the L2 together (lanes beyond that would slow each other down), the
  * largest meshes first; among members of the same number of lanes, realisations are assigned to
  * lanes longest-first (cost ~ particles + mesh cells x log N) and run back to back on their lane.
- * cola_batch_run enqueues cola_run (2LPT + n_step PM steps +
- * P(k) in nbins bins) of every realisation, forked from and joined back into `stream`:
+ * cola_batch_run enqueues cola_run (2LPT + n_step PM steps + P(k) in nbins bins) of every realisation,
+ * forked from and joined back into `stream`:
  *   use_graph = 0 : plain launches;
  *   use_graph = 1 : the first call runs once eagerly (warm-up, then synchronises), captures the
  *                   whole launch sequence into a CUDA graph and launches it; later calls only

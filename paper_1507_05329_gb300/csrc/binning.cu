@@ -4,7 +4,7 @@
 // particles of one lattice plane are spread over tens of mesh planes (§2.3 mesh; displacements of
 // ~8 cells rms at a = 1 for the 0.78 Mpc/h cells of the 1536^3 mesh), so visiting them in lattice
 // order touches far more mesh than the L2 holds.  Each step therefore
-//   1. counts particles per tile of T x T x TZ mesh cells (T = 8 across, TZ = 32 along z) from the
+//   1. counts particles per tile of T x T x TZ mesh cells (T = 8 across, TZ = 64 along z) from the
 //      fixed-point base cell (the same integer cell as the deposit), with warp-aggregated atomics;
 //   2. scans the counts into offsets;
 //   3. scatters packed lattice coordinates into their tile's list.  A particle whose base cell
@@ -14,8 +14,8 @@
 //      particles that fall inside the tile in shared memory (64-bit integers, exact) and writes
 //      the whole tile once with plain stores: no clearing pass and no global atomics on the mesh;
 //   5. gathers the force and applies the kick and drift tile by tile (primary entries only): the
-//      CTA first copies the tile's force values with a one-cell halo ((T+1)^2 (TZ+1) x 3 floats,
-//      32 KB) into shared memory with coalesced loads, then interpolates from shared memory.  The
+//      CTA first copies the tile's force values with a one-cell halo ((T+1)^2 (TZ+1) x 3 floats in
+//      padded rows, 66 KB) into shared memory with coalesced loads, then interpolates from shared memory.  The
 //      tile index runs fastest along z, so neighbouring tiles (which share halos) run together.
 // The order of particles inside a tile's list depends on atomic timing, but neither result does:
 // integer sums are order independent and every particle's gather is computed on its own.
@@ -509,10 +509,10 @@ constexpr int kHx = kT + 1, kHp = (kTz + 1 + 3) & ~3;
 constexpr int kGatherFloats = 3 * kHx * kHx * kHp;
 constexpr int kBulkWaitLimit = 1 << 22;   // polls of the staging barrier before the CTA gives up
 
-// Stage a tile's forces: one cp.async.bulk of the tile's z extent (32 cells, fewer in the last tile; a
+// Stage a tile's forces: one cp.async.bulk of the tile's z extent (64 cells, fewer in the last tile; a
 // multiple of 4: the mesh side is, where this kernel runs) per force row, all completing on the mbarrier
 // at bar_sa, plus each row's periodic halo cell by a 4-byte cp.async (committed as one group).  Rows start
-// 16-byte aligned (z0 a multiple of 32, rows of 2 pc floats with pc even).  Called by every thread of the
+// 16-byte aligned (z0 a multiple of 64, rows of 2 pc floats with pc even).  Called by every thread of the
 // block; contains a barrier.
 __device__ __forceinline__ void gather_stage(float* fsm, unsigned bar_sa, int nm, int x0, int y0, int z0,
                                              const float* f0, const float* f1,

@@ -38,7 +38,15 @@ double realisation_cost(const cola_params& p) {
 // Eight equal members of two steps in a graph, microseconds with 1 / 2 / 4 / 8 lanes (126 MB of L2):
 // 64^3 723 / 422 / 290 / 216, 96^3 1294 / 828 / 647 / 703, 128^3 1764 / 1399 / 1500 / 1691,
 // 192^3 4647 / 5144 / 5795 / 5855, 256^3 9199 / 8737 / 9604 / 9843, 320^3 18259 / 17986 / 19685 / 20126;
-// four of 192^3 with 192^3 particles 7315 / 10097 / 10211.
+// four of 192^3 with 192^3 particles 7315 / 10097 / 10211.  Denser lattices have no term of their own, since the
+// same widths suit them: eight with as many particles as cells, 64^3 1082 / 766 / 569 / 527, 96^3 2313 / 1912 /
+// 1843 / 1869 (on the rule's 5), 128^3 4474 / 4255 (the rule's 2).
+// Two lanes would suit a group of 256^3 alone (5%; 320^3 1% either way in two measurements), but then one of
+// 256^3 shares a group with the 128^3 ones: beside seven of them 2610 against 2442.  Groups wait for one another,
+// because a large member beside small ones mostly loses more than they overlap.  This rule / without the wait /
+// every member on any of 8 lanes: one of 320^3 and fifteen of 64^3 2693 / 2843 / 2840, one of 256^3 and seven of
+// 128^3 2442 / 2597 / 2630, four of 192^3 and sixteen of 64^3 2760 / 2761 / 3405, two of 320^3, four of 192^3,
+// eight of 128^3 and sixteen of 64^3 8719 / 9030 / 9730, six of 128^3 and twenty-four of 32^3 2048 / 1910 / 4342.
 int lane_width(int n, int l2_bytes, int lanes) {
   const double fit = (double)l2_bytes / (28.0 * n * n * n);
   return (int)std::min((double)lanes, std::max(1.0, std::floor(fit)));

@@ -15,10 +15,11 @@ namespace cola {
 // dependent launch): the kernel must begin with after_previous(), which waits until that one has completed
 // and its writes are visible.  No kernel lets its successor in before its own blocks have ended (with an
 // early release the successor's waiting blocks took the last wave's resources: 512^3/768^3 steps 4%
-// slower).  A kernel reads what the previous one may have written with plain loads only: neither __ldg nor
-// a const __restrict__ pointer, which the compiler may read ahead of the wait; tables written once (twiddles,
-// wave numbers, amplitudes) keep them.  Before -> after: 32^3/64^3 realisation of two steps 150 -> 85 us,
-// 96^3/192^3 step 264 -> 242, adjoint 64^3/128^3 2218 -> 1716, P(k) 128^3/256^3 303 -> 275.
+// slower).  A kernel reads what the previous one may have written with plain or streaming (__ldcs) loads, which
+// stay behind the wait: neither __ldg nor a const __restrict__ pointer, which the compiler may read ahead of
+// it; tables written once (twiddles, wave numbers, amplitudes) keep them.  Before -> after: 32^3/64^3
+// realisation of two steps 150 -> 85 us, 96^3/192^3 step 264 -> 242, adjoint 64^3/128^3 2218 -> 1716, P(k)
+// 128^3/256^3 303 -> 275.
 template <class... P, class... A>
 inline void launch_after(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A&&... args) {
   cudaLaunchAttribute attr{};
@@ -293,7 +294,7 @@ int launch_gather(const ParticleGeom& pg, const float* const f[3], long long rs,
                   float* force_out, float* s, float* v, const float* psi1, const float* psi2,
                   const KickDrift* kd, int* flags, cudaStream_t st);
 
-// Spatial binning by tiles of 8 x 8 x 32 mesh cells (binning.cu).
+// Spatial binning by tiles of 8 x 8 x 64 mesh cells (binning.cu).
 struct BinGeom {
   int nt;      // tiles per axis across z
   int nz;      // tiles along z

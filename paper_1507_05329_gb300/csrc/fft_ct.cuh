@@ -4,9 +4,10 @@
 //
 // Every pass reads a tile of pencils from HBM once, runs the groups of the length's plan (fft_plan.h) on
 // it through shared memory and writes it once; the first group loads straight from HBM and the last
-// stores straight to it.  Strided passes (y, x) take tiles of 8 adjacent columns (64-byte row segments; 4 beyond 1536),
-// lanes running over the columns first; the contiguous passes (z) take pairs of real rows as complex
-// rows, lanes running along the row, so that their global accesses are whole 128-byte lines.
+// stores straight to it.  Strided passes (y, x) take tiles of 8 adjacent columns (64-byte row segments; 16
+// from 144 to 320 points, 4 beyond 1536: PenCfg), lanes running over the columns first; the contiguous passes
+// (z) take pairs of real rows as complex rows, lanes running along the row, so that their global accesses are
+// whole 128-byte lines.
 #pragma once
 #include "fft_core.cuh"
 #include "fft_plan.h"

@@ -34,8 +34,9 @@ struct FftOps {
 
 namespace ct {
 
-// Every even length 2^a 3^b 5^c from 18 to 1024, and the longer ones whose tile of 8 columns fits a CTA
-// in few stages: the meshes and lattices in use.  Other lengths take the run-time plans of fft_generic.cu.
+// Every even length 2^a 3^b 5^c from 18 to 1024, and of the longer ones the mesh sides in use: 1280, 1536 and
+// 2048.  Each length costs build time, not speed, so the other long ones (1080 to 2000, of which those up to 1500
+// would hold a tile of 8 columns just as well) and the shortest take the run-time plans of fft_generic.cu.
 #ifdef COLA_CT_TEST_SIZES
 constexpr int kCtSizes[] = {COLA_CT_TEST_SIZES};
 #else

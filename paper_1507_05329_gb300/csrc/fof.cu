@@ -24,7 +24,8 @@ namespace cola {
 namespace {
 
 constexpr int kFlagIterations = 4;   // union-find did not converge (never expected; reported)
-// 649 us at 128^3/256^3 with 8 cells per particle; 741 with 27, 971 with 64 (clearing and scanning them).
+// Kernel time of a call at 128^3/256^3: 649 us with 8 cells per particle; 741 with 27, 971 with 64 (clearing and
+// scanning them).
 constexpr double kCellsPerParticle = 8.0;
 
 int check_launch(const char* what) {
@@ -206,7 +207,7 @@ __global__ void __launch_bounds__(256) k_fof_first(int n, const uint4* rec, cons
 // in a dense halo, where a record has hundreds of friends, they are passed over by the root that comes
 // with their coordinates.  (In lattice order, 27 cells of side l looked up one by one, 134 M of them, and
 // two root searches for every friend, 128^3/256^3 at b = 0.2 took 1225 us for the links and 1240 us for
-// scanning the cells; in sorted order with one pass 1000 and 40; now 280 for both passes.)
+// scanning the cells; in sorted order with one pass 1000 and 40; now 280 to 340 for both passes.)
 template <bool ONE>
 __global__ void __launch_bounds__(256) k_fof_link(int n, const uint4* rec, const unsigned* off,
                                                   FofGeom f, int* parent, int* flags) {
